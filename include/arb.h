@@ -289,7 +289,7 @@ arb_status arb_rollback(arb_ctx *ctx, int32_t batch, int32_t *seq_lens, const in
  *   decisions  uint8 [n_steps]: 1 = escalate to the target, 0 = keep the draft step.  Ties: RSD escalates
  *              at s_d == tau; the oracle rules keep the draft at Delta == tau / s_t == s_d; among equal
  *              advantages the budgeted rule takes the lower index first.
- *   stats      nullable; zeroed on `stream`, then filled by the kernel (sums in fp64).
+ *   stats      nullable; overwritten by the kernel (sums in fp64).
  * Delta and every comparison are taken in fp32 (IEEE subtraction, no flush to zero).
  * Errors: ARB_ERR_INVALID_ARG (null pointer, unknown kind, s_t missing), ARB_ERR_UNSUPPORTED (budgeted
  * rule beyond 65536 steps).

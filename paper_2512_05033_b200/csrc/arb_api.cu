@@ -149,7 +149,8 @@ arb_status arb_create(arb_ctx **out, int device, size_t workspace_bytes) {
     const size_t rot_ints = (size_t)kRotSets * kRotCounters + kRotSets + 8;
     ok = ok && guarded_malloc(c, &c->rot, sizeof(int) * rot_ints);
     ok = ok && cudaMemset(c->rot, 0, sizeof(int) * rot_ints) == cudaSuccess;
-    ok = ok && guarded_malloc(c, &c->spearman_acc, 4 * sizeof(double));
+    ok = ok && guarded_malloc(c, &c->rank_ws, rank_ws_bytes());
+    ok = ok && cudaMemset(c->rank_ws, 0, 256) == cudaSuccess;
     c->chunk_ws_bytes = 2 * c->workspace_bytes;   // partials of long step chunks that are split over their keys
     ok = ok && guarded_malloc(c, &c->chunk_ws, c->chunk_ws_bytes);
     ok = ok && guarded_malloc(c, &c->step_hint, decode_step_hint_bytes(sms));
@@ -168,7 +169,7 @@ arb_status arb_create(arb_ctx **out, int device, size_t workspace_bytes) {
         guarded_free(c->workspace);
         guarded_free(c->counters);
         guarded_free(c->rot);
-        guarded_free(c->spearman_acc);
+        guarded_free(c->rank_ws);
         guarded_free(c->chunk_ws);
         guarded_free(c->step_hint);
         cudaFree(c->guards_dev);
@@ -189,7 +190,7 @@ arb_status arb_destroy(arb_ctx *ctx) {
     guarded_free(c->workspace);
     guarded_free(c->counters);
     guarded_free(c->rot);
-    guarded_free(c->spearman_acc);
+    guarded_free(c->rank_ws);
     guarded_free(c->chunk_ws);
     guarded_free(c->step_hint);
     cudaFree(c->guards_dev);

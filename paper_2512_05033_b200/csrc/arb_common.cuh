@@ -62,7 +62,8 @@ struct Ctx {
     int *rot = nullptr;
     uint32_t decode_gen = 1000;          // generation of the next tensor-core decode call
     uint32_t rot_wait_through = 0;        // tensor-core decode calls up to this generation wait for their predecessor
-    double *spearman_acc = nullptr;       // three fp64 accumulators of arb_spearman
+    char *rank_ws = nullptr;              // arb_policy, arb_spearman: two arrival counters (zero between calls), then at 256 the
+                                          // statistics of a policy's CTAs and the ranks of two samples
     int *step_hint = nullptr;             // single-launch decode: the page tiles each CTA streamed last (arb_decode_step.cu)
     int step_min_chunk = 16;              // single-launch decode: fewest pages worth giving a CTA
     int step_boundary_pct = 100;          // single-launch decode: what a (sequence, kv head) boundary inside a CTA's range counts for
@@ -75,6 +76,8 @@ struct Ctx {
     const unsigned char **guards_dev = nullptr;
     unsigned long long *guard_bad = nullptr;
 };
+
+constexpr size_t kPolicyPartBytes = 8192;   // of rank_ws: the statistics of a policy's CTAs
 
 constexpr int kRotSets = 4;
 constexpr int kRotCounters = 1 << 16;
@@ -317,6 +320,9 @@ arb_status launch_phase_lens(Ctx *ctx, int batch, const int32_t *step_lens, cons
 arb_status launch_phase_lens_tokens(Ctx *ctx, int batch, const int32_t *step_lens, const uint8_t *decisions, int want,
                                     int n_tokens, int32_t *out, cudaStream_t stream);
 arb_status launch_spearman(Ctx *ctx, int n, const float *x, const float *y, double *rho, cudaStream_t stream);
+size_t rank_ws_bytes();
+arb_status launch_policy_budget(Ctx *ctx, int n, const float *s_d, const float *s_t, int budget, uint8_t *decisions,
+                                arb_policy_stats *stats, cudaStream_t stream);
 arb_status launch_policy(Ctx *ctx, int kind, int n_steps, const float *s_d, const float *s_t, float tau, int budget,
                          uint8_t *decisions, arb_policy_stats *stats, cudaStream_t stream);
 arb_status launch_route_classes(Ctx *ctx, int dtype, int mode, int n_steps, int hidden_dim, int n_classes,

@@ -4,10 +4,7 @@
 //   RSD baseline (Section 3.1 of the paper): the step is accepted iff s_d > tau, so escalated iff s_d <= tau.
 //   Oracle threshold (Section 4.1): escalate iff Delta = s_t - s_d > tau.
 //   Oracle arg max (Section 4.1): keep the higher-scoring step; escalate iff s_t > s_d.
-//   Budgeted oracle (Appendix B, Theorem): escalate the min(budget, #{Delta > 0}) steps with the largest
-//   positive Delta; equal advantages go to the lower index.  Done by counting, not sorting: step i's
-//   rank is the number of steps that come before it in (Delta descending, index ascending) order, and
-//   every thread finds its own rank against tiles of Delta staged in shared memory.
+//   Budgeted oracle (Appendix B, Theorem): needs an order over the steps, see arb_rank.cu.
 // Each kernel also accumulates the escalation count, the wasted escalations of Section 3.2 (escalated
 // although s_t <= s_d), the realised score sum_i (a_i ? s_t : s_d) and the gain sum_i a_i (s_t - s_d).
 // Delta is one fp32 subtraction, not flushed to zero for subnormal results, so that the decision is
@@ -16,11 +13,6 @@
 // C-way heads (Section 6.1, ablation): one warp per step computes the C logits (softmax head) or one
 // logit against C - 1 ordered cut points (ordinal head), the class probabilities, the expected class
 // level scaled to [0, 1] as the routing score, and the threshold decision (a tie accepts).
-//
-// Spearman's rho (the rank correlation the paper reports between router scores and the oracle advantage,
-// Section 4.2 "Evaluation" and Tables 1-3): ranks by counting -- rank_i = #{x_j < x_i} + (#{x_j = x_i} + 1) / 2,
-// ties sharing the mean of the ranks they span -- for both samples in one pass over shared-memory tiles,
-// then the three centred sums of the Pearson formula in fp64 and a one-thread kernel for the quotient.
 #include "arb_common.cuh"
 
 namespace arb {
@@ -28,6 +20,7 @@ namespace arb {
 namespace {
 
 constexpr int kPolicyThreads = 256;
+constexpr int kPolicyMaxCtas = 256;
 
 __device__ __forceinline__ float sub_ieee(float a, float b) {
     float r;
@@ -35,114 +28,76 @@ __device__ __forceinline__ float sub_ieee(float a, float b) {
     return r;
 }
 
-// block-wide sums of the four statistics, then one atomic each
-__device__ __forceinline__ void add_stats(arb_policy_stats *stats, unsigned esc, unsigned wasted, double realised,
-                                          double gain) {
-    __shared__ unsigned s_esc[kPolicyThreads / 32], s_wst[kPolicyThreads / 32];
-    __shared__ double s_real[kPolicyThreads / 32], s_gain[kPolicyThreads / 32];
+// block-wide sums of the four statistics, in thread 0
+__device__ __forceinline__ void block_stats(arb_policy_stats &v) {
+    __shared__ arb_policy_stats part[kPolicyThreads / 32];
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) {
-        esc += __shfl_xor_sync(0xffffffffu, esc, off);
-        wasted += __shfl_xor_sync(0xffffffffu, wasted, off);
-        realised += __shfl_xor_sync(0xffffffffu, realised, off);
-        gain += __shfl_xor_sync(0xffffffffu, gain, off);
+        v.escalated += __shfl_xor_sync(0xffffffffu, v.escalated, off);
+        v.wasted += __shfl_xor_sync(0xffffffffu, v.wasted, off);
+        v.realised += __shfl_xor_sync(0xffffffffu, v.realised, off);
+        v.gain += __shfl_xor_sync(0xffffffffu, v.gain, off);
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) { s_esc[warp] = esc; s_wst[warp] = wasted; s_real[warp] = realised; s_gain[warp] = gain; }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < kPolicyThreads / 32; ++w) {
-            esc += s_esc[w]; wasted += s_wst[w]; realised += s_real[w]; gain += s_gain[w];
+            v.escalated += part[w].escalated;
+            v.wasted += part[w].wasted;
+            v.realised += part[w].realised;
+            v.gain += part[w].gain;
         }
-        if (esc) atomicAdd(&stats->escalated, esc);
-        if (wasted) atomicAdd(&stats->wasted, wasted);
-        atomicAdd(&stats->realised, realised);
-        atomicAdd(&stats->gain, gain);
     }
 }
 
+// One launch, statistics included: every CTA leaves its sums, the last to finish adds them up in CTA order (so the
+// same scores give the same bits).  Launch-bound at the sizes of a split; with the statistics zeroed by a copy engine
+// and added by fp64 atomics it was two stream operations, and the sums came out in any order.
 __global__ void __launch_bounds__(kPolicyThreads)
-policy_kernel(int kind, int n, const float *__restrict__ s_d, const float *__restrict__ s_t, float tau, int budget,
-              uint8_t *__restrict__ decisions, arb_policy_stats *stats) {
-    __shared__ float tile[kPolicyThreads];
-    const int i = blockIdx.x * kPolicyThreads + threadIdx.x;
-    const bool live = i < n;
-    const float sd = live ? s_d[i] : 0.f;
-    const float st = (live && s_t != nullptr) ? s_t[i] : sd;
-    const float delta = sub_ieee(st, sd);
-    int a = 0;
-    if (kind == ARB_POLICY_RSD) {
-        a = live && !(sd > tau);
-    } else if (kind == ARB_POLICY_ORACLE_THRESHOLD) {
-        a = live && delta > tau;
-    } else if (kind == ARB_POLICY_ORACLE_ARGMAX) {
-        a = live && st > sd;
-    } else {
-        // rank of step i in (Delta descending, index ascending) order; uniform trip count per block
-        int rank = 0;
-        for (int j0 = 0; j0 < n; j0 += kPolicyThreads) {
-            const int j = j0 + threadIdx.x;
-            __syncthreads();
-            tile[threadIdx.x] = j < n ? sub_ieee(s_t[j], s_d[j]) : -INFINITY;
-            __syncthreads();
-            const int m = min(kPolicyThreads, n - j0);
-            for (int k = 0; k < m; ++k) {
-                const float dj = tile[k];
-                rank += (dj > delta) || (dj == delta && j0 + k < i);
-            }
-        }
-        a = live && delta > 0.f && rank < budget;
+policy_kernel(int kind, int n, const float *__restrict__ s_d, const float *__restrict__ s_t, float tau,
+              uint8_t *__restrict__ decisions, arb_policy_stats *stats, arb_policy_stats *part, int *done) {
+    __shared__ int last;
+    arb_policy_stats v = {0u, 0u, 0.0, 0.0};
+    for (int i = blockIdx.x * kPolicyThreads + threadIdx.x; i < n; i += (int)gridDim.x * kPolicyThreads) {
+        const float sd = s_d[i];
+        const float st = s_t != nullptr ? s_t[i] : sd;
+        bool a;
+        if (kind == ARB_POLICY_RSD) a = !(sd > tau);
+        else if (kind == ARB_POLICY_ORACLE_THRESHOLD) a = sub_ieee(st, sd) > tau;
+        else a = st > sd;
+        decisions[i] = a ? 1 : 0;
+        v.escalated += a;
+        v.wasted += a && !(st > sd);
+        v.realised += (double)(a ? st : sd);
+        v.gain += a ? (double)st - (double)sd : 0.0;
     }
-    if (live) decisions[i] = (uint8_t)a;
-    if (stats != nullptr) {   // uniform: every thread of the block takes part in the reduction
-        const bool w = a && !(st > sd);
-        add_stats(stats, (unsigned)a, (unsigned)w, live ? (double)(a ? st : sd) : 0.0,
-                  a ? (double)st - (double)sd : 0.0);
-    }
-}
-
-__global__ void __launch_bounds__(kPolicyThreads)
-spearman_rank_kernel(int n, const float *__restrict__ x, const float *__restrict__ y, double *__restrict__ acc) {
-    __shared__ float xs[kPolicyThreads], ys[kPolicyThreads];
-    __shared__ double red[3][kPolicyThreads / 32];
-    const int i = blockIdx.x * kPolicyThreads + threadIdx.x;
-    const bool live = i < n;
-    const float xi = live ? x[i] : 0.f, yi = live ? y[i] : 0.f;
-    int lx = 0, ex = 0, ly = 0, ey = 0;
-    for (int j0 = 0; j0 < n; j0 += kPolicyThreads) {
-        const int j = j0 + threadIdx.x;
-        __syncthreads();
-        xs[threadIdx.x] = j < n ? x[j] : 0.f;
-        ys[threadIdx.x] = j < n ? y[j] : 0.f;
-        __syncthreads();
-        const int m = min(kPolicyThreads, n - j0);
-        for (int k = 0; k < m; ++k) {
-            lx += xs[k] < xi; ex += xs[k] == xi;
-            ly += ys[k] < yi; ey += ys[k] == yi;
-        }
-    }
-    const double mean = ((double)n + 1.0) * 0.5;
-    const double dx = live ? (double)lx + ((double)ex + 1.0) * 0.5 - mean : 0.0;
-    const double dy = live ? (double)ly + ((double)ey + 1.0) * 0.5 - mean : 0.0;
-    double v[3] = {dx * dy, dx * dx, dy * dy};
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-        if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = v[q];
+    if (stats == nullptr) return;
+    block_stats(v);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = v;
+        __threadfence();
+        last = atomicAdd(done, 1) == (int)gridDim.x - 1;
     }
     __syncthreads();
-    if (threadIdx.x < 3) {
-        double t = 0.0;
-        for (int w = 0; w < kPolicyThreads / 32; ++w) t += red[threadIdx.x][w];
-        atomicAdd(&acc[threadIdx.x], t);
+    if (!last) return;
+    __threadfence();
+    v = {0u, 0u, 0.0, 0.0};
+    if (threadIdx.x < gridDim.x) {   // kPolicyMaxCtas == kPolicyThreads: at most one record per thread
+        const arb_policy_stats *p = part + threadIdx.x;
+        v.escalated = __ldcg(&p->escalated);
+        v.wasted = __ldcg(&p->wasted);
+        v.realised = __ldcg(&p->realised);
+        v.gain = __ldcg(&p->gain);
+    }
+    block_stats(v);
+    if (threadIdx.x == 0) {
+        *stats = v;
+        *done = 0;
     }
 }
-
-__global__ void spearman_finish_kernel(int n, const double *__restrict__ acc, double *__restrict__ rho) {
-    const double sxy = acc[0], sxx = acc[1], syy = acc[2];
-    *rho = (n < 2 || !(sxx > 0.0) || !(syy > 0.0)) ? __longlong_as_double(0x7ff8000000000000ll) : sxy / sqrt(sxx * syy);
-}
+static_assert(kPolicyMaxCtas <= kPolicyThreads, "one record per thread of the last CTA");
+static_assert(kPolicyMaxCtas * sizeof(arb_policy_stats) <= kPolicyPartBytes, "the records of a call");
 
 constexpr int kHeadWarps = 4;
 
@@ -249,20 +204,12 @@ route_classes_kernel(const HeadArgs a) {
 
 arb_status launch_policy(Ctx *ctx, int kind, int n_steps, const float *s_d, const float *s_t, float tau, int budget,
                          uint8_t *decisions, arb_policy_stats *stats, cudaStream_t stream) {
-    if (stats != nullptr && cudaMemsetAsync(stats, 0, sizeof(arb_policy_stats), stream) != cudaSuccess) return ARB_ERR_CUDA;
-    const int grid = (n_steps + kPolicyThreads - 1) / kPolicyThreads;
-    policy_kernel<<<grid, kPolicyThreads, 0, stream>>>(kind, n_steps, s_d, s_t, tau, budget, decisions, stats);
-    ctx->launches++;
-    return cudaGetLastError() == cudaSuccess ? ARB_OK : ARB_ERR_CUDA;
-}
-
-arb_status launch_spearman(Ctx *ctx, int n, const float *x, const float *y, double *rho, cudaStream_t stream) {
-    if (cudaMemsetAsync(ctx->spearman_acc, 0, 3 * sizeof(double), stream) != cudaSuccess) return ARB_ERR_CUDA;
-    if (n > 0) {
-        spearman_rank_kernel<<<(n + kPolicyThreads - 1) / kPolicyThreads, kPolicyThreads, 0, stream>>>(n, x, y, ctx->spearman_acc);
-        ctx->launches++;
-    }
-    spearman_finish_kernel<<<1, 1, 0, stream>>>(n, ctx->spearman_acc, rho);
+    if (kind == ARB_POLICY_ORACLE_BUDGET) return launch_policy_budget(ctx, n_steps, s_d, s_t, budget, decisions, stats, stream);
+    const int need = (n_steps + kPolicyThreads - 1) / kPolicyThreads;
+    const int grid = need < kPolicyMaxCtas ? need : kPolicyMaxCtas;
+    policy_kernel<<<grid, kPolicyThreads, 0, stream>>>(kind, n_steps, s_d, s_t, tau, decisions, stats,
+                                                       reinterpret_cast<arb_policy_stats *>(ctx->rank_ws + 256),
+                                                       reinterpret_cast<int *>(ctx->rank_ws) + 1);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? ARB_OK : ARB_ERR_CUDA;
 }

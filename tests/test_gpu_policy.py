@@ -221,3 +221,30 @@ def test_quantising_append_matches_oracle(dtype, D):
     assert st == 0 and c.poll_status() == 0
     assert torch.equal(dk.cpu(), k_ref) and torch.equal(dv.cpu(), v_ref)          # codes: bit-exact
     assert np.array_equal(dseq.cpu().numpy(), sl_ref)
+
+
+@pytest.mark.parametrize("n", [1, 1024, 8193, 65536])
+@pytest.mark.parametrize("levels", [0, 3])
+def test_ranks_and_budget_at_the_edges_of_the_cluster(n, levels):
+    """One cluster of eight CTAs holds 8 * 2^k values: sizes around its capacities, all values distinct (levels 0)
+    and three levels (runs of equals across every CTA).  Decisions and counters are whole numbers; rho is a
+    quotient of exact integer sums on both sides, so a few units of 2^-53."""
+    import math
+    from paper_2512_05033_b200 import binding
+    c = H.ctx()
+    g = torch.Generator().manual_seed(n + levels)
+    sd, st = torch.rand(n, generator=g), torch.rand(n, generator=g)
+    if levels:
+        sd, st = torch.zeros(n), (torch.randint(0, levels, (n,), generator=g) + 1).float() / 4
+    stats = c.new_policy_stats("cuda")
+    for budget in (0, 1, n // 3 + 1, n - 1, n, 2 * n):
+        dec = c.policy(binding.POLICY_ORACLE_BUDGET, sd.cuda(), st.cuda(), budget=budget, stats=stats)
+        got, (ref, rs) = c.policy_stats(stats), oracle.policy(binding.POLICY_ORACLE_BUDGET, sd, st, budget=budget)
+        assert np.array_equal(dec.cpu().numpy(), ref), budget
+        assert (got["escalated"], got["wasted"]) == (rs["escalated"], rs["wasted"])
+        assert abs(got["realised"] - rs["realised"]) <= 1e-9 * max(1.0, abs(rs["realised"]))
+    y = torch.randn(n, generator=g)
+    y[: n // 2] = -0.0 if levels else y[: n // 2]
+    ref, rho = oracle.spearman(st, y), float(c.spearman(st.cuda(), y.cuda()).item())
+    assert (math.isnan(ref) and math.isnan(rho)) or abs(ref - rho) <= 1e-12, (rho, ref)
+    assert c.poll_status() == 0
