@@ -363,7 +363,7 @@ arb_status arb_kv_append(arb_ctx *ctx, const arb_attn_params *params, int32_t to
  * untouched (pools, length), its out row is zero-filled and ARB_DEV_BAD_SEQ_LEN is raised; a sequence whose
  * new row would land on a page outside the pool keeps its length and pools, raises ARB_DEV_BAD_PAGE, and its
  * out row is unspecified but finite-safe (as for arb_attn).  q_lens other than 0 and 1 count as 0 with the
- * status bit.  bf16 / head_dim 128 / g <= 8 run as one kernel; other shapes as the two calls above.
+ * status bit.  bf16 runs as one kernel, fp32 as the two calls above.
  * Asynchronous on `stream`; launched as a programmatic dependent of the kernel before it (it touches no
  * memory before that kernel has completed, so this is safe behind any kernel).
  */

@@ -232,7 +232,7 @@ arb_status arb_attn(arb_ctx *ctx, const arb_attn_params *params, const void *q, 
     const bool maybe_decode = params->max_q_len == 1 || params->total_q > params->max_q_len;
     const bool tensor_cores = (params->flags & ARB_ATTN_NO_TENSOR_CORES) == 0;
     if (maybe_decode) {
-        // bf16 / head_dim 128: a call that is one of a back-to-back series (ARB_ATTN_OVERLAP_PREVIOUS) takes the
+        // bf16: a call that is one of a back-to-back series (ARB_ATTN_OVERLAP_PREVIOUS) takes the
         // two-kernel form, whose calls stream under one another's tails; a call on its own takes the single
         // launch, which is what finishes a lone call soonest.
         const bool series = (params->flags & ARB_ATTN_OVERLAP_PREVIOUS) != 0;
@@ -248,9 +248,8 @@ arb_status arb_attn(arb_ctx *ctx, const arb_attn_params *params, const void *q, 
         if (st != ARB_OK) return st;
     }
     if (params->max_q_len >= 2) {
-        // Step chunks: bf16 chunks of head_dim 128 go to the tcgen05 kernel (from kChunkMmaMinRows
-        // rows on, i.e. all of them); the rest, and every fp32 chunk, to the CUDA-core kernel.  Both
-        // kernels decide per sequence on the device.
+        // Step chunks: bf16 chunks go to the tcgen05 kernel (from kChunkMmaMinRows rows on, i.e. all of them),
+        // fp32 chunks to the CUDA-core kernel.  Both kernels decide per sequence on the device.
         int skip_rows = 0;
         if (tensor_cores && chunk_mma_supported(*params)) {
             st = launch_chunk_mma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
@@ -283,7 +282,7 @@ arb_status arb_decode_step(arb_ctx *ctx, const arb_attn_params *params, const vo
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if ((params->flags & ARB_ATTN_NO_TENSOR_CORES) == 0 && decode_step_supported(*params))
         return launch_decode_step(c, *params, q, k_new, v_new, k_pages, v_pages, nullptr, block_table, seq_lens, q_lens, out, s);
-    // shapes the single launch does not serve (fp32, head_dim 64): the same step as two launches
+    // what the single launch does not serve (fp32): the same step as two launches
     st = launch_kv_append(c, *params, params->total_q, k_new, v_new, block_table, seq_lens, q_lens, 1, k_pages, v_pages, s);
     if (st != ARB_OK) return st;
     note_unnumbered_decode(c, decode_workspace_bytes(*params, c->num_sms));

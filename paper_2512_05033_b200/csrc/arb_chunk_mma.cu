@@ -1,4 +1,4 @@
-// Step-chunk attention on the 5th-generation tensor cores (tcgen05 + TMEM), bf16, head_dim 128.
+// Step-chunk attention on the 5th-generation tensor cores (tcgen05 + TMEM), bf16, head_dim 128 or 64.
 //
 // A chunk of n query tokens against one KV head is a contraction over shared operands: the
 // M = n * group query rows (token-major, the group's heads of one token are consecutive rows) all read
@@ -15,7 +15,7 @@
 //     O += P V       tcgen05.mma with P as the TMEM A operand and the V tile read MN-major straight
 //                    from its page layout; fp32 accumulator in the group's 128 TMEM columns for O
 //
-// TMEM: S 0-127 (one region for both groups), P_A 128-191, P_B 192-255, O_A 256-383, O_B 384-511.  The
+// TMEM at head_dim 128: S 0-127 (one region for both groups), P_A 128-191, P_B 192-255, O_A 256-383, O_B 384-511.  The
 // work of an item is a sequence of units (one group on one KV tile; the groups alternate).  S of a unit is
 // wanted only until its group holds it in registers, so one S region serves both groups, and with P in
 // columns of its own the next unit's Q K^T runs under this unit's exponentials: a softmax group goes from
@@ -46,11 +46,9 @@ namespace arb {
 
 namespace {
 
-constexpr int kD = 128;           // head_dim
 constexpr int kBM = 128;          // query rows per row tile; a work item is a pair of row tiles
 constexpr int kBN = 128;          // keys per KV tile
 constexpr int kTilePages = kBN / kPage;
-constexpr int kStages = 2;
 constexpr int kSoftmaxThreads = 128;        // per row tile
 constexpr int kThreads = 3 * kSoftmaxThreads;   // two softmax groups and a group of service warps; registers are
                                                 // handed out per 128 threads, so the third group's spare warps cost none
@@ -66,15 +64,13 @@ constexpr int kWideners = 3;                      // warps per operand in the E4
 static_assert(kWideners == 3 && kWideners <= 4, "a slot per widening warp; every warp has a pair in every full tile");
 __host__ __device__ constexpr int threads_of(bool e4m3) { return e4m3 ? 4 * kSoftmaxThreads : kThreads; }
 constexpr int kHalfBytes = 128 * 128;      // [128 rows x 64 bf16]: one 128-byte-swizzled half tile
-constexpr int kTileBytes = 2 * kHalfBytes;  // [128 x 128] bf16
 constexpr int kBoxBytes = kPage * 128;      // one TMA box: 16 rows x 64 bf16
 constexpr int kStagePages = 6;              // E4M3: pages of codes in flight per operand ...
 constexpr int kStagePairs = kStagePages / 2;   // ... asked for, waited for and widened two at a time
 constexpr int kTilePairs = kTilePages / 2;
-constexpr int kCodePageBytes = kPage * kD;  // 2 KB: one (page, kv head) tile of codes
-constexpr uint32_t kTmemCols = 512;         // S (shared): columns 0..127, P of group A: 128..191, of B: 192..255,
-constexpr uint32_t kPCol = 128;             // O of group A: 256..383, of B: 384..511
-constexpr uint32_t kOCol = 256;
+constexpr int kCodePageBytes = kPage * 128; // 2 KB: one (page, kv head) tile of codes
+constexpr uint32_t kTmemCols = 512;         // S (shared): columns 0..127; then P of group A, P of B, O of A, O of B
+constexpr uint32_t kPCol = 128;
 constexpr float kRescaleThreshold = 8.0f;   // log2 units
 constexpr int kItemSlots = 8;               // work items announced ahead of their use
 constexpr int kPrefetchTiles = 4;            // K/V tiles asked into L2 ahead of the ring
@@ -91,8 +87,27 @@ constexpr int kSplitMaxParts = 32;          // a warp's lanes cover the parts in
 // sequences of at least kFillMinTiles tiles.
 constexpr int kFillMinTiles = 8;
 constexpr int kFillPartTiles = 4;
-constexpr size_t kSlotFloats = (size_t)kBM * kD + 2 * kBM;   // one row tile's partial: O as [32 groups of 4 dims][128 rows][4],
-                                                             // so that the rows' 16-byte pieces lie side by side; then (max, sum) [128][2]
+// one row tile's partial: O as [groups of 4 dims][128 rows][4], so that the rows' 16-byte pieces lie side by side; then
+// (max, sum) [128][2]
+__host__ __device__ constexpr size_t slot_floats(int head_dim) { return (size_t)kBM * head_dim + 2 * kBM; }
+
+// What depends on the head dimension.  64-dimension heads: half the bytes per tile, so twice the ring stages; and TMEM has
+// room for P as two bf16 terms (p = hi + lo, 16 significant bits): the second product is run for both.  The MMAs of an HD = 64
+// unit take half the tensor time, so the second term is hidden under the exponentials, and the weights keep what the
+// CUDA-core kernel that served these chunks before kept (fp32, far below the rounding of the output).  Measured: the
+// step-scoring batch with 64-dimension heads 14.1 ms -> 0.42 ms, a batch of 16 short steps over 1k-8k keys 1.33 ms -> 0.09 ms.
+template <int HD>
+struct Shape {
+    static constexpr int kHalves = HD / 64;                       // 128-byte-swizzled 64-dimension pieces of a row
+    static constexpr int kTileBytes = kHalves * kHalfBytes;       // [128 x HD] bf16
+    static constexpr int kStages = HD == 64 ? 4 : 2;
+    static constexpr bool kSplitP = HD == 64;
+    static constexpr uint32_t kPCols = kSplitP ? kBN : kBN / 2;   // two keys per column, hi then lo
+    static constexpr uint32_t kOCol = kPCol + 2 * kPCols;
+    static constexpr size_t kSlotFloats = slot_floats(HD);
+    static_assert(kOCol + 2 * HD <= kTmemCols, "TMEM columns");
+};
+constexpr int kMaxStages = 4;
 
 struct MmaArgs {
     const char *q;
@@ -117,10 +132,10 @@ struct MmaArgs {
 
 struct Bars {
     uint64_t q_full;             // both softmax groups wrote their Q tiles
-    uint64_t k_full[kStages];    // TMA bytes of a K tile landed
-    uint64_t v_full[kStages];
-    uint64_t k_empty[kStages];   // the first products that read the K stage have completed
-    uint64_t v_empty[kStages];   // the second products that read the V stage have completed
+    uint64_t k_full[kMaxStages];    // TMA bytes of a K tile landed
+    uint64_t v_full[kMaxStages];
+    uint64_t k_empty[kMaxStages];   // the first products that read the K stage have completed
+    uint64_t v_empty[kMaxStages];   // the second products that read the V stage have completed
     uint64_t s_full[2];          // S = Q K^T of row tile A / B is in TMEM
     uint64_t p_full[2];          // P of row tile A / B is in TMEM (over S)
     uint64_t o_full[2];          // O += P V of row tile A / B has completed
@@ -134,14 +149,17 @@ struct Bars {
     int abort;
 };
 
-constexpr size_t kSmemFixed = 1024 /*alignment*/ + 2 * kTileBytes /*Q of A, B*/ + 2 * kStages * kTileBytes /*K, V*/ +
-                              sizeof(Bars);
+template <int HD>
+constexpr size_t smem_fixed() {
+    return 1024 /*alignment*/ + 2 * Shape<HD>::kTileBytes /*Q of A, B*/ + 2 * Shape<HD>::kStages * Shape<HD>::kTileBytes /*K, V*/ + sizeof(Bars);
+}
 
 constexpr size_t kCodeStageBytes = 2 * kStagePages * kCodePageBytes;   // E4M3: staging of both operands
 constexpr int kMaxBatchE4m3 = 320;   // the staging takes 24 KB of what the plan tables of a larger batch would need
 
-inline size_t mma_smem_bytes(int batch, bool e4m3 = false) {
-    return kSmemFixed + (e4m3 ? kCodeStageBytes : 0) + sizeof(int) * (7 * (size_t)batch + 2);
+template <int HD>
+inline size_t mma_smem_bytes(int batch, bool e4m3) {
+    return smem_fixed<HD>() + (e4m3 ? kCodeStageBytes : 0) + sizeof(int) * (7 * (size_t)batch + 2);
 }
 
 // ---- tcgen05 / TMA wrappers -------------------------------------------------------------------
@@ -198,13 +216,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes
     return d;
 }
 
-// Instruction descriptor of kind::f16: fp32 accumulator, A and B both bf16 or both f16, M = 128, N = 128.
-__host__ __device__ constexpr uint32_t instr_desc(bool b_mn_major, bool f16 = false) {
+// Instruction descriptor of kind::f16: fp32 accumulator, A and B both bf16 or both f16, M = 128.
+__host__ __device__ constexpr uint32_t instr_desc(int n, bool b_mn_major, bool f16) {
     return (1u << 4)                       // accumulator format: f32
            | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10)   // A, B format: f16 = 0, bf16 = 1
            | (0u << 15)                    // A is K-major
            | ((b_mn_major ? 1u : 0u) << 16)
-           | ((uint32_t)(kBN >> 3) << 17)  // N
+           | ((uint32_t)(n >> 3) << 17)    // N
            | ((uint32_t)(kBM >> 4) << 24); // M
 }
 
@@ -469,9 +487,14 @@ __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, in
     return true;
 }
 
-template <int G, bool E4M3>
+template <int G, bool E4M3, int HD>
 __global__ void __launch_bounds__(threads_of(E4M3), 1)
 chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map) {
+    using Sh = Shape<HD>;
+    constexpr int kTileBytes = Sh::kTileBytes, kStages = Sh::kStages;
+    constexpr uint32_t kPCols = Sh::kPCols, kOCol = Sh::kOCol;
+    constexpr size_t kSlotFloats = Sh::kSlotFloats;
+    static_assert(!E4M3 || HD == 128, "the code cache has 128-dimension rows");
     extern __shared__ char smem_raw[];
     char *base = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     char *q_s = base;                                  // [row tile A, B][2 halves][128 rows][128 B]
@@ -575,7 +598,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             // ring (two tiles deep) only has to cover the L2 latency, not the DRAM latency
             auto prefetch_pages = [&](int pf) {
                 if ((unsigned)pf < (unsigned)a.num_pages && !helper) {
-                    constexpr int kPageBytes = kPage * kD * (E4M3 ? 1 : 2);
+                    constexpr int kPageBytes = kPage * HD * (E4M3 ? 1 : 2);
                     const char *src = pool + ((size_t)pf * Hkv + w.kvh) * kPageBytes;
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(kPageBytes) : "memory");
                 }
@@ -679,9 +702,9 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                     if (lane == 0) ok = mbar_wait(&empty[s], par ^ 1u, abort, a.status);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                     if (ok) {
-                        if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)npages * 2u * kBoxBytes);
+                        if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)npages * Sh::kHalves * kBoxBytes);
                         __syncwarp();
-                        if (lane < 16 && pg < npages)
+                        if (lane < 8 * Sh::kHalves && pg < npages)
                             tma_box_load(ring + s * kTileBytes + half * kHalfBytes + pg * kBoxBytes, map, half * 64, row, &full[s]);
                     }
                 }
@@ -700,7 +723,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         // complete costs about a hundred cycles, so one thread issuing both kinds leaves the tensor core idle while it
         // looks at its barriers.
         if (lane == 0) {
-            constexpr uint32_t idesc_qk = instr_desc(false, E4M3);
+            constexpr uint32_t idesc_qk = instr_desc(kBN, false, E4M3);
             const uint32_t q_addr = smem_u32(q_s);
             uint32_t it = 0, nitem = 0, nproc = 0;   // KV tiles so far, items, items with work
             uint32_t nfree[2] = {0u, 0u};            // S loads so far per group
@@ -716,7 +739,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 ++nproc;
                 const bool lone = w.rows[1] == 0;
                 const int units = lone ? w.ntiles : 2 * w.ntiles;
-                // S of unit u: 8 steps of 16 dims, 4 per 64-dim half; K-major operands, SBO = 8 rows.  A K stage is
+                // S of unit u: steps of 16 dims, 4 per 64-dim half; K-major operands, SBO = 8 rows.  A K stage is
                 // waited for by the first unit that reads it and released behind the last one.
                 auto issue_qk = [&](int u) {
                     const uint32_t itx = it + (lone ? u : (u >> 1)), s = itx % kStages;
@@ -725,7 +748,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                     const uint32_t k_addr = smem_u32(k_s + s * kTileBytes);
                     tc_fence_after();
 #pragma unroll
-                    for (int ks = 0; ks < kD / 16; ++ks) {
+                    for (int ks = 0; ks < HD / 16; ++ks) {
                         const uint32_t off = (ks >> 2) * kHalfBytes + (ks & 3) * 32;
                         mma_f16_ss(tmem, smem_desc(q_addr + qt * kTileBytes + off, 16, 1024),
                                    smem_desc(k_addr + off, 16, 1024), idesc_qk, ks > 0 ? 1u : 0u);
@@ -747,7 +770,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
     } else if (warp == kPvWarp) {
         // ================================ MMA issue: O += P V =======================================
         if (lane == 0) {
-            constexpr uint32_t idesc_pv = instr_desc(true, E4M3);
+            constexpr uint32_t idesc_pv = instr_desc(HD, true, E4M3);
             uint32_t it = 0, nitem = 0, itg[2] = {0u, 0u};  // KV tiles so far, items, units so far per group
             Item w;
             for (;; ++nitem) {
@@ -760,7 +783,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 const bool lone = w.rows[1] == 0;
                 const int units = lone ? w.ntiles : 2 * w.ntiles;
                 // O of the unit's group += P V: 8 steps of 16 keys; P from the group's TMEM columns (two keys per
-                // column, 8 columns per step); V MN-major: 64-dim halves LBO apart, 8-key groups SBO apart.  A V stage
+                // column, 8 columns per step; with a split P all steps of hi, then all of lo); V MN-major: 64-dim halves LBO apart, 8-key groups SBO apart.  A V stage
                 // is waited for by the first unit that reads it and released behind the last one.
                 for (int u = 0; u < units; ++u) {
                     const uint32_t itx = it + (lone ? u : (u >> 1)), s = itx % kStages;
@@ -770,9 +793,9 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                     mbar_wait(&bars->p_full[g], itg[g] & 1u, abort, a.status);
                     tc_fence_after();
 #pragma unroll
-                    for (int ks = 0; ks < kBN / 16; ++ks)
-                        mma_f16_ts(tmem + kOCol + g * kBN, tmem + kPCol + g * (kBN / 2) + ks * 8,
-                                   smem_desc(v_addr + ks * 2 * 1024, kHalfBytes, 1024), idesc_pv,
+                    for (int ks = 0; ks < (int)kPCols / 8; ++ks)
+                        mma_f16_ts(tmem + kOCol + g * HD, tmem + kPCol + g * kPCols + ks * 8,
+                                   smem_desc(v_addr + (ks % (kBN / 16)) * 2 * 1024, kHalfBytes, 1024), idesc_pv,
                                    (u >= 2 || ks > 0) ? 1u : 0u);
                     mma_commit(&bars->o_full[g]);
                     ++itg[g];
@@ -791,8 +814,8 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         const int grp = warp >> 2, tg = tid & (kSoftmaxThreads - 1);
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;  // this warp's TMEM lane quadrant
         const uint32_t s_tmem = tmem + lane_base;                                  // S: one region for both groups
-        const uint32_t p_tmem = tmem + lane_base + kPCol + grp * (kBN / 2);        // this group's P
-        const uint32_t o_tmem = tmem + lane_base + kOCol + grp * kBN;
+        const uint32_t p_tmem = tmem + lane_base + kPCol + grp * kPCols;           // this group's P
+        const uint32_t o_tmem = tmem + lane_base + kOCol + grp * HD;
         char *q_tile = q_s + grp * kTileBytes;
         const int swz = tg & 7;
         uint32_t it = 0, itg = 0, nitem = 0;  // KV tiles so far: of all items, of those this group has worked on
@@ -813,12 +836,12 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             const int r = min(w.r_begin + (lone ? 0 : grp * kBM) + tg, w.rows_total - 1);
             const int tok = r / G, head = r - tok * G;
             const int lim = w.L - w.n + tok + 1;  // keys this row may see
-            const size_t grow = ((size_t)(w.qrow0 + tok) * a.Hq + w.kvh * G + head) * kD;
-            // ---- Q tile: row `tg`, 16 chunks of 8 dims, chunk c of a half stored at c ^ (row & 7)
+            const size_t grow = ((size_t)(w.qrow0 + tok) * a.Hq + w.kvh * G + head) * HD;
+            // ---- Q tile: row `tg`, chunks of 8 dims, chunk c of a half stored at c ^ (row & 7)
             if (!(lone && grp == 1)) {   // (the second group of such an item reads Q tile A as well)
                 const uint4 *src = reinterpret_cast<const uint4 *>(a.q + grow * 2);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
+                for (int c = 0; c < HD / 8; ++c) {
                     uint4 v = row_ok ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
                     if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
                         v.x = bf16x2_to_f16x2(v.x); v.y = bf16x2_to_f16x2(v.y);
@@ -878,7 +901,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 }
                 if (__any_sync(0xffffffffu, rescale)) {
 #pragma unroll 1
-                    for (int c4 = 0; c4 < 4; ++c4) {
+                    for (int c4 = 0; c4 < HD / 32; ++c4) {
                         uint32_t o[32];
                         tmem_ld32(o_tmem + c4 * 32, o);
                         tmem_wait_ld();
@@ -898,7 +921,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 uint64_t l2[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
                 for (int c4 = 0; c4 < 4; ++c4) {
-                    uint32_t pk[16];
+                    uint32_t pk[16], pl[Sh::kSplitP ? 16 : 1];
 #pragma unroll
                     for (int k = 0; k < 16; ++k) {
                         const uint64_t t = fma_f32x2(pack_f32x2(__uint_as_float(v[c4 * 32 + 2 * k]),
@@ -907,9 +930,12 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                         unpack_f32x2(t, t0, t1);
                         const float e0 = fast_exp2(t0), e1 = fast_exp2(t1);
                         pk[k] = E4M3 ? pack_f16(e0, e1) : pack_bf16(e0, e1);
+                        if constexpr (Sh::kSplitP)   // what the rounding left over, to 8 more bits
+                            pl[k] = pack_bf16(e0 - __uint_as_float(pk[k] << 16), e1 - __uint_as_float(pk[k] & 0xffff0000u));
                         l2[k & 3] = add_f32x2(l2[k & 3], pack_f32x2(e0, e1));
                     }
                     tmem_st16(p_tmem + c4 * 16, pk);
+                    if constexpr (Sh::kSplitP) tmem_st16(p_tmem + kBN / 2 + c4 * 16, pl);
                 }
                 {
                     float x0, x1, y0, y1;
@@ -927,8 +953,9 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                         char *vrow = v_s + s * kTileBytes + tg * 128;
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
-                            *reinterpret_cast<uint4 *>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
-                            *reinterpret_cast<uint4 *>(vrow + kHalfBytes + c * 16) = make_uint4(0, 0, 0, 0);
+#pragma unroll
+                            for (int h = 0; h < Sh::kHalves; ++h)
+                                *reinterpret_cast<uint4 *>(vrow + h * kHalfBytes + c * 16) = make_uint4(0, 0, 0, 0);
                         }
                     }
                 }
@@ -943,7 +970,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             if (lone) {
                 // The two groups hold O, max and sum over the even and over the odd KV tiles of the same rows.  They
                 // exchange (max, sum) through the shared memory of Q tile B, which such an item does not use, and
-                // each merges and writes 64 of the 128 dimensions: thread tg of either group owns TMEM lane tg and
+                // each merges and writes half of the dimensions: thread tg of either group owns TMEM lane tg and
                 // reads that lane of both O.
                 float2 *ml = reinterpret_cast<float2 *>(q_s + kTileBytes);
                 ml[grp * kSoftmaxThreads + tg] = make_float2(m_used, l_sum);
@@ -961,10 +988,10 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 const bool slot_in = !w.split || ARB_IN_RANGE(a.status, w.slot, a.split_cap);
                 float *po = a.split_ws + (size_t)(w.split && slot_in ? w.slot : 0) * kSlotFloats;
                 const float norm = w.split ? (E4M3 ? a.v_scale : 1.0f) : (E4M3 ? a.v_scale : 1.0f) / l;
-                const uint32_t oa = tmem + lane_base + kOCol, ob = oa + kBN;
+                const uint32_t oa = tmem + lane_base + kOCol, ob = oa + HD;
                 uint4 *dst = reinterpret_cast<uint4 *>(a.out + grow * 2);
 #pragma unroll 1
-                for (int c4 = 2 * grp; c4 < 2 * grp + 2; ++c4) {
+                for (int c4 = HD / 64 * grp; c4 < HD / 64 * (grp + 1); ++c4) {
                     uint32_t va[32];
                     float o[32];
                     tmem_ld32(oa + c4 * 32, va);
@@ -998,7 +1025,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                     }
                 }
                 if (w.split && grp == 0 && row_ok && slot_in)
-                    *reinterpret_cast<float2 *>(po + (size_t)kBM * kD + tg * 2) = make_float2(m, l);
+                    *reinterpret_cast<float2 *>(po + (size_t)kBM * HD + tg * 2) = make_float2(m, l);
                 tc_fence_before();
                 continue;
             }
@@ -1007,7 +1034,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 const bool slot_in = ARB_IN_RANGE(a.status, w.slot + grp, a.split_cap);
                 float *po = a.split_ws + (size_t)(slot_in ? w.slot + grp : 0) * kSlotFloats;
 #pragma unroll 1
-                for (int c4 = 0; c4 < 4; ++c4) {
+                for (int c4 = 0; c4 < HD / 32; ++c4) {
                     uint32_t v[32];
                     tmem_ld32(o_tmem + c4 * 32, v);
                     tmem_wait_ld();
@@ -1022,14 +1049,14 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                                 make_uint4(v[qd * 4], v[qd * 4 + 1], v[qd * 4 + 2], v[qd * 4 + 3]);
                     }
                 }
-                if (row_ok && slot_in) *reinterpret_cast<float2 *>(po + (size_t)kBM * kD + tg * 2) = make_float2(m_used, l_sum);
+                if (row_ok && slot_in) *reinterpret_cast<float2 *>(po + (size_t)kBM * HD + tg * 2) = make_float2(m_used, l_sum);
                 tc_fence_before();
                 continue;
             }
             const float inv_l = (E4M3 ? a.v_scale : 1.0f) / l_sum;
             uint4 *dst = reinterpret_cast<uint4 *>(a.out + grow * 2);
 #pragma unroll 1
-            for (int c4 = 0; c4 < 4; ++c4) {
+            for (int c4 = 0; c4 < HD / 32; ++c4) {
                 uint32_t v[32];
                 tmem_ld32(o_tmem + c4 * 32, v);
                 tmem_wait_ld();
@@ -1060,22 +1087,23 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
 
 // ---- merge of the parts of split sequences -------------------------------------------------------------
 // Runs behind chunk_mma_kernel on the stream.  Every CTA rebuilds the plan, then takes jobs in turn: a job
-// is a quarter (32 dimensions) of one row tile of a split sequence, one thread per query row:
+// is 32 dimensions of one row tile of a split sequence, one thread per query row:
 //     m = max_p m_p,  w_p = 2^(m_p - m),  out = sum_p w_p O_p / sum_p w_p l_p.
 // Partials are laid out so that the threads of a warp (consecutive rows) read consecutive 16-byte pieces.
 constexpr int kCombineThreads = kBM;
 constexpr int kCombineDims = 32;    // dimensions of a row per job
 
-template <int G>
+template <int G, int HD>
 __global__ void __launch_bounds__(kCombineThreads)
 chunk_combine_kernel(const MmaArgs a) {
+    constexpr size_t kSlotFloats = Shape<HD>::kSlotFloats;
     extern __shared__ int plan_smem[];
     const Plan pl = plan_arrays(plan_smem, a.batch);
     const int tid = threadIdx.x;
     const int B = a.batch, Hkv = a.Hkv;
     pdl_enter();
     make_plan<G>(a, pl, tid, kCombineThreads, nullptr);
-    constexpr int kQuarters = kD / kCombineDims;
+    constexpr int kPieces = HD / kCombineDims;
     int job = 0;
     for (int r = 0; r < B; ++r) {
         const int P = pl.parts[r];
@@ -1083,13 +1111,13 @@ chunk_combine_kernel(const MmaArgs a) {
         const int sb = pl.sorted[r], pairs = pl.pairs[sb];
         const int n = a.q_lens[sb], L = a.seq_lens[sb], rows_total = n * G;
         const int T = part_tiles(L, P);
-        const int njobs = Hkv * pairs * 2 * kQuarters;
+        const int njobs = Hkv * pairs * 2 * kPieces;
         // the jobs of this sequence that fall to this CTA
         int j = (int)blockIdx.x - job % (int)gridDim.x;
         if (j < 0) j += (int)gridDim.x;
         job += njobs;
         for (; j < njobs; j += (int)gridDim.x) {
-            const int qd = j % kQuarters, jt = j / kQuarters;
+            const int qd = j % kPieces, jt = j / kPieces;
             const int g = jt & 1, pt = (jt >> 1) % pairs, kvh = (jt >> 1) / pairs;
             const int r_begin = pt * 2 * kBM;
             const int rows_here = max(0, min(kBM, rows_total - r_begin - g * kBM));
@@ -1100,7 +1128,7 @@ chunk_combine_kernel(const MmaArgs a) {
             const size_t part_stride = 2 * kSlotFloats;
             float m = -INFINITY;
             for (int p = 0; p < nparts; ++p)
-                m = fmaxf(m, __ldcg(slot0 + p * part_stride + (size_t)kBM * kD + tid * 2));   // part 0 sees key 0: finite
+                m = fmaxf(m, __ldcg(slot0 + p * part_stride + (size_t)kBM * HD + tid * 2));   // part 0 sees key 0: finite
             float l = 0.f;
             float4 acc[kCombineDims / 4];
 #pragma unroll
@@ -1111,7 +1139,7 @@ chunk_combine_kernel(const MmaArgs a) {
 #pragma unroll
                 for (int c = 0; c < kCombineDims / 4; ++c)
                     o[c] = __ldcg(reinterpret_cast<const float4 *>(sp + ((size_t)(qd * (kCombineDims / 4) + c) * kBM + tid) * 4));
-                const float2 ml = __ldcg(reinterpret_cast<const float2 *>(sp + (size_t)kBM * kD + tid * 2));
+                const float2 ml = __ldcg(reinterpret_cast<const float2 *>(sp + (size_t)kBM * HD + tid * 2));
                 const float w = fast_exp2(ml.x - m);
                 l = fmaf(w, ml.y, l);
 #pragma unroll
@@ -1124,7 +1152,7 @@ chunk_combine_kernel(const MmaArgs a) {
             }
             const int rr = r_begin + g * kBM + tid;
             const int tok = rr / G, head = rr - tok * G;
-            const size_t grow = ((size_t)(pl.row0[sb] + tok) * a.Hq + kvh * G + head) * kD + (size_t)qd * kCombineDims;
+            const size_t grow = ((size_t)(pl.row0[sb] + tok) * a.Hq + kvh * G + head) * HD + (size_t)qd * kCombineDims;
             const float inv = 1.0f / l;
             uint4 *dst = reinterpret_cast<uint4 *>(a.out + grow * 2);
 #pragma unroll
@@ -1140,25 +1168,25 @@ chunk_combine_kernel(const MmaArgs a) {
     }
 }
 
-template <int G, bool E4M3>
+template <int G, bool E4M3, int HD>
 arb_status launch_one(Ctx *ctx, const MmaArgs &a, const CUtensorMap &km, const CUtensorMap &vm, int max_items,
                       cudaStream_t stream) {
-    const size_t smem = mma_smem_bytes(a.batch, E4M3);
+    const size_t smem = mma_smem_bytes<HD>(a.batch, E4M3);
     static bool attr_set[64] = {};
     if (!attr_set[ctx->device & 63]) {
-        if (cudaFuncSetAttribute(chunk_mma_kernel<G, E4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)mma_smem_bytes(E4M3 ? kMaxBatchE4m3 : kMaxBatch, E4M3)) != cudaSuccess)
+        if (cudaFuncSetAttribute(chunk_mma_kernel<G, E4M3, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)mma_smem_bytes<HD>(E4M3 ? kMaxBatchE4m3 : kMaxBatch, E4M3)) != cudaSuccess)
             return ARB_ERR_CUDA;
         attr_set[ctx->device & 63] = true;
     }
     const int grid = max_items < ctx->num_sms ? max_items : ctx->num_sms;
-    const cudaError_t err = launch_pdl(chunk_mma_kernel<G, E4M3>, dim3(grid), dim3(threads_of(E4M3)), smem, stream, a, km, vm);
+    const cudaError_t err = launch_pdl(chunk_mma_kernel<G, E4M3, HD>, dim3(grid), dim3(threads_of(E4M3)), smem, stream, a, km, vm);
     ctx->launches++;
     if (err != cudaSuccess) return ARB_ERR_CUDA;
     // the merge of split sequences, when the block table is long enough for a sequence to be split at all
     if (a.split_cap > 0) {
         const size_t csmem = sizeof(int) * (7 * (size_t)a.batch + 2);
-        const cudaError_t cerr = launch_pdl(chunk_combine_kernel<G>, dim3(4 * ctx->num_sms), dim3(kCombineThreads), csmem, stream, a);
+        const cudaError_t cerr = launch_pdl(chunk_combine_kernel<G, HD>, dim3(4 * ctx->num_sms), dim3(kCombineThreads), csmem, stream, a);
         ctx->launches++;
         if (cerr != cudaSuccess) return ARB_ERR_CUDA;
     }
@@ -1169,17 +1197,25 @@ arb_status launch_one(Ctx *ctx, const MmaArgs &a, const CUtensorMap &km, const C
 
 bool chunk_mma_supported(const arb_attn_params &p) {
     const int g = p.num_q_heads / p.num_kv_heads;
-    return p.dtype == ARB_BF16 && p.head_dim == kD && p.max_q_len >= 2 && p.max_q_len * g >= kChunkMmaMinRows &&
+    return p.dtype == ARB_BF16 && (p.head_dim == 64 || p.head_dim == 128) && p.max_q_len >= 2 && p.max_q_len * g >= kChunkMmaMinRows &&
            tma_available();
 }
 
 namespace {
 
+template <int G>
+arb_status launch_g(Ctx *ctx, const MmaArgs &a, bool e4m3, int head_dim, const CUtensorMap &km, const CUtensorMap &vm,
+                    int max_items, cudaStream_t stream) {
+    if (e4m3) return launch_one<G, true, 128>(ctx, a, km, vm, max_items, stream);
+    if (head_dim == 64) return launch_one<G, false, 64>(ctx, a, km, vm, max_items, stream);
+    return launch_one<G, false, 128>(ctx, a, km, vm, max_items, stream);
+}
+
 arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages, const void *v_pages,
                            bool e4m3, float k_scale, float v_scale, const int32_t *block_table, const int32_t *seq_lens,
                            const int32_t *q_lens, void *out, cudaStream_t stream) {
     alignas(64) CUtensorMap km, vm;
-    const PoolView view = e4m3 ? PoolView::kE4m3 : PoolView::kBf16HalfRows;
+    const PoolView view = e4m3 ? PoolView::kE4m3 : p.head_dim == 64 ? PoolView::kBf16D64 : PoolView::kBf16HalfRows;
     if (!pool_map(ctx, &km, k_pages, p.num_pages, p.num_kv_heads, view) ||
         !pool_map(ctx, &vm, v_pages, p.num_pages, p.num_kv_heads, view))
         return ARB_ERR_CUDA;
@@ -1201,7 +1237,7 @@ arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, co
     a.min_rows = kChunkMmaMinRows;
     a.work_counter = ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 1;
     a.split_ws = ctx->chunk_ws;
-    a.split_cap = (int)(ctx->chunk_ws_bytes / (kSlotFloats * sizeof(float)));
+    a.split_cap = (int)(ctx->chunk_ws_bytes / (slot_floats(p.head_dim) * sizeof(float)));
     // Can a sequence of this call be split at all?  Long ones from kSplitMinTiles tiles on; shorter ones only in a call
     // whose work items may fail to fill the machine.  The host knows the rows: at most `batch` of them are decode rows,
     // the others sit in row-tile pairs of 256, one work item per pair and KV head.
@@ -1218,23 +1254,15 @@ arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, co
     long long bound = (long long)p.num_kv_heads * ((long long)p.total_q * g / kBM + p.batch);
     if (a.split_cap > 0) bound *= kSplitMaxParts;   // every item of a split sequence comes once per part
     const int max_items = (int)(bound < 1 ? 1 : (bound > (1 << 30) ? (1 << 30) : bound));
-    switch (e4m3 ? g + 8 : g) {
-        case 1: return launch_one<1, false>(ctx, a, km, vm, max_items, stream);
-        case 2: return launch_one<2, false>(ctx, a, km, vm, max_items, stream);
-        case 3: return launch_one<3, false>(ctx, a, km, vm, max_items, stream);
-        case 4: return launch_one<4, false>(ctx, a, km, vm, max_items, stream);
-        case 5: return launch_one<5, false>(ctx, a, km, vm, max_items, stream);
-        case 6: return launch_one<6, false>(ctx, a, km, vm, max_items, stream);
-        case 7: return launch_one<7, false>(ctx, a, km, vm, max_items, stream);
-        case 8: return launch_one<8, false>(ctx, a, km, vm, max_items, stream);
-        case 9: return launch_one<1, true>(ctx, a, km, vm, max_items, stream);
-        case 10: return launch_one<2, true>(ctx, a, km, vm, max_items, stream);
-        case 11: return launch_one<3, true>(ctx, a, km, vm, max_items, stream);
-        case 12: return launch_one<4, true>(ctx, a, km, vm, max_items, stream);
-        case 13: return launch_one<5, true>(ctx, a, km, vm, max_items, stream);
-        case 14: return launch_one<6, true>(ctx, a, km, vm, max_items, stream);
-        case 15: return launch_one<7, true>(ctx, a, km, vm, max_items, stream);
-        case 16: return launch_one<8, true>(ctx, a, km, vm, max_items, stream);
+    switch (g) {
+        case 1: return launch_g<1>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
+        case 2: return launch_g<2>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
+        case 3: return launch_g<3>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
+        case 4: return launch_g<4>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
+        case 5: return launch_g<5>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
+        case 6: return launch_g<6>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
+        case 7: return launch_g<7>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
+        case 8: return launch_g<8>(ctx, a, e4m3, p.head_dim, km, vm, max_items, stream);
         default: return ARB_ERR_UNSUPPORTED;
     }
 }

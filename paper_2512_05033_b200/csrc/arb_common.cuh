@@ -12,7 +12,7 @@ namespace arb {
 constexpr int kPage = 16;             // tokens per KV page
 constexpr int kMaxBatch = 1024;       // sequences per call (prefix tables live in shared memory)
 constexpr int kMaxGroup = 8;          // query heads per KV head
-// q_len * group from which a bf16, head_dim-128 chunk goes to the tcgen05 kernel: every chunk.  A tile with few
+// q_len * group from which a bf16 chunk goes to the tcgen05 kernel: every chunk.  A tile with few
 // query rows wastes tensor-core rows, but the tile streams a sequence's keys once, at memory speed, where the
 // CUDA-core kernel re-reads them per query row (measured on rounds of short steps: 0.76 ms against 0.12 ms per
 // call; the threshold used to be 64 rows).

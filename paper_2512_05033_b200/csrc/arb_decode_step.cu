@@ -1,4 +1,4 @@
-// One decode token in one launch (bf16, head_dim 128, group size <= 8): the cache write of the token's new
+// One decode token in one launch (bf16, head_dim 64 or 128, group size <= 8): the cache write of the token's new
 // K/V rows, split-KV attention over the paged cache, the split combine and the length update, all in one
 // kernel.  This is what a token of a draft or target step costs in Algorithm 1 of the paper ("Sample draft
 // step" / "Sample target step": z_i ~ q(z_i | x, z_<i), Section 3.1): every call of that chain reads what the
@@ -41,21 +41,26 @@ namespace arb {
 
 namespace {
 
-constexpr int kCW = 8;                        // consumer warps
-constexpr int kCT = kCW * 32;                 // consumer threads
-constexpr int kProdWarp = kCW;                // the producer warp
-constexpr int kAuxWarp = kCW + 1;             // bookkeeping: length update, rows of refused sequences
-constexpr int kNT = kCT + 64;
-constexpr int kTileBytes = kPage * kD * 2;    // 4 KB: one (page, kv head) tile of K or of V
-constexpr int kHalfTile = kTileBytes / 2;
+constexpr int kHalfTile = kPage * 128;        // 2 KB: 64 dimensions of a (page, kv head) tile of K or of V
 constexpr int kCodeTileBytes = kPage * kD;    // 2 KB: the same tile of an E4M3 cache
 constexpr int kI4CodeBytes = kPage * kD / 2;  // 1 KB: the same tile of a 4-bit cache (16 rows x 64 bytes, not swizzled) ...
 constexpr int kI4ScaleBytes = kPage * 4;      // ... followed by the 16 fp32 scales of its rows
 constexpr int kI4StageBytes = 1152;           // both, rounded up to 128
 enum { kKvBf16 = 0, kKvE4m3 = 1, kKvI4 = 2 }; // the cache a kernel instance reads
-constexpr int kBatch = 32;                    // producer lanes issuing side by side
+constexpr int kCW = 8;                        // consumer warps
+constexpr int kCT = kCW * 32;                 // consumer threads
+constexpr int kProdWarp = kCW;                // the producer warps, and behind them one for bookkeeping: length update,
+                                              // rows of refused sequences
+// A warp issues a tiled copy every hundred cycles or so, whatever it brings.  Tiles of 4 KB (bf16, head_dim 128) come faster
+// than HBM that way, from one warp (a second one makes every lone call 0.8 us slower: 14.6 -> 15.4 us per draft-shaped
+// token).  Where a tile is 2 KB or less two warps issue, one K and one V: a token of 16 x 8 kv heads of 64 dimensions
+// (150 MB) 38 -> 32 us, draft-shaped tokens over 4-bit codes 17.6 -> 16.7 us, over E4M3 codes 5 % less.
+template <int KV, int HD>
+__host__ __device__ constexpr int producer_warps() { return KV == kKvBf16 && HD == 128 ? 1 : 2; }
+template <int KV, int HD>
+__host__ __device__ constexpr int step_threads() { return 32 * (kCW + producer_warps<KV, HD>() + 1); }
+
 constexpr int kParked = 2;                    // segment results parked in shared memory before they are written
-constexpr int kOStride = kD + 4;              // floats between two heads of a warp record (spreads the banks)
 // What a boundary costs is time (the warps meet, a second arrival, perhaps a second merge), a few microseconds
 // whatever the call's size: as pages it is the CTA's even share, but no more than this many.
 constexpr int kBoundaryCap = 32;
@@ -103,19 +108,21 @@ struct Tail {
     int last[kParked];
 };
 
-template <int G>
+template <int G, int HD>
 struct Cfg {
+    static constexpr int kOStride = HD + 4;               // floats between two heads of a warp record (spreads the banks)
     static constexpr int GP = (G + 3) / 4 * 4;
     static constexpr int WREC = 2 * 8 + G * kOStride;     // warp record: [m[8] | l[8] | o[G][kOStride]]
-    static constexpr int REC = 2 * GP + G * kD;           // parked record: [m[GP] | l[GP] | o[G][D]]
+    static constexpr int REC = 2 * GP + G * HD;           // parked record: [m[GP] | l[GP] | o[G][D]]
     static constexpr int OSM_BYTES = kCW * WREC * 4;
     static constexpr int PARK_BYTES = kParked * REC * 4;
 };
 
 // E4M3: the ring holds tiles of codes; every consumer warp has a widened K tile and a widened V tile of its own
-template <int G, int STAGES, int KV>
+template <int G, int STAGES, int KV, int HD>
 size_t smem_bytes(int batch) {
-    using C = Cfg<G>;
+    using C = Cfg<G, HD>;
+    constexpr int kTileBytes = HD / 64 * kHalfTile;
     const size_t wide = (size_t)kCW * 2 * kTileBytes;
     const size_t tiles = KV == kKvE4m3 ? (size_t)STAGES * kCodeTileBytes + wide
                          : KV == kKvI4 ? (size_t)STAGES * kI4StageBytes + wide : (size_t)STAGES * kTileBytes;
@@ -290,20 +297,30 @@ __device__ __forceinline__ void parts_of(const Plan &pl, Segment &s) {
     s.nparts = pl.cta_of(s.b, s.kvh, pages, pages - 1) - s.c_first + 1;
 }
 
-template <int G, int STAGES, bool APPEND, int KV>
-__global__ void __launch_bounds__(kNT, 1)
+// Head dimension 64: a tile is 2 KB (one box), the products have half the steps, and the softmax weights enter the
+// second product as two bf16 terms (p = hi + lo: 16 significant bits, like the fp32 weights of the CUDA-core kernel this
+// form replaced, to within the rounding of the output); the memory system sets the pace, so the second term costs nothing.
+template <int G, int STAGES, bool APPEND, int KV, int HD>
+__global__ void __launch_bounds__(step_threads<KV, HD>(), 1)
 decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map) {
-    using C = Cfg<G>;
+    constexpr int kProducers = producer_warps<KV, HD>();
+    constexpr int kAuxWarp = kCW + kProducers, kNT = step_threads<KV, HD>();
+    constexpr int kOwnStages = STAGES / kProducers;             // of one producer warp
+    constexpr int kBatch = kOwnStages < 32 ? kOwnStages : 32;   // lanes of a producer warp issuing side by side
+    using C = Cfg<G, HD>;
     using Tail = arb::Tail<STAGES>;
-    constexpr int GP = C::GP, WREC = C::WREC, REC = C::REC;
+    constexpr int GP = C::GP, WREC = C::WREC, REC = C::REC, kOStride = C::kOStride;
+    constexpr int kD = HD, kTileBytes = HD / 64 * kHalfTile;   // a tile of a bf16 cache, and of widened codes
+    constexpr bool SPLIT_P = HD == 64;
     constexpr bool E4M3 = KV == kKvE4m3, I4 = KV == kKvI4, WIDE = KV != kKvBf16;
     constexpr int kStageBytes = E4M3 ? kCodeTileBytes : I4 ? kI4StageBytes : kTileBytes;   // a ring stage
     constexpr int kTxBytes = I4 ? kI4CodeBytes + kI4ScaleBytes : kStageBytes;               // what the copies of a stage bring
     constexpr int kRowBytes = E4M3 ? kD : I4 ? kD / 2 : kD * 2;         // bytes of a cache row
     constexpr int kWideBytes = WIDE ? kCW * 2 * kTileBytes : 0;         // codes: a widened K and V tile per consumer warp
     constexpr int kRingBytes = STAGES * kStageBytes + kWideBytes;       // the merges use all of it
+    static_assert(!WIDE || HD == 128, "code caches have 128-dimension rows");
     static_assert(G >= 1 && G <= 8, "the group's heads are the 8 columns of the tile");
-    static_assert(STAGES % (2 * kCW) == 0 && kBatch <= STAGES, "a ring stage always belongs to the same warp of a segment");
+    static_assert(STAGES % (2 * kCW) == 0, "a ring stage always belongs to the same warp of a segment");
 
     extern __shared__ char smem_raw[];
     char *base = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -475,13 +492,15 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     }
     volatile int *abort = &tail->abort;
 
-    if (warp == kProdWarp) {
-        // ================================ producer warp ==========================================
+    if (warp >= kProdWarp) {
+        // ================================ producer warps ===========================================
         // The CTA's flat range of (sequence, kv head, page) triples goes through in groups of 32: lane i finds
         // triple i of the group (a short walk up the prefix table from the range's first sequence) and fetches its block-table entry; the entries
         // of the next group are asked for before the tiles of this one are issued, so that the look-up is off the
         // path after the first group, across sequence boundaries too.  Tiles enter the ring page by page, K then
-        // V; lanes 0 .. kBatch-1 each own one stage at a time.
+        // V.  Two warps issue them, one K and one V, where a tile is 2 KB or less: see producer_warps.  Lanes
+        // 0 .. kBatch-1 of a warp each own one stage at a time.
+        const int pw = warp - kProdWarp;
         const int nflat = r1 - r0;
         auto tile_row = [&](int r) -> int {   // first row, in the 2-D view of the pool, of the tile of flat triple r
             const int lo = pl.seq_of(r, seq0);
@@ -496,39 +515,42 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             }
             return (pid * Hkv + kvh) * kPage;
         };
-        uint32_t c = 0;
         int row_next = lane < nflat ? tile_row(r0 + lane) : 0;
-        if (lane == 0) {
+        if (lane == 0 && pw == 0) {
             hint[0] = a.hint_tag;
             hint[1] = nflat;
         }
         for (int g0 = 0; g0 < nflat; g0 += 32) {
             const int row_cur = row_next;
-            if (g0 + lane < min(nflat, kHintPages)) hint[4 + g0 + lane] = row_cur;
-            const int ntiles = 2 * min(32, nflat - g0);
+            if (pw == 0 && g0 + lane < min(nflat, kHintPages)) hint[4 + g0 + lane] = row_cur;
+            const int ntiles = (2 / kProducers) * min(32, nflat - g0);   // of this warp
 #pragma unroll 1
             for (int i0 = 0; i0 < ntiles; i0 += kBatch) {
                 // the next group's look-up goes out behind this group's first copies, not in front of them
                 if (i0 == kBatch && g0 + 32 + lane < nflat) row_next = tile_row(r0 + g0 + 32 + lane);
                 const int i = i0 + lane;
-                const int row = __shfl_sync(0xffffffffu, row_cur, (i >> 1) & 31);
-                const uint32_t cc = c + i, st = cc % STAGES, par = (cc / STAGES) & 1u;
-                const CUtensorMap *map = (i & 1) ? &v_map : &k_map;
-                // The lanes wait for 32 different stages.  A blocking wait would put the whole warp to sleep until its
+                const int t = kProducers * i + pw;   // tile of the group: page t / 2, K or V
+                const bool is_v = (t & 1) != 0;
+                const CUtensorMap *map = is_v ? &v_map : &k_map;
+                const int row = __shfl_sync(0xffffffffu, row_cur, (t >> 1) & 31);
+                const uint32_t cc = 2u * (uint32_t)g0 + (uint32_t)t, st = cc % STAGES, par = (cc / STAGES) & 1u;
+                // The lanes wait for different stages.  A blocking wait would put the whole warp to sleep until its
                 // time limit whenever one stage is not free yet, and copies for stages that are would go out late, in
                 // clumps (seen: 0.7 us apart).  So the warp polls, converged: every round each lane tests its own
                 // stage without blocking and issues its copy the moment the stage is free.
-                bool pending = i < ntiles && ARB_IN_RANGE(a.status, row, (long long)a.num_pages * Hkv * kPage);
+                bool pending = lane < kBatch && i < ntiles && ARB_IN_RANGE(a.status, row, (long long)a.num_pages * Hkv * kPage);
                 const long long t0 = clock64();
                 while (__any_sync(0xffffffffu, pending)) {
                     if (pending && mbar_test_wait(&tail->empty[st], par ^ 1u)) {
                         mbar_arrive_expect_tx(&tail->full[st], kTxBytes);
                         if constexpr (I4) {   // 16 rows x 64 bytes of codes, then the rows' 16 scales
                             tma_box_load(ring + st * kStageBytes, map, 0, row, &tail->full[st]);
-                            bulk_load(ring + st * kStageBytes + kI4CodeBytes, ((i & 1) ? a.v_scales : a.k_scales) + row,
+                            bulk_load(ring + st * kStageBytes + kI4CodeBytes, (is_v ? a.v_scales : a.k_scales) + row,
                                       kI4ScaleBytes, &tail->full[st]);
                         } else if constexpr (E4M3) {
                             tma_box_load(ring + st * kStageBytes, map, 0, row, &tail->full[st]);   // 16 rows x 128 codes
+                        } else if constexpr (HD == 64) {
+                            tma_box_load(ring + st * kTileBytes, map, 0, row, &tail->full[st]);    // 16 rows x 64 dims
                         } else if (a.whole_rows) {
                             tma_box_load3(ring + st * kTileBytes, map, 0, row, 0, &tail->full[st]);
                         } else {
@@ -547,14 +569,13 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 }
             }
             if (ntiles <= kBatch && g0 + 32 + lane < nflat) row_next = tile_row(r0 + g0 + 32 + lane);
-            c += ntiles;
         }
         // After a timeout the consumers may have left copies unconsumed: wait (bounded) for the last ring's
         // worth, so that no copy is in flight into this CTA's shared memory when it exits.
         if (lane == 0 && *abort) {
-            const uint32_t n = c < (uint32_t)STAGES ? c : (uint32_t)STAGES;
-            for (uint32_t i = 0; i < n; ++i) {
-                const uint32_t cc = c - 1 - i;
+            const int own = (2 / kProducers) * nflat, n = min(own, kOwnStages);
+            for (int i = 0; i < n; ++i) {
+                const uint32_t cc = (uint32_t)(kProducers * (own - 1 - i) + pw);
                 const long long t0 = clock64();
                 while (!mbar_try_wait(&tail->full[cc % STAGES], (cc / STAGES) & 1u) && clock64() - t0 < (1ll << 24)) {
                 }
@@ -627,13 +648,13 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         n_parked = 0;
     };
 
-    // B fragments of q^T (128 dims x 8 heads): k-slice ks holds dims 16 ks + 2 tq, + 1 and + 8 of head gq.  The
+    // B fragments of q^T (kD dims x 8 heads): k-slice ks holds dims 16 ks + 2 tq, + 1 and + 8 of head gq.  The
     // fragments of the next segment are asked for while this one streams.
-    uint32_t qb[8][2], qn[8][2];
-    auto load_q = [&](const Segment &g, uint32_t (&dst)[8][2]) {
+    uint32_t qb[kD / 16][2], qn[kD / 16][2];
+    auto load_q = [&](const Segment &g, uint32_t (&dst)[kD / 16][2]) {
         const char *qh = a.q + ((size_t)row0[g.b] * a.Hq + g.kvh * G + (head_ok ? gq : 0)) * kD * 2;
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
+        for (int ks = 0; ks < kD / 16; ++ks) {
             dst[ks][0] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + tq * 4)) : 0u;
             dst[ks][1] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + 16 + tq * 4)) : 0u;
             if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
@@ -664,7 +685,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             patch = last_pg >= s.pg0 && last_pg < s.pg1 && ((last_pg - s.pg0) % kCW) == warp;
             if (patch) {
                 const char *src = (lane < 16 ? a.k_new : a.v_new) + ((size_t)qrow * Hkv + s.kvh) * kD * 2 + (lane & 15) * 16;
-                new_row = __ldg(reinterpret_cast<const uint4 *>(src));
+                const bool in_row = (lane & 15) < kD / 8;
+                if (in_row) new_row = __ldg(reinterpret_cast<const uint4 *>(src));
                 const int pid = a.block_table[(size_t)s.b * a.max_pages + last_pg];
                 const bool store = (unsigned)pid < (unsigned)a.num_pages && ARB_IN_RANGE(a.status, qrow, a.rows);
                 // (a page outside the pool: the producer has raised ARB_DEV_BAD_PAGE; nothing is written)
@@ -714,7 +736,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                     }
                     new_row = make_uint4(e4m3x2_to_f16x2((uint16_t)code[0]), e4m3x2_to_f16x2((uint16_t)code[1]),
                                          e4m3x2_to_f16x2((uint16_t)code[2]), e4m3x2_to_f16x2((uint16_t)code[3]));
-                } else if (store) {
+                } else if (store && in_row) {
                     char *dst = (lane < 16 ? a.k_pool : a.v_pool) +
                                 (((size_t)pid * Hkv + s.kvh) * kPage + new_slot) * (kD * 2) + (lane & 15) * 16;
                     *reinterpret_cast<uint4 *>(dst) = new_row;
@@ -723,11 +745,11 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         }
 
         // this lane's columns (heads h0, h1): running max (the same in the 8 lanes of a column pair), its share of
-        // the sum, and 8 m-tiles of O^T: o[mt][0..1] = dim 16 mt + gq of heads h0, h1; o[mt][2..3] = dim + 8
+        // the sum, and the m-tiles of O^T: o[mt][0..1] = dim 16 mt + gq of heads h0, h1; o[mt][2..3] = dim + 8
         float m_run0 = -INFINITY, m_run1 = -INFINITY, l_run0 = 0.f, l_run1 = 0.f;
-        float o[8][4];
+        float o[kD / 16][4];
 #pragma unroll
-        for (int mt = 0; mt < 8; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
+        for (int mt = 0; mt < kD / 16; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
 
         for (int gi = warp; gi < seg_pages; gi += kCW) {
             const int pg = s.pg0 + gi;
@@ -756,7 +778,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                     tile_p = wide_k;
                 }
                 if (patch_here) {
-                    if (lane < 16) *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane)) = new_row;
+                    if (lane < kD / 8) *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane)) = new_row;
                     if constexpr (I4) {
                         const float ns = __shfl_sync(0xffffffffu, new_scale, 0);
                         if (gq == new_slot) ksc0 = ns;
@@ -766,7 +788,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 }
                 const uint32_t tile = smem_u32(tile_p);
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
+                for (int ks = 0; ks < kD / 16; ++ks) {
                     uint32_t af[4];   // rows: keys; matrices: (keys 0-7 | 8-15) x (dims 16 ks + 0-7 | 8-15)
                     ldmatrix_x4(tile + tile_off((lane & 7) + ((lane >> 3) & 1) * 8, 2 * ks + (lane >> 4)), af);
                     if (ks & 1) mma_16816<E4M3>(sb, af, qb[ks][0], qb[ks][1]);
@@ -804,7 +826,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             const float p10 = fast_exp2(s10 - mn0), p11 = fast_exp2(s11 - mn1);
             uint32_t w0 = E4M3 ? pack_f16(p00, p01) : pack_bf16(p00, p01);   // key gq:     heads h0, h1
             uint32_t w1 = E4M3 ? pack_f16(p10, p11) : pack_bf16(p10, p11);   // key gq + 8
-            if constexpr (I4) {   // (the weights that reach the tensor core carry the value scales: packed below)
+            if constexpr (I4 || SPLIT_P) {   // (4-bit: the weights that reach the tensor core carry the value scales, packed below)
                 l_run0 = fmaf(l_run0, f0, p00 + p10);
                 l_run1 = fmaf(l_run1, f1, p01 + p11);
             } else if constexpr (E4M3) {
@@ -816,17 +838,21 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 l_run1 = fmaf(l_run1, f1, __uint_as_float(w0 & 0xffff0000u) + __uint_as_float(w1 & 0xffff0000u));
             }
             // B fragment of P^T (16 keys x 8 heads): keys 2 tq, + 1 (and + 8) of head gq
-            uint32_t pb0 = 0, pb1 = 0;
+            uint32_t pb0 = 0, pb1 = 0, lb0 = 0, lb1 = 0;
             if constexpr (!I4) {
                 pb0 = movmatrix_trans(w0);
                 pb1 = movmatrix_trans(w1);
             }
+            if constexpr (SPLIT_P) {   // what the rounding to bf16 left over
+                lb0 = movmatrix_trans(pack_bf16(p00 - __uint_as_float(w0 << 16), p01 - __uint_as_float(w0 & 0xffff0000u)));
+                lb1 = movmatrix_trans(pack_bf16(p10 - __uint_as_float(w1 << 16), p11 - __uint_as_float(w1 & 0xffff0000u)));
+            }
             if (__any_sync(0xffffffffu, f0 != 1.0f || f1 != 1.0f)) {
 #pragma unroll
-                for (int mt = 0; mt < 8; ++mt) { o[mt][0] *= f0; o[mt][1] *= f1; o[mt][2] *= f0; o[mt][3] *= f1; }
+                for (int mt = 0; mt < kD / 16; ++mt) { o[mt][0] *= f0; o[mt][1] *= f1; o[mt][2] *= f0; o[mt][3] *= f1; }
             }
 
-            // ---- O^T += V^T P^T: 8 m-tiles of 16 dims ---------------------------------------------------
+            // ---- O^T += V^T P^T: m-tiles of 16 dims ---------------------------------------------------
             {
                 const uint32_t cv = ck + 1u, st = cv % STAGES, par = (cv / STAGES) & 1u;
                 mbar_wait(&tail->full[st], par, abort, a.status);
@@ -845,7 +871,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                     tile_p = wide_v;
                 }
                 if (patch_here) {
-                    if (lane >= 16) *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane - 16)) = new_row;
+                    if (lane >= 16 && lane - 16 < kD / 8)
+                        *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane - 16)) = new_row;
                     if constexpr (I4) {
                         const float ns = __shfl_sync(0xffffffffu, new_scale, 16);
                         if (gq == new_slot) vsc0 = ns;
@@ -862,16 +889,17 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 if (ntok < kPage) {
                     // slots past the sequence end may hold anything; they must not reach the tensor core, not even
                     // times zero: blank them in shared memory
-                    for (int i = lane; i < (kPage - ntok) * 16; i += 32)
-                        *reinterpret_cast<uint4 *>(tile_p + tile_off(ntok + (i >> 4), i & 15)) = make_uint4(0, 0, 0, 0);
+                    for (int i = lane; i < (kPage - ntok) * (kD / 8); i += 32)
+                        *reinterpret_cast<uint4 *>(tile_p + tile_off(ntok + i / (kD / 8), i % (kD / 8))) = make_uint4(0, 0, 0, 0);
                     __syncwarp();
                 }
                 const uint32_t tile = smem_u32(tile_p);
 #pragma unroll
-                for (int mt = 0; mt < 8; ++mt) {
+                for (int mt = 0; mt < kD / 16; ++mt) {
                     uint32_t af[4];   // transposed on the way: rows dims (16 mt + 0-7 | 8-15), columns keys (0-7 | 8-15)
                     ldmatrix_x4_trans(tile + tile_off((lane & 7) + (lane >> 4) * 8, 2 * mt + ((lane >> 3) & 1)), af);
                     mma_16816<E4M3>(o[mt], af, pb0, pb1);
+                    if constexpr (SPLIT_P) mma_16816<false>(o[mt], af, lb0, lb1);
                 }
                 __syncwarp();
                 if constexpr (!WIDE) {
@@ -894,7 +922,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             rec[8 + h0] = l_run0; rec[8 + h1] = l_run1;
         }
 #pragma unroll
-        for (int mt = 0; mt < 8; ++mt) {
+        for (int mt = 0; mt < kD / 16; ++mt) {
             const int d = 16 * mt + gq;
             if (h0 < G) { rec[16 + h0 * kOStride + d] = o[mt][0]; rec[16 + h0 * kOStride + d + 8] = o[mt][2]; }
             if (h1 < G) { rec[16 + h1 * kOStride + d] = o[mt][1]; rec[16 + h1 * kOStride + d + 8] = o[mt][3]; }
@@ -927,7 +955,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         s = s_next;
         have = have_next;
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) { qb[ks][0] = qn[ks][0]; qb[ks][1] = qn[ks][1]; }
+        for (int ks = 0; ks < kD / 16; ++ks) { qb[ks][0] = qn[ks][0]; qb[ks][1] = qn[ks][1]; }
     }
     if (n_parked > 0) flush();
 
@@ -1026,16 +1054,17 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
 // Ring stages.  What is in flight per SM is stages x bytes of a stage, and it has to cover latency x bandwidth: 32 tiles
 // of a bf16 cache are 128 KB; the tiles of the code caches are 2 KB and 1.1 KB, so their rings are deeper (with 32
 // stages a large call over 4-bit codes could keep 16 KB per SM in flight: 1.4 TB/s).  The widened tiles of the code
-// forms take 64 KB beside the ring.
-template <int KV>
-constexpr int stages_of() { return KV == kKvBf16 ? 32 : KV == kKvE4m3 ? 48 : 80; }
+// forms take 64 KB beside the ring.  Tiles of 64-dimension heads are 2 KB: 64 stages keep the same 128 KB in flight.
+template <int KV, int HD>
+constexpr int stages_of() { return KV == kKvBf16 ? (HD == 64 ? 64 : 32) : KV == kKvE4m3 ? 48 : 80; }
 
-template <int G, bool APPEND, int KV>
+template <int G, bool APPEND, int KV, int HD = 128>
 arb_status launch_variant(Ctx *ctx, const StepArgs &a, const CUtensorMap &km, const CUtensorMap &vm, cudaStream_t stream) {
+    constexpr int STAGES = stages_of<KV, HD>();
     static bool attr_set[64] = {};
     if (!attr_set[ctx->device & 63]) {
-        if (cudaFuncSetAttribute(decode_step_kernel<G, stages_of<KV>(), APPEND, KV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem_bytes<G, stages_of<KV>(), KV>(kMaxBatch)) != cudaSuccess)
+        if (cudaFuncSetAttribute(decode_step_kernel<G, STAGES, APPEND, KV, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem_bytes<G, STAGES, KV, HD>(kMaxBatch)) != cudaSuccess)
             return ARB_ERR_CUDA;
         attr_set[ctx->device & 63] = true;
     }
@@ -1044,21 +1073,25 @@ arb_status launch_variant(Ctx *ctx, const StepArgs &a, const CUtensorMap &km, co
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctx->num_sms);
-    cfg.blockDim = dim3(kNT);
-    cfg.dynamicSmemBytes = smem_bytes<G, stages_of<KV>(), KV>(a.batch);
+    cfg.blockDim = dim3(step_threads<KV, HD>());
+    cfg.dynamicSmemBytes = smem_bytes<G, STAGES, KV, HD>(a.batch);
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, decode_step_kernel<G, stages_of<KV>(), APPEND, KV>, a, km, vm) != cudaSuccess) return ARB_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, decode_step_kernel<G, STAGES, APPEND, KV, HD>, a, km, vm) != cudaSuccess) return ARB_ERR_CUDA;
     ctx->launches++;
     return ARB_OK;
 }
 
 // The E4M3 and the 4-bit forms exist with the cache write only (decode alone over an E4M3 cache is arb_attn_decode_e4m3).
 template <int G>
-arb_status launch_g(Ctx *ctx, const StepArgs &a, int kv, const CUtensorMap &km, const CUtensorMap &vm, cudaStream_t stream) {
+arb_status launch_g(Ctx *ctx, const StepArgs &a, int kv, int head_dim, const CUtensorMap &km, const CUtensorMap &vm,
+                    cudaStream_t stream) {
     if (kv == kKvE4m3) return launch_variant<G, true, kKvE4m3>(ctx, a, km, vm, stream);
     if (kv == kKvI4) return launch_variant<G, true, kKvI4>(ctx, a, km, vm, stream);
+    if (head_dim == 64)
+        return a.k_new != nullptr ? launch_variant<G, true, kKvBf16, 64>(ctx, a, km, vm, stream)
+                                  : launch_variant<G, false, kKvBf16, 64>(ctx, a, km, vm, stream);
     return a.k_new != nullptr ? launch_variant<G, true, kKvBf16>(ctx, a, km, vm, stream)
                               : launch_variant<G, false, kKvBf16>(ctx, a, km, vm, stream);
 }
@@ -1069,7 +1102,7 @@ size_t decode_step_hint_bytes(int num_sms) { return sizeof(int) * (size_t)num_sm
 
 bool decode_step_supported(const arb_attn_params &p) {
     const int g = p.num_q_heads / p.num_kv_heads;
-    return p.dtype == ARB_BF16 && p.head_dim == kD && g >= 1 && g <= 8 && tma_available();
+    return p.dtype == ARB_BF16 && (p.head_dim == 64 || p.head_dim == 128) && g >= 1 && g <= 8 && tma_available();
 }
 
 // k_new == nullptr: attention only (seq_lens is not written).  scales != nullptr: an E4M3 cache with scales =
@@ -1091,6 +1124,10 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
     } else if (e4m3) {
         if (!pool_map(ctx, &km, k_pages, p.num_pages, p.num_kv_heads, PoolView::kE4m3) ||
             !pool_map(ctx, &vm, v_pages, p.num_pages, p.num_kv_heads, PoolView::kE4m3))
+            return ARB_ERR_CUDA;
+    } else if (p.head_dim == 64) {
+        if (!pool_map(ctx, &km, k_pages, p.num_pages, p.num_kv_heads, PoolView::kBf16D64) ||
+            !pool_map(ctx, &vm, v_pages, p.num_pages, p.num_kv_heads, PoolView::kBf16D64))
             return ARB_ERR_CUDA;
     } else {
         whole_rows = pool_map(ctx, &km, k_pages, p.num_pages, p.num_kv_heads, PoolView::kBf16WholeRows) &&
@@ -1143,14 +1180,14 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
     a.v_scales = v_row_scales;
     const int kv = i4 ? kKvI4 : e4m3 ? kKvE4m3 : kKvBf16;
     switch (g) {
-        case 1: return launch_g<1>(ctx, a, kv, km, vm, stream);
-        case 2: return launch_g<2>(ctx, a, kv, km, vm, stream);
-        case 3: return launch_g<3>(ctx, a, kv, km, vm, stream);
-        case 4: return launch_g<4>(ctx, a, kv, km, vm, stream);
-        case 5: return launch_g<5>(ctx, a, kv, km, vm, stream);
-        case 6: return launch_g<6>(ctx, a, kv, km, vm, stream);
-        case 7: return launch_g<7>(ctx, a, kv, km, vm, stream);
-        case 8: return launch_g<8>(ctx, a, kv, km, vm, stream);
+        case 1: return launch_g<1>(ctx, a, kv, p.head_dim, km, vm, stream);
+        case 2: return launch_g<2>(ctx, a, kv, p.head_dim, km, vm, stream);
+        case 3: return launch_g<3>(ctx, a, kv, p.head_dim, km, vm, stream);
+        case 4: return launch_g<4>(ctx, a, kv, p.head_dim, km, vm, stream);
+        case 5: return launch_g<5>(ctx, a, kv, p.head_dim, km, vm, stream);
+        case 6: return launch_g<6>(ctx, a, kv, p.head_dim, km, vm, stream);
+        case 7: return launch_g<7>(ctx, a, kv, p.head_dim, km, vm, stream);
+        case 8: return launch_g<8>(ctx, a, kv, p.head_dim, km, vm, stream);
         default: return ARB_ERR_UNSUPPORTED;
     }
 }

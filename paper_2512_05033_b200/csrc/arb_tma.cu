@@ -40,11 +40,11 @@ struct MapEntry {
 
 bool tma_available() { return encode_tiled_fn() != nullptr; }
 
-bool encode_pool_map(CUtensorMap *map, const void *pool, int num_pages, int num_kv_heads, bool e4m3) {
+bool encode_pool_map(CUtensorMap *map, const void *pool, int num_pages, int num_kv_heads, int head_dim, bool e4m3) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)kD, (cuuint64_t)num_pages * num_kv_heads * kPage};
-    const cuuint64_t strides[1] = {(cuuint64_t)kD * (e4m3 ? 1 : 2)};
+    const cuuint64_t dims[2] = {(cuuint64_t)head_dim, (cuuint64_t)num_pages * num_kv_heads * kPage};
+    const cuuint64_t strides[1] = {(cuuint64_t)head_dim * (e4m3 ? 1 : 2)};
     const cuuint32_t box[2] = {(cuuint32_t)(e4m3 ? kD : 64), (cuuint32_t)kPage};
     const cuuint32_t estr[2] = {1, 1};
     return fn(map, e4m3 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
@@ -86,7 +86,7 @@ namespace {
 bool encode_view(CUtensorMap *map, const void *pool, int num_pages, int num_kv_heads, PoolView view) {
     if (view == PoolView::kI4) return encode_pool_map_i4(map, pool, num_pages, num_kv_heads);
     if (view == PoolView::kBf16WholeRows) return encode_pool_map3(map, pool, num_pages, num_kv_heads);
-    return encode_pool_map(map, pool, num_pages, num_kv_heads, view == PoolView::kE4m3);
+    return encode_pool_map(map, pool, num_pages, num_kv_heads, view == PoolView::kBf16D64 ? 64 : kD, view == PoolView::kE4m3);
 }
 }  // namespace
 

@@ -631,3 +631,29 @@ def test_e4m3_chunk_peaked_and_bad_lengths():
     assert c.poll_status() == binding.DEV_BAD_SEQ_LEN
     assert float(out2[40:47].abs().max()) == 0.0
     assert torch.equal(out2[:40], out[:40]) and torch.equal(out2[47:], out[47:])
+
+
+HEAD64_CASES = [
+    # (Hq, Hkv, seq_lens, q_lens): bf16, head_dim 64, on the tensor cores
+    (4, 4, [2, 16, 129], [2, 3, 17]),                        # g = 1: smallest chunks, a chunk that is the whole sequence
+    (32, 8, [300, 5000, 77, 256], [64, 1, 30, 128]),         # g = 4: full row tiles, lone tiles, a decode row
+    (14, 2, [1300, 128, 127], [19, 18, 37]),                 # g = 7: 133, 126 and 259 rows, around one and two row tiles
+    (16, 2, [2600, 1100], [33, 1]),                          # g = 8: few items, cut over the keys
+    (8, 1, [26000], [40]),                                   # a long sequence, split and merged
+    (12, 2, [1, 17, 3001, 640], [1, 1, 1, 1]),               # decode rows only
+]
+
+
+@pytest.mark.parametrize("q_std", [1.0, 5.0])
+@pytest.mark.parametrize("case", HEAD64_CASES)
+def test_head64_on_the_tensor_cores_matches_oracle(case, q_std):
+    """The weights enter the second product as two bf16 terms (relative 2^-17 left over), so the error is the rounding
+    of the output, half an ulp = 2^-9 relative, and the fp32 path: the bar of the CUDA-core kernels, peaked too."""
+    Hq, Hkv, sl, ql = case
+    inp = wl.small_attn_case(len(sl), Hq, Hkv, 64, BF, sl, ql, seed=640 + Hq, q_std=q_std)
+    out, bits = H.gpu_attn(inp)
+    ref, st = H.oracle_attn(inp)
+    assert bits == 0 and st == 0
+    assert np.isfinite(out).all()
+    err = np.abs(out - ref)
+    assert (err <= 2.0 ** -8 * np.abs(ref) + 1e-3).all(), err.max()

@@ -55,7 +55,9 @@ STEP_CASES = [
     (2, 8, 8, 128, BF, [260, 100], [1, 1]),                             # g = 1
     (16, 32, 8, 128, BF, [100 * i + 7 for i in range(16)], [1] * 16),   # many short segments per CTA
     (1, 8, 2, 64, F32, [512], [1]),                                     # the tiny config's shape: two launches inside
-    (2, 6, 2, 64, BF, [700, 70], [1, 1]),                               # bf16, head_dim 64: two launches inside
+    (2, 6, 2, 64, BF, [700, 70], [1, 1]),                               # bf16, head_dim 64
+    (5, 32, 8, 64, BF, [0, 15, 16, 4001, 9000], [1, 1, 1, 1, 1]),       # ... an empty sequence, page edges, long ones
+    (3, 16, 2, 64, BF, [2100, 900, 31], [1, 0, 1]),                     # ... g = 8, an idle slot
 ]
 
 
