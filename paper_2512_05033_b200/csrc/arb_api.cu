@@ -248,8 +248,9 @@ arb_status arb_attn(arb_ctx *ctx, const arb_attn_params *params, const void *q, 
         if (st != ARB_OK) return st;
     }
     if (params->max_q_len >= 2) {
-        // Step chunks: bf16 chunks go to the tcgen05 kernel (from kChunkMmaMinRows rows on, i.e. all of them),
-        // fp32 chunks to the CUDA-core kernel.  Both kernels decide per sequence on the device.
+        // Step chunks: fp32 chunks have a kernel of their own; bf16 chunks go to the tcgen05 kernel (from
+        // kChunkMmaMinRows rows on, i.e. all of them).  The kernels decide per sequence on the device.
+        if (params->dtype == ARB_F32) return launch_chunk_f32(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
         int skip_rows = 0;
         if (tensor_cores && chunk_mma_supported(*params)) {
             st = launch_chunk_mma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);

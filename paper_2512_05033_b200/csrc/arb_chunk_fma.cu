@@ -1,7 +1,6 @@
 // Step-chunk attention, CUDA-core path: one CTA per (query row, kv head).
 //
-// This is the path for chunks the tensor-core kernel does not take: fp32 inputs (whose 1e-5 tolerance
-// rules out tf32), head_dim 64, groups above 8, and every chunk when ARB_ATTN_NO_TENSOR_CORES is set.  It
+// This is the path of every bf16 chunk when ARB_ATTN_NO_TENSOR_CORES is set (for comparison: fp32 weights).  It
 // also zero-fills the rows of chunk sequences whose lengths are invalid, whatever their size.  Query token i of
 // a chunk of n tokens sits at position pos = L - n + i and attends keys 0..pos; the causal mask is
 // just each row's own key count.  K and V rows are read straight from global memory with 16-byte
@@ -267,9 +266,6 @@ arb_status launch_chunk_fma(Ctx *ctx, const arb_attn_params &p, const void *q, c
     if (p.dtype == ARB_BF16) {
         if (p.head_dim == 128) return launch_g<__nv_bfloat16, 128>(ctx, g, a, p.total_q, stream);
         if (p.head_dim == 64) return launch_g<__nv_bfloat16, 64>(ctx, g, a, p.total_q, stream);
-    } else if (p.dtype == ARB_F32) {
-        if (p.head_dim == 128) return launch_g<float, 128>(ctx, g, a, p.total_q, stream);
-        if (p.head_dim == 64) return launch_g<float, 64>(ctx, g, a, p.total_q, stream);
     }
     return ARB_ERR_UNSUPPORTED;
 }

@@ -297,6 +297,9 @@ arb_status launch_chunk_fma(Ctx *ctx, const arb_attn_params &p, const void *q, c
                             const void *v_pages, const int32_t *block_table, const int32_t *seq_lens,
                             const int32_t *q_lens, void *out, int n_lo, int n_hi, int skip_rows,
                             cudaStream_t stream);
+arb_status launch_chunk_f32(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages, const void *v_pages,
+                            const int32_t *block_table, const int32_t *seq_lens, const int32_t *q_lens, void *out,
+                            cudaStream_t stream);
 bool chunk_mma_supported(const arb_attn_params &p);
 bool decode_mma_supported(const arb_attn_params &p);
 arb_status launch_decode_mma(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages,

@@ -657,3 +657,38 @@ def test_head64_on_the_tensor_cores_matches_oracle(case, q_std):
     assert np.isfinite(out).all()
     err = np.abs(out - ref)
     assert (err <= 2.0 ** -8 * np.abs(ref) + 1e-3).all(), err.max()
+
+
+FP32_CHUNK_CASES = [
+    # (Hq, Hkv, D, seq_lens, q_lens): row tiles of 64, key tiles of 32, the list of units cut over the CTAs
+    (4, 4, 64, [2, 31, 32, 33], [2, 2, 31, 33]),             # g = 1: one key tile, its edges
+    (8, 2, 128, [1700, 900, 64], [100, 1, 16]),              # g = 4: ragged row tiles beside a decode row
+    (14, 2, 64, [3000, 640], [10, 19]),                      # g = 7: 70 and 133 rows, one and five beyond a tile
+    (16, 2, 128, [65, 4097], [8, 8]),                        # g = 8: exactly one row tile
+    (8, 1, 64, [9000], [2]),                                 # one row tile over every CTA: the longest merge
+]
+
+
+@pytest.mark.parametrize("ws", [0, 1_300_000])
+@pytest.mark.parametrize("case", FP32_CHUNK_CASES)
+def test_fp32_chunk_matches_oracle(case, ws):
+    """fp32 products and sums: 1e-5.  A small workspace has no room for partials: the row tiles stay whole.  Slots past
+    every row's position hold NaN."""
+    from paper_2512_05033_b200 import binding
+    Hq, Hkv, D, sl, ql = case
+    inp = wl.small_attn_case(len(sl), Hq, Hkv, D, F32, sl, ql, seed=320 + Hq, q_std=2.0, extra_tokens=20)
+    for b, L in enumerate(sl):
+        for j in range(L, L + 20):
+            pg = int(inp.block_table[b, j // wl.PAGE])
+            inp.k_pages[pg, :, j % wl.PAGE] = float("nan")
+            inp.v_pages[pg, :, j % wl.PAGE] = float("nan")
+    ref, st = H.oracle_attn(inp)
+    if ws == 0:
+        out, bits = H.gpu_attn(inp)
+    else:
+        c, d = binding.Context(0, workspace_bytes=ws), inp.to("cuda")
+        out = c.attn(d.q, d.k_pages, d.v_pages, d.block_table, d.seq_lens, d.q_lens, max(ql)).double().cpu().numpy()
+        bits = c.poll_status()
+        c.close()
+    assert bits == 0 and st == 0
+    H.assert_close(out, ref, F32)
