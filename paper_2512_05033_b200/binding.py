@@ -1,8 +1,10 @@
-"""ctypes binding of the C-ABI library ``libarb.so`` (``include/arb.h``).
+"""Binding of the C-ABI library ``libarb.so`` (``include/arb.h``).
 
 Argument marshalling only: every step of the path runs in the CUDA kernels.  torch supplies device
-memory and streams; raw pointers cross the boundary.  Importing this module fails loudly when the
-library has not been built (``python -m paper_2512_05033_b200.build``): there is no fallback.
+memory and streams; raw pointers cross the boundary.  The calls of a token's path go through the extension
+module ``_native`` (csrc/native_binding.cpp), which checks the tensors and calls the C ABI; set-up, the pointer-level calls
+and the self-tests through ctypes.  Importing this module fails loudly when either has not been built
+(``python -m paper_2512_05033_b200.build``): there is no fallback.
 """
 from __future__ import annotations
 
@@ -22,6 +24,12 @@ if not _LIB_PATH.exists():
         "(python -m paper_2512_05033_b200.build); there is no CPU fallback")
 
 lib = ctypes.CDLL(str(_LIB_PATH))
+
+try:
+    from . import _native
+except ImportError as e:
+    raise ImportError("the extension module _native is missing: build it first (python -m paper_2512_05033_b200.build)") from e
+_native.bind(lib._handle)
 
 ARB_OK = 0
 ARB_ERR_INVALID_ARG, ARB_ERR_UNSUPPORTED, ARB_ERR_WORKSPACE, ARB_ERR_CUDA, ARB_ERR_DEVICE_STATUS = 1, 2, 3, 4, 5
@@ -184,11 +192,13 @@ class Context:
         with torch.cuda.device(self.device):
             _check(lib.arb_create(ctypes.byref(h), self.device.index or 0, workspace_bytes), "arb_create")
         self._h = h
+        self._p = int(h.value)   # the handle as the extension module takes it
 
     def close(self):
         if getattr(self, "_h", None):
             lib.arb_destroy(self._h)
             self._h = None
+            self._p = None
 
     def __del__(self):
         try:
@@ -210,12 +220,10 @@ class Context:
         """out[total_q, Hq, D] = paged GQA attention; all tensors on the device.  Asynchronous."""
         if out is None:
             out = torch.empty_like(q)
-        p = params or self.params_for(q, k_pages, block_table, max_q_len, softmax_scale)
-        st = lib.arb_attn(self._h, ctypes.byref(p), _dev(q, "q"), _dev(k_pages, "k_pages", q.dtype),
-                          _dev(v_pages, "v_pages", q.dtype), _dev(block_table, "block_table", torch.int32),
-                          _dev(seq_lens, "seq_lens", torch.int32), _dev(q_lens, "q_lens", torch.int32),
-                          _dev(out, "out", q.dtype), _stream_ptr(stream))
-        _check(st, "arb_attn")
+        st = _native.attn(self._p, q, k_pages, v_pages, block_table, seq_lens, q_lens, max_q_len, out, softmax_scale, stream,
+                          params)
+        if st:
+            _check(st, "arb_attn")
         return out
 
     def attn_raw(self, p: AttnParams, q_ptr, k_ptr, v_ptr, bt_ptr, sl_ptr, ql_ptr, out_ptr, stream_ptr) -> int:
@@ -228,14 +236,10 @@ class Context:
         Synchronises the stream before returning."""
         if out_host is None:
             out_host = torch.empty_like(q_host, pin_memory=True)
-        for t in (q_host, block_table_host, seq_lens_host, q_lens_host, out_host):
-            if t.is_cuda or not t.is_contiguous():
-                raise ValueError("host tensors must be contiguous CPU tensors")
-        p = self.params_for(q_host, k_pages, block_table_host, max_q_len, softmax_scale)
-        st = lib.arb_attn_host(self._h, ctypes.byref(p), q_host.data_ptr(), _dev(k_pages, "k_pages"),
-                               _dev(v_pages, "v_pages"), block_table_host.data_ptr(), seq_lens_host.data_ptr(),
-                               q_lens_host.data_ptr(), out_host.data_ptr(), _stream_ptr(stream))
-        _check(st, "arb_attn_host")
+        st = _native.attn_host(self._p, q_host, k_pages, v_pages, block_table_host, seq_lens_host, q_lens_host, max_q_len,
+                               out_host, softmax_scale, 0, stream, 0)
+        if st:
+            _check(st, "arb_attn_host")
         return out_host
 
     def attn_host_raw(self, p: AttnParams, q_ptr, k_ptr, v_ptr, bt_ptr, sl_ptr, ql_ptr, out_ptr, stream_ptr) -> int:
@@ -246,15 +250,10 @@ class Context:
                         out_host, softmax_scale: float = 0.0, flags: int = 0, stream=None):
         """First half of the pipelined host call: enqueues copies and kernels and returns; out_host (pinned) holds
         the result once attn_host_wait() has returned."""
-        for t in (q_host, block_table_host, seq_lens_host, q_lens_host, out_host):
-            if t.is_cuda or not t.is_contiguous():
-                raise ValueError("host tensors must be contiguous CPU tensors")
-        p = self.params_for(q_host, k_pages, block_table_host, max_q_len, softmax_scale)
-        p.flags = flags
-        st = lib.arb_attn_host_begin(self._h, ctypes.byref(p), q_host.data_ptr(), _dev(k_pages, "k_pages"),
-                                     _dev(v_pages, "v_pages"), block_table_host.data_ptr(), seq_lens_host.data_ptr(),
-                                     q_lens_host.data_ptr(), out_host.data_ptr(), _stream_ptr(stream))
-        _check(st, "arb_attn_host_begin")
+        st = _native.attn_host(self._p, q_host, k_pages, v_pages, block_table_host, seq_lens_host, q_lens_host, max_q_len,
+                               out_host, softmax_scale, flags, stream, 1)
+        if st:
+            _check(st, "arb_attn_host_begin")
         return out_host
 
     def attn_host_begin_raw(self, p: AttnParams, q_ptr, k_ptr, v_ptr, bt_ptr, sl_ptr, ql_ptr, out_ptr, stream_ptr) -> int:
@@ -264,7 +263,7 @@ class Context:
 
     def attn_host_wait(self):
         """Blocks until every attn_host_begin of this context has delivered its result."""
-        _check(lib.arb_attn_host_wait(self._h), "arb_attn_host_wait")
+        _check(_native.attn_host_wait(self._p), "arb_attn_host_wait")
 
     # -- arb_decode_step ----------------------------------------------------------------------
     def decode_step(self, q, k_new, v_new, k_pages, v_pages, block_table, seq_lens, q_lens, out=None,
@@ -273,13 +272,10 @@ class Context:
         including them, seq_lens += q_lens (in place).  Asynchronous."""
         if out is None:
             out = torch.empty_like(q)
-        p = params or self.params_for(q, k_pages, block_table, 1, softmax_scale)
-        st = lib.arb_decode_step(self._h, ctypes.byref(p), _dev(q, "q"), _dev(k_new, "k_new", q.dtype),
-                                 _dev(v_new, "v_new", q.dtype), _dev(k_pages, "k_pages", q.dtype),
-                                 _dev(v_pages, "v_pages", q.dtype), _dev(block_table, "block_table", torch.int32),
-                                 _dev(seq_lens, "seq_lens", torch.int32), _dev(q_lens, "q_lens", torch.int32),
-                                 _dev(out, "out", q.dtype), _stream_ptr(stream))
-        _check(st, "arb_decode_step")
+        st = _native.decode_step(self._p, q, k_new, v_new, k_pages, v_pages, block_table, seq_lens, q_lens, out,
+                                 softmax_scale, stream, params)
+        if st:
+            _check(st, "arb_decode_step")
         return out
 
     # -- arb_decode_step_e4m3 -----------------------------------------------------------------
@@ -290,15 +286,10 @@ class Context:
         the codes including them, seq_lens += q_lens (in place).  Asynchronous."""
         if out is None:
             out = torch.empty_like(q)
-        p = params or self.params_for(q, k_codes, block_table, 1, softmax_scale)
-        st = lib.arb_decode_step_e4m3(self._h, ctypes.byref(p), _dev(q, "q", torch.bfloat16),
-                                      _dev(k_new, "k_new", torch.bfloat16), _dev(v_new, "v_new", torch.bfloat16),
-                                      _dev(k_codes, "k_codes", torch.uint8), _dev(v_codes, "v_codes", torch.uint8),
-                                      float(k_scale), float(v_scale), float(k_inv_scale), float(v_inv_scale),
-                                      _dev(block_table, "block_table", torch.int32),
-                                      _dev(seq_lens, "seq_lens", torch.int32), _dev(q_lens, "q_lens", torch.int32),
-                                      _dev(out, "out", torch.bfloat16), _stream_ptr(stream))
-        _check(st, "arb_decode_step_e4m3")
+        st = _native.decode_step_e4m3(self._p, q, k_new, v_new, k_codes, v_codes, k_scale, v_scale, k_inv_scale, v_inv_scale,
+                                      block_table, seq_lens, q_lens, out, softmax_scale, stream, params)
+        if st:
+            _check(st, "arb_decode_step_e4m3")
         return out
 
     # -- arb_decode_step_i4 -------------------------------------------------------------------
@@ -308,57 +299,37 @@ class Context:
         rows are quantised into the pools, out = attention over scale * code including them, seq_lens += q_lens."""
         if out is None:
             out = torch.empty_like(q)
-        if params is None:
-            num_pages, Hkv, P, _ = k_codes.shape
-            B, max_pages = block_table.shape
-            params = attn_params(_dtype_code(q), B, q.shape[1], Hkv, q.shape[2], num_pages, max_pages, q.shape[0], 1,
-                                 softmax_scale, P, 0)
-        st = lib.arb_decode_step_i4(self._h, ctypes.byref(params), _dev(q, "q", torch.bfloat16),
-                                    _dev(k_new, "k_new", torch.bfloat16), _dev(v_new, "v_new", torch.bfloat16),
-                                    _dev(k_codes, "k_codes", torch.uint8), _dev(v_codes, "v_codes", torch.uint8),
-                                    _dev(k_scales, "k_scales", torch.float32), _dev(v_scales, "v_scales", torch.float32),
-                                    _dev(block_table, "block_table", torch.int32),
-                                    _dev(seq_lens, "seq_lens", torch.int32), _dev(q_lens, "q_lens", torch.int32),
-                                    _dev(out, "out", torch.bfloat16), _stream_ptr(stream))
-        _check(st, "arb_decode_step_i4")
+        st = _native.decode_step_i4(self._p, q, k_new, v_new, k_codes, v_codes, k_scales, v_scales, block_table, seq_lens,
+                                    q_lens, out, softmax_scale, stream, params)
+        if st:
+            _check(st, "arb_decode_step_i4")
         return out
 
     # -- arb_kv_append_i4 ---------------------------------------------------------------------
     def kv_append_i4(self, k_new, v_new, block_table, seq_lens, new_lens, k_codes, v_codes, k_scales, v_scales,
                      update_lens: bool = True, stream=None):
         """In place: the new rows are quantised to the 4-bit format and written behind each sequence's tokens."""
-        num_pages, Hkv, P, half = k_codes.shape
-        B, max_pages = block_table.shape
-        p = attn_params(_dtype_code(k_new), B, Hkv, Hkv, 2 * half, num_pages, max_pages, 0, 0, 0.0, P, 0)
-        st = lib.arb_kv_append_i4(self._h, ctypes.byref(p), k_new.shape[0], _dev(k_new, "k_new", torch.bfloat16),
-                                  _dev(v_new, "v_new", torch.bfloat16), _dev(block_table, "block_table", torch.int32),
-                                  _dev(seq_lens, "seq_lens", torch.int32), _dev(new_lens, "new_lens", torch.int32),
-                                  1 if update_lens else 0, _dev(k_codes, "k_codes", torch.uint8),
-                                  _dev(v_codes, "v_codes", torch.uint8), _dev(k_scales, "k_scales", torch.float32),
-                                  _dev(v_scales, "v_scales", torch.float32), _stream_ptr(stream))
-        _check(st, "arb_kv_append_i4")
+        _check(_native.kv_append_i4(self._p, k_new, v_new, block_table, seq_lens, new_lens, k_codes, v_codes, k_scales,
+                                    v_scales, 1 if update_lens else 0, stream), "arb_kv_append_i4")
 
     # -- arb_route ----------------------------------------------------------------------------
     def route(self, hidden, w, b: float, tau: float, scores=None, decisions=None, stream=None):
         """scores fp32 [S] = sigmoid(hidden . w + b); decisions uint8 [S] = (score > tau)."""
-        S, H = hidden.shape
         if scores is None:
-            scores = torch.empty(S, dtype=torch.float32, device=hidden.device)
+            scores = torch.empty(hidden.shape[0], dtype=torch.float32, device=hidden.device)
         if decisions is None:
-            decisions = torch.empty(S, dtype=torch.uint8, device=hidden.device)
-        st = lib.arb_route(self._h, _dtype_code(hidden), S, H, _dev(hidden, "hidden"), _dev(w, "w", hidden.dtype),
-                           float(b), float(tau), _dev(scores, "scores", torch.float32),
-                           _dev(decisions, "decisions", torch.uint8), _stream_ptr(stream))
-        _check(st, "arb_route")
+            decisions = torch.empty(hidden.shape[0], dtype=torch.uint8, device=hidden.device)
+        st = _native.route(self._p, hidden, w, b, tau, scores, decisions, stream)
+        if st:
+            _check(st, "arb_route")
         return scores, decisions
 
     # -- arb_rollback -------------------------------------------------------------------------
     def rollback(self, seq_lens, step_lens, decisions=None, stream=None):
         """In place: seq_lens[i] -= step_lens[i] where decisions is None or decisions[i] != 0."""
-        dp = None if decisions is None else _dev(decisions, "decisions", torch.uint8)
-        st = lib.arb_rollback(self._h, seq_lens.shape[0], _dev(seq_lens, "seq_lens", torch.int32),
-                              _dev(step_lens, "step_lens", torch.int32), dp, _stream_ptr(stream))
-        _check(st, "arb_rollback")
+        st = _native.rollback(self._p, seq_lens, step_lens, decisions, stream)
+        if st:
+            _check(st, "arb_rollback")
         return seq_lens
 
     # -- arb_attn_decode_e4m3 -----------------------------------------------------------------
@@ -367,13 +338,10 @@ class Context:
         """Decode attention (q_len 1 or 0) over an E4M3 cache; q and out bf16.  Asynchronous."""
         if out is None:
             out = torch.empty_like(q)
-        p = params or self.params_for(q, k_codes, block_table, 1, softmax_scale, flags=flags)
-        st = lib.arb_attn_decode_e4m3(self._h, ctypes.byref(p), _dev(q, "q", torch.bfloat16),
-                                      _dev(k_codes, "k_codes", torch.uint8), _dev(v_codes, "v_codes", torch.uint8),
-                                      float(k_scale), float(v_scale), _dev(block_table, "block_table", torch.int32),
-                                      _dev(seq_lens, "seq_lens", torch.int32), _dev(q_lens, "q_lens", torch.int32),
-                                      _dev(out, "out", torch.bfloat16), _stream_ptr(stream))
-        _check(st, "arb_attn_decode_e4m3")
+        st = _native.attn_e4m3(self._p, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, 1, out,
+                               softmax_scale, flags, stream, params, 1)
+        if st:
+            _check(st, "arb_attn_decode_e4m3")
         return out
 
     # -- arb_attn_e4m3 ------------------------------------------------------------------------
@@ -382,29 +350,20 @@ class Context:
         """Attention (decode rows and step chunks) over an E4M3 cache; q and out bf16.  Asynchronous."""
         if out is None:
             out = torch.empty_like(q)
-        p = params or self.params_for(q, k_codes, block_table, max_q_len, softmax_scale)
-        st = lib.arb_attn_e4m3(self._h, ctypes.byref(p), _dev(q, "q", torch.bfloat16),
-                               _dev(k_codes, "k_codes", torch.uint8), _dev(v_codes, "v_codes", torch.uint8),
-                               float(k_scale), float(v_scale), _dev(block_table, "block_table", torch.int32),
-                               _dev(seq_lens, "seq_lens", torch.int32), _dev(q_lens, "q_lens", torch.int32),
-                               _dev(out, "out", torch.bfloat16), _stream_ptr(stream))
-        _check(st, "arb_attn_e4m3")
+        st = _native.attn_e4m3(self._p, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, max_q_len, out,
+                               softmax_scale, 0, stream, params, 0)
+        if st:
+            _check(st, "arb_attn_e4m3")
         return out
 
     # -- arb_kv_append_e4m3 -------------------------------------------------------------------
     def kv_append_e4m3(self, k_new, v_new, k_inv_scale: float, v_inv_scale: float, block_table, seq_lens, new_lens,
                        k_codes, v_codes, update_lens: bool = True, stream=None):
         """In place: the new rows are quantised to E4M3 (x * inv_scale) and written behind each sequence's tokens."""
-        num_pages, Hkv, P, D = k_codes.shape
-        B, max_pages = block_table.shape
-        p = attn_params(_dtype_code(k_new), B, Hkv, Hkv, D, num_pages, max_pages, 0, 0, 0.0, P, 0)
-        st = lib.arb_kv_append_e4m3(self._h, ctypes.byref(p), k_new.shape[0], _dev(k_new, "k_new"),
-                                    _dev(v_new, "v_new", k_new.dtype), float(k_inv_scale), float(v_inv_scale),
-                                    _dev(block_table, "block_table", torch.int32), _dev(seq_lens, "seq_lens", torch.int32),
-                                    _dev(new_lens, "new_lens", torch.int32), 1 if update_lens else 0,
-                                    _dev(k_codes, "k_codes", torch.uint8), _dev(v_codes, "v_codes", torch.uint8),
-                                    _stream_ptr(stream))
-        _check(st, "arb_kv_append_e4m3")
+        st = _native.kv_append_e4m3(self._p, k_new, v_new, k_inv_scale, v_inv_scale, block_table, seq_lens, new_lens, k_codes,
+                                    v_codes, 1 if update_lens else 0, stream)
+        if st:
+            _check(st, "arb_kv_append_e4m3")
         return seq_lens
 
     # -- arb_spearman -------------------------------------------------------------------------
@@ -412,9 +371,7 @@ class Context:
         """rho (device float64 [1]) = Spearman's rank correlation of two fp32 device vectors."""
         if rho is None:
             rho = torch.empty(1, dtype=torch.float64, device=x.device)
-        st = lib.arb_spearman(self._h, x.shape[0], _dev(x, "x", torch.float32), _dev(y, "y", torch.float32),
-                              _dev(rho, "rho", torch.float64), _stream_ptr(stream))
-        _check(st, "arb_spearman")
+        _check(_native.spearman(self._p, x, y, rho, stream), "arb_spearman")
         return rho
 
     # -- arb_phase_lens -----------------------------------------------------------------------
@@ -422,21 +379,18 @@ class Context:
         """out int32 [B]: lengths of the next call of a phase of the step loop (see arb_phase_lens)."""
         if out is None:
             out = torch.empty_like(step_lens)
-        dp = None if decisions is None else _dev(decisions, "decisions", torch.uint8)
-        st = lib.arb_phase_lens(self._h, step_lens.shape[0], _dev(step_lens, "step_lens", torch.int32), dp, int(want),
-                                int(t), _dev(out, "out", torch.int32), _stream_ptr(stream))
-        _check(st, "arb_phase_lens")
+        st = _native.phase_lens(self._p, step_lens, decisions, want, t, -1, out, stream)
+        if st:
+            _check(st, "arb_phase_lens")
         return out
 
     def phase_lens_tokens(self, step_lens, n_tokens: int, decisions=None, want: int = 1, out=None, stream=None):
         """out int32 [n_tokens, B]: row t = phase_lens(..., t=t), all rows in one launch."""
-        B = step_lens.shape[0]
         if out is None:
-            out = torch.empty(n_tokens, B, dtype=torch.int32, device=step_lens.device)
-        dp = None if decisions is None else _dev(decisions, "decisions", torch.uint8)
-        st = lib.arb_phase_lens_tokens(self._h, B, _dev(step_lens, "step_lens", torch.int32), dp, int(want), int(n_tokens),
-                                       _dev(out, "out", torch.int32), _stream_ptr(stream))
-        _check(st, "arb_phase_lens_tokens")
+            out = torch.empty(n_tokens, step_lens.shape[0], dtype=torch.int32, device=step_lens.device)
+        st = _native.phase_lens(self._p, step_lens, decisions, want, -1, n_tokens, out, stream)
+        if st:
+            _check(st, "arb_phase_lens_tokens")
         return out
 
     # -- arb_policy ---------------------------------------------------------------------------
@@ -445,14 +399,11 @@ class Context:
         """Escalation decisions uint8 [N] from PRM scores (fp32 device tensors).  `stats`, if given, is a
         device tensor of 3 float64 that receives the arb_policy_stats record (two uint32 counters, then the
         realised score and the gain); read it with policy_stats()."""
-        n = s_d.shape[0]
         if decisions is None:
-            decisions = torch.empty(n, dtype=torch.uint8, device=s_d.device)
-        sp = None if stats is None else _dev(stats, "stats", torch.float64)
-        tp = None if s_t is None else _dev(s_t, "s_t", torch.float32)
-        st = lib.arb_policy(self._h, kind, n, _dev(s_d, "s_d", torch.float32), tp, float(tau), int(budget),
-                            _dev(decisions, "decisions", torch.uint8), sp, _stream_ptr(stream))
-        _check(st, "arb_policy")
+            decisions = torch.empty(s_d.shape[0], dtype=torch.uint8, device=s_d.device)
+        st = _native.policy(self._p, kind, s_d, s_t, tau, budget, decisions, stats, stream)
+        if st:
+            _check(st, "arb_policy")
         return decisions
 
     @staticmethod
@@ -471,36 +422,24 @@ class Context:
     def route_classes(self, mode: int, hidden, w, b, tau: float, probs=None, scores=None, decisions=None,
                       stream=None):
         """C-way head: returns (probs fp32 [S, C], scores fp32 [S], decisions uint8 [S]).  b: C host floats."""
-        S, H = hidden.shape
-        C = len(b)
+        S, b = hidden.shape[0], tuple(float(x) for x in b)
         if probs is None:
-            probs = torch.empty(S, C, dtype=torch.float32, device=hidden.device)
+            probs = torch.empty(S, len(b), dtype=torch.float32, device=hidden.device)
         if scores is None:
             scores = torch.empty(S, dtype=torch.float32, device=hidden.device)
         if decisions is None:
             decisions = torch.empty(S, dtype=torch.uint8, device=hidden.device)
-        bh = (ctypes.c_float * C)(*[float(x) for x in b])
-        st = lib.arb_route_classes(self._h, _dtype_code(hidden), mode, S, H, C, _dev(hidden, "hidden"),
-                                   _dev(w, "w", hidden.dtype), bh, float(tau), _dev(probs, "probs", torch.float32),
-                                   _dev(scores, "scores", torch.float32), _dev(decisions, "decisions", torch.uint8),
-                                   _stream_ptr(stream))
-        _check(st, "arb_route_classes")
+        _check(_native.route_classes(self._p, mode, hidden, w, b, tau, probs, scores, decisions, stream), "arb_route_classes")
         return probs, scores, decisions
 
     # -- arb_kv_append ------------------------------------------------------------------------
     def kv_append(self, k_new, v_new, block_table, seq_lens, new_lens, k_pages, v_pages, update_lens: bool = True,
                   stream=None):
         """In place: the new tokens' K/V go behind each sequence's cached tokens; seq_lens += new_lens."""
-        num_pages, Hkv, P, D = k_pages.shape
-        B, max_pages = block_table.shape
-        p = attn_params(_dtype_code(k_pages), B, Hkv, Hkv, D, num_pages, max_pages, 0, 0, 0.0, P, 0)
-        total_new = k_new.shape[0]
-        st = lib.arb_kv_append(self._h, ctypes.byref(p), total_new, _dev(k_new, "k_new", k_pages.dtype),
-                               _dev(v_new, "v_new", k_pages.dtype), _dev(block_table, "block_table", torch.int32),
-                               _dev(seq_lens, "seq_lens", torch.int32), _dev(new_lens, "new_lens", torch.int32),
-                               1 if update_lens else 0, _dev(k_pages, "k_pages"), _dev(v_pages, "v_pages", k_pages.dtype),
-                               _stream_ptr(stream))
-        _check(st, "arb_kv_append")
+        st = _native.kv_append(self._p, k_new, v_new, block_table, seq_lens, new_lens, k_pages, v_pages,
+                               1 if update_lens else 0, stream)
+        if st:
+            _check(st, "arb_kv_append")
         return seq_lens
 
     # -- self-test ----------------------------------------------------------------------------

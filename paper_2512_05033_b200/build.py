@@ -1,4 +1,5 @@
-"""Build libarb.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Build libarb.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _native.so (the per-call part of the
+Python binding) with g++ against torch's headers.
 
     python -m paper_2512_05033_b200.build [--force] [--verbose] [--checks]
 
@@ -9,9 +10,11 @@ ARB_LIB_VARIANT=checks is set; it is for test runs, not for timing.
 from __future__ import annotations
 
 import concurrent.futures
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 from pathlib import Path
 
 HERE = Path(__file__).resolve().parent
@@ -60,7 +63,22 @@ def build(force: bool = False, verbose: bool = False, checks: bool = False) -> P
         subprocess.check_call([NVCC, "-shared", "-Wno-deprecated-gpu-targets", "-o", str(tmp), *map(str, objs),
                                "-lcudart"])
         os.replace(tmp, LIB)
+    build_native(force)
     return LIB
+
+
+def build_native(force: bool = False) -> Path:
+    src, out = CSRC / "native_binding.cpp", HERE / "_native.so"
+    if force or _stale(out, [src, HERE.parent / "include" / "arb.h"]):
+        torch_dir = Path(importlib.util.find_spec("torch").origin).parent   # not imported: only its headers and libraries
+        inc, lib = torch_dir / "include", torch_dir / "lib"
+        tmp = out.with_suffix(f".tmp{os.getpid()}.so")
+        subprocess.check_call(["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden",
+                               f"-I{sysconfig.get_paths()['include']}", f"-I{inc}", f"-I{inc / 'torch/csrc/api/include'}",
+                               f"-I{Path(NVCC).parent.parent / 'include'}", str(src), "-o", str(tmp), f"-L{lib}",
+                               "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+        os.replace(tmp, out)
+    return out
 
 
 if __name__ == "__main__":
