@@ -25,16 +25,25 @@
 //     tile in shared memory (the tile arrives with whatever the slot held) and stores it to the pool; the
 //     lengths move forward once every CTA has read them (a counter in the prologue tells the last reader).
 //
-// The template parameter KV names the cache.  Compiled a second time (KV = E4M3) the kernel serves an E4M3 cache (arb_decode_step_e4m3: the token
-// of a quantised draft).  A page tile is 2 KB of codes; the consumer warp that owns it widens it to f16 (exact) into
-// a tile of its own in shared memory, laid out like a bf16 tile, frees the ring stage at once, and runs the same
-// fragment loads and MMAs on f16 operands (q converted bf16 -> f16, P rounded to f16).  The token's new rows are
+// The template parameter KV names the cache.  Compiled a second time (KV = E4M3) the kernel serves an E4M3 cache
+// (arb_decode_step_e4m3: the token of a quantised draft).  A page tile is 2 KB of codes, widened to f16 (exact) on its way
+// into the MMA fragments, f16 MMAs (q converted bf16 -> f16, P rounded to f16).  The token's new rows are
 // quantised by the warp that patches them in (x * inv_scale, nearest code, saturating: the arithmetic of
-// arb_kv_append_e4m3), stored to the pool as codes and patched into the widened tile.
+// arb_kv_append_e4m3) and stored to the pool as codes.
 // A third time (KV = 4-bit; arb_decode_step_i4) it serves a cache of 4-bit codes with one fp32 scale per (token, kv head)
-// row: a stage is 1 KB of codes and the rows' 16 scales; the consumer warp widens the codes to bf16 (exact), keeps the
-// scales of its two keys in registers, multiplies them into the scores and into the weights, and runs the bf16 MMAs; the
+// row: a stage is 1 KB of codes and the rows' 16 scales; codes widen to bf16 (exact), the scales of a lane's two keys
+// multiply the scores and the weights, and the MMAs are the bf16 ones; the
 // token's rows are quantised in the kernel (row max by shuffles, IEEE divisions, nearest with ties to even).
+//
+// Fragments out of codes.  The sum over dimensions may run in any order and the rows of O^T may stand for any dimensions, so a
+// lane takes what lies together: for S^T the 32 dimensions 32 tq .. of key rows gq and gq + 8 (step ks: dimensions
+// 32 tq + 4 ks ..; q is loaded in the same order), for O^T the 16 dimensions 16 gq .. of its four key rows, two rows' codes
+// sorted into pairs by byte permutes (accumulator rows gq and gq + 8 of m-tile mt: dimensions 16 gq + 2 mt and + 1).  A page
+// is 4 + 4 16-byte loads of codes and two or three instructions per fragment register.  Widened into a tile in shared
+// memory and read back by ldmatrix, which this replaced, a page took a warp 1.4 us and the consumers set the pace of
+// every call: tokens of the target shape (16 sequences of 4k to 32k, 8 kv heads) E4M3 199 -> 108 us (6.0 TB/s, 0.93 of the
+// measured copy rate), 4-bit 192 -> 138 us (2.5 TB/s; the copies' issue and the page chain share the time: 132 us without
+// the scales' copies, 118 without the products); the draft shape 16.5 -> 14.4 us, either cache.
 #include "arb_decode_tc.cuh"
 
 namespace arb {
@@ -118,14 +127,11 @@ struct Cfg {
     static constexpr int PARK_BYTES = kParked * REC * 4;
 };
 
-// E4M3: the ring holds tiles of codes; every consumer warp has a widened K tile and a widened V tile of its own
 template <int G, int STAGES, int KV, int HD>
 size_t smem_bytes(int batch) {
     using C = Cfg<G, HD>;
     constexpr int kTileBytes = HD / 64 * kHalfTile;
-    const size_t wide = (size_t)kCW * 2 * kTileBytes;
-    const size_t tiles = KV == kKvE4m3 ? (size_t)STAGES * kCodeTileBytes + wide
-                         : KV == kKvI4 ? (size_t)STAGES * kI4StageBytes + wide : (size_t)STAGES * kTileBytes;
+    const size_t tiles = (size_t)STAGES * (KV == kKvE4m3 ? kCodeTileBytes : KV == kKvI4 ? kI4StageBytes : kTileBytes);
     return 1024 + tiles + C::OSM_BYTES + C::PARK_BYTES + sizeof(Tail<STAGES>) + sizeof(int) * (4 * (size_t)batch + 3 + 8);
 }
 
@@ -168,45 +174,40 @@ __device__ __forceinline__ uint32_t e4m3x2_from_f32(float lo, float hi) {
     asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// A warp widens a tile of codes (16 rows x 128 B, 128-byte swizzle) into an f16 tile laid out like a bf16 tile:
-// lane (r, h) = (lane / 2, lane % 2) takes the 64 codes of half h of row r, four 16-byte pieces in, eight out.
-__device__ __forceinline__ void widen_tile(const char *codes, char *dst, int lane) {
-    const int r = lane >> 1, h = lane & 1;
-#pragma unroll
-    for (int c4 = 0; c4 < 4; ++c4) {
-        const int c = 4 * h + c4;
-        const uint4 cd = *reinterpret_cast<const uint4 *>(codes + r * 128 + ((c ^ (r & 7)) << 4));
-        uint4 lo, hi;
-        lo.x = e4m3x2_to_f16x2((uint16_t)cd.x); lo.y = e4m3x2_to_f16x2((uint16_t)(cd.x >> 16));
-        lo.z = e4m3x2_to_f16x2((uint16_t)cd.y); lo.w = e4m3x2_to_f16x2((uint16_t)(cd.y >> 16));
-        hi.x = e4m3x2_to_f16x2((uint16_t)cd.z); hi.y = e4m3x2_to_f16x2((uint16_t)(cd.z >> 16));
-        hi.z = e4m3x2_to_f16x2((uint16_t)cd.w); hi.w = e4m3x2_to_f16x2((uint16_t)(cd.w >> 16));
-        *reinterpret_cast<uint4 *>(dst + tile_off(r, 2 * c)) = lo;
-        *reinterpret_cast<uint4 *>(dst + tile_off(r, 2 * c + 1)) = hi;
-    }
+// 4-bit cache: a 32-bit word holds 8 dimensions as nibbles (code + 8), nibble i and nibble i + 4 being the neighbouring
+// dimensions 2i and 2i + 1.  Moved to bits 3-6 under the exponent of 16, a nibble is the bf16 number 16 + nibble = code +
+// kI4Bias: two integer instructions per pair.  The products run on the biased numbers (small whole numbers, exact) and the
+// bias comes off again in fp32: S starts from -kI4Bias * sum(q), and one more MMA against a constant sums what the weights
+// add to every row of O^T.
+constexpr float kI4Bias = 24.0f;
+constexpr uint32_t kI4BiasPair = 0x41C041C0u;   // kI4Bias as two bf16
+__device__ __forceinline__ uint32_t i4_pair_to_bf16x2(uint32_t w, int i) {
+    return ((i == 0 ? w << 3 : w >> (4 * i - 3)) & 0x00780078u) | 0x41804180u;
 }
 
-// 4-bit cache: a 32-bit word holds 8 dimensions as nibbles (code + 8), nibble i and nibble i + 4 being the neighbouring
-// dimensions 2i and 2i + 1.  (word >> 4i) & 0x000F000F | 0x43004300 is the bf16 pair (128 + nibble i, 128 + nibble i + 4)
-// -- a bf16 with exponent 2^7 counts in ones -- and subtracting 136 leaves the two codes, exactly.
-__device__ __forceinline__ uint4 i4_word_to_bf16x8(uint32_t w) {
-    uint32_t r[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t biased = ((w >> (4 * i)) & 0x000F000Fu) | 0x43004300u;
-        asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r[i]) : "r"(biased), "r"(0x3F803F80u), "r"(0xC308C308u));
+// Codes of one key row for S^T -> the two registers of k-step ks: row = this lane's 32 dimensions (8 or 4 words).
+template <bool E4M3>
+__device__ __forceinline__ void k_fragment(const uint32_t *row, int ks, uint32_t &a0, uint32_t &a2) {
+    if constexpr (E4M3) {
+        a0 = e4m3x2_to_f16x2((uint16_t)row[ks]);
+        a2 = e4m3x2_to_f16x2((uint16_t)(row[ks] >> 16));
+    } else {
+        a0 = i4_pair_to_bf16x2(row[ks >> 1], 2 * (ks & 1));
+        a2 = i4_pair_to_bf16x2(row[ks >> 1], 2 * (ks & 1) + 1);
     }
-    return make_uint4(r[0], r[1], r[2], r[3]);
 }
-// A warp widens a tile of 4-bit codes (16 rows x 64 bytes, plain row-major) into a bf16 tile laid out like a tile of
-// a bf16 cache: lane (r, h) = (lane / 2, lane % 2) takes the 32 bytes (64 dimensions) of half h of row r.
-__device__ __forceinline__ void widen_tile_i4(const char *codes, char *dst, int lane) {
-    const int r = lane >> 1, h = lane & 1;
-    const uint4 c0 = *reinterpret_cast<const uint4 *>(codes + r * 64 + h * 32);
-    const uint4 c1 = *reinterpret_cast<const uint4 *>(codes + r * 64 + h * 32 + 16);
-    const uint32_t w[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4 *>(dst + tile_off(r, 8 * h + i)) = i4_word_to_bf16x8(w[i]);
+// Codes of two neighbouring key rows for O^T, 16 dimensions each (4 or 2 words) -> the registers of m-tile mt: the two
+// keys' values of dimension 2 mt (a0) and 2 mt + 1 (a1) of the 16.
+template <bool E4M3>
+__device__ __forceinline__ void v_fragment(const uint32_t *ra, const uint32_t *rb, int mt, uint32_t &a0, uint32_t &a1) {
+    if constexpr (E4M3) {
+        const uint32_t pair = __byte_perm(ra[mt >> 1], rb[mt >> 1], (mt & 1) ? 0x7362 : 0x5140);
+        a0 = e4m3x2_to_f16x2((uint16_t)pair);
+        a1 = e4m3x2_to_f16x2((uint16_t)(pair >> 16));
+    } else {
+        a0 = i4_pair_to_bf16x2(__byte_perm(ra[mt >> 2], rb[mt >> 2], 0x5410), mt & 3);
+        a1 = i4_pair_to_bf16x2(__byte_perm(ra[mt >> 2], rb[mt >> 2], 0x7632), mt & 3);
+    }
 }
 
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -310,15 +311,15 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     using C = Cfg<G, HD>;
     using Tail = arb::Tail<STAGES>;
     constexpr int GP = C::GP, WREC = C::WREC, REC = C::REC, kOStride = C::kOStride;
-    constexpr int kD = HD, kTileBytes = HD / 64 * kHalfTile;   // a tile of a bf16 cache, and of widened codes
+    constexpr int kD = HD, kTileBytes = HD / 64 * kHalfTile;   // a tile of a bf16 cache
     constexpr bool SPLIT_P = HD == 64;
-    constexpr bool E4M3 = KV == kKvE4m3, I4 = KV == kKvI4, WIDE = KV != kKvBf16;
+    constexpr bool E4M3 = KV == kKvE4m3, I4 = KV == kKvI4, CODES = KV != kKvBf16;
     constexpr int kStageBytes = E4M3 ? kCodeTileBytes : I4 ? kI4StageBytes : kTileBytes;   // a ring stage
     constexpr int kTxBytes = I4 ? kI4CodeBytes + kI4ScaleBytes : kStageBytes;               // what the copies of a stage bring
     constexpr int kRowBytes = E4M3 ? kD : I4 ? kD / 2 : kD * 2;         // bytes of a cache row
-    constexpr int kWideBytes = WIDE ? kCW * 2 * kTileBytes : 0;         // codes: a widened K and V tile per consumer warp
-    constexpr int kRingBytes = STAGES * kStageBytes + kWideBytes;       // the merges use all of it
-    static_assert(!WIDE || HD == 128, "code caches have 128-dimension rows");
+    constexpr int kRingBytes = STAGES * kStageBytes;                    // the merges use all of it
+    constexpr int kRowWords = E4M3 ? 8 : 4;                             // 32-bit words of codes a lane takes per key row for S^T
+    static_assert(!CODES || HD == 128, "code caches have 128-dimension rows");
     static_assert(G >= 1 && G <= 8, "the group's heads are the 8 columns of the tile");
     static_assert(STAGES % (2 * kCW) == 0, "a ring stage always belongs to the same warp of a segment");
 
@@ -655,16 +656,16 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         const char *qh = a.q + ((size_t)row0[g.b] * a.Hq + g.kvh * G + (head_ok ? gq : 0)) * kD * 2;
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) {
+            if constexpr (CODES) {   // dimensions 32 tq + 4 ks .. + 3, in the order the codes come in
+                const uint2 w = head_ok ? __ldg(reinterpret_cast<const uint2 *>(qh + tq * 64 + ks * 8)) : make_uint2(0u, 0u);
+                dst[ks][0] = E4M3 ? bf16x2_to_f16x2(w.x) : w.x;   // (the operands of one MMA share a type)
+                dst[ks][1] = E4M3 ? bf16x2_to_f16x2(w.y) : w.y;
+                continue;
+            }
             dst[ks][0] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + tq * 4)) : 0u;
             dst[ks][1] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + 16 + tq * 4)) : 0u;
-            if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
-                dst[ks][0] = bf16x2_to_f16x2(dst[ks][0]);
-                dst[ks][1] = bf16x2_to_f16x2(dst[ks][1]);
-            }
         }
     };
-    // E4M3: this warp's widened K and V tiles
-    char *wide_k = ring + STAGES * kStageBytes + warp * 2 * kTileBytes, *wide_v = wide_k + kTileBytes;
     Segment s_next;
     int seq_at = seq0;
     bool have = next_segment(cur, r1, seq_at, pl, s);
@@ -679,7 +680,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         const int seg_pages = s.pg1 - s.pg0;
         const int last_pg = (s.L - 1) / kPage, new_slot = (s.L - 1) % kPage;
         bool patch = false;
-        uint4 new_row = make_uint4(0, 0, 0, 0);
+        uint4 new_row = make_uint4(0, 0, 0, 0);   // bf16 cache: 16 bytes of the row; code caches: the codes (x, and y for E4M3)
         float new_scale = 0.f;   // 4-bit cache: the scale of the new K row (lanes 0..15) / V row (lanes 16..31)
         if constexpr (APPEND) {
             patch = last_pg >= s.pg0 && last_pg < s.pg1 && ((last_pg - s.pg0) % kCW) == warp;
@@ -719,10 +720,10 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                         *reinterpret_cast<uint32_t *>((lane < 16 ? a.k_pool : a.v_pool) + slot_row * (kD / 2) + (lane & 15) * 4) = word;
                         if ((lane & 15) == 0) (lane < 16 ? a.k_scales : a.v_scales)[slot_row] = new_scale;
                     }
-                    new_row = i4_word_to_bf16x8(word);
+                    new_row.x = word;
                 } else if constexpr (E4M3) {
                     // quantise this lane's eight values as arb_kv_append_e4m3 does (x * inv_scale in fp32, nearest code,
-                    // ties to even, saturating), store the codes, and keep their widened form for the tile
+                    // ties to even, saturating), store the codes, and keep them for the tile
                     const float inv = lane < 16 ? a.k_inv_scale : a.v_inv_scale;
                     const uint32_t w[4] = {new_row.x, new_row.y, new_row.z, new_row.w};
                     uint32_t code[4];
@@ -734,8 +735,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                                     (((size_t)pid * Hkv + s.kvh) * kPage + new_slot) * kD + (lane & 15) * 8;
                         *reinterpret_cast<uint2 *>(dst) = make_uint2(code[0] | (code[1] << 16), code[2] | (code[3] << 16));
                     }
-                    new_row = make_uint4(e4m3x2_to_f16x2((uint16_t)code[0]), e4m3x2_to_f16x2((uint16_t)code[1]),
-                                         e4m3x2_to_f16x2((uint16_t)code[2]), e4m3x2_to_f16x2((uint16_t)code[3]));
+                    new_row.x = code[0] | (code[1] << 16);
+                    new_row.y = code[2] | (code[3] << 16);
                 } else if (store && in_row) {
                     char *dst = (lane < 16 ? a.k_pool : a.v_pool) +
                                 (((size_t)pid * Hkv + s.kvh) * kPage + new_slot) * (kD * 2) + (lane & 15) * 16;
@@ -747,6 +748,20 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         // this lane's columns (heads h0, h1): running max (the same in the 8 lanes of a column pair), its share of
         // the sum, and the m-tiles of O^T: o[mt][0..1] = dim 16 mt + gq of heads h0, h1; o[mt][2..3] = dim + 8
         float m_run0 = -INFINITY, m_run1 = -INFINITY, l_run0 = 0.f, l_run1 = 0.f;
+        float q_bias0 = 0.f, q_bias1 = 0.f;         // 4-bit cache: what the codes' bias adds to the scores of heads h0, h1, negated
+        float o_bias[4] = {0.f, 0.f, 0.f, 0.f};     // ... and (the first two) to every row of O^T
+        if constexpr (I4) {
+            float sum = 0.f;   // of head gq: this lane's 32 dimensions, then the row's four lanes
+#pragma unroll
+            for (int ks = 0; ks < kD / 16; ++ks)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    sum += __uint_as_float(qb[ks][i] << 16) + __uint_as_float(qb[ks][i] & 0xffff0000u);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+            q_bias0 = -kI4Bias * __shfl_sync(0xffffffffu, sum, 4 * h0);
+            q_bias1 = -kI4Bias * __shfl_sync(0xffffffffu, sum, 4 * h1);
+        }
         float o[kD / 16][4];
 #pragma unroll
         for (int mt = 0; mt < kD / 16; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
@@ -758,44 +773,67 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             const uint32_t ck = seg_base + 2u * (uint32_t)gi;
 
             // ---- S^T = K q^T: 16 keys x 8 heads, two accumulators so that the chain is four deep ----------
-            float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
+            float sa[4] = {q_bias0, q_bias1, q_bias0, q_bias1}, sb[4] = {0.f, 0.f, 0.f, 0.f};
             float ksc0 = 1.f, ksc1 = 1.f, vsc0 = 1.f, vsc1 = 1.f;   // 4-bit cache: the scales of keys gq and gq + 8
             {
                 const uint32_t st = ck % STAGES, par = (ck / STAGES) & 1u;
                 mbar_wait(&tail->full[st], par, abort, a.status);
                 char *tile_p = ring + st * kStageBytes;
-                if constexpr (WIDE) {   // widen into this warp's tile; the ring stage is free at once
+                if constexpr (CODES) {   // the codes come into registers; the ring stage is free at once
+                    uint32_t row0_w[kRowWords], row1_w[kRowWords];
+#pragma unroll
+                    for (int c = 0; c < kRowWords / 4; ++c) {
+                        const int at = E4M3 ? (((2 * tq + c) ^ (gq & 7)) << 4) : tq * 16;   // (rows gq and gq + 8: same swizzle)
+                        const char *src = tile_p + gq * (E4M3 ? 128 : 64) + at;
+                        const uint4 x = *reinterpret_cast<const uint4 *>(src);
+                        const uint4 y = *reinterpret_cast<const uint4 *>(src + 8 * (E4M3 ? 128 : 64));
+                        row0_w[4 * c] = x.x; row0_w[4 * c + 1] = x.y; row0_w[4 * c + 2] = x.z; row0_w[4 * c + 3] = x.w;
+                        row1_w[4 * c] = y.x; row1_w[4 * c + 1] = y.y; row1_w[4 * c + 2] = y.z; row1_w[4 * c + 3] = y.w;
+                    }
                     if constexpr (I4) {
-                        widen_tile_i4(tile_p, wide_k, lane);
                         const float *sc = reinterpret_cast<const float *>(tile_p + kI4CodeBytes);
                         ksc0 = sc[gq];
                         ksc1 = sc[gq + 8];
-                    } else {
-                        widen_tile(tile_p, wide_k, lane);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&tail->empty[st]);
-                    tile_p = wide_k;
-                }
-                if (patch_here) {
-                    if (lane < kD / 8) *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane)) = new_row;
-                    if constexpr (I4) {
-                        const float ns = __shfl_sync(0xffffffffu, new_scale, 0);
-                        if (gq == new_slot) ksc0 = ns;
-                        if (gq + 8 == new_slot) ksc1 = ns;
+                    if (patch_here) {   // lanes 0..15 hold the new K row, dimensions 8 lane ..
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t x = __shfl_sync(0xffffffffu, new_row.x, 4 * tq + j);
+                            const uint32_t y = E4M3 ? __shfl_sync(0xffffffffu, new_row.y, 4 * tq + j) : 0u;
+                            const int w = E4M3 ? 2 * j : j;
+                            if (gq == new_slot) { row0_w[w] = x; if (E4M3) row0_w[w + 1] = y; }
+                            if (gq + 8 == new_slot) { row1_w[w] = x; if (E4M3) row1_w[w + 1] = y; }
+                        }
+                        if constexpr (I4) {
+                            const float ns = __shfl_sync(0xffffffffu, new_scale, 0);
+                            if (gq == new_slot) ksc0 = ns;
+                            if (gq + 8 == new_slot) ksc1 = ns;
+                        }
+                    }
+#pragma unroll
+                    for (int ks = 0; ks < kD / 16; ++ks) {
+                        uint32_t af[4];
+                        k_fragment<E4M3>(row0_w, ks, af[0], af[2]);
+                        k_fragment<E4M3>(row1_w, ks, af[1], af[3]);
+                        if (ks & 1) mma_16816<E4M3>(sb, af, qb[ks][0], qb[ks][1]);
+                        else mma_16816<E4M3>(sa, af, qb[ks][0], qb[ks][1]);
+                    }
+                } else {
+                    if (patch_here) {
+                        if (lane < kD / 8) *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane)) = new_row;
+                        __syncwarp();
+                    }
+                    const uint32_t tile = smem_u32(tile_p);
+#pragma unroll
+                    for (int ks = 0; ks < kD / 16; ++ks) {
+                        uint32_t af[4];   // rows: keys; matrices: (keys 0-7 | 8-15) x (dims 16 ks + 0-7 | 8-15)
+                        ldmatrix_x4(tile + tile_off((lane & 7) + ((lane >> 3) & 1) * 8, 2 * ks + (lane >> 4)), af);
+                        if (ks & 1) mma_16816<E4M3>(sb, af, qb[ks][0], qb[ks][1]);
+                        else mma_16816<E4M3>(sa, af, qb[ks][0], qb[ks][1]);
                     }
                     __syncwarp();
-                }
-                const uint32_t tile = smem_u32(tile_p);
-#pragma unroll
-                for (int ks = 0; ks < kD / 16; ++ks) {
-                    uint32_t af[4];   // rows: keys; matrices: (keys 0-7 | 8-15) x (dims 16 ks + 0-7 | 8-15)
-                    ldmatrix_x4(tile + tile_off((lane & 7) + ((lane >> 3) & 1) * 8, 2 * ks + (lane >> 4)), af);
-                    if (ks & 1) mma_16816<E4M3>(sb, af, qb[ks][0], qb[ks][1]);
-                    else mma_16816<E4M3>(sa, af, qb[ks][0], qb[ks][1]);
-                }
-                __syncwarp();
-                if constexpr (!WIDE) {
                     if (patch_here) fence_proxy_async_smem();   // the stage's next writer is the TMA unit
                     if (lane == 0) mbar_arrive(&tail->empty[st]);
                 }
@@ -850,6 +888,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             if (__any_sync(0xffffffffu, f0 != 1.0f || f1 != 1.0f)) {
 #pragma unroll
                 for (int mt = 0; mt < kD / 16; ++mt) { o[mt][0] *= f0; o[mt][1] *= f1; o[mt][2] *= f0; o[mt][3] *= f1; }
+                if constexpr (I4) { o_bias[0] *= f0; o_bias[1] *= f1; }
             }
 
             // ---- O^T += V^T P^T: m-tiles of 16 dims ---------------------------------------------------
@@ -857,52 +896,89 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 const uint32_t cv = ck + 1u, st = cv % STAGES, par = (cv / STAGES) & 1u;
                 mbar_wait(&tail->full[st], par, abort, a.status);
                 char *tile_p = ring + st * kStageBytes;
-                if constexpr (WIDE) {
+                if constexpr (CODES) {
+                    constexpr int kVWords = kRowWords / 2;   // of this lane's 16 dimensions
+                    const int key[4] = {2 * tq, 2 * tq + 1, 2 * tq + 8, 2 * tq + 9};
+                    uint32_t vw[4][kVWords];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if constexpr (E4M3) {
+                            const uint4 x = *reinterpret_cast<const uint4 *>(tile_p + key[j] * 128 + ((gq ^ (key[j] & 7)) << 4));
+                            vw[j][0] = x.x; vw[j][1] = x.y; vw[j][2] = x.z; vw[j][3] = x.w;
+                        } else {
+                            const uint2 x = *reinterpret_cast<const uint2 *>(tile_p + key[j] * 64 + gq * 8);
+                            vw[j][0] = x.x; vw[j][1] = x.y;
+                        }
+                    }
                     if constexpr (I4) {
-                        widen_tile_i4(tile_p, wide_v, lane);
                         const float *sc = reinterpret_cast<const float *>(tile_p + kI4CodeBytes);
                         vsc0 = k0 ? sc[gq] : 0.f;        // (the scale of a slot past the sequence end may be anything)
                         vsc1 = k1 ? sc[gq + 8] : 0.f;
-                    } else {
-                        widen_tile(tile_p, wide_v, lane);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&tail->empty[st]);
-                    tile_p = wide_v;
-                }
-                if (patch_here) {
-                    if (lane >= 16 && lane - 16 < kD / 8)
-                        *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane - 16)) = new_row;
+                    if (patch_here) {   // lanes 16..31 hold the new V row, dimensions 8 (lane - 16) ..
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const uint32_t x = __shfl_sync(0xffffffffu, new_row.x, 16 + 2 * gq + j);
+                            const uint32_t y = E4M3 ? __shfl_sync(0xffffffffu, new_row.y, 16 + 2 * gq + j) : 0u;
+                            const int w = E4M3 ? 2 * j : j;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                if (key[i] == new_slot) { vw[i][w] = x; if (E4M3) vw[i][w + 1] = y; }
+                        }
+                        if constexpr (I4) {
+                            const float ns = __shfl_sync(0xffffffffu, new_scale, 16);
+                            if (gq == new_slot) vsc0 = ns;
+                            if (gq + 8 == new_slot) vsc1 = ns;
+                        }
+                    }
+                    if constexpr (I4) {   // a value is scale * code: the weight of a key takes its row's scale
+                        w0 = pack_bf16(p00 * vsc0, p01 * vsc0);
+                        w1 = pack_bf16(p10 * vsc1, p11 * vsc1);
+                        pb0 = movmatrix_trans(w0);
+                        pb1 = movmatrix_trans(w1);
+                    } else if (ntok < kPage) {   // codes past the sequence end may be NaN: not even times zero
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (key[j] >= ntok) {
+#pragma unroll
+                                for (int w = 0; w < kVWords; ++w) vw[j][w] = 0u;
+                            }
+                    }
+#pragma unroll
+                    for (int mt = 0; mt < kD / 16; ++mt) {
+                        uint32_t af[4];
+                        v_fragment<E4M3>(vw[0], vw[1], mt, af[0], af[1]);
+                        v_fragment<E4M3>(vw[2], vw[3], mt, af[2], af[3]);
+                        mma_16816<E4M3>(o[mt], af, pb0, pb1);
+                    }
                     if constexpr (I4) {
-                        const float ns = __shfl_sync(0xffffffffu, new_scale, 16);
-                        if (gq == new_slot) vsc0 = ns;
-                        if (gq + 8 == new_slot) vsc1 = ns;
+                        const uint32_t af[4] = {kI4BiasPair, kI4BiasPair, kI4BiasPair, kI4BiasPair};
+                        mma_16816<false>(o_bias, af, pb0, pb1);
+                    }
+                } else {
+                    if (patch_here) {
+                        if (lane >= 16 && lane - 16 < kD / 8)
+                            *reinterpret_cast<uint4 *>(tile_p + tile_off(new_slot, lane - 16)) = new_row;
+                        __syncwarp();
+                    }
+                    if (ntok < kPage) {
+                        // slots past the sequence end may hold anything; they must not reach the tensor core, not even
+                        // times zero: blank them in shared memory
+                        for (int i = lane; i < (kPage - ntok) * (kD / 8); i += 32)
+                            *reinterpret_cast<uint4 *>(tile_p + tile_off(ntok + i / (kD / 8), i % (kD / 8))) = make_uint4(0, 0, 0, 0);
+                        __syncwarp();
+                    }
+                    const uint32_t tile = smem_u32(tile_p);
+#pragma unroll
+                    for (int mt = 0; mt < kD / 16; ++mt) {
+                        uint32_t af[4];   // transposed on the way: rows dims (16 mt + 0-7 | 8-15), columns keys (0-7 | 8-15)
+                        ldmatrix_x4_trans(tile + tile_off((lane & 7) + (lane >> 4) * 8, 2 * mt + ((lane >> 3) & 1)), af);
+                        mma_16816<E4M3>(o[mt], af, pb0, pb1);
+                        if constexpr (SPLIT_P) mma_16816<false>(o[mt], af, lb0, lb1);
                     }
                     __syncwarp();
-                }
-                if constexpr (I4) {   // a value is scale * code: the weight of a key takes its row's scale
-                    w0 = pack_bf16(p00 * vsc0, p01 * vsc0);
-                    w1 = pack_bf16(p10 * vsc1, p11 * vsc1);
-                    pb0 = movmatrix_trans(w0);
-                    pb1 = movmatrix_trans(w1);
-                }
-                if (ntok < kPage) {
-                    // slots past the sequence end may hold anything; they must not reach the tensor core, not even
-                    // times zero: blank them in shared memory
-                    for (int i = lane; i < (kPage - ntok) * (kD / 8); i += 32)
-                        *reinterpret_cast<uint4 *>(tile_p + tile_off(ntok + i / (kD / 8), i % (kD / 8))) = make_uint4(0, 0, 0, 0);
-                    __syncwarp();
-                }
-                const uint32_t tile = smem_u32(tile_p);
-#pragma unroll
-                for (int mt = 0; mt < kD / 16; ++mt) {
-                    uint32_t af[4];   // transposed on the way: rows dims (16 mt + 0-7 | 8-15), columns keys (0-7 | 8-15)
-                    ldmatrix_x4_trans(tile + tile_off((lane & 7) + (lane >> 4) * 8, 2 * mt + ((lane >> 3) & 1)), af);
-                    mma_16816<E4M3>(o[mt], af, pb0, pb1);
-                    if constexpr (SPLIT_P) mma_16816<false>(o[mt], af, lb0, lb1);
-                }
-                __syncwarp();
-                if constexpr (!WIDE) {
                     if (patch_here || ntok < kPage) fence_proxy_async_smem();
                     if (lane == 0) mbar_arrive(&tail->empty[st]);
                 }
@@ -923,6 +999,13 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         }
 #pragma unroll
         for (int mt = 0; mt < kD / 16; ++mt) {
+            if constexpr (CODES) {   // dimensions 16 gq + 2 mt and + 1
+                const int d = 16 * gq + 2 * mt;
+                if constexpr (I4) { o[mt][0] -= o_bias[0]; o[mt][1] -= o_bias[1]; o[mt][2] -= o_bias[0]; o[mt][3] -= o_bias[1]; }
+                if (h0 < G) *reinterpret_cast<float2 *>(rec + 16 + h0 * kOStride + d) = make_float2(o[mt][0], o[mt][2]);
+                if (h1 < G) *reinterpret_cast<float2 *>(rec + 16 + h1 * kOStride + d) = make_float2(o[mt][1], o[mt][3]);
+                continue;
+            }
             const int d = 16 * mt + gq;
             if (h0 < G) { rec[16 + h0 * kOStride + d] = o[mt][0]; rec[16 + h0 * kOStride + d + 8] = o[mt][2]; }
             if (h1 < G) { rec[16 + h1 * kOStride + d] = o[mt][1]; rec[16 + h1 * kOStride + d + 8] = o[mt][3]; }
@@ -1053,10 +1136,9 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
 // kernel's CTAs leave anyway.
 // Ring stages.  What is in flight per SM is stages x bytes of a stage, and it has to cover latency x bandwidth: 32 tiles
 // of a bf16 cache are 128 KB; the tiles of the code caches are 2 KB and 1.1 KB, so their rings are deeper (with 32
-// stages a large call over 4-bit codes could keep 16 KB per SM in flight: 1.4 TB/s).  The widened tiles of the code
-// forms take 64 KB beside the ring.  Tiles of 64-dimension heads are 2 KB: 64 stages keep the same 128 KB in flight.
+// stages a large call over 4-bit codes could keep 16 KB per SM in flight: 1.4 TB/s).  Tiles of 64-dimension heads are 2 KB: 64 stages keep the same 128 KB in flight.
 template <int KV, int HD>
-constexpr int stages_of() { return KV == kKvBf16 ? (HD == 64 ? 64 : 32) : KV == kKvE4m3 ? 48 : 80; }
+constexpr int stages_of() { return KV == kKvBf16 ? (HD == 64 ? 64 : 32) : KV == kKvE4m3 ? 64 : 128; }
 
 template <int G, bool APPEND, int KV, int HD = 128>
 arb_status launch_variant(Ctx *ctx, const StepArgs &a, const CUtensorMap &km, const CUtensorMap &vm, cudaStream_t stream) {

@@ -194,6 +194,7 @@ E4M3_STEP_CASES = [
     (5, 16, 2, [2100, 5, 900, 77, 4000], [1, 0, 1, 0, 1]),
     (1, 5, 1, [40000], [1]),
     (2, 8, 8, [260, 100], [1, 1]),
+    (32, 28, 4, list(range(32)), [1] * 32),                             # the new row in every slot of a page
 ]
 KS, VS = 0.011, 0.017     # N(0,1) values / scale reach about 400: the whole range of the format is used
 
