@@ -69,7 +69,8 @@ __host__ __device__ constexpr int producer_warps() { return KV == kKvBf16 && HD 
 template <int KV, int HD>
 __host__ __device__ constexpr int step_threads() { return 32 * (kCW + producer_warps<KV, HD>() + 1); }
 
-constexpr int kParked = 2;                    // segment results parked in shared memory before they are written
+constexpr int kMergeBatch = 12;               // parts of a split item merged per round of loads, straight into registers ...
+constexpr int kDirectParts = 2 * kMergeBatch; // ... up to this many; more go through the ring in one bulk copy
 // What a boundary costs is time (the warps meet, a second arrival, perhaps a second merge), a few microseconds
 // whatever the call's size: as pages it is the CTA's even share, but no more than this many.
 constexpr int kBoundaryCap = 32;
@@ -114,7 +115,7 @@ struct Tail {
     uint64_t empty[STAGES];
     uint64_t merge_bar;   // the bulk copies of a merge
     int abort;
-    int last[kParked];
+    int last[2];
 };
 
 template <int G, int HD>
@@ -122,9 +123,7 @@ struct Cfg {
     static constexpr int kOStride = HD + 4;               // floats between two heads of a warp record (spreads the banks)
     static constexpr int GP = (G + 3) / 4 * 4;
     static constexpr int WREC = 2 * 8 + G * kOStride;     // warp record: [m[8] | l[8] | o[G][kOStride]]
-    static constexpr int REC = 2 * GP + G * HD;           // parked record: [m[GP] | l[GP] | o[G][D]]
     static constexpr int OSM_BYTES = kCW * WREC * 4;
-    static constexpr int PARK_BYTES = kParked * REC * 4;
 };
 
 template <int G, int STAGES, int KV, int HD>
@@ -132,16 +131,11 @@ size_t smem_bytes(int batch) {
     using C = Cfg<G, HD>;
     constexpr int kTileBytes = HD / 64 * kHalfTile;
     const size_t tiles = (size_t)STAGES * (KV == kKvE4m3 ? kCodeTileBytes : KV == kKvI4 ? kI4StageBytes : kTileBytes);
-    return 1024 + tiles + C::OSM_BYTES + C::PARK_BYTES + sizeof(Tail<STAGES>) + sizeof(int) * (4 * (size_t)batch + 3 + 8);
+    return 1024 + tiles + C::OSM_BYTES + sizeof(Tail<STAGES>) + sizeof(int) * (4 * (size_t)batch + 3 + 8);
 }
 
-struct Parked {
-    int bk, nparts, c_first;
-    size_t out_base;
-};
-
-struct Pending {   // a split (sequence, kv head) this CTA was the last to reach
-    int slot0, nparts;
+struct Split {   // a (sequence, kv head) of which this CTA holds a part
+    int bk, slot0, nparts;
     size_t out_base;
 };
 
@@ -310,7 +304,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     constexpr int kBatch = kOwnStages < 32 ? kOwnStages : 32;   // lanes of a producer warp issuing side by side
     using C = Cfg<G, HD>;
     using Tail = arb::Tail<STAGES>;
-    constexpr int GP = C::GP, WREC = C::WREC, REC = C::REC, kOStride = C::kOStride;
+    constexpr int GP = C::GP, WREC = C::WREC, kOStride = C::kOStride;
     constexpr int kD = HD, kTileBytes = HD / 64 * kHalfTile;   // a tile of a bf16 cache
     constexpr bool SPLIT_P = HD == 64;
     constexpr bool E4M3 = KV == kKvE4m3, I4 = KV == kKvI4, CODES = KV != kKvBf16;
@@ -327,8 +321,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     char *base = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     char *ring = base;
     float *osm = reinterpret_cast<float *>(base + kRingBytes);
-    float *park = reinterpret_cast<float *>(base + kRingBytes + C::OSM_BYTES);
-    Tail *tail = reinterpret_cast<Tail *>(base + kRingBytes + C::OSM_BYTES + C::PARK_BYTES);
+    Tail *tail = reinterpret_cast<Tail *>(base + kRingBytes + C::OSM_BYTES);
     int *pref = reinterpret_cast<int *>(tail + 1);
     int *row0 = pref + a.batch + 1;
     int *act = row0 + a.batch + 1;
@@ -592,61 +585,17 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     uint32_t seg_base = 0;                     // ring counter of the segment's first tile
     int cur = r0;
     Segment s;
-    int n_parked = 0, pend_n = 0;
-    Parked pk[kParked];
-    Pending pend[2];
-
-    // Writes what is parked: whole (sequence, kv head)s to `out`, parts of split ones to the workspace, followed
-    // by the arrival at the item's counter.  The last to arrive notes the merge for the epilogue.
-    auto flush = [&]() {
-        bool any_multi = false;
-        for (int j = 0; j < n_parked; ++j) {
-            const float *rec = park + j * REC;
-            if (pk[j].nparts == 1) {
-                if (!ARB_IN_RANGE(a.status, pk[j].out_base + G * kD - 1, (size_t)a.rows * a.Hq * kD)) continue;
-                for (int idx = tid; idx < G * kD; idx += kCT)
-                    reinterpret_cast<__nv_bfloat16 *>(a.out)[pk[j].out_base + idx] =
-                        __float2bfloat16_rn(rec[2 * GP + idx] / rec[GP + idx / kD]);
-            } else {
-                any_multi = true;
-                const size_t slot = (size_t)pk[j].bk + blockIdx.x;
-                if (!ARB_IN_RANGE(a.status, slot, a.slots)) continue;
-                for (int idx = tid; idx < G * kD / 4; idx += kCT)
-                    reinterpret_cast<float4 *>(a.part_o + slot * G * kD)[idx] =
-                        reinterpret_cast<const float4 *>(rec + 2 * GP)[idx];
-                if (tid < G) {
-                    a.part_ml[(slot * GP + tid) * 2 + 0] = rec[tid];
-                    a.part_ml[(slot * GP + tid) * 2 + 1] = rec[GP + tid];
-                }
-            }
-        }
-        if (any_multi) {
-            __threadfence();
-            asm volatile("fence.proxy.async;" ::: "memory");   // the partials are read back through bulk copies
-            named_barrier(1, kCT);
-            if (tid == 0) {
-                int old[kParked];
-                for (int j = 0; j < n_parked; ++j)
-                    old[j] = pk[j].nparts > 1 ? atomicAdd(&a.counters[pk[j].bk], 1) : -1;
-                for (int j = 0; j < n_parked; ++j) {
-                    const int last = pk[j].nparts > 1 && old[j] == pk[j].nparts - 1;
-                    if (last) a.counters[pk[j].bk] = 0;   // everyone has arrived: ready for the next call
-                    tail->last[j] = last;
-                }
-                __threadfence();
-            }
-            named_barrier(1, kCT);
-            for (int j = 0; j < n_parked; ++j) {
-                if (pk[j].nparts > 1 && tail->last[j] && pend_n < 2) {
-                    pend[pend_n].slot0 = pk[j].bk + pk[j].c_first;
-                    pend[pend_n].nparts = pk[j].nparts;
-                    pend[pend_n].out_base = pk[j].out_base;
-                    ++pend_n;
-                }
-            }
-        }
-        named_barrier(1, kCT);   // parking slots and flags are free again
-        n_parked = 0;
+    // Only the first and the last segment of a CTA's range can be parts of a split item.
+    int n_split = 0;
+    Split sp[2];
+    constexpr int VECS = G * kD / 4;   // 4-dimension pieces of the group's outputs, one per consumer thread
+    constexpr int kPartBytes = G * kD * 4;
+    static_assert(VECS <= kCT, "one piece per consumer thread");
+    const int eh = tid / (kD / 4);     // head of this thread's piece
+    auto write_row = [&](size_t out_base, float4 x, float inv) {
+        if (!ARB_IN_RANGE(a.status, out_base + G * kD - 1, (size_t)a.rows * a.Hq * kD)) return;
+        *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + out_base + (size_t)tid * 4) =
+            make_uint2(pack_bf16(x.x * inv, x.y * inv), pack_bf16(x.z * inv, x.w * inv));
     };
 
     // B fragments of q^T (kD dims x 8 heads): k-slice ks holds dims 16 ks + 2 tq, + 1 and + 8 of head gq.  The
@@ -1010,52 +959,113 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             if (h0 < G) { rec[16 + h0 * kOStride + d] = o[mt][0]; rec[16 + h0 * kOStride + d + 8] = o[mt][2]; }
             if (h1 < G) { rec[16 + h1 * kOStride + d] = o[mt][1]; rec[16 + h1 * kOStride + d + 8] = o[mt][3]; }
         }
-        if (n_parked == kParked) flush();   // uniform across the consumer threads
         named_barrier(1, kCT);
-        float *dst = park + n_parked * REC;
-        for (int idx = tid; idx < G * kD; idx += kCT) {
-            const int h = idx / kD, d = idx - h * kD;
-            float M = -INFINITY;
+        // A whole item goes to `out`, a part of a split one to the workspace, from the registers the merge leaves it in.
+        parts_of(pl, s);
+        const size_t out_base = ((size_t)qrow * a.Hq + s.kvh * G) * kD;
+        const size_t slot = (size_t)s.bk + blockIdx.x;
+        if (tid < VECS) {
+            float M = -INFINITY, mw[kCW];
 #pragma unroll
-            for (int w = 0; w < kCW; ++w) M = fmaxf(M, osm[w * WREC + h]);
-            float l = 0.f, acc = 0.f;
+            for (int w = 0; w < kCW; ++w) { mw[w] = osm[w * WREC + eh]; M = fmaxf(M, mw[w]); }
+            float l = 0.f;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int w = 0; w < kCW; ++w) {
-                const float ff = fast_exp2(osm[w * WREC + h] - M);   // 0 for a warp that had no page
-                l = fmaf(ff, osm[w * WREC + 8 + h], l);
-                acc = fmaf(ff, osm[w * WREC + 16 + h * kOStride + d], acc);
+                const float ff = fast_exp2(mw[w] - M);   // 0 for a warp that had no page
+                const float4 v = *reinterpret_cast<const float4 *>(osm + w * WREC + 16 + eh * kOStride + (tid % (kD / 4)) * 4);
+                l = fmaf(ff, osm[w * WREC + 8 + eh], l);
+                x.x = fmaf(ff, v.x, x.x); x.y = fmaf(ff, v.y, x.y); x.z = fmaf(ff, v.z, x.z); x.w = fmaf(ff, v.w, x.w);
             }
-            dst[2 * GP + idx] = E4M3 ? acc * a.v_scale : acc;   // values of an E4M3 cache are v_scale * code
-            if (d == 0) { dst[h] = M; dst[GP + h] = l; }
+            if constexpr (E4M3) { x.x *= a.v_scale; x.y *= a.v_scale; x.z *= a.v_scale; x.w *= a.v_scale; }   // values are v_scale * code
+            if (s.nparts == 1) {
+                write_row(out_base, x, 1.0f / l);
+            } else if (ARB_IN_RANGE(a.status, slot, a.slots)) {
+                reinterpret_cast<float4 *>(a.part_o + slot * G * kD)[tid] = x;
+                if (tid % (kD / 4) == 0) *reinterpret_cast<float2 *>(a.part_ml + (slot * GP + eh) * 2) = make_float2(M, l);
+            }
         }
-        parts_of(pl, s);
-        pk[n_parked].bk = s.bk;
-        pk[n_parked].nparts = s.nparts;
-        pk[n_parked].c_first = s.c_first;
-        pk[n_parked].out_base = ((size_t)qrow * a.Hq + s.kvh * G) * kD;
-        ++n_parked;
-        named_barrier(1, kCT);   // warp records are free for the next segment
+        if (s.nparts > 1) {
+            const Split here = {s.bk, s.bk + s.c_first, s.nparts, out_base};
+            if (n_split++ == 0) sp[0] = here; else sp[1] = here;
+        }
+        if (have_next) named_barrier(1, kCT);   // warp records are free for the next segment
         s = s_next;
         have = have_next;
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) { qb[ks][0] = qn[ks][0]; qb[ks][1] = qn[ks][1]; }
     }
-    if (n_parked > 0) flush();
+    if (n_split == 0) return;
+    // Arrivals.  The barrier orders every thread's partials before thread 0's fence, whose release covers them; the last to
+    // arrive at an item acquires what the others released.  (A fence by every thread, and parking the results in shared memory
+    // first, cost 1.7 us more: a draft-shaped token 14.6 -> 12.9 us with the merge below, one of a single sequence of 256
+    // tokens 9.4 -> 7.1 us.)
+    named_barrier(1, kCT);
+    if (tid == 0) {
+        __threadfence();
+        int old[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (j < n_split) old[j] = atomicAdd(&a.counters[sp[j].bk], 1);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int last = j < n_split && old[j] == sp[j].nparts - 1;
+            if (last) a.counters[sp[j].bk] = 0;   // everyone has arrived: ready for the next call
+            tail->last[j] = last;
+        }
+        __threadfence();
+    }
+    named_barrier(1, kCT);
+    const bool last0 = tail->last[0] != 0, last1 = tail->last[1] != 0;
+    const int pend_n = (last0 ? 1 : 0) + (last1 ? 1 : 0);
+    if (pend_n == 0) return;
+    const Split pend[2] = {last0 ? sp[0] : sp[1], sp[1]};
 
     // ---- merges of the split (sequence, kv head)s this CTA was the last to reach ------------------------
     //     m = max_p m_p,  w_p = 2^(m_p - m),  out = sum_p w_p o_p / sum_p w_p l_p,
-    // one 4-dimension piece of the group's G x 128 outputs per thread.  The parts of an item lie in consecutive
-    // workspace slots, and the ring is idle by now (every tile has been consumed, the producer issues nothing
-    // more): one bulk copy brings the (max, sum) records, one the partial outputs -- a single round trip however
-    // many parts there are -- and the sum runs out of shared memory.  More parts than the ring holds go in pieces.
-    constexpr int VECS = G * kD / 4;
-    constexpr int kPartBytes = G * kD * 4;
-    static_assert(VECS <= kCT, "one piece per consumer thread");
-    if (pend_n == 0) return;
+    // one 4-dimension piece of the group's outputs per thread.  The parts of an item lie in consecutive workspace slots.  A few
+    // parts (the usual call: 148 CTAs over 16 items is 10 each) are loaded into registers, a round trip per kMergeBatch of them.
+    // Many parts (one sequence over the whole machine) come through the ring, which is idle by now (every tile has been
+    // consumed, the producer issues nothing more): one bulk copy brings the (max, sum) records, one the partial outputs, and
+    // the sum runs out of shared memory; more parts than the ring holds go in pieces.
+    if (max(pend[0].nparts, pend_n > 1 ? pend[1].nparts : 0) <= kDirectParts) {
+        if (tid >= VECS) return;
+#pragma unroll 1
+        for (int j = 0; j < pend_n; ++j) {
+            const Split it = j == 0 ? pend[0] : pend[1];
+            float M = -INFINITY, l = 0.f;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int p0 = 0; p0 < it.nparts; p0 += kMergeBatch) {
+                float2 ml[kMergeBatch];
+                float4 v[kMergeBatch];
+#pragma unroll
+                for (int p = 0; p < kMergeBatch; ++p) {
+                    const bool in = p0 + p < it.nparts;
+                    const size_t slot = (size_t)it.slot0 + p0 + p;
+                    ml[p] = in ? __ldcg(reinterpret_cast<const float2 *>(a.part_ml) + slot * GP + eh) : make_float2(-INFINITY, 0.f);
+                    v[p] = in ? __ldcg(reinterpret_cast<const float4 *>(a.part_o) + slot * VECS + tid) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                float mb = M;
+#pragma unroll
+                for (int p = 0; p < kMergeBatch; ++p) mb = fmaxf(mb, ml[p].x);
+                const float f = fast_exp2(M - mb);
+                M = mb;
+                l *= f; x.x *= f; x.y *= f; x.z *= f; x.w *= f;
+#pragma unroll
+                for (int p = 0; p < kMergeBatch; ++p) {
+                    const float w = fast_exp2(ml[p].x - M);
+                    l = fmaf(w, ml[p].y, l);
+                    x.x = fmaf(w, v[p].x, x.x); x.y = fmaf(w, v[p].y, x.y); x.z = fmaf(w, v[p].z, x.z); x.w = fmaf(w, v[p].w, x.w);
+                }
+            }
+            write_row(it.out_base, x, 1.0f / l);
+        }
+        return;
+    }
     // up to two merges, each in its own half of the ring, their first copies in flight together
     const int cap = kRingBytes / pend_n;
     const bool mine = tid < VECS;
-    const int e = mine ? tid : 0, eh = e / (kD / 4);
+    const int e = mine ? tid : 0, he = e / (kD / 4);
     uint32_t merge_phase = 0;
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
     float4 x[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
@@ -1075,10 +1085,10 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         const float4 *po_s = reinterpret_cast<const float4 *>(ring + j * cap + ml_area(j));
         const int np = min(per_piece(j), pend[j].nparts - p0);
         if (p0 == 0)
-            for (int p = 0; p < pend[j].nparts; ++p) m[j] = fmaxf(m[j], ml_s[p * GP + eh].x);
+            for (int p = 0; p < pend[j].nparts; ++p) m[j] = fmaxf(m[j], ml_s[p * GP + he].x);
 #pragma unroll 4
         for (int p = 0; p < np; ++p) {
-            const float2 ml = ml_s[(p0 + p) * GP + eh];
+            const float2 ml = ml_s[(p0 + p) * GP + he];
             const float w = fast_exp2(ml.x - m[j]);
             const float4 v = po_s[p * VECS + e];
             l[j] = fmaf(w, ml.y, l[j]);
@@ -1095,7 +1105,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         for (int j = 0; j < 2; ++j) more = more || (j < pend_n && done[j] < pend[j].nparts);
         if (!more) break;
         if (tid == 0) {
-            asm volatile("fence.proxy.async;" ::: "memory");
+            asm volatile("fence.proxy.async;" ::: "memory");   // the partials were written by ordinary stores
             uint32_t bytes = 0;
             // the expected bytes are known before the copies are issued: same arithmetic as issue()
 #pragma unroll
@@ -1120,13 +1130,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-        if (j < pend_n && mine && ARB_IN_RANGE(a.status, pend[j].out_base + G * kD - 1, (size_t)a.rows * a.Hq * kD)) {
-            const float inv = 1.0f / l[j];
-            uint2 o2;
-            o2.x = pack_bf16(x[j].x * inv, x[j].y * inv);
-            o2.y = pack_bf16(x[j].z * inv, x[j].w * inv);
-            *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + pend[j].out_base + (size_t)e * 4) = o2;
-        }
+        if (j < pend_n && mine) write_row(pend[j].out_base, x[j], 1.0f / l[j]);
     }
 }
 
