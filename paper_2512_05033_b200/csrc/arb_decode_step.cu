@@ -60,14 +60,12 @@ constexpr int kCW = 8;                        // consumer warps
 constexpr int kCT = kCW * 32;                 // consumer threads
 constexpr int kProdWarp = kCW;                // the producer warps, and behind them one for bookkeeping: length update,
                                               // rows of refused sequences
-// A warp issues a tiled copy every hundred cycles or so, whatever it brings.  Tiles of 4 KB (bf16, head_dim 128) come faster
-// than HBM that way, from one warp (a second one makes every lone call 0.8 us slower: 14.6 -> 15.4 us per draft-shaped
-// token).  Where a tile is 2 KB or less two warps issue, one K and one V: a token of 16 x 8 kv heads of 64 dimensions
-// (150 MB) 38 -> 32 us, draft-shaped tokens over 4-bit codes 17.6 -> 16.7 us, over E4M3 codes 5 % less.
-template <int KV, int HD>
-__host__ __device__ constexpr int producer_warps() { return KV == kKvBf16 && HD == 128 ? 1 : 2; }
-template <int KV, int HD>
-__host__ __device__ constexpr int step_threads() { return 32 * (kCW + producer_warps<KV, HD>() + 1); }
+// A warp issues a tiled copy every hundred cycles or so, whatever it brings, so two warps issue, one K and one V.  Against one
+// warp: rounds of the step loop 1196 -> 1137 us, a token of 8 x 8 kv heads over 1k to 8k 30.2 -> 28.9 us, draft-shaped
+// tokens the same within 1 %, and where a tile is 2 KB or less more: 16 x 8 kv heads of 64 dimensions (150 MB) 38 -> 32 us,
+// draft-shaped tokens over 4-bit codes 17.6 -> 16.7 us.
+constexpr int kAuxWarp = kCW + 2;
+constexpr int kNT = 32 * (kCW + 3);
 
 constexpr int kMergeBatch = 12;               // parts of a split item merged per round of loads, straight into registers ...
 constexpr int kDirectParts = 2 * kMergeBatch; // ... up to this many; more go through the ring in one bulk copy
@@ -79,7 +77,10 @@ constexpr int kBoundaryCap = 32;
 // (the bookkeeping warp does, off every other warp's path): in a chain of dependent calls the bytes of call n + 1
 // cross from HBM while call n is in its latency-bound tail.  A prefetch is a hint: rows are range-checked, a stale or
 // foreign record costs some bandwidth and nothing else, and every real read comes after the wait.
-constexpr int kHintPages = 64;
+// 24 pages are about what HBM delivers while a kernel ends and the next one finds its plan.  More only stand in the way of the
+// lengths and the table: 64 / 32 / 24 / 16 / 8 pages, draft-shaped token 12.6 / 12.4 / 12.1 / 12.2 / 12.3 us, 32 x 8 kv
+// heads of 200 to 900 tokens 20.1 / 18.5 / 18.4 / 18.9 / 18.9 us, rounds of the step loop alike.
+constexpr int kHintPages = 24;
 constexpr int kHintStride = kHintPages + 4;   // [tag, count, -, -, rows ...]
 
 struct StepArgs {
@@ -98,6 +99,7 @@ struct StepArgs {
     int hint_tag;      // shape of this call; a record with another tag is ignored
     uint32_t *status;
     int batch, Hq, Hkv, num_pages, max_pages;
+    uint32_t grid_inv; // floor(2^32 / CTAs) + 1
     int whole_rows;    // the tensor maps are 3-D: one copy per page tile instead of one per half
     int slots;         // partial slots in the workspace region (bounds-check build)
     int rows;          // rows of q and out
@@ -131,7 +133,7 @@ size_t smem_bytes(int batch) {
     using C = Cfg<G, HD>;
     constexpr int kTileBytes = HD / 64 * kHalfTile;
     const size_t tiles = (size_t)STAGES * (KV == kKvE4m3 ? kCodeTileBytes : KV == kKvI4 ? kI4StageBytes : kTileBytes);
-    return 1024 + tiles + C::OSM_BYTES + sizeof(Tail<STAGES>) + sizeof(int) * (4 * (size_t)batch + 3 + 8);
+    return 1024 + tiles + C::OSM_BYTES + sizeof(Tail<STAGES>) + sizeof(int) * (4 * (size_t)batch + 3);
 }
 
 struct Split {   // a (sequence, kv head) of which this CTA holds a part
@@ -296,11 +298,9 @@ __device__ __forceinline__ void parts_of(const Plan &pl, Segment &s) {
 // second product as two bf16 terms (p = hi + lo: 16 significant bits, like the fp32 weights of the CUDA-core kernel this
 // form replaced, to within the rounding of the output); the memory system sets the pace, so the second term costs nothing.
 template <int G, int STAGES, bool APPEND, int KV, int HD>
-__global__ void __launch_bounds__(step_threads<KV, HD>(), 1)
+__global__ void __launch_bounds__(kNT, 1)
 decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map) {
-    constexpr int kProducers = producer_warps<KV, HD>();
-    constexpr int kAuxWarp = kCW + kProducers, kNT = step_threads<KV, HD>();
-    constexpr int kOwnStages = STAGES / kProducers;             // of one producer warp
+    constexpr int kOwnStages = STAGES / 2;             // of one producer warp
     constexpr int kBatch = kOwnStages < 32 ? kOwnStages : 32;   // lanes of a producer warp issuing side by side
     using C = Cfg<G, HD>;
     using Tail = arb::Tail<STAGES>;
@@ -326,7 +326,6 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     int *row0 = pref + a.batch + 1;
     int *act = row0 + a.batch + 1;
     int *slen = act + a.batch + 1;
-    int *plan_s = slen + a.batch;    // [8]: this CTA's cut, worked out by warp 0
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int B = a.batch, Hkv = a.Hkv;
@@ -348,6 +347,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         row0[0] = 0;
         act[0] = 0;
     }
+    __syncthreads();   // the barriers are initialised: off the path that begins below
     int *hint = a.hint + (size_t)blockIdx.x * kHintStride;
     if (warp == kAuxWarp) {
         // the tiles this CTA streamed last time are asked into L2 while the predecessor is still at work
@@ -367,52 +367,90 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     // Everything below may read what the kernel before this one wrote (lengths, q, new rows, the cache).
     wait_for_predecessor();
 
-    // ---- prologue: lengths -> page counts and q row offsets (the bookkeeping warp joins when the plan is there) ----
-    constexpr int kPT = kNT - 32;   // threads of the prologue: all but the bookkeeping warp
-    if (warp == kAuxWarp) {
-        asm volatile("bar.sync 3, %0;" ::"r"(kNT) : "memory");
-    } else {
-    for (int b = tid; b < B; b += kPT) {
-        const int n = a.q_lens[b], L0 = a.seq_lens[b];
-        const bool ok = step_ok<APPEND>(n, L0, a.max_pages);
-        const int L = L0 + (APPEND ? 1 : 0);
-        pref[b + 1] = ok ? (L + kPage - 1) / kPage * Hkv : 0;
-        row0[b + 1] = n > 0 ? n : 0;
-        act[b + 1] = ok ? 1 : 0;
-        slen[b] = L;
-    }
-    named_barrier(2, kPT);
-    if (warp == 0) {
-        int carry_p = 0, carry_r = 0, carry_a = 0;
-        for (int b0 = 0; b0 < B; b0 += 32) {
-            const int b = b0 + lane;
-            int vp = b < B ? pref[b + 1] : 0;
-            int vr = b < B ? row0[b + 1] : 0;
-            int va = b < B ? act[b + 1] : 0;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int tp = __shfl_up_sync(0xffffffffu, vp, off);
-                const int tr = __shfl_up_sync(0xffffffffu, vr, off);
-                const int ta = __shfl_up_sync(0xffffffffu, va, off);
-                if (lane >= off) { vp += tp; vr += tr; va += ta; }
-            }
-            if (b < B) { pref[b + 1] = vp + carry_p; row0[b + 1] = vr + carry_r; act[b + 1] = va + carry_a; }
-            carry_p += __shfl_sync(0xffffffffu, vp, 31);
-            carry_r += __shfl_sync(0xffffffffu, vr, 31);
-            carry_a += __shfl_sync(0xffffffffu, va, 31);
-        }
-        // The cut, while the warp is at it: an even share of the padded list per CTA; both ends of this CTA's range
-        // are looked up with one ballot per 32 sequences (the padded starts ascend, so the sequence that holds a
-        // position is the last one that starts at or before it) instead of a search in every warp.
-        __syncwarp();
-        Plan pl;
-        pl.pref = pref; pl.act = act; pl.slen = slen; pl.B = B; pl.Hkv = Hkv;
-        const int total = pref[B], items = act[B] * Hkv, grid = (int)gridDim.x;
-        const int even = max(a.min_chunk, fast_div(total + grid - 1, grid));
+    // ---- prologue: lengths -> page counts and q row offsets -------------------------------------------------
+    // Every warp works the plan out for itself: nothing but its own loads and shuffles lies between the predecessor's end
+    // and a warp's first look-up.  (One warp planning for all, with two barriers and a search of its tables, took 1.2 us; a
+    // draft-shaped token 12.9 -> 12.6 us, one of a single 256-token sequence 6.8 -> 6.5 us.)  All warps store the same values
+    // into the tables.  A batch of more than 32 is loaded by the whole block first.
+    Plan pl;
+    pl.pref = pref; pl.act = act; pl.slen = slen; pl.B = B; pl.Hkv = Hkv;
+    // total work and items -> what a boundary counts for, the padded list's length, the even share of it
+    const int grid = (int)gridDim.x;
+    auto per_cta = [&](int x) -> int {   // ceil(x / grid) through the launch's reciprocal, which is at most one too large
+        const uint32_t y = (uint32_t)(x + grid - 1), q = __umulhi(y, a.grid_inv);
+        return (int)(q * (uint32_t)grid > y ? q - 1 : q);
+    };
+    auto shares = [&](int total, int items) {
+        const int even = max(a.min_chunk, per_cta(total));
         pl.pen = items > 1 ? (min(even, kBoundaryCap) * a.boundary_pct + 99) / 100 : 0;
         pl.total_padded = total + pl.pen * items;
-        pl.chunk = max(a.min_chunk, fast_div(pl.total_padded + grid - 1, grid));
-        int ends[2], seq0 = 0;
+        pl.chunk = max(a.min_chunk, per_cta(pl.total_padded));
+    };
+    int ends[2], seq0 = 0;   // this CTA's range, and the sequence it begins in
+    auto lengths_of = [&](int b, int &pages, int &rows, int &ok, int &L) {
+        const int n = a.q_lens[b], L0 = a.seq_lens[b];
+        ok = step_ok<APPEND>(n, L0, a.max_pages) ? 1 : 0;
+        L = L0 + (APPEND ? 1 : 0);
+        pages = ok ? (L + kPage - 1) / kPage * Hkv : 0;
+        rows = n > 0 ? n : 0;
+    };
+    auto scan3 = [&](int &vp, int &vr, int &va) {
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int tp = __shfl_up_sync(0xffffffffu, vp, off);
+            const int tr = __shfl_up_sync(0xffffffffu, vr, off);
+            const int ta = __shfl_up_sync(0xffffffffu, va, off);
+            if (lane >= off) { vp += tp; vr += tr; va += ta; }
+        }
+    };
+    if (B <= 32) {
+        int vp = 0, vr = 0, va = 0, L = 0;
+        if (lane < B) lengths_of(lane, vp, vr, va, L);
+        const int own = vp, ok = va;
+        scan3(vp, vr, va);
+        if (lane < B) { pref[lane + 1] = vp; row0[lane + 1] = vr; act[lane + 1] = va; slen[lane] = L; }
+        const int total = __shfl_sync(0xffffffffu, vp, 31);
+        shares(total, __shfl_sync(0xffffffffu, va, 31) * Hkv);
+        // the lane whose sequence holds an end of the range works it out (see Plan)
+        const int pages = ok ? (L + kPage - 1) / kPage : 0, item = pages + pl.pen;
+        const int first = vp - own + pl.pen * Hkv * (va - ok);
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            const long long rel = (long long)(blockIdx.x + w) * pl.chunk - first;
+            const bool here = ok && rel >= 0 && rel < (long long)item * Hkv;
+            const int r = here ? (int)rel : 0, kvh = fast_div(r, max(item, 1));
+            const int pos = vp - own + kvh * pages + max(0, r - kvh * item - pl.pen);
+            const unsigned mask = __ballot_sync(0xffffffffu, here);
+            const int src = __ffs(mask) - 1;
+            const int at = __shfl_sync(0xffffffffu, pos, src & 31);
+            ends[w] = mask ? at : total;   // nobody's: behind the end of the list
+            if (w == 0) seq0 = max(src, 0);
+        }
+        __syncwarp();
+    } else {
+        for (int b = tid; b < B; b += kNT) {
+            int vp, vr, va, L;
+            lengths_of(b, vp, vr, va, L);
+            pref[b + 1] = vp; row0[b + 1] = vr; act[b + 1] = va; slen[b] = L;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            int carry_p = 0, carry_r = 0, carry_a = 0;
+            for (int b0 = 0; b0 < B; b0 += 32) {
+                const int b = b0 + lane;
+                int vp = b < B ? pref[b + 1] : 0, vr = b < B ? row0[b + 1] : 0, va = b < B ? act[b + 1] : 0;
+                scan3(vp, vr, va);
+                if (b < B) { pref[b + 1] = vp + carry_p; row0[b + 1] = vr + carry_r; act[b + 1] = va + carry_a; }
+                carry_p += __shfl_sync(0xffffffffu, vp, 31);
+                carry_r += __shfl_sync(0xffffffffu, vr, 31);
+                carry_a += __shfl_sync(0xffffffffu, va, 31);
+            }
+        }
+        __syncthreads();
+        // both ends of the range with one ballot per 32 sequences: the padded starts ascend, so the sequence that holds a
+        // position is the last one that starts at or before it
+        const int total = pref[B];
+        shares(total, act[B] * Hkv);
 #pragma unroll
         for (int w = 0; w < 2; ++w) {
             const long long t = (long long)(blockIdx.x + w) * pl.chunk;
@@ -425,23 +463,16 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             ends[w] = t >= pl.total_padded ? total : pl.real_in(best, t);
             if (w == 0) seq0 = best;
         }
-        if (lane == 0) {
-            plan_s[0] = ends[0];
-            plan_s[1] = ends[1];
-            plan_s[2] = pl.pen;
-            plan_s[3] = pl.chunk;
-            plan_s[4] = seq0;
-        }
     }
-    named_barrier(2, kPT);
-    asm volatile("bar.arrive 3, %0;" ::"r"(kNT) : "memory");   // the plan is there: the bookkeeping warp may go on
-    }
+    // Named barrier 3 counts the warps that have read the lengths: the bookkeeping warp waits for it, the others pass.
+    if (warp != kAuxWarp) asm volatile("bar.arrive 3, %0;" ::"r"(kNT) : "memory");
 
     if (warp == kAuxWarp) {
         // ================================ bookkeeping warp ==========================================
-        // Lengths: every CTA has its copy in shared memory by now.  The CTA whose count completes the grid
+        // Lengths: once every warp has read them, the CTA counts itself in.  The CTA whose count completes the grid
         // knows that nobody will read seq_lens again and moves them forward: for the sequences that take part
         // and whose new row has a page inside the pool to go to (the same test the writer of the row makes).
+        asm volatile("bar.sync 3, %0;" ::"r"(kNT) : "memory");
         if constexpr (APPEND) {
             int last = 0;
             if (lane == 0) last = atomicAdd(a.lens_counter, 1) == (int)gridDim.x - 1;
@@ -470,16 +501,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         return;
     }
 
-    Plan pl;
-    pl.pref = pref;
-    pl.act = act;
-    pl.slen = slen;
-    pl.B = B;
-    pl.Hkv = Hkv;
-    const int r0 = plan_s[0], r1 = plan_s[1], seq0 = plan_s[4];
-    pl.pen = plan_s[2];
-    pl.chunk = plan_s[3];
-    pl.total_padded = 0;   // only the cut needs it
+    const int r0 = ends[0], r1 = ends[1];
     if (r0 >= r1) {
         if (tid == 0) hint[1] = 0;   // nothing streamed: nothing to ask for next time
         return;
@@ -492,9 +514,11 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         // triple i of the group (a short walk up the prefix table from the range's first sequence) and fetches its block-table entry; the entries
         // of the next group are asked for before the tiles of this one are issued, so that the look-up is off the
         // path after the first group, across sequence boundaries too.  Tiles enter the ring page by page, K then
-        // V.  Two warps issue them, one K and one V, where a tile is 2 KB or less: see producer_warps.  Lanes
+        // V: one warp issues the K tiles, one the V tiles.  Lanes
         // 0 .. kBatch-1 of a warp each own one stage at a time.
         const int pw = warp - kProdWarp;
+        const bool is_v = pw != 0;
+        const CUtensorMap *map = is_v ? &v_map : &k_map;
         const int nflat = r1 - r0;
         auto tile_row = [&](int r) -> int {   // first row, in the 2-D view of the pool, of the tile of flat triple r
             const int lo = pl.seq_of(r, seq0);
@@ -517,22 +541,19 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         for (int g0 = 0; g0 < nflat; g0 += 32) {
             const int row_cur = row_next;
             if (pw == 0 && g0 + lane < min(nflat, kHintPages)) hint[4 + g0 + lane] = row_cur;
-            const int ntiles = (2 / kProducers) * min(32, nflat - g0);   // of this warp
+            const int npages = min(32, nflat - g0);
 #pragma unroll 1
-            for (int i0 = 0; i0 < ntiles; i0 += kBatch) {
+            for (int i0 = 0; i0 < npages; i0 += kBatch) {
                 // the next group's look-up goes out behind this group's first copies, not in front of them
                 if (i0 == kBatch && g0 + 32 + lane < nflat) row_next = tile_row(r0 + g0 + 32 + lane);
                 const int i = i0 + lane;
-                const int t = kProducers * i + pw;   // tile of the group: page t / 2, K or V
-                const bool is_v = (t & 1) != 0;
-                const CUtensorMap *map = is_v ? &v_map : &k_map;
-                const int row = __shfl_sync(0xffffffffu, row_cur, (t >> 1) & 31);
-                const uint32_t cc = 2u * (uint32_t)g0 + (uint32_t)t, st = cc % STAGES, par = (cc / STAGES) & 1u;
+                const int row = __shfl_sync(0xffffffffu, row_cur, i & 31);
+                const uint32_t cc = 2u * (uint32_t)(g0 + i) + (uint32_t)pw, st = cc % STAGES, par = (cc / STAGES) & 1u;
                 // The lanes wait for different stages.  A blocking wait would put the whole warp to sleep until its
                 // time limit whenever one stage is not free yet, and copies for stages that are would go out late, in
                 // clumps (seen: 0.7 us apart).  So the warp polls, converged: every round each lane tests its own
                 // stage without blocking and issues its copy the moment the stage is free.
-                bool pending = lane < kBatch && i < ntiles && ARB_IN_RANGE(a.status, row, (long long)a.num_pages * Hkv * kPage);
+                bool pending = lane < kBatch && i < npages && ARB_IN_RANGE(a.status, row, (long long)a.num_pages * Hkv * kPage);
                 const long long t0 = clock64();
                 while (__any_sync(0xffffffffu, pending)) {
                     if (pending && mbar_test_wait(&tail->empty[st], par ^ 1u)) {
@@ -562,14 +583,14 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                     }
                 }
             }
-            if (ntiles <= kBatch && g0 + 32 + lane < nflat) row_next = tile_row(r0 + g0 + 32 + lane);
+            if (npages <= kBatch && g0 + 32 + lane < nflat) row_next = tile_row(r0 + g0 + 32 + lane);
         }
         // After a timeout the consumers may have left copies unconsumed: wait (bounded) for the last ring's
         // worth, so that no copy is in flight into this CTA's shared memory when it exits.
         if (lane == 0 && *abort) {
-            const int own = (2 / kProducers) * nflat, n = min(own, kOwnStages);
+            const int n = min(nflat, kOwnStages);
             for (int i = 0; i < n; ++i) {
-                const uint32_t cc = (uint32_t)(kProducers * (own - 1 - i) + pw);
+                const uint32_t cc = (uint32_t)(2 * (nflat - 1 - i) + pw);
                 const long long t0 = clock64();
                 while (!mbar_try_wait(&tail->full[cc % STAGES], (cc / STAGES) & 1u) && clock64() - t0 < (1ll << 24)) {
                 }
@@ -1159,7 +1180,7 @@ arb_status launch_variant(Ctx *ctx, const StepArgs &a, const CUtensorMap &km, co
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctx->num_sms);
-    cfg.blockDim = dim3(step_threads<KV, HD>());
+    cfg.blockDim = dim3(kNT);
     cfg.dynamicSmemBytes = smem_bytes<G, STAGES, KV, HD>(a.batch);
     cfg.stream = stream;
     cfg.attrs = attr;
@@ -1248,6 +1269,7 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
                        ((uint32_t)p.num_pages * 2246822519u) ^ ((uint32_t)p.max_pages_per_seq * 3266489917u)) | 1;
     a.status = ctx->status;
     a.batch = p.batch;
+    a.grid_inv = (uint32_t)((1ull << 32) / (unsigned)ctx->num_sms) + 1u;
     a.Hq = p.num_q_heads;
     a.Hkv = p.num_kv_heads;
     a.num_pages = p.num_pages;
