@@ -248,18 +248,13 @@ arb_status arb_attn(arb_ctx *ctx, const arb_attn_params *params, const void *q, 
         if (st != ARB_OK) return st;
     }
     if (params->max_q_len >= 2) {
-        // Step chunks: fp32 chunks have a kernel of their own; bf16 chunks go to the tcgen05 kernel (from
-        // kChunkMmaMinRows rows on, i.e. all of them).  The kernels decide per sequence on the device.
+        // Step chunks: fp32 chunks have a kernel of their own, bf16 chunks go to the tcgen05 kernel, however few rows they
+        // have: a tile with few query rows wastes tensor-core rows, but streams a sequence's keys once, at memory speed, where
+        // the CUDA-core kernel re-reads them per query row (rounds of short steps: 0.76 ms against 0.12 ms per call).
         if (params->dtype == ARB_F32) return launch_chunk_f32(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
-        int skip_rows = 0;
-        if (tensor_cores && chunk_mma_supported(*params)) {
-            st = launch_chunk_mma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
-            if (st != ARB_OK) return st;
-            skip_rows = kChunkMmaMinRows;
-        }
-        st = launch_chunk_fma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, 2,
-                              params->max_q_len, skip_rows, s);
-        if (st != ARB_OK) return st;
+        if (tensor_cores && chunk_mma_supported(*params))
+            return launch_chunk_mma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
+        return launch_chunk_fma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
     }
     return ARB_OK;
 }
@@ -682,13 +677,7 @@ arb_status arb_attn_e4m3(arb_ctx *ctx, const arb_attn_params *params, const void
         if (st != ARB_OK) return st;
     }
     if (params->max_q_len >= 2) {
-        st = launch_chunk_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, s);
-        if (st != ARB_OK) return st;
-        // the CUDA-core chunk kernel reads no key here: every chunk of valid lengths has gone to the tensor cores; it
-        // zero-fills the rows of sequences whose lengths are not (status bit) and otherwise leaves at once
-        st = launch_chunk_fma(c, *params, q, k_codes, v_codes, block_table, seq_lens, q_lens, out, 2, params->max_q_len,
-                              kChunkMmaMinRows, s);
-        if (st != ARB_OK) return st;
+        return launch_chunk_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, s);
     }
     return ARB_OK;
 }
@@ -741,7 +730,8 @@ arb_status arb_poll_status(arb_ctx *ctx, arb_stream_t stream, uint32_t *bits) {
     if (cudaMemcpyAsync(&host, c->status, sizeof(host), cudaMemcpyDeviceToHost, s) != cudaSuccess) return ARB_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return ARB_ERR_CUDA;
     if (bits) *bits = host;
-    if (host != 0) {  // a kernel that gave up may have left arrival counters behind
+    if (host != 0) {  // a kernel that gave up may have left arrival counters behind (the word between the two is the generation)
+        if (cudaMemsetAsync(c->rot + (size_t)kRotSets * kRotCounters + kRotSets + 1, 0, sizeof(int) * 7, s) != cudaSuccess) return ARB_ERR_CUDA;
         if (cudaMemsetAsync(c->counters, 0, sizeof(int) * (c->counters_len + 4), s) != cudaSuccess) return ARB_ERR_CUDA;
         if (cudaMemsetAsync(c->rot, 0, sizeof(int) * ((size_t)kRotSets * kRotCounters + kRotSets), s) != cudaSuccess)
             return ARB_ERR_CUDA;

@@ -1,7 +1,6 @@
 // Step-chunk attention, CUDA-core path: one CTA per (query row, kv head).
 //
-// This is the path of every bf16 chunk when ARB_ATTN_NO_TENSOR_CORES is set (for comparison: fp32 weights).  It
-// also zero-fills the rows of chunk sequences whose lengths are invalid, whatever their size.  Query token i of
+// This is the path of every bf16 chunk when ARB_ATTN_NO_TENSOR_CORES is set (for comparison: fp32 weights).  Query token i of
 // a chunk of n tokens sits at position pos = L - n + i and attends keys 0..pos; the causal mask is
 // just each row's own key count.  K and V rows are read straight from global memory with 16-byte
 // loads (the rows of one chunk are re-read by neighbouring CTAs out of L2); each group of lanes that
@@ -26,9 +25,6 @@ struct ChunkArgs {
     char *out;
     uint32_t *status;
     int batch, Hq, Hkv, num_pages, max_pages;
-    int n_lo, n_hi;  // this kernel owns the sequences with n_lo <= q_len <= n_hi ...
-    int skip_rows;   // ... except valid ones with q_len * group >= skip_rows (> 0): the tensor-core kernel has them
-    const int *needed;  // with skip_rows > 0: written by the tensor-core kernel, 0 = nothing is left for this one
     int jobs;        // (query row, kv head) pairs: total_q * Hkv; the CTAs take them in turn
     float scale_log2;
 };
@@ -54,14 +50,13 @@ __device__ void chunk_fma_job(const ChunkArgs &a, int job, float *rec, const int
     }
     const int b = lo;
     const int n = a.q_lens[b], L = a.seq_lens[b];
-    if (n < a.n_lo || n > a.n_hi) return;  // another kernel owns this sequence
+    if (n < 2) return;  // a decode row: another kernel has it
     T *orow = reinterpret_cast<T *>(a.out) + ((size_t)row * a.Hq + kvh * G) * D;
     if (L < n || L > a.max_pages * kPage) {
         if (tid == 0) atomicOr(a.status, (uint32_t)ARB_DEV_BAD_SEQ_LEN);
         for (int idx = tid; idx < G * D; idx += kThreads) orow[idx] = Elt<T>::from_float(0.f);
         return;
     }
-    if (a.skip_rows > 0 && n * G >= a.skip_rows) return;
     const int i = row - row0[b];
     const int nkeys = L - n + i + 1;
     const int npages = (nkeys + kPage - 1) / kPage;
@@ -172,7 +167,6 @@ __global__ void __launch_bounds__(kThreads) chunk_fma_kernel(const ChunkArgs a) 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int B = a.batch;
     pdl_enter();
-    if (a.skip_rows > 0 && a.needed != nullptr && *a.needed == 0) return;  // the usual case: every chunk was large
 
     if (tid == 0) row0[0] = 0;
     for (int b = tid; b < B; b += kThreads) row0[b + 1] = max(a.q_lens[b], 0);
@@ -192,8 +186,7 @@ __global__ void __launch_bounds__(kThreads) chunk_fma_kernel(const ChunkArgs a) 
         }
     }
     __syncthreads();
-    // the grid is bounded (a call whose chunks all went to the tensor cores would otherwise start, and end at once,
-    // one CTA per query row and kv head): the CTAs take the jobs in turn
+    // the grid is bounded: the CTAs take the jobs in turn
     for (int job = blockIdx.x; job < a.jobs; job += gridDim.x) {
         chunk_fma_job<T, D, G>(a, job, rec, row0);
         __syncthreads();   // the records are free again
@@ -238,9 +231,7 @@ arb_status launch_g(Ctx *ctx, int g, const ChunkArgs &a, int total_q, cudaStream
 
 arb_status launch_chunk_fma(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages,
                             const void *v_pages, const int32_t *block_table, const int32_t *seq_lens,
-                            const int32_t *q_lens, void *out, int n_lo, int n_hi, int skip_rows,
-                            cudaStream_t stream) {
-    const int *needed = skip_rows > 0 ? ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 2 : nullptr;
+                            const int32_t *q_lens, void *out, cudaStream_t stream) {
     ChunkArgs a;
     a.q = static_cast<const char *>(q);
     a.k_pages = static_cast<const char *>(k_pages);
@@ -255,10 +246,6 @@ arb_status launch_chunk_fma(Ctx *ctx, const arb_attn_params &p, const void *q, c
     a.Hkv = p.num_kv_heads;
     a.num_pages = p.num_pages;
     a.max_pages = p.max_pages_per_seq;
-    a.n_lo = n_lo;
-    a.n_hi = n_hi;
-    a.skip_rows = skip_rows;
-    a.needed = needed;
     a.jobs = p.total_q * p.num_kv_heads;
     const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * 1.4426950408889634f;

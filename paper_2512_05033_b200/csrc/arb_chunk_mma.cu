@@ -28,8 +28,9 @@
 // tiled TMA copies (one 16 x 64 box per page and half of head_dim, landing in the canonical swizzled
 // layout) into a two-stage ring.  Roles: warps 0-3 softmax group A, warps 4-7 group B (softmax and epilogue),
 // warp 8 TMA producer of K, warp 10 of V, warp 9 issue of Q K^T and TMEM allocation, warp 11 issue of P V.  Work items are
-// handed out dynamically, longest sequences first: the K producer takes the next item from an atomic
-// counter and announces it to the other roles through a small queue in shared memory.  Every mbarrier wait
+// handed out dynamically, longest sequences first: a CTA begins with the item of its own number, then the K producer takes
+// the next one from an atomic counter (the take that ends the call leaves it at zero) and announces it to the other roles
+// through a small queue in shared memory.  Every mbarrier wait
 // is bounded; TMEM is released on every path.
 //
 // The same kernel, compiled a second time (template parameter E4M3), reads an E4M3 KV cache (one byte per element;
@@ -118,9 +119,7 @@ struct MmaArgs {
     char *out;
     uint32_t *status;
     int batch, Hq, Hkv, num_pages, max_pages;
-    int min_rows;  // sequences with q_len * group >= min_rows are handled here
-    int *work_counter;  // [0] next work item, [1] set if a chunk sequence is left for the CUDA-core kernel;
-                        // both zeroed on the stream before the launch
+    int *work_counter;  // work items taken beyond every CTA's first; zero between calls
     float *split_ws;    // partial results of split sequences, kSlotFloats per (item, row tile)
     int split_cap;      // slots that fit there
     int fill_ctas;      // CTAs a call should keep busy: a call with fewer than half as many work items has its
@@ -351,17 +350,17 @@ __device__ __forceinline__ Plan plan_arrays(int *base, int B) {
     return pl;
 }
 
-// Fills the plan; every thread of the block takes part.  small_flag (nullable): set to 1 by block 0 if a
-// chunk sequence is left for the CUDA-core kernel.
+// A chunk whose lengths fit: what this kernel serves.  One whose lengths do not has its rows zero-filled.
+__device__ __forceinline__ bool chunk_ok(const MmaArgs &a, int n, int L) { return n >= 2 && L >= n && L <= a.max_pages * kPage; }
+
+// Fills the plan; every thread of the block takes part.
 template <int G>
-__device__ void make_plan(const MmaArgs &a, Plan pl, int tid, int nthreads, int *small_flag) {
+__device__ void make_plan(const MmaArgs &a, Plan pl, int tid, int nthreads) {
     const int B = a.batch, Hkv = a.Hkv, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) { pl.pref[0] = 0; pl.row0[0] = 0; }
     for (int b = tid; b < B; b += nthreads) {
         const int n = a.q_lens[b], L = a.seq_lens[b];
-        int pairs = 0;
-        if (n >= 2 && n * G >= a.min_rows && L >= n && L <= a.max_pages * kPage) pairs = (n * G + 2 * kBM - 1) / (2 * kBM);
-        if (small_flag != nullptr && blockIdx.x == 0 && n >= 2 && pairs == 0) atomicOr(small_flag, 1);  // small, or invalid lengths
+        const int pairs = chunk_ok(a, n, L) ? (n * G + 2 * kBM - 1) / (2 * kBM) : 0;
         pl.pairs[b] = pairs;
         pl.key[b] = pairs > 0 ? L : -1;
         pl.row0[b + 1] = n > 0 ? n : 0;
@@ -538,8 +537,18 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         mbar_fence_init();
     }
     wait_for_predecessor();   // everything below reads what the kernel before this one may have written
-    make_plan<G>(a, pl, tid, threads_of(E4M3), a.work_counter + 1);
-    const int total = pl.pref[B];
+    make_plan<G>(a, pl, tid, threads_of(E4M3));
+    for (int b = blockIdx.x; b < B; b += gridDim.x) {
+        const int n = a.q_lens[b];
+        if (n < 2 || pl.pairs[b] > 0) continue;
+        if (tid == 0) atomicOr(a.status, (uint32_t)ARB_DEV_BAD_SEQ_LEN);
+        for (int i = pl.row0[b]; i < pl.row0[b] + n; ++i) {
+            if (!ARB_IN_RANGE(a.status, i, a.rows)) break;
+            uint4 *o = reinterpret_cast<uint4 *>(a.out + (size_t)i * a.Hq * HD * 2);
+            for (int c = tid; c < a.Hq * HD / 8; c += threads_of(E4M3)) o[c] = make_uint4(0, 0, 0, 0);
+        }
+    }
+    const int total = pl.pref[B], workers = min(total, (int)gridDim.x);   // CTAs that take items
     if ((int)blockIdx.x >= total) return;  // nothing for this CTA; no TMEM taken, no barrier pending
 
     if (warp == kMmaWarp) tmem_alloc(&bars->tmem_base, kTmemCols);
@@ -574,7 +583,13 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             int item = total;
             if (lane == 0) {
                 if (!is_v && !helper) {
-                    if (mbar_wait(&bars->item_empty[slot], qpar ^ 1u, abort, a.status)) item = atomicAdd(a.work_counter, 1);
+                    if (nq == 0) {
+                        item = blockIdx.x;
+                    } else if (mbar_wait(&bars->item_empty[slot], qpar ^ 1u, abort, a.status)) {
+                        const int taken = atomicAdd(a.work_counter, 1);   // `total` takes a call: the last of every CTA finds nothing
+                        if (taken == total - 1) *a.work_counter = 0;
+                        item = workers + taken;
+                    }
                     bars->item_id[slot] = item;
                     mbar_arrive(&bars->item_full[slot]);
                 } else if (mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) {
@@ -1102,7 +1117,7 @@ chunk_combine_kernel(const MmaArgs a) {
     const int tid = threadIdx.x;
     const int B = a.batch, Hkv = a.Hkv;
     pdl_enter();
-    make_plan<G>(a, pl, tid, kCombineThreads, nullptr);
+    make_plan<G>(a, pl, tid, kCombineThreads);
     constexpr int kPieces = HD / kCombineDims;
     int job = 0;
     for (int r = 0; r < B; ++r) {
@@ -1196,9 +1211,7 @@ arb_status launch_one(Ctx *ctx, const MmaArgs &a, const CUtensorMap &km, const C
 }  // namespace
 
 bool chunk_mma_supported(const arb_attn_params &p) {
-    const int g = p.num_q_heads / p.num_kv_heads;
-    return p.dtype == ARB_BF16 && (p.head_dim == 64 || p.head_dim == 128) && p.max_q_len >= 2 && p.max_q_len * g >= kChunkMmaMinRows &&
-           tma_available();
+    return p.dtype == ARB_BF16 && (p.head_dim == 64 || p.head_dim == 128) && p.max_q_len >= 2 && tma_available();
 }
 
 namespace {
@@ -1234,7 +1247,6 @@ arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, co
     a.num_pages = p.num_pages;
     a.max_pages = p.max_pages_per_seq;
     a.rows = p.total_q;
-    a.min_rows = kChunkMmaMinRows;
     a.work_counter = ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 1;
     a.split_ws = ctx->chunk_ws;
     a.split_cap = (int)(ctx->chunk_ws_bytes / (slot_floats(p.head_dim) * sizeof(float)));
@@ -1245,7 +1257,6 @@ arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, co
     const long long least_items = (long long)p.num_kv_heads * (((long long)p.total_q - p.batch) * (p.num_q_heads / p.num_kv_heads) / (2 * kBM));
     a.fill_ctas = (2 * least_items <= ctx->num_sms && max_tiles >= kFillMinTiles) ? ctx->num_sms : 0;
     if (max_tiles <= kSplitMinTiles && a.fill_ctas == 0) a.split_cap = 0;
-    if (cudaMemsetAsync(a.work_counter, 0, 2 * sizeof(int), stream) != cudaSuccess) return ARB_ERR_CUDA;
     const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * k_scale * 1.4426950408889634f;
     a.v_scale = v_scale;

@@ -12,11 +12,6 @@ namespace arb {
 constexpr int kPage = 16;             // tokens per KV page
 constexpr int kMaxBatch = 1024;       // sequences per call (prefix tables live in shared memory)
 constexpr int kMaxGroup = 8;          // query heads per KV head
-// q_len * group from which a bf16 chunk goes to the tcgen05 kernel: every chunk.  A tile with few
-// query rows wastes tensor-core rows, but the tile streams a sequence's keys once, at memory speed, where the
-// CUDA-core kernel re-reads them per query row (measured on rounds of short steps: 0.76 ms against 0.12 ms per
-// call; the threshold used to be 64 rows).
-constexpr int kChunkMmaMinRows = 2;
 constexpr int kDecodeMmaMinGroup = 1; // group size from which bf16 / head_dim 128 decode uses warp-level MMA
 constexpr long long kWaitCycles = 1ll << 31;  // bound of every mbarrier wait (about a second)
 
@@ -295,8 +290,7 @@ arb_status launch_decode(Ctx *ctx, const arb_attn_params &p, const void *q, cons
                          const int32_t *q_lens, void *out, cudaStream_t stream);
 arb_status launch_chunk_fma(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages,
                             const void *v_pages, const int32_t *block_table, const int32_t *seq_lens,
-                            const int32_t *q_lens, void *out, int n_lo, int n_hi, int skip_rows,
-                            cudaStream_t stream);
+                            const int32_t *q_lens, void *out, cudaStream_t stream);
 arb_status launch_chunk_f32(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages, const void *v_pages,
                             const int32_t *block_table, const int32_t *seq_lens, const int32_t *q_lens, void *out,
                             cudaStream_t stream);
