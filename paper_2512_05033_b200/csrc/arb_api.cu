@@ -231,15 +231,17 @@ arb_status arb_attn(arb_ctx *ctx, const arb_attn_params *params, const void *q, 
     // (the host knows only the total and the maximum of q_lens).
     const bool maybe_decode = params->max_q_len == 1 || params->total_q > params->max_q_len;
     const bool tensor_cores = (params->flags & ARB_ATTN_NO_TENSOR_CORES) == 0;
+    bool beside = false;   // decode rows and chunks of the call run side by side
     if (maybe_decode) {
         // bf16: a call that is one of a back-to-back series (ARB_ATTN_OVERLAP_PREVIOUS) takes the
         // two-kernel form, whose calls stream under one another's tails; a call on its own takes the single
         // launch, which is what finishes a lone call soonest.
         const bool series = (params->flags & ARB_ATTN_OVERLAP_PREVIOUS) != 0;
-        if (tensor_cores && !series && decode_step_supported(*params))
-            st = launch_decode_step(c, *params, q, nullptr, nullptr, const_cast<void *>(k_pages),
-                                    const_cast<void *>(v_pages), nullptr, block_table, const_cast<int32_t *>(seq_lens), q_lens, out, s);
-        else if (tensor_cores && decode_mma_supported(*params))
+        if (tensor_cores && !series && decode_step_supported(*params)) {
+            beside = params->max_q_len >= 2 && chunk_mma_supported(*params);
+            st = launch_decode_step(c, *params, q, nullptr, nullptr, const_cast<void *>(k_pages), const_cast<void *>(v_pages),
+                                    nullptr, block_table, const_cast<int32_t *>(seq_lens), q_lens, out, s, beside);
+        } else if (tensor_cores && decode_mma_supported(*params))
             st = launch_decode_mma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
         else {
             note_unnumbered_decode(c, decode_workspace_bytes(*params, c->num_sms));  // region 0, no generation number
@@ -253,7 +255,7 @@ arb_status arb_attn(arb_ctx *ctx, const arb_attn_params *params, const void *q, 
         // the CUDA-core kernel re-reads them per query row (rounds of short steps: 0.76 ms against 0.12 ms per call).
         if (params->dtype == ARB_F32) return launch_chunk_f32(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
         if (tensor_cores && chunk_mma_supported(*params))
-            return launch_chunk_mma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
+            return launch_chunk_mma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, beside, s);
         return launch_chunk_fma(c, *params, q, k_pages, v_pages, block_table, seq_lens, q_lens, out, s);
     }
     return ARB_OK;
@@ -332,7 +334,7 @@ arb_status arb_decode_step_i4(arb_ctx *ctx, const arb_attn_params *params, const
     if (decode_workspace_bytes(*params, c->num_sms) > c->workspace_bytes) return ARB_ERR_WORKSPACE;
     if (!decode_step_supported(*params)) return ARB_ERR_UNSUPPORTED;
     return launch_decode_step(c, *params, q, k_new, v_new, k_codes, v_codes, nullptr, block_table, seq_lens, q_lens, out,
-                              reinterpret_cast<cudaStream_t>(stream), k_scales, v_scales);
+                              reinterpret_cast<cudaStream_t>(stream), false, k_scales, v_scales);
 }
 
 arb_status arb_attn_decode_static(const arb_attn_params *params, const void *q, const void *k_pages,

@@ -124,6 +124,7 @@ struct MmaArgs {
     int split_cap;      // slots that fit there
     int fill_ctas;      // CTAs a call should keep busy: a call with fewer than half as many work items has its
                         // sequences cut over their keys as well (0: never)
+    int beside;         // the kernel before this one is the decode rows of the same call: it is waited for at the end
     int rows;           // rows of q and out (bounds-check build)
     float scale_log2;   // softmax scale (times the key scale of an E4M3 cache) * log2(e)
     float v_scale;      // value scale of an E4M3 cache, 1 otherwise
@@ -536,7 +537,10 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         bars->abort = 0;
         mbar_fence_init();
     }
-    wait_for_predecessor();   // everything below reads what the kernel before this one may have written
+    // Everything below reads what the kernel before this one may have written.  The decode rows of the same call write nothing
+    // of it, and let this kernel start only when what ran before them has completed; they are waited for at the end, so
+    // that this kernel's completion implies theirs.
+    if (!a.beside) wait_for_predecessor();
     make_plan<G>(a, pl, tid, threads_of(E4M3));
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
         const int n = a.q_lens[b];
@@ -549,7 +553,10 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         }
     }
     const int total = pl.pref[B], workers = min(total, (int)gridDim.x);   // CTAs that take items
-    if ((int)blockIdx.x >= total) return;  // nothing for this CTA; no TMEM taken, no barrier pending
+    if ((int)blockIdx.x >= total) {   // nothing for this CTA; no TMEM taken, no barrier pending
+        if (a.beside) wait_for_predecessor();
+        return;
+    }
 
     if (warp == kMmaWarp) tmem_alloc(&bars->tmem_base, kTmemCols);
     tc_fence_before();
@@ -1098,6 +1105,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
     }
+    if (a.beside) wait_for_predecessor();
 }
 
 // ---- merge of the parts of split sequences -------------------------------------------------------------
@@ -1226,7 +1234,7 @@ arb_status launch_g(Ctx *ctx, const MmaArgs &a, bool e4m3, int head_dim, const C
 
 arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages, const void *v_pages,
                            bool e4m3, float k_scale, float v_scale, const int32_t *block_table, const int32_t *seq_lens,
-                           const int32_t *q_lens, void *out, cudaStream_t stream) {
+                           const int32_t *q_lens, void *out, bool beside, cudaStream_t stream) {
     alignas(64) CUtensorMap km, vm;
     const PoolView view = e4m3 ? PoolView::kE4m3 : p.head_dim == 64 ? PoolView::kBf16D64 : PoolView::kBf16HalfRows;
     if (!pool_map(ctx, &km, k_pages, p.num_pages, p.num_kv_heads, view) ||
@@ -1247,6 +1255,7 @@ arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, co
     a.num_pages = p.num_pages;
     a.max_pages = p.max_pages_per_seq;
     a.rows = p.total_q;
+    a.beside = beside ? 1 : 0;
     a.work_counter = ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 1;
     a.split_ws = ctx->chunk_ws;
     a.split_cap = (int)(ctx->chunk_ws_bytes / (slot_floats(p.head_dim) * sizeof(float)));
@@ -1282,8 +1291,8 @@ arb_status launch_chunk_tc(Ctx *ctx, const arb_attn_params &p, const void *q, co
 
 arb_status launch_chunk_mma(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_pages,
                             const void *v_pages, const int32_t *block_table, const int32_t *seq_lens,
-                            const int32_t *q_lens, void *out, cudaStream_t stream) {
-    return launch_chunk_tc(ctx, p, q, k_pages, v_pages, false, 1.0f, 1.0f, block_table, seq_lens, q_lens, out, stream);
+                            const int32_t *q_lens, void *out, bool beside, cudaStream_t stream) {
+    return launch_chunk_tc(ctx, p, q, k_pages, v_pages, false, 1.0f, 1.0f, block_table, seq_lens, q_lens, out, beside, stream);
 }
 
 // step chunks over an E4M3 cache (q, out bf16): keys are k_scale * code, values v_scale * code
@@ -1291,7 +1300,7 @@ arb_status launch_chunk_e4m3(Ctx *ctx, const arb_attn_params &p, const void *q, 
                              const void *v_codes, float k_scale, float v_scale, const int32_t *block_table,
                              const int32_t *seq_lens, const int32_t *q_lens, void *out, cudaStream_t stream) {
     if (p.num_q_heads / p.num_kv_heads > 8 || p.batch > kMaxBatchE4m3 || !tma_available()) return ARB_ERR_UNSUPPORTED;
-    return launch_chunk_tc(ctx, p, q, k_codes, v_codes, true, k_scale, v_scale, block_table, seq_lens, q_lens, out, stream);
+    return launch_chunk_tc(ctx, p, q, k_codes, v_codes, true, k_scale, v_scale, block_table, seq_lens, q_lens, out, false, stream);
 }
 
 }  // namespace arb

@@ -83,6 +83,16 @@ constexpr int kBoundaryCap = 32;
 constexpr int kHintPages = 24;
 constexpr int kHintStride = kHintPages + 4;   // [tag, count, -, -, rows ...]
 
+// The decode rows of a call with chunks stream while the chunks compute, on SMs of their own: alone an SM draws about 77 GB/s
+// (65 of them 5 TB/s), beside chunks less.  Both kinds of work are known from the lengths; the decode rows get the share of
+// the SMs that kBesideWeight times their work is of the whole, counted in page tiles: a page of a kv head is 1, 128 keys of a
+// pair of chunk row tiles are kBesidePairTile (2.3 us against 0.106 us), of a lone row tile kBesideLoneTile.  A serving
+// iteration (32 decode rows, 32 steps, lognormal lengths) 806 -> 748 us, 900 -> 874 us under the power cap (weights 1.33 /
+// 1.9 / 2.6 / 3.5: 813 / 749 / 746 / 769 us); one 16-token step beside 15 decode rows of 4k to 32k 217 -> 199 us (on a fixed
+// 65 SMs 271), four of 32 tokens beside 60 rows of 500 to 3000 114 -> 100 us, one of 8 beside 7 draft-shaped rows 33 -> 24 us.
+constexpr float kBesideWeight = 2.2f;
+constexpr int kBesidePairTile = 22, kBesideLoneTile = 13;
+
 struct StepArgs {
     const char *q;
     const char *k_new, *v_new;   // [rows, Hkv, D]; null: no cache write, seq_lens already count the token
@@ -100,6 +110,7 @@ struct StepArgs {
     uint32_t *status;
     int batch, Hq, Hkv, num_pages, max_pages;
     uint32_t grid_inv; // floor(2^32 / CTAs) + 1
+    int beside;        // the kernel launched next runs beside this one (see launch_decode_step)
     int whole_rows;    // the tensor maps are 3-D: one copy per page tile instead of one per half
     int slots;         // partial slots in the workspace region (bounds-check build)
     int rows;          // rows of q and out
@@ -330,7 +341,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int B = a.batch, Hkv = a.Hkv;
 
-    let_successor_start();
+    if (!a.beside) let_successor_start();
     if (tid == kCT) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&k_map)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&v_map)) : "memory");
@@ -366,6 +377,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     }
     // Everything below may read what the kernel before this one wrote (lengths, q, new rows, the cache).
     wait_for_predecessor();
+    if (a.beside) let_successor_start();   // the successor does not wait for this kernel, but it may read what the predecessor wrote
 
     // ---- prologue: lengths -> page counts and q row offsets -------------------------------------------------
     // Every warp works the plan out for itself: nothing but its own loads and shuffles lies between the predecessor's end
@@ -375,12 +387,24 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     Plan pl;
     pl.pref = pref; pl.act = act; pl.slen = slen; pl.B = B; pl.Hkv = Hkv;
     // total work and items -> what a boundary counts for, the padded list's length, the even share of it
-    const int grid = (int)gridDim.x;
-    auto per_cta = [&](int x) -> int {   // ceil(x / grid) through the launch's reciprocal, which is at most one too large
-        const uint32_t y = (uint32_t)(x + grid - 1), q = __umulhi(y, a.grid_inv);
-        return (int)(q * (uint32_t)grid > y ? q - 1 : q);
+    int ctas = (int)gridDim.x;   // that take part
+    auto per_cta = [&](int x) -> int {   // ceil(x / ctas), mostly through the launch's reciprocal, which is at most one too large
+        if (a.beside) return fast_div(x + ctas - 1, ctas);
+        const uint32_t y = (uint32_t)(x + ctas - 1), q = __umulhi(y, a.grid_inv);
+        return (int)(q * (uint32_t)ctas > y ? q - 1 : q);
     };
-    auto shares = [&](int total, int items) {
+    auto chunk_work = [&](int n, int L) -> float {   // of one sequence, in page tiles
+        if (n < 2 || L < n) return 0.f;
+        const int tiles = (n * G + 127) / 128;
+        return (float)Hkv * (float)((L + 127) / 128) * (float)((tiles >> 1) * kBesidePairTile + (tiles & 1) * kBesideLoneTile);
+    };
+    auto shares = [&](int total, int items, float chunks) {
+        if (a.beside) {
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) chunks += __shfl_xor_sync(0xffffffffu, chunks, off);
+            const float mine = kBesideWeight * (float)total;
+            ctas = min(ctas, max(4, __float2int_ru((float)ctas * __fdividef(mine, mine + chunks + 1.f))));
+        }
         const int even = max(a.min_chunk, per_cta(total));
         pl.pen = items > 1 ? (min(even, kBoundaryCap) * a.boundary_pct + 99) / 100 : 0;
         pl.total_padded = total + pl.pen * items;
@@ -406,11 +430,11 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     if (B <= 32) {
         int vp = 0, vr = 0, va = 0, L = 0;
         if (lane < B) lengths_of(lane, vp, vr, va, L);
-        const int own = vp, ok = va;
+        const int own = vp, ok = va, rows = vr;
         scan3(vp, vr, va);
         if (lane < B) { pref[lane + 1] = vp; row0[lane + 1] = vr; act[lane + 1] = va; slen[lane] = L; }
         const int total = __shfl_sync(0xffffffffu, vp, 31);
-        shares(total, __shfl_sync(0xffffffffu, va, 31) * Hkv);
+        shares(total, __shfl_sync(0xffffffffu, va, 31) * Hkv, a.beside ? chunk_work(rows, L) : 0.f);
         // the lane whose sequence holds an end of the range works it out (see Plan)
         const int pages = ok ? (L + kPage - 1) / kPage : 0, item = pages + pl.pen;
         const int first = vp - own + pl.pen * Hkv * (va - ok);
@@ -450,7 +474,10 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         // both ends of the range with one ballot per 32 sequences: the padded starts ascend, so the sequence that holds a
         // position is the last one that starts at or before it
         const int total = pref[B];
-        shares(total, act[B] * Hkv);
+        float chunks = 0.f;
+        if (a.beside)
+            for (int b = lane; b < B; b += 32) chunks += chunk_work(row0[b + 1] - row0[b], slen[b]);
+        shares(total, act[B] * Hkv, chunks);
 #pragma unroll
         for (int w = 0; w < 2; ++w) {
             const long long t = (long long)(blockIdx.x + w) * pl.chunk;
@@ -1215,9 +1242,12 @@ bool decode_step_supported(const arb_attn_params &p) {
 // k_new == nullptr: attention only (seq_lens is not written).  scales != nullptr: an E4M3 cache with scales =
 // {k_scale, v_scale, k_inv_scale, v_inv_scale}; k_row_scales != nullptr: a 4-bit cache with its two scale pools
 // (k_new is required for both); neither: a bf16 cache.
+// beside: the decode rows of a call that has chunks too.  The chunk kernel, launched next, reads and writes nothing that this
+// one does, so it starts as soon as this kernel's predecessor is known to have completed, and this one takes only its share
+// of the SMs (kBesideWeight).
 arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_new, const void *v_new,
                               void *k_pages, void *v_pages, const float *scales, const int32_t *block_table,
-                              int32_t *seq_lens, const int32_t *q_lens, void *out, cudaStream_t stream,
+                              int32_t *seq_lens, const int32_t *q_lens, void *out, cudaStream_t stream, bool beside,
                               float *k_row_scales, float *v_row_scales) {
     alignas(64) CUtensorMap km, vm;
     const bool e4m3 = scales != nullptr, i4 = k_row_scales != nullptr;
@@ -1265,10 +1295,11 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
     a.counters = ctx->rot;                                                       // [kRotCounters]
     a.lens_counter = ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 4;
     a.hint = ctx->step_hint;
-    a.hint_tag = (int)(((uint32_t)p.batch * 2654435761u) ^ ((uint32_t)p.num_kv_heads * 40503u) ^
-                       ((uint32_t)p.num_pages * 2246822519u) ^ ((uint32_t)p.max_pages_per_seq * 3266489917u)) | 1;
+    a.hint_tag = ((int)(((uint32_t)p.batch * 2654435761u) ^ ((uint32_t)p.num_kv_heads * 40503u) ^
+                       ((uint32_t)p.num_pages * 2246822519u) ^ ((uint32_t)p.max_pages_per_seq * 3266489917u)) & ~3) | (beside ? 3 : 1);   // (another cut: another record)
     a.status = ctx->status;
     a.batch = p.batch;
+    a.beside = beside ? 1 : 0;
     a.grid_inv = (uint32_t)((1ull << 32) / (unsigned)ctx->num_sms) + 1u;
     a.Hq = p.num_q_heads;
     a.Hkv = p.num_kv_heads;

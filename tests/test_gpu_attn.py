@@ -692,3 +692,29 @@ def test_fp32_chunk_matches_oracle(case, ws):
         c.close()
     assert bits == 0 and st == 0
     H.assert_close(out, ref, F32)
+
+
+BESIDE_CASES = [
+    # (Hq, Hkv, D, seq_lens, q_lens): decode rows and chunks of one call side by side, the SMs shared by their work
+    (12, 2, 128, [40, 5000], [1, 2]),                                  # next to no decode work: the fewest CTAs
+    (12, 2, 128, [9000, 30], [1, 4]),                                  # nearly all decode work
+    (32, 8, 128, [300 + 37 * i for i in range(33)], [1, 9, 1] * 11),   # more than 32 sequences: the other plan
+    (16, 2, 64, [700, 2, 4000, 90], [1, 2, 40, 1]),
+]
+
+
+@pytest.mark.parametrize("case", BESIDE_CASES)
+def test_decode_rows_beside_chunks_match_oracle(case):
+    """... and what follows on the stream sees both: the output is overwritten and the call repeated back to back."""
+    Hq, Hkv, D, sl, ql = case
+    inp = wl.small_attn_case(len(sl), Hq, Hkv, D, BF, sl, ql, seed=720 + Hq)
+    ref, st = H.oracle_attn(inp)
+    d, c = inp.to("cuda"), H.ctx()
+    out, copies = torch.empty_like(d.q), []
+    for _ in range(4):
+        out.fill_(float("nan"))
+        c.attn(d.q, d.k_pages, d.v_pages, d.block_table, d.seq_lens, d.q_lens, max(ql), out=out)
+        copies.append(out.clone())
+    assert c.poll_status() == 0 and st == 0
+    for got in copies:
+        H.assert_close(got.double().cpu().numpy(), ref, BF, tight=3e-3)
