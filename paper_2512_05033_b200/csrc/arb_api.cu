@@ -72,6 +72,19 @@ struct DeviceGuard {
 
 namespace {
 
+// Decode rows over an E4M3 cache: a call of a back-to-back series takes the two-kernel form, a call on its own the single
+// launch: a target-shaped call 112 -> 104 us, a draft-shaped one 18.9 -> 10.5 us, two sequences of 300 to 500 tokens 11.2 ->
+// 6.6 us, and one launch instead of two in front of the chunks of a mixed one.
+arb_status decode_e4m3(Ctx *c, const arb_attn_params &p, const void *q, const uint8_t *k_codes, const uint8_t *v_codes, float k_scale,
+                       float v_scale, const int32_t *block_table, const int32_t *seq_lens, const int32_t *q_lens, void *out,
+                       bool beside, cudaStream_t s) {
+    if ((p.flags & ARB_ATTN_OVERLAP_PREVIOUS) || !decode_step_supported(p))
+        return launch_decode_e4m3(c, p, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, s);
+    const float scales[4] = {k_scale, v_scale, 1.0f, 1.0f};
+    return launch_decode_step(c, p, q, nullptr, nullptr, const_cast<uint8_t *>(k_codes), const_cast<uint8_t *>(v_codes), scales,
+                              block_table, const_cast<int32_t *>(seq_lens), q_lens, out, s, beside);
+}
+
 bool pipe_setup(Ctx *c) {
     if (c->pipe_ready) return true;
     bool ok = cudaStreamCreateWithFlags(&c->in_stream, cudaStreamNonBlocking) == cudaSuccess;
@@ -652,8 +665,8 @@ arb_status arb_attn_decode_e4m3(arb_ctx *ctx, const arb_attn_params *params, con
     if (!aligned16(q) || !aligned16(out) || !aligned16(k_codes) || !aligned16(v_codes)) return ARB_ERR_INVALID_ARG;
     Ctx *c = reinterpret_cast<Ctx *>(ctx);
     if (decode_workspace_bytes(*params, c->num_sms) > c->workspace_bytes) return ARB_ERR_WORKSPACE;
-    return launch_decode_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out,
-                              reinterpret_cast<cudaStream_t>(stream));
+    return decode_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, false,
+                       reinterpret_cast<cudaStream_t>(stream));
 }
 
 arb_status arb_attn_e4m3(arb_ctx *ctx, const arb_attn_params *params, const void *q, const uint8_t *k_codes,
@@ -674,12 +687,13 @@ arb_status arb_attn_e4m3(arb_ctx *ctx, const arb_attn_params *params, const void
     if (decode_workspace_bytes(*params, c->num_sms) > c->workspace_bytes) return ARB_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const bool maybe_decode = params->max_q_len == 1 || params->total_q > params->max_q_len;
+    const bool beside = maybe_decode && params->max_q_len >= 2 && (params->flags & ARB_ATTN_OVERLAP_PREVIOUS) == 0;
     if (maybe_decode) {
-        st = launch_decode_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, s);
+        st = decode_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, beside, s);
         if (st != ARB_OK) return st;
     }
     if (params->max_q_len >= 2) {
-        return launch_chunk_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, s);
+        return launch_chunk_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, beside, s);
     }
     return ARB_OK;
 }

@@ -1298,9 +1298,9 @@ arb_status launch_chunk_mma(Ctx *ctx, const arb_attn_params &p, const void *q, c
 // step chunks over an E4M3 cache (q, out bf16): keys are k_scale * code, values v_scale * code
 arb_status launch_chunk_e4m3(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_codes,
                              const void *v_codes, float k_scale, float v_scale, const int32_t *block_table,
-                             const int32_t *seq_lens, const int32_t *q_lens, void *out, cudaStream_t stream) {
+                             const int32_t *seq_lens, const int32_t *q_lens, void *out, bool beside, cudaStream_t stream) {
     if (p.num_q_heads / p.num_kv_heads > 8 || p.batch > kMaxBatchE4m3 || !tma_available()) return ARB_ERR_UNSUPPORTED;
-    return launch_chunk_tc(ctx, p, q, k_codes, v_codes, true, k_scale, v_scale, block_table, seq_lens, q_lens, out, false, stream);
+    return launch_chunk_tc(ctx, p, q, k_codes, v_codes, true, k_scale, v_scale, block_table, seq_lens, q_lens, out, beside, stream);
 }
 
 }  // namespace arb

@@ -304,7 +304,7 @@ arb_status launch_chunk_mma(Ctx *ctx, const arb_attn_params &p, const void *q, c
                             const int32_t *q_lens, void *out, bool beside, cudaStream_t stream);
 arb_status launch_chunk_e4m3(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_codes,
                              const void *v_codes, float k_scale, float v_scale, const int32_t *block_table,
-                             const int32_t *seq_lens, const int32_t *q_lens, void *out, cudaStream_t stream);
+                             const int32_t *seq_lens, const int32_t *q_lens, void *out, bool beside, cudaStream_t stream);
 arb_status launch_route(Ctx *ctx, int dtype, int n_steps, int hidden_dim, const void *hidden, const void *w,
                         float b, float tau, float *scores, uint8_t *decisions, cudaStream_t stream);
 arb_status launch_rollback(Ctx *ctx, int batch, int32_t *seq_lens, const int32_t *step_lens,

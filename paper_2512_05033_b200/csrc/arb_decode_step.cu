@@ -1217,11 +1217,13 @@ arb_status launch_variant(Ctx *ctx, const StepArgs &a, const CUtensorMap &km, co
     return ARB_OK;
 }
 
-// The E4M3 and the 4-bit forms exist with the cache write only (decode alone over an E4M3 cache is arb_attn_decode_e4m3).
+// The 4-bit form exists with the cache write only.
 template <int G>
 arb_status launch_g(Ctx *ctx, const StepArgs &a, int kv, int head_dim, const CUtensorMap &km, const CUtensorMap &vm,
                     cudaStream_t stream) {
-    if (kv == kKvE4m3) return launch_variant<G, true, kKvE4m3>(ctx, a, km, vm, stream);
+    if (kv == kKvE4m3)
+        return a.k_new != nullptr ? launch_variant<G, true, kKvE4m3>(ctx, a, km, vm, stream)
+                                  : launch_variant<G, false, kKvE4m3>(ctx, a, km, vm, stream);
     if (kv == kKvI4) return launch_variant<G, true, kKvI4>(ctx, a, km, vm, stream);
     if (head_dim == 64)
         return a.k_new != nullptr ? launch_variant<G, true, kKvBf16, 64>(ctx, a, km, vm, stream)
@@ -1241,7 +1243,7 @@ bool decode_step_supported(const arb_attn_params &p) {
 
 // k_new == nullptr: attention only (seq_lens is not written).  scales != nullptr: an E4M3 cache with scales =
 // {k_scale, v_scale, k_inv_scale, v_inv_scale}; k_row_scales != nullptr: a 4-bit cache with its two scale pools
-// (k_new is required for both); neither: a bf16 cache.
+// (k_new is required); neither: a bf16 cache.
 // beside: the decode rows of a call that has chunks too.  The chunk kernel, launched next, reads and writes nothing that this
 // one does, so it starts as soon as this kernel's predecessor is known to have completed, and this one takes only its share
 // of the SMs (kBesideWeight).
@@ -1251,7 +1253,7 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
                               float *k_row_scales, float *v_row_scales) {
     alignas(64) CUtensorMap km, vm;
     const bool e4m3 = scales != nullptr, i4 = k_row_scales != nullptr;
-    if ((e4m3 || i4) && k_new == nullptr) return ARB_ERR_INVALID_ARG;
+    if (i4 && k_new == nullptr) return ARB_ERR_INVALID_ARG;
     if (e4m3 && i4) return ARB_ERR_INVALID_ARG;
     bool whole_rows = false;
     if (i4) {
