@@ -472,7 +472,8 @@ __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, in
     const int r = item - pl.pref[lo];
     it.kvh = r / (pairs * P);
     const int rem = r - it.kvh * pairs * P;
-    const int pt = rem / P, part = rem - pt * P;
+    const int later = rem / P, part = rem - later * P;
+    const int pt = pairs - 1 - later;   // from the last pair of a sequence, which sees most keys, to the first
     it.r_begin = pt * 2 * kBM;
     it.rows[0] = min(kBM, it.rows_total - it.r_begin);
     it.rows[1] = max(0, min(kBM, it.rows_total - it.r_begin - kBM));
