@@ -130,8 +130,17 @@ struct MmaArgs {
     float v_scale;      // value scale of an E4M3 cache, 1 otherwise
 };
 
+// A work item: up to two consecutive row tiles (A, B) of one (sequence, kv head), over the KV tiles
+// [t0, t0 + ntiles) of the keys they see.  They share every K/V tile that is loaded; B may be missing
+// (rows[1] == 0).  `split`: the sequence's keys are cut into parts and this item leaves partials in
+// slots `slot` (tile A) and `slot + 1` (tile B).
+struct Item {
+    int b, kvh, n, L, rows_total, r_begin, rows[2], kv_len, t0, ntiles, qrow0, slot;   // ntiles < 0: there are no more
+    int split;
+};
+
 struct Bars {
-    uint64_t q_full;             // both softmax groups wrote their Q tiles
+    uint64_t q_full[2];          // Q tile A / B is written (a lone row tile: A alone)
     uint64_t k_full[kMaxStages];    // TMA bytes of a K tile landed
     uint64_t v_full[kMaxStages];
     uint64_t k_empty[kMaxStages];   // the first products that read the K stage have completed
@@ -144,6 +153,7 @@ struct Bars {
     uint64_t item_full[kItemSlots];   // the producer warp has fetched the next work item
     uint64_t item_empty[kItemSlots];  // the MMA thread, the V producer and the softmax threads have read it
     uint64_t code_full[2][kStagePages];   // E4M3: a page of codes of K / of V has landed in its staging slot
+    Item item[kItemSlots];            // (E4M3: the number alone)
     int item_id[kItemSlots];
     uint32_t tmem_base;
     int abort;
@@ -154,12 +164,13 @@ constexpr size_t smem_fixed() {
     return 1024 /*alignment*/ + 2 * Shape<HD>::kTileBytes /*Q of A, B*/ + 2 * Shape<HD>::kStages * Shape<HD>::kTileBytes /*K, V*/ + sizeof(Bars);
 }
 
+constexpr size_t kMlBytes = 2 * kSoftmaxThreads * sizeof(float2);
 constexpr size_t kCodeStageBytes = 2 * kStagePages * kCodePageBytes;   // E4M3: staging of both operands
 constexpr int kMaxBatchE4m3 = 320;   // the staging takes 24 KB of what the plan tables of a larger batch would need
 
 template <int HD>
 inline size_t mma_smem_bytes(int batch, bool e4m3) {
-    return smem_fixed<HD>() + (e4m3 ? kCodeStageBytes : 0) + sizeof(int) * (7 * (size_t)batch + 2);
+    return smem_fixed<HD>() + (e4m3 ? kCodeStageBytes : HD == 64 ? kMlBytes : 0) + sizeof(int) * (7 * (size_t)batch + 2);
 }
 
 // ---- tcgen05 / TMA wrappers -------------------------------------------------------------------
@@ -319,14 +330,8 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return r;
 }
 
-// A work item: up to two consecutive row tiles (A, B) of one (sequence, kv head), over the KV tiles
-// [t0, t0 + ntiles) of the keys they see.  They share every K/V tile that is loaded; B may be missing
-// (rows[1] == 0).  `split`: the sequence's keys are cut into parts and this item leaves partials in
-// slots `slot` (tile A) and `slot + 1` (tile B).
-struct Item {
-    int b, kvh, n, L, rows_total, r_begin, rows[2], kv_len, t0, ntiles, qrow0, slot;
-    bool split;
-};
+template <int N>
+struct IntC { static constexpr int value = N; };
 
 // The tables every CTA (and the combine kernel) derives from the lengths, in shared memory.
 struct Plan {
@@ -452,11 +457,22 @@ __device__ __forceinline__ int pair_kv_len(int L, int n, int rows_total, int r_b
 }
 __device__ __forceinline__ int part_tiles(int L, int P) {
     const int nt = (L + kBN - 1) / kBN;
-    return (nt + P - 1) / P;
+    return P > 1 ? (nt + P - 1) / P : nt;
 }
 
+// a / b for 0 <= a < 2^24, 0 < b, through the float reciprocal with a correction step: every role works an item out between
+// two items, and an integer division is some forty dependent instructions
+__device__ __forceinline__ int item_div(int a, int b) {
+    if (a >= (1 << 24)) return a / b;
+    int q = __float2int_rz(__fdividef((float)a, (float)b));
+    const int r = a - q * b;
+    if (r < 0) --q; else if (r >= b) ++q;
+    return q;
+}
+
+// Item number -> what it is, out of the plan's tables alone (a round trip to global memory here is one per item).
 template <int G>
-__device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, int B, int Hkv, const MmaArgs &a, Item &it) {
+__device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, int B, int Hkv, Item &it) {
     if (item >= total) return false;
     int lo = 0, hi = B;
     while (hi - lo > 1) {
@@ -465,14 +481,14 @@ __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, in
     }
     const int sb = pl.sorted[lo];  // pref runs over the sequences in serving order
     it.b = sb;
-    it.n = a.q_lens[sb];
-    it.L = a.seq_lens[sb];
+    it.n = pl.row0[sb + 1] - pl.row0[sb];
+    it.L = pl.key[sb];
     it.rows_total = it.n * G;
     const int pairs = pl.pairs[sb], P = pl.parts[lo];
     const int r = item - pl.pref[lo];
-    it.kvh = r / (pairs * P);
+    it.kvh = item_div(r, pairs * P);
     const int rem = r - it.kvh * pairs * P;
-    const int later = rem / P, part = rem - later * P;
+    const int later = P > 1 ? item_div(rem, P) : rem, part = rem - later * P;
     const int pt = pairs - 1 - later;   // from the last pair of a sequence, which sees most keys, to the first
     it.r_begin = pt * 2 * kBM;
     it.rows[0] = min(kBM, it.rows_total - it.r_begin);
@@ -502,7 +518,9 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
     char *k_s = base + 2 * kTileBytes;                 // [stage][2 halves][128 keys][128 B]
     char *v_s = k_s + kStages * kTileBytes;
     char *code_s = v_s + kStages * kTileBytes;         // E4M3: [K, V][kStagePages][16 rows][128 B of codes]
-    Bars *bars = reinterpret_cast<Bars *>(code_s + (E4M3 ? kCodeStageBytes : 0));
+    // (max, sum) of a lone row tile's two groups: the first half of Q tile B, which such an item does not use
+    float2 *ml = reinterpret_cast<float2 *>(HD == 64 ? code_s : q_s + kTileBytes);
+    Bars *bars = reinterpret_cast<Bars *>(code_s + (E4M3 ? kCodeStageBytes : HD == 64 ? kMlBytes : 0));
     const Plan pl = plan_arrays(reinterpret_cast<int *>(bars + 1), a.batch);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -510,7 +528,8 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
 
     let_successor_start();
     if (tid == 0) {
-        mbar_init(&bars->q_full, 2 * kSoftmaxThreads);
+        mbar_init(&bars->q_full[0], kSoftmaxThreads);
+        mbar_init(&bars->q_full[1], kSoftmaxThreads);
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&bars->k_full[s], E4M3 ? kWideners : 1);   // E4M3: every widening warp of the operand arrives
             mbar_init(&bars->v_full[s], E4M3 ? kWideners : 1);
@@ -566,6 +585,15 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
     const uint32_t tmem = bars->tmem_base;
     volatile int *abort = &bars->abort;
 
+    // What an announced item is.  The K warp works it out once for all roles; in the E4M3 form, whose K warps are its bottleneck,
+    // every role for itself (486 against 468 us per step-scoring batch the other way).
+    auto read_item = [&](uint32_t slot, Item &w) {
+        if constexpr (E4M3) {
+            if (!get_item<G>(bars->item_id[slot], total, pl, B, Hkv, w)) w.ntiles = -1;
+        } else {
+            w = bars->item[slot];
+        }
+    };
     const bool helper = E4M3 && warp >= kKHelpWarp;                          // a widening warp of the fourth group
     const int widx = helper ? 1 + (warp & 1) : 0;                            // which of the operand's wideners
     if (warp >= 2 * kSoftmaxThreads / 32) {   // the service warps
@@ -588,25 +616,37 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         Item w;
         for (uint32_t nq = 0;; ++nq) {
             const uint32_t slot = nq % kItemSlots, qpar = (nq / kItemSlots) & 1u;
-            int item = total;
-            if (lane == 0) {
-                if (!is_v && !helper) {
-                    if (nq == 0) {
-                        item = blockIdx.x;
-                    } else if (mbar_wait(&bars->item_empty[slot], qpar ^ 1u, abort, a.status)) {
+            if (!is_v && !helper) {
+                int item = blockIdx.x;
+                if (nq > 0) {
+                    item = total;
+                    if (lane == 0 && mbar_wait(&bars->item_empty[slot], qpar ^ 1u, abort, a.status)) {
                         const int taken = atomicAdd(a.work_counter, 1);   // `total` takes a call: the last of every CTA finds nothing
                         if (taken == total - 1) *a.work_counter = 0;
                         item = workers + taken;
                     }
+                    item = __shfl_sync(0xffffffffu, item, 0);
+                }
+                if (E4M3 && lane == 0) {
                     bars->item_id[slot] = item;
                     mbar_arrive(&bars->item_full[slot]);
-                } else if (mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) {
-                    item = bars->item_id[slot];
-                    mbar_arrive(&bars->item_empty[slot]);
                 }
+                if (!get_item<G>(item, total, pl, B, Hkv, w)) w.ntiles = -1;
+                if (!E4M3 && lane == 0) {
+                    bars->item[slot] = w;
+                    mbar_arrive(&bars->item_full[slot]);
+                }
+            } else {
+                bool there = true;
+                if (lane == 0) there = mbar_wait(&bars->item_full[slot], qpar, abort, a.status);
+                there = __shfl_sync(0xffffffffu, there ? 1 : 0, 0) != 0;
+                __syncwarp();   // lane 0's wait covers what the other lanes read (a shuffle alone orders no memory)
+                read_item(slot, w);
+                if (!there) w.ntiles = -1;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars->item_empty[slot]);
             }
-            item = __shfl_sync(0xffffffffu, item, 0);
-            if (!get_item<G>(item, total, pl, B, Hkv, a, w)) break;
+            if (w.ntiles < 0) break;
             // Block-table entries are read one step before they are used (the tile's own pages one tile
             // ahead, the pages to ask into L2 one tile before the request), so that no global-memory round
             // trip sits between two tiles.  Lanes 0-7: the pages of a tile; -1 marks "no such page".
@@ -748,18 +788,16 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         if (lane == 0) {
             constexpr uint32_t idesc_qk = instr_desc(kBN, false, E4M3);
             const uint32_t q_addr = smem_u32(q_s);
-            uint32_t it = 0, nitem = 0, nproc = 0;   // KV tiles so far, items, items with work
+            uint32_t it = 0, nitem = 0, nq[2] = {0u, 0u};   // KV tiles so far, items, Q tiles A and B so far
             uint32_t nfree[2] = {0u, 0u};            // S loads so far per group
             Item w;
             for (;; ++nitem) {
                 const uint32_t slot = nitem % kItemSlots, qpar = (nitem / kItemSlots) & 1u;
                 if (!mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) break;
-                const int item = bars->item_id[slot];
+                read_item(slot, w);
                 mbar_arrive(&bars->item_empty[slot]);
-                if (!get_item<G>(item, total, pl, B, Hkv, a, w)) break;
+                if (w.ntiles < 0) break;
                 if (w.ntiles == 0) continue;   // a part the pair sees nothing of: no role does anything for it
-                mbar_wait(&bars->q_full, nproc & 1u, abort, a.status);
-                ++nproc;
                 const bool lone = w.rows[1] == 0;
                 const int units = lone ? w.ntiles : 2 * w.ntiles;
                 // S of unit u: steps of 16 dims, 4 per 64-dim half; K-major operands, SBO = 8 rows.  A K stage is
@@ -767,6 +805,10 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 auto issue_qk = [&](int u) {
                     const uint32_t itx = it + (lone ? u : (u >> 1)), s = itx % kStages;
                     const int g = u & 1, qt = lone ? 0 : g;
+                    if (u == 0 || (u == 1 && !lone)) {
+                        mbar_wait(&bars->q_full[u], nq[u] & 1u, abort, a.status);
+                        ++nq[u];
+                    }
                     if (lone || g == 0) mbar_wait(&bars->k_full[s], (itx / kStages) & 1u, abort, a.status);
                     const uint32_t k_addr = smem_u32(k_s + s * kTileBytes);
                     tc_fence_after();
@@ -799,9 +841,9 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             for (;; ++nitem) {
                 const uint32_t slot = nitem % kItemSlots, qpar = (nitem / kItemSlots) & 1u;
                 if (!mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) break;
-                const int item = bars->item_id[slot];
+                read_item(slot, w);
                 mbar_arrive(&bars->item_empty[slot]);
-                if (!get_item<G>(item, total, pl, B, Hkv, a, w)) break;
+                if (w.ntiles < 0) break;
                 if (w.ntiles == 0) continue;
                 const bool lone = w.rows[1] == 0;
                 const int units = lone ? w.ntiles : 2 * w.ntiles;
@@ -839,51 +881,92 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         const uint32_t s_tmem = tmem + lane_base;                                  // S: one region for both groups
         const uint32_t p_tmem = tmem + lane_base + kPCol + grp * kPCols;           // this group's P
         const uint32_t o_tmem = tmem + lane_base + kOCol + grp * HD;
-        char *q_tile = q_s + grp * kTileBytes;
-        const int swz = tg & 7;
         uint32_t it = 0, itg = 0, nitem = 0;  // KV tiles so far: of all items, of those this group has worked on
         uint32_t nlone = 0;                   // items with one row tile so far
-        Item w;
+        // 16-byte chunk c (8 dims) of row r of a [128 x HD] tile: at c ^ (row & 7) of its 64-dim half
+        auto chunk_at = [](char *tile, int r, int c) -> char * { return tile + (c >> 3) * kHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4); };
+        constexpr int kLanesPerRow = HD / 8, kRowsPerPass = 32 / kLanesPerRow;
+        const int warp_row = tg & ~31;   // a warp loads and stores the 32 rows of its own TMEM lanes, neighbouring lanes a row:
+                                         // a row per lane instead touches 32 lines per instruction, 2 us per tile each way
+        // (with the item's decoding done once per CTA: prompts of 256 to 2048 tokens, six key tiles an item, 209 -> 183 us, the
+        // step-scoring batch with 64-dimension heads 415 -> 382 us, a 16-token step 31 -> 29 us)
+        auto row_offset = [&](const Item &w, int r) -> size_t {   // of query row r of the sequence in q and out, elements
+            const int tok = r / G;
+            return ((size_t)(w.qrow0 + tok) * a.Hq + w.kvh * G + (r - tok * G)) * HD;
+        };
+        auto load_q = [&](const Item &w, int r_first, int rows) {   // the group's Q tile
+            char *tile = q_s + grp * kTileBytes;
+#pragma unroll 8
+            for (int i = 0; i < 32 / kRowsPerPass; ++i) {
+                const int row = warp_row + i * kRowsPerPass + lane / kLanesPerRow, c = lane % kLanesPerRow;
+                const bool ok = row < rows;
+                const char *src = a.q + (row_offset(w, min(r_first + row, w.rows_total - 1)) + c * 8) * 2;
+                if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
+                    uint4 v = ok ? __ldg(reinterpret_cast<const uint4 *>(src)) : make_uint4(0, 0, 0, 0);
+                    v.x = bf16x2_to_f16x2(v.x); v.y = bf16x2_to_f16x2(v.y);
+                    v.z = bf16x2_to_f16x2(v.z); v.w = bf16x2_to_f16x2(v.w);
+                    *reinterpret_cast<uint4 *>(chunk_at(tile, row, c)) = v;
+                } else {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                                 ::"r"(smem_u32(chunk_at(tile, row, c))), "l"(src), "r"(ok ? 16 : 0) : "memory");
+                }
+            }
+            if constexpr (!E4M3) asm volatile("cp.async.wait_all;" ::: "memory");
+            fence_async_smem();   // the reader is the tensor core
+        };
+        // Writes the chunks c0 .. c0 + N - 1 of this warp's rows, which its lanes have left in `tile` (the Q tile of an item
+        // that is through with it), to out.
+        auto store_rows = [&](const Item &w, char *tile, int r_first, int rows, int c0, auto n_chunks) {
+            constexpr int N = decltype(n_chunks)::value, kPass = 32 / N;
+            __syncwarp();
+#pragma unroll 4
+            for (int i = 0; i < 32 / kPass; ++i) {
+                const int row = warp_row + i * kPass + lane / N, c = c0 + lane % N;
+                if (row < rows) {
+                    const int r = r_first + row;
+                    if (!ARB_IN_RANGE(a.status, w.qrow0 + r / G, a.rows)) continue;
+                    *reinterpret_cast<uint4 *>(a.out + (row_offset(w, r) + c * 8) * 2) = *reinterpret_cast<const uint4 *>(chunk_at(tile, row, c));
+                }
+            }
+        };
         for (;; ++nitem) {
             const uint32_t slot = nitem % kItemSlots, qpar = (nitem / kItemSlots) & 1u;
-            if (!mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) break;
-            const int item = bars->item_id[slot];
-            mbar_arrive(&bars->item_empty[slot]);
-            if (!get_item<G>(item, total, pl, B, Hkv, a, w)) break;
-            if (w.ntiles == 0) continue;   // a part the pair sees nothing of
+            // The branches on a wait's result and on the item leave the loop, so nothing else brings the lanes of a warp back
+            // together, and the tcgen05 loads and stores below want the whole warp: it meets here and behind every wait.
+            const bool there = mbar_wait(&bars->item_full[slot], qpar, abort, a.status);
+            if (!__all_sync(0xffffffffu, there)) break;
+            // read where it stands, and given back when the item is done: the registers of the loop below are all spoken for
+            Item mine;
+            if constexpr (E4M3) {
+                read_item(slot, mine);
+                mbar_arrive(&bars->item_empty[slot]);
+            }
+            const Item &w = E4M3 ? mine : bars->item[slot];
+            if (w.ntiles < 0) break;
+            if (w.ntiles == 0) {   // a part the pair sees nothing of
+                if constexpr (!E4M3) mbar_arrive(&bars->item_empty[slot]);
+                continue;
+            }
             // An item with one row tile is worked on by both groups: even KV tiles by group A, odd ones by group B,
             // each with an O of its own, merged in the epilogue.
             const bool lone = w.rows[1] == 0;
-            const int rows_here = lone ? w.rows[0] : w.rows[grp];
-            const bool row_ok = tg < rows_here;
-            const int r = min(w.r_begin + (lone ? 0 : grp * kBM) + tg, w.rows_total - 1);
-            const int tok = r / G, head = r - tok * G;
+            const int tok = min(w.r_begin + (lone ? 0 : grp * kBM) + tg, w.rows_total - 1) / G;
             const int lim = w.L - w.n + tok + 1;  // keys this row may see
-            const size_t grow = ((size_t)(w.qrow0 + tok) * a.Hq + w.kvh * G + head) * HD;
-            // ---- Q tile: row `tg`, chunks of 8 dims, chunk c of a half stored at c ^ (row & 7)
-            if (!(lone && grp == 1)) {   // (the second group of such an item reads Q tile A as well)
-                const uint4 *src = reinterpret_cast<const uint4 *>(a.q + grow * 2);
-#pragma unroll
-                for (int c = 0; c < HD / 8; ++c) {
-                    uint4 v = row_ok ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
-                    if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
-                        v.x = bf16x2_to_f16x2(v.x); v.y = bf16x2_to_f16x2(v.y);
-                        v.z = bf16x2_to_f16x2(v.z); v.w = bf16x2_to_f16x2(v.w);
-                    }
-                    *reinterpret_cast<uint4 *>(q_tile + (c >> 3) * kHalfBytes + tg * 128 + (((c & 7) ^ swz) << 4)) = v;
-                }
-                fence_async_smem();
+            if (!(lone && grp == 1)) {   // (the second group of a lone row tile reads Q tile A as well)
+                load_q(w, w.r_begin + (lone ? 0 : grp * kBM), lone ? w.rows[0] : w.rows[grp]);
+                mbar_arrive(&bars->q_full[grp]);
             }
-            mbar_arrive(&bars->q_full);
             float m_used = -INFINITY, l_sum = 0.f;
+            const int ntiles = w.ntiles, t0 = w.t0, kv_len = w.kv_len;   // what the loop needs
             const uint32_t it0 = it;
-            it += w.ntiles;
-            const int my_tiles = lone ? (w.ntiles + 1 - grp) / 2 : w.ntiles;   // KV tiles this group works on
-            for (int j = lone ? grp : 0, jt = 0; j < w.ntiles; j += lone ? 2 : 1, ++itg, ++jt) {
+            it += ntiles;
+            const int my_tiles = lone ? (ntiles + 1 - grp) / 2 : ntiles;   // KV tiles this group works on
+            for (int j = lone ? grp : 0, jt = 0; j < ntiles; j += lone ? 2 : 1, ++itg, ++jt) {
                 const uint32_t s = (it0 + j) % kStages, par = ((it0 + j) / kStages) & 1u;
-                const int key0 = (w.t0 + j) * kBN;
+                const int key0 = (t0 + j) * kBN;
                 const int nvis = lim - key0;  // columns < nvis are visible to this row (may be <= 0)
                 mbar_wait(&bars->s_full[grp], itg & 1u, abort, a.status);
+                __syncwarp();
                 tc_fence_after();
                 // ---- the whole row of S (128 scores) comes into registers with one round trip
                 uint32_t v[kBN];
@@ -920,6 +1003,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 // (it was issued when the group delivered that P, a whole softmax pass ago)
                 if (jt > 0) {
                     mbar_wait(&bars->o_full[grp], (itg - 1u) & 1u, abort, a.status);
+                    __syncwarp();
                     tc_fence_after();
                 }
                 if (__any_sync(0xffffffffu, rescale)) {
@@ -969,7 +1053,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 tmem_wait_st();
                 // ---- V rows past the last visible key of the item (stale slots, pages never loaded)
                 //      must not reach the tensor core, not even times zero
-                const int nvalid = w.kv_len - key0;
+                const int nvalid = kv_len - key0;
                 if (nvalid < kBN && (grp == 0 || lone)) {   // the P of group A (of a pair) is waited for first
                     mbar_wait(&bars->v_full[s], par, abort, a.status);
                     if (tg >= nvalid) {
@@ -986,21 +1070,22 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 tc_fence_before();
                 mbar_arrive(&bars->p_full[grp]);
             }
-            // ---- epilogue: O / l, bf16, one 256-byte row per thread
+            const int r_first = w.r_begin + (w.rows[1] == 0 ? 0 : grp * kBM), rows_here = w.rows[1] == 0 ? w.rows[0] : w.rows[grp];
+            const bool row_ok = tg < rows_here;
+            // ---- epilogue: O / l, bf16, one row of the output per thread
             if (my_tiles > 0) mbar_wait(&bars->o_full[grp], (itg - 1u) & 1u, abort, a.status);
+            __syncwarp();
             tc_fence_after();
-            const bool row_in = ARB_IN_RANGE(a.status, w.qrow0 + tok, a.rows);
             if (lone) {
                 // The two groups hold O, max and sum over the even and over the odd KV tiles of the same rows.  They
-                // exchange (max, sum) through the shared memory of Q tile B, which such an item does not use, and
-                // each merges and writes half of the dimensions: thread tg of either group owns TMEM lane tg and
+                // exchange (max, sum) through shared memory, and each merges and writes half of the dimensions: thread tg of either group owns TMEM lane tg and
                 // reads that lane of both O.
-                float2 *ml = reinterpret_cast<float2 *>(q_s + kTileBytes);
                 ml[grp * kSoftmaxThreads + tg] = make_float2(m_used, l_sum);
                 tc_fence_before();
                 mbar_arrive(&bars->ml_full);
                 mbar_wait(&bars->ml_full, nlone & 1u, abort, a.status);
                 ++nlone;
+                __syncwarp();
                 tc_fence_after();
                 const float2 ml0 = ml[tg], ml1 = ml[kSoftmaxThreads + tg];
                 const bool two = w.ntiles > 1;                       // else group B has worked on nothing: its O is undefined
@@ -1010,9 +1095,10 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 const float l = ml0.y * w0 + (two ? ml1.y * w1 : 0.f);
                 const bool slot_in = !w.split || ARB_IN_RANGE(a.status, w.slot, a.split_cap);
                 float *po = a.split_ws + (size_t)(w.split && slot_in ? w.slot : 0) * kSlotFloats;
+                // (staged where neither the other group nor (max, sum) is: tile A, or the second half of tile B)
+                char *stage = q_s + grp * kTileBytes;
                 const float norm = w.split ? (E4M3 ? a.v_scale : 1.0f) : (E4M3 ? a.v_scale : 1.0f) / l;
                 const uint32_t oa = tmem + lane_base + kOCol, ob = oa + HD;
-                uint4 *dst = reinterpret_cast<uint4 *>(a.out + grow * 2);
 #pragma unroll 1
                 for (int c4 = HD / 64 * grp; c4 < HD / 64 * (grp + 1); ++c4) {
                     uint32_t va[32];
@@ -1035,7 +1121,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                                 *reinterpret_cast<float4 *>(po + ((size_t)(c4 * 8 + qd) * kBM + tg) * 4) =
                                     make_float4(o[qd * 4], o[qd * 4 + 1], o[qd * 4 + 2], o[qd * 4 + 3]);
                         }
-                    } else if (row_ok && row_in) {
+                    } else {
 #pragma unroll
                         for (int qd = 0; qd < 4; ++qd) {
                             uint4 o4;
@@ -1043,16 +1129,14 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                             o4.y = pack_bf16(o[qd * 8 + 2], o[qd * 8 + 3]);
                             o4.z = pack_bf16(o[qd * 8 + 4], o[qd * 8 + 5]);
                             o4.w = pack_bf16(o[qd * 8 + 6], o[qd * 8 + 7]);
-                            dst[c4 * 4 + qd] = o4;
+                            *reinterpret_cast<uint4 *>(chunk_at(stage, tg, c4 * 4 + qd)) = o4;
                         }
                     }
                 }
+                if (!w.split) store_rows(w, stage, r_first, rows_here, HD / 16 * grp, IntC<HD / 16>());
                 if (w.split && grp == 0 && row_ok && slot_in)
                     *reinterpret_cast<float2 *>(po + (size_t)kBM * HD + tg * 2) = make_float2(m, l);
-                tc_fence_before();
-                continue;
-            }
-            if (w.split) {
+            } else if (w.split) {
                 // one part of a split sequence: leave the un-normalised O row and its (max, sum)
                 const bool slot_in = ARB_IN_RANGE(a.status, w.slot + grp, a.split_cap);
                 float *po = a.split_ws + (size_t)(slot_in ? w.slot + grp : 0) * kSlotFloats;
@@ -1073,17 +1157,14 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                     }
                 }
                 if (row_ok && slot_in) *reinterpret_cast<float2 *>(po + (size_t)kBM * HD + tg * 2) = make_float2(m_used, l_sum);
-                tc_fence_before();
-                continue;
-            }
-            const float inv_l = (E4M3 ? a.v_scale : 1.0f) / l_sum;
-            uint4 *dst = reinterpret_cast<uint4 *>(a.out + grow * 2);
+            } else {
+                const float inv_l = (E4M3 ? a.v_scale : 1.0f) / l_sum;
+                char *stage = q_s + grp * kTileBytes;   // the group's last product has read its Q tile
 #pragma unroll 1
-            for (int c4 = 0; c4 < HD / 32; ++c4) {
-                uint32_t v[32];
-                tmem_ld32(o_tmem + c4 * 32, v);
-                tmem_wait_ld();
-                if (row_ok && row_in) {
+                for (int c4 = 0; c4 < HD / 32; ++c4) {
+                    uint32_t v[32];
+                    tmem_ld32(o_tmem + c4 * 32, v);
+                    tmem_wait_ld();
 #pragma unroll
                     for (int qd = 0; qd < 4; ++qd) {
                         uint4 o4;
@@ -1091,10 +1172,13 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                         o4.y = pack_bf16(__uint_as_float(v[qd * 8 + 2]) * inv_l, __uint_as_float(v[qd * 8 + 3]) * inv_l);
                         o4.z = pack_bf16(__uint_as_float(v[qd * 8 + 4]) * inv_l, __uint_as_float(v[qd * 8 + 5]) * inv_l);
                         o4.w = pack_bf16(__uint_as_float(v[qd * 8 + 6]) * inv_l, __uint_as_float(v[qd * 8 + 7]) * inv_l);
-                        dst[c4 * 4 + qd] = o4;
+                        *reinterpret_cast<uint4 *>(chunk_at(stage, tg, c4 * 4 + qd)) = o4;
                     }
                 }
+                store_rows(w, stage, r_first, rows_here, 0, IntC<HD / 8>());
             }
+            __syncwarp();   // the warp's rows of the tile are read before the next item's Q takes their place
+            if constexpr (!E4M3) mbar_arrive(&bars->item_empty[slot]);
             tc_fence_before();
         }
     }
