@@ -1,4 +1,4 @@
-// The two operations on whole score vectors that need an order: Spearman's rho and the budgeted oracle.
+// The two operations on whole score vectors that need an order: Spearman's rho and the budgeted oracle rule.
 //
 // Spearman's rho (the rank correlation the paper reports between router scores and the oracle advantage,
 // Section 4.2 "Evaluation" and Tables 1-3): ranks with ties sharing the mean of the ranks they span, then the
