@@ -182,14 +182,14 @@ __device__ __forceinline__ uint32_t e4m3x2_from_f32(float lo, float hi) {
     return r;
 }
 // 4-bit cache: a 32-bit word holds 8 dimensions as nibbles (code + 8), nibble i and nibble i + 4 being the neighbouring
-// dimensions 2i and 2i + 1.  Moved to bits 3-6 under the exponent of 16, a nibble is the bf16 number 16 + nibble = code +
-// kI4Bias: two integer instructions per pair.  The products run on the biased numbers (small whole numbers, exact) and the
-// bias comes off again in fp32: S starts from -kI4Bias * sum(q), and one more MMA against a constant sums what the weights
-// add to every row of O^T.
-constexpr float kI4Bias = 24.0f;
-constexpr uint32_t kI4BiasPair = 0x41C041C0u;   // kI4Bias as two bf16
+// dimensions 2i and 2i + 1.  A nibble in the low bits of the bf16 128 counts in ones (128 + nibble); one exact
+// subtraction of 136 leaves the code.  The codes themselves enter the products: left biased (the number 16 + nibble is an
+// instruction cheaper) they make every partial sum of S = q . k carry 24 sum(q), and a q with one large component then
+// lost what the other dimensions add.
 __device__ __forceinline__ uint32_t i4_pair_to_bf16x2(uint32_t w, int i) {
-    return ((i == 0 ? w << 3 : w >> (4 * i - 3)) & 0x00780078u) | 0x41804180u;
+    uint32_t r;
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(((w >> (4 * i)) & 0x000F000Fu) | 0x43004300u), "r"(0x3F803F80u), "r"(0xC308C308u));
+    return r;
 }
 
 // Codes of one key row for S^T -> the two registers of k-step ks: row = this lane's 32 dimensions (8 or 4 words).
@@ -745,20 +745,6 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         // this lane's columns (heads h0, h1): running max (the same in the 8 lanes of a column pair), its share of
         // the sum, and the m-tiles of O^T: o[mt][0..1] = dim 16 mt + gq of heads h0, h1; o[mt][2..3] = dim + 8
         float m_run0 = -INFINITY, m_run1 = -INFINITY, l_run0 = 0.f, l_run1 = 0.f;
-        float q_bias0 = 0.f, q_bias1 = 0.f;         // 4-bit cache: what the codes' bias adds to the scores of heads h0, h1, negated
-        float o_bias[4] = {0.f, 0.f, 0.f, 0.f};     // ... and (the first two) to every row of O^T
-        if constexpr (I4) {
-            float sum = 0.f;   // of head gq: this lane's 32 dimensions, then the row's four lanes
-#pragma unroll
-            for (int ks = 0; ks < kD / 16; ++ks)
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    sum += __uint_as_float(qb[ks][i] << 16) + __uint_as_float(qb[ks][i] & 0xffff0000u);
-            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-            q_bias0 = -kI4Bias * __shfl_sync(0xffffffffu, sum, 4 * h0);
-            q_bias1 = -kI4Bias * __shfl_sync(0xffffffffu, sum, 4 * h1);
-        }
         float o[kD / 16][4];
 #pragma unroll
         for (int mt = 0; mt < kD / 16; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
@@ -770,7 +756,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             const uint32_t ck = seg_base + 2u * (uint32_t)gi;
 
             // ---- S^T = K q^T: 16 keys x 8 heads, two accumulators so that the chain is four deep ----------
-            float sa[4] = {q_bias0, q_bias1, q_bias0, q_bias1}, sb[4] = {0.f, 0.f, 0.f, 0.f};
+            float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
             float ksc0 = 1.f, ksc1 = 1.f, vsc0 = 1.f, vsc1 = 1.f;   // 4-bit cache: the scales of keys gq and gq + 8
             {
                 const uint32_t st = ck % STAGES, par = (ck / STAGES) & 1u;
@@ -885,7 +871,6 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             if (__any_sync(0xffffffffu, f0 != 1.0f || f1 != 1.0f)) {
 #pragma unroll
                 for (int mt = 0; mt < kD / 16; ++mt) { o[mt][0] *= f0; o[mt][1] *= f1; o[mt][2] *= f0; o[mt][3] *= f1; }
-                if constexpr (I4) { o_bias[0] *= f0; o_bias[1] *= f1; }
             }
 
             // ---- O^T += V^T P^T: m-tiles of 16 dims ---------------------------------------------------
@@ -950,10 +935,6 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                         v_fragment<E4M3>(vw[2], vw[3], mt, af[2], af[3]);
                         mma_16816<E4M3>(o[mt], af, pb0, pb1);
                     }
-                    if constexpr (I4) {
-                        const uint32_t af[4] = {kI4BiasPair, kI4BiasPair, kI4BiasPair, kI4BiasPair};
-                        mma_16816<false>(o_bias, af, pb0, pb1);
-                    }
                 } else {
                     if (patch_here) {
                         if (lane >= 16 && lane - 16 < kD / 8)
@@ -998,7 +979,6 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         for (int mt = 0; mt < kD / 16; ++mt) {
             if constexpr (CODES) {   // dimensions 16 gq + 2 mt and + 1
                 const int d = 16 * gq + 2 * mt;
-                if constexpr (I4) { o[mt][0] -= o_bias[0]; o[mt][1] -= o_bias[1]; o[mt][2] -= o_bias[0]; o[mt][3] -= o_bias[1]; }
                 if (h0 < G) *reinterpret_cast<float2 *>(rec + 16 + h0 * kOStride + d) = make_float2(o[mt][0], o[mt][2]);
                 if (h1 < G) *reinterpret_cast<float2 *>(rec + 16 + h1 * kOStride + d) = make_float2(o[mt][1], o[mt][3]);
                 continue;

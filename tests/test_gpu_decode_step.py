@@ -390,6 +390,29 @@ def _live(codes, scales, inp, lens):
     return codes, s
 
 
+def test_decode_step_i4_keeps_small_dimensions_beside_a_large_one():
+    """A query component of 2^20 against codes that are 0 in its dimension: every product there is exactly 0, so the
+    scores are sums of at most 128 products below 7 * 5 and the bar of the other cases holds.  (Partial sums that carried a
+    multiple of sum(q) would be rounded to whole units.)"""
+    sl = [700, 31, 1600]
+    inp = wl.small_attn_case(3, 12, 2, 128, BF, [n + 1 for n in sl], [1] * 3, seed=990)
+    inp.seq_lens.sub_(1)
+    inp.q[..., 0] = 2.0 ** 20
+    inp.k_pages[..., 0] = 0.0
+    kc, ks = map(torch.from_numpy, oracle.i4_encode(inp.k_pages))
+    vc, vs = map(torch.from_numpy, oracle.i4_encode(inp.v_pages))
+    k_new, v_new = _new_rows(inp, 3, 991)
+    k_new[..., 0] = 0.0
+    c, d = H.ctx(), inp.to("cuda")
+    out = c.decode_step_i4(d.q, k_new.cuda(), v_new.cuda(), kc.cuda(), vc.cuda(), ks.cuda(), vs.cuda(), d.block_table,
+                           d.seq_lens, d.q_lens)
+    assert c.poll_status() == 0
+    ok, ov, oks, ovs, osl, st = oracle.kv_append_i4(k_new, v_new, inp.block_table, inp.seq_lens, inp.q_lens, kc, vc, ks, vs)
+    ref, st2 = oracle.attn_i4(inp.q, ok, ov, oks, ovs, inp.block_table, osl, inp.q_lens)
+    assert st == 0 and st2 == 0
+    _i4_close(out, ref, ovs)
+
+
 def test_decode_step_i4_chain_in_place_and_as_a_graph():
     c = H.ctx()
     B, T = 5, 10
