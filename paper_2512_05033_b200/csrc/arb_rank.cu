@@ -307,7 +307,7 @@ policy_budget_kernel(int n, int lg, const float *__restrict__ s_d, const float *
     const int m = 1 << lg, per = m / kThreads, base = me * m;
     const uint32_t below = (1u << lane) - 1u;
 
-    // the bits of a positive float order as the float does; 0: not worth a call
+    // the bits of a positive float order as the float does, infinity last; 0: not worth a call (a NaN advantage is not)
     uint32_t key[kMaxPer];
 #pragma unroll
     for (int j = 0; j < kMaxPer; ++j) {
@@ -315,7 +315,7 @@ policy_budget_kernel(int n, int lg, const float *__restrict__ s_d, const float *
         const int i = base + j * kThreads + tid;
         if (j < per && i < n) {
             const uint32_t d = __float_as_uint(sub_ieee(s_t[i], s_d[i]));
-            if ((int)d > 0) key[j] = d;
+            if ((int)d > 0 && d <= 0x7f800000u) key[j] = d;
         }
     }
     for (int i = tid; i < kPasses * kDigits; i += kThreads) (&s.hist[0][0])[i] = 0;

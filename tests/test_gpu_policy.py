@@ -248,3 +248,26 @@ def test_ranks_and_budget_at_the_edges_of_the_cluster(n, levels):
     ref, rho = oracle.spearman(st, y), float(c.spearman(st.cuda(), y.cuda()).item())
     assert (math.isnan(ref) and math.isnan(rho)) or abs(ref - rho) <= 1e-12, (rho, ref)
     assert c.poll_status() == 0
+
+
+@pytest.mark.parametrize("n", [9, 3000])
+def test_budget_takes_infinite_advantages_first_and_nan_never(n):
+    """An advantage that is NaN (a NaN score, inf - inf) is not positive: it is not escalated and uses up no budget."""
+    from paper_2512_05033_b200 import binding
+    c = H.ctx()
+    sd, st = _scores(n, 70 + n)
+    nan, inf = float("nan"), float("inf")
+    sd[:9] = torch.tensor([nan, 0.1, -nan, inf, -inf, 0.2, inf, -inf, nan])
+    st[:9] = torch.tensor([0.9, nan, -nan, inf, -inf, inf, 0.5, 0.5, inf])
+    perm = torch.randperm(n, generator=torch.Generator().manual_seed(n))
+    sd, st = sd[perm].contiguous(), st[perm].contiguous()
+    bad = torch.isnan(st - sd)                                # the oracle's sort has no place for a NaN: an advantage of 0
+    osd, ost = torch.where(bad, 0.5, sd), torch.where(bad, 0.5, st)
+    assert int(bad.sum()) == 6
+    stats = c.new_policy_stats("cuda")
+    for budget in (0, 1, 2, 3, n // 3, n):
+        dec = c.policy(binding.POLICY_ORACLE_BUDGET, sd.cuda(), st.cuda(), budget=budget, stats=stats)
+        got, (ref, rs) = c.policy_stats(stats), oracle.policy(binding.POLICY_ORACLE_BUDGET, osd, ost, budget=budget)
+        assert np.array_equal(dec.cpu().numpy(), ref), budget
+        assert (got["escalated"], got["wasted"]) == (rs["escalated"], rs["wasted"])
+    assert c.poll_status() == 0
