@@ -150,6 +150,7 @@ struct Bars {
     uint64_t o_full[2];          // O += P V of row tile A / B has completed
     uint64_t s_free[2];          // group A / B holds the S it was given in registers: the S region is free
     uint64_t ml_full;            // an item with one row tile: both softmax groups have left their (max, sum)
+    uint64_t ml_free;            // ... and every softmax thread has read them
     uint64_t item_full[kItemSlots];   // the producer warp has fetched the next work item
     uint64_t item_empty[kItemSlots];  // the MMA thread, the V producer and the softmax threads have read it
     uint64_t code_full[2][kStagePages];   // E4M3: a page of codes of K / of V has landed in its staging slot
@@ -169,9 +170,11 @@ constexpr size_t kCodeStageBytes = 2 * kStagePages * kCodePageBytes;   // E4M3: 
 constexpr int kMaxBatchE4m3 = 320;   // the staging takes 24 KB of what the plan tables of a larger batch would need
 
 template <int HD>
-inline size_t mma_smem_bytes(int batch, bool e4m3) {
+constexpr size_t mma_smem_bytes(int batch, bool e4m3) {
     return smem_fixed<HD>() + (e4m3 ? kCodeStageBytes : HD == 64 ? kMlBytes : 0) + sizeof(int) * (7 * (size_t)batch + 2);
 }
+
+static_assert(mma_smem_bytes<128>(kMaxBatchE4m3, true) <= 227 * 1024 && mma_smem_bytes<128>(kMaxBatch, false) <= 227 * 1024, "shared memory of a CTA");
 
 // ---- tcgen05 / TMA wrappers -------------------------------------------------------------------
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -545,6 +548,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         mbar_init(&bars->s_free[0], kSoftmaxThreads);
         mbar_init(&bars->s_free[1], kSoftmaxThreads);
         mbar_init(&bars->ml_full, 2 * kSoftmaxThreads);
+        mbar_init(&bars->ml_free, 2 * kSoftmaxThreads);
         for (int i = 0; i < kItemSlots; ++i) {
             mbar_init(&bars->item_full[i], 1);
             // the two MMA threads, the V warp, the softmax threads (E4M3: and the four helping warps)
@@ -952,6 +956,9 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             const bool lone = w.rows[1] == 0;
             const int tok = min(w.r_begin + (lone ? 0 : grp * kBM) + tg, w.rows_total - 1) / G;
             const int lim = w.L - w.n + tok + 1;  // keys this row may see
+            // The (max, sum) of the lone row tile before must have been read by every thread before Q tile B, or the next
+            // lone tile's (max, sum), takes their place.
+            if (nlone > 0) mbar_wait(&bars->ml_free, (nlone - 1u) & 1u, abort, a.status);
             if (!(lone && grp == 1)) {   // (the second group of a lone row tile reads Q tile A as well)
                 load_q(w, w.r_begin + (lone ? 0 : grp * kBM), lone ? w.rows[0] : w.rows[grp]);
                 mbar_arrive(&bars->q_full[grp]);
@@ -1088,6 +1095,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 __syncwarp();
                 tc_fence_after();
                 const float2 ml0 = ml[tg], ml1 = ml[kSoftmaxThreads + tg];
+                mbar_arrive(&bars->ml_free);
                 const bool two = w.ntiles > 1;                       // else group B has worked on nothing: its O is undefined
                 const float m = fmaxf(ml0.x, two ? ml1.x : -INFINITY);
                 const float w0 = ml0.x == -INFINITY ? 0.f : fast_exp2(ml0.x - m);

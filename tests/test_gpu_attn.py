@@ -718,3 +718,35 @@ def test_decode_rows_beside_chunks_match_oracle(case):
     assert c.poll_status() == 0 and st == 0
     for got in copies:
         H.assert_close(got.double().cpu().numpy(), ref, BF, tight=3e-3)
+
+
+LONE_CASES = [
+    # (Hq, Hkv, seq_lens, q_lens): row tiles in threes (a lone one before its sequence's pair), and lone row tiles over a
+    # single key tile one behind the other
+    (32, 8, [400 + 7 * i for i in range(24)], [96] * 24),
+    (32, 8, [128 - i for i in range(40)], [2 + i % 31 for i in range(40)]),
+    (28, 4, [1000 + 61 * i for i in range(20)] + [100] * 20, [18 + 37 * (i % 2) for i in range(40)]),
+]
+
+
+@pytest.mark.parametrize("e4m3", [False, True])
+@pytest.mark.parametrize("case", LONE_CASES)
+def test_lone_row_tiles_followed_by_others(case, e4m3):
+    """The two softmax groups of a lone row tile exchange (max, sum) through shared memory that the next item uses again:
+    more items than CTAs, so that every CTA takes several, the same bits call after call."""
+    Hq, Hkv, sl, ql = case
+    inp = wl.small_attn_case(len(sl), Hq, Hkv, 128, BF, sl, ql, seed=810 + Hq)
+    c, d = H.ctx(), inp.to("cuda")
+    if e4m3:
+        kc, vc = (torch.from_numpy(oracle.e4m3_encode(p, 1 / 0.0125)) for p in (inp.k_pages, inp.v_pages))
+        ref, st = oracle.attn_e4m3(inp.q, kc, vc, 0.0125, 0.0125, inp.block_table, inp.seq_lens, inp.q_lens)
+        dk, dv = kc.cuda(), vc.cuda()
+        call = lambda out: c.attn_e4m3(d.q, dk, dv, 0.0125, 0.0125, d.block_table, d.seq_lens, d.q_lens, max(ql), out=out)
+    else:
+        ref, st = H.oracle_attn(inp)
+        call = lambda out: c.attn(d.q, d.k_pages, d.v_pages, d.block_table, d.seq_lens, d.q_lens, max(ql), out=out)
+    outs = [call(torch.full_like(d.q, float("nan"))) for _ in range(12)]
+    assert c.poll_status() == 0 and st == 0
+    H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
+    for o in outs[1:]:
+        assert torch.equal(o, outs[0])
