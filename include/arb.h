@@ -103,7 +103,9 @@ typedef struct {
     int32_t page_size;         /* 16 */
     int32_t num_pages;         /* pages in the pool that k_pages / v_pages point to */
     int32_t max_pages_per_seq; /* row length of block_table */
-    int32_t total_q;           /* sum of q_lens (rows of q and out); the host knows it */
+    int32_t total_q;           /* sum of q_lens (rows of q and out); the host knows it.  Step chunks: should the lengths on
+                                  the device add up to more, rows from total_q on are neither read nor written, and a step
+                                  longer than total_q counts as a bad length */
     int32_t max_q_len;         /* max of q_lens; 1 selects the decode kernel alone */
     float softmax_scale;       /* <= 0 selects 1/sqrt(head_dim) */
     uint32_t flags;            /* ARB_ATTN_* bits, 0 for none */

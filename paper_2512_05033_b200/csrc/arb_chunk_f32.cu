@@ -55,6 +55,10 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool real
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(real ? 16 : 0) : "memory");
 }
 
+// Tokens of a sequence that q and out have rows for: all of them, unless the q_lens on the device add up to more than the
+// caller's total_q.
+__device__ __forceinline__ int rows_there(const F32Args &a, int qrow0, int n) { return qrow0 < 0 ? 0 : max(0, min(n, a.rows - qrow0)); }
+
 // One row tile over the key tiles [t0, t1); nparts > 1: leaves partial `slot` and merges if it is the last to arrive.
 template <int D, int G>
 __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, int t0, int t1, int qrow0, int nparts,
@@ -63,6 +67,7 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
     constexpr int kLaneRows = D == 128 ? 8 : 4;     // rows of O a lane holds, 4 dimensions each
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = a.q_lens[b], L = a.seq_lens[b], rows = n * G, r_begin = rt * kRows;
+    const int there = rows_there(a, qrow0, n) * G;   // rows that q and out have
     const int kv_len = L - n + (min(r_begin + kRows, rows) - 1) / G + 1;   // keys the tile's last row sees
     t1 = min(t1, (kv_len + kKeys - 1) / kKeys);
     auto row_of = [&](int i) -> size_t {   // first element of row i of the tile in q and out
@@ -75,7 +80,7 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
     for (int i = tid; i < kRows * kVecs; i += kThreads) {
         const int r = i / kVecs, c = i - r * kVecs;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r_begin + r < rows) {
+        if (r_begin + r < there) {
             x = __ldg(reinterpret_cast<const float4 *>(a.q + row_of(r)) + c);
             x.x *= a.scale_log2; x.y *= a.scale_log2; x.z *= a.scale_log2; x.w *= a.scale_log2;
         }
@@ -203,7 +208,7 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
 #pragma unroll
         for (int r = 0; r < kLaneRows; ++r) {
             const int i = warp * kWarpRows + orow + r;
-            if (r_begin + i < rows && ARB_IN_RANGE(a.status, qrow0 + (r_begin + i) / G, a.rows)) {
+            if (r_begin + i < there && ARB_IN_RANGE(a.status, qrow0 + (r_begin + i) / G, a.rows)) {
                 const float inv = s.row[warp][orow + r];
                 *reinterpret_cast<float4 *>(a.out + row_of(i) + odim) =
                     make_float4(o[r][0] * inv, o[r][1] * inv, o[r][2] * inv, o[r][3] * inv);
@@ -236,7 +241,7 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
     // m = max_p m_p, w_p = 2^(m_p - m), out = sum_p w_p o_p / sum_p w_p l_p; part 0 sees key 0: m is finite
     const float *p0 = a.partials + (size_t)slot_first * slot_floats<D>();
     const int i = tid / (kThreads / kRows), c0 = tid % (kThreads / kRows);   // four threads per row
-    if (r_begin + i >= rows || !ARB_IN_RANGE(a.status, qrow0 + (r_begin + i) / G, a.rows)) return;
+    if (r_begin + i >= there || !ARB_IN_RANGE(a.status, qrow0 + (r_begin + i) / G, a.rows)) return;
     float M = -INFINITY;
 #pragma unroll 8
     for (int p = 0; p < nparts; ++p) M = fmaxf(M, __ldcg(p0 + p * slot_floats<D>() + kRows * D + i));
@@ -274,7 +279,7 @@ chunk_f32_kernel(const F32Args a) {
     pdl_enter();
     auto shape = [&](int b, int &rts, int &kts) {   // row tiles and key tiles of a sequence this kernel serves
         const int n = a.q_lens[b], L = a.seq_lens[b];
-        const bool ok = n >= 2 && L >= n && L <= a.max_pages * kPage;
+        const bool ok = n >= 2 && n <= a.rows && L >= n && L <= a.max_pages * kPage;
         rts = ok ? (n * G + kRows - 1) / kRows : 0;
         kts = ok ? (L + kKeys - 1) / kKeys : 0;
         return n >= 2 && !ok;
@@ -307,7 +312,7 @@ chunk_f32_kernel(const F32Args a) {
         int rts, kts;
         if (!shape(b, rts, kts)) continue;
         if (tid == 0) atomicOr(a.status, (uint32_t)ARB_DEV_BAD_SEQ_LEN);
-        for (size_t i = tid; i < (size_t)(row0[b + 1] - row0[b]) * a.Hq * D; i += kThreads) a.out[(size_t)row0[b] * a.Hq * D + i] = 0.f;
+        for (size_t i = tid; i < (size_t)rows_there(a, row0[b], row0[b + 1] - row0[b]) * a.Hq * D; i += kThreads) a.out[(size_t)row0[b] * a.Hq * D + i] = 0.f;
     }
     const long long total = units[B];
     if (total == 0) return;

@@ -360,7 +360,16 @@ __device__ __forceinline__ Plan plan_arrays(int *base, int B) {
 }
 
 // A chunk whose lengths fit: what this kernel serves.  One whose lengths do not has its rows zero-filled.
-__device__ __forceinline__ bool chunk_ok(const MmaArgs &a, int n, int L) { return n >= 2 && L >= n && L <= a.max_pages * kPage; }
+__device__ __forceinline__ bool chunk_ok(const MmaArgs &a, int n, int L) {
+    return n >= 2 && n <= a.rows && L >= n && L <= a.max_pages * kPage;
+}
+
+// Query rows (tokens times heads of the group) of a sequence that q and out have: all of them, unless the q_lens on the
+// device add up to more than the caller's total_q.
+template <int G>
+__device__ __forceinline__ int rows_there(const MmaArgs &a, int qrow0, int n) {
+    return qrow0 < 0 ? 0 : max(0, min(n, a.rows - qrow0)) * G;
+}
 
 // Fills the plan; every thread of the block takes part.
 template <int G>
@@ -475,9 +484,9 @@ __device__ __forceinline__ int item_div(int a, int b) {
 
 // Item number -> what it is, out of the plan's tables alone (a round trip to global memory here is one per item).
 template <int G>
-__device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, int B, int Hkv, Item &it) {
+__device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, const MmaArgs &a, Item &it) {
     if (item >= total) return false;
-    int lo = 0, hi = B;
+    int lo = 0, hi = a.batch;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (pl.pref[mid] <= item) lo = mid; else hi = mid;
@@ -494,8 +503,10 @@ __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, in
     const int later = P > 1 ? item_div(rem, P) : rem, part = rem - later * P;
     const int pt = pairs - 1 - later;   // from the last pair of a sequence, which sees most keys, to the first
     it.r_begin = pt * 2 * kBM;
-    it.rows[0] = min(kBM, it.rows_total - it.r_begin);
-    it.rows[1] = max(0, min(kBM, it.rows_total - it.r_begin - kBM));
+    it.qrow0 = pl.row0[sb];
+    const int rows = rows_there<G>(a, it.qrow0, it.n);
+    it.rows[0] = max(0, min(kBM, rows - it.r_begin));
+    it.rows[1] = max(0, min(kBM, rows - it.r_begin - kBM));
     it.kv_len = pair_kv_len<G>(it.L, it.n, it.rows_total, it.r_begin);   // keys the pair's last row sees
     const int nt_pair = (it.kv_len + kBN - 1) / kBN;
     const int T = part_tiles(it.L, P);
@@ -503,7 +514,6 @@ __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, in
     it.ntiles = max(0, min(it.t0 + T, nt_pair) - it.t0);   // 0: nothing of this part is visible to the pair
     it.split = P > 1;
     it.slot = pl.sslot[lo] + ((it.kvh * pairs + pt) * P + part) * 2;
-    it.qrow0 = pl.row0[sb];
     return true;
 }
 
@@ -570,8 +580,8 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         const int n = a.q_lens[b];
         if (n < 2 || pl.pairs[b] > 0) continue;
         if (tid == 0) atomicOr(a.status, (uint32_t)ARB_DEV_BAD_SEQ_LEN);
-        for (int i = pl.row0[b]; i < pl.row0[b] + n; ++i) {
-            if (!ARB_IN_RANGE(a.status, i, a.rows)) break;
+        const int there = rows_there<1>(a, pl.row0[b], n);
+        for (int i = pl.row0[b]; i < pl.row0[b] + there; ++i) {
             uint4 *o = reinterpret_cast<uint4 *>(a.out + (size_t)i * a.Hq * HD * 2);
             for (int c = tid; c < a.Hq * HD / 8; c += threads_of(E4M3)) o[c] = make_uint4(0, 0, 0, 0);
         }
@@ -593,7 +603,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
     // every role for itself (486 against 468 us per step-scoring batch the other way).
     auto read_item = [&](uint32_t slot, Item &w) {
         if constexpr (E4M3) {
-            if (!get_item<G>(bars->item_id[slot], total, pl, B, Hkv, w)) w.ntiles = -1;
+            if (!get_item<G>(bars->item_id[slot], total, pl, a, w)) w.ntiles = -1;
         } else {
             w = bars->item[slot];
         }
@@ -635,7 +645,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                     bars->item_id[slot] = item;
                     mbar_arrive(&bars->item_full[slot]);
                 }
-                if (!get_item<G>(item, total, pl, B, Hkv, w)) w.ntiles = -1;
+                if (!get_item<G>(item, total, pl, a, w)) w.ntiles = -1;
                 if (!E4M3 && lane == 0) {
                     bars->item[slot] = w;
                     mbar_arrive(&bars->item_full[slot]);
@@ -904,7 +914,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             for (int i = 0; i < 32 / kRowsPerPass; ++i) {
                 const int row = warp_row + i * kRowsPerPass + lane / kLanesPerRow, c = lane % kLanesPerRow;
                 const bool ok = row < rows;
-                const char *src = a.q + (row_offset(w, min(r_first + row, w.rows_total - 1)) + c * 8) * 2;
+                const char *src = a.q + (ok ? (row_offset(w, r_first + row) + c * 8) * 2 : 0);
                 if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
                     uint4 v = ok ? __ldg(reinterpret_cast<const uint4 *>(src)) : make_uint4(0, 0, 0, 0);
                     v.x = bf16x2_to_f16x2(v.x); v.y = bf16x2_to_f16x2(v.y);
@@ -1225,7 +1235,7 @@ chunk_combine_kernel(const MmaArgs a) {
         const int P = pl.parts[r];
         if (P <= 1) continue;
         const int sb = pl.sorted[r], pairs = pl.pairs[sb];
-        const int n = a.q_lens[sb], L = a.seq_lens[sb], rows_total = n * G;
+        const int n = a.q_lens[sb], L = a.seq_lens[sb], rows_total = n * G, rows = rows_there<G>(a, pl.row0[sb], n);
         const int T = part_tiles(L, P);
         const int njobs = Hkv * pairs * 2 * kPieces;
         // the jobs of this sequence that fall to this CTA
@@ -1236,7 +1246,7 @@ chunk_combine_kernel(const MmaArgs a) {
             const int qd = j % kPieces, jt = j / kPieces;
             const int g = jt & 1, pt = (jt >> 1) % pairs, kvh = (jt >> 1) / pairs;
             const int r_begin = pt * 2 * kBM;
-            const int rows_here = max(0, min(kBM, rows_total - r_begin - g * kBM));
+            const int rows_here = max(0, min(kBM, rows - r_begin - g * kBM));
             if (tid >= rows_here) continue;
             const int nt_pair = (pair_kv_len<G>(L, n, rows_total, r_begin) + kBN - 1) / kBN;
             const int nparts = min(P, (nt_pair + T - 1) / T);   // parts the pair sees something of

@@ -750,3 +750,41 @@ def test_lone_row_tiles_followed_by_others(case, e4m3):
     H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
     for o in outs[1:]:
         assert torch.equal(o, outs[0])
+
+
+@pytest.mark.parametrize("dtype,D", [(BF, 128), (BF, 64), (F32, 128), ("e4m3", 128)])
+@pytest.mark.parametrize("Hq,Hkv,sl,ql,rows", [
+    (8, 2, [300, 90, 500], [40, 7, 60], 90),             # the last sequence's rows 43 .. 59 are missing
+    (32, 8, [700, 5000, 260], [30, 1, 200], 31),         # ... all of them
+    (8, 1, [26000, 26000, 3], [20, 30, 9], 33),          # a split sequence cut short; a bad length behind the end
+])
+def test_rows_beyond_total_q_are_left_alone(dtype, D, Hq, Hkv, sl, ql, rows):
+    """q_lens on the device that add up to more than the caller's total_q: the rows there are come out as ever, and nothing
+    behind them is written (the buffers go on, so that a stray access shows and does not fault)."""
+    from paper_2512_05033_b200 import binding
+    e4m3 = dtype == "e4m3"
+    dt = BF if e4m3 else dtype
+    inp = wl.small_attn_case(len(sl), Hq, Hkv, D, dt, [max(a, b) for a, b in zip(sl, ql)], ql, seed=830 + Hq)
+    inp.seq_lens.copy_(torch.tensor(sl))
+    c, d = H.ctx(), inp.to("cuda")
+    out = torch.full_like(d.q, 4096.0)
+    most = max(n for n in ql if n <= rows)
+    if e4m3:
+        kc, vc = (torch.from_numpy(oracle.e4m3_encode(p, 1 / 0.0125)) for p in (inp.k_pages, inp.v_pages))
+        ref, st = oracle.attn_e4m3(inp.q, kc, vc, 0.0125, 0.0125, inp.block_table, inp.seq_lens, inp.q_lens)
+        c.attn_e4m3(d.q[:rows], kc.cuda(), vc.cuda(), 0.0125, 0.0125, d.block_table, d.seq_lens, d.q_lens,
+                    most, out=out[:rows])
+    else:
+        ref, st = H.oracle_attn(inp)
+        c.attn(d.q[:rows], d.k_pages, d.v_pages, d.block_table, d.seq_lens, d.q_lens, most, out=out[:rows])
+    bits = c.poll_status()
+    got = out.double().cpu().numpy()
+    assert (got[rows:] == 4096.0).all(), "a row behind total_q was written"
+    bad = [n > rows or n > a for n, a in zip(ql, sl)]    # a step longer than total_q counts as a bad length
+    assert bits == (binding.DEV_BAD_SEQ_LEN if any(bad) else 0)
+    at = 0
+    for n, b in zip(ql, bad):
+        if b:
+            ref[at:at + n] = 0.0
+        at += n
+    H.assert_close(got[:rows], ref[:rows], dt, tight=3e-3 if dt == BF else None)
