@@ -482,8 +482,10 @@ __device__ __forceinline__ int item_div(int a, int b) {
     return q;
 }
 
-// Item number -> what it is, out of the plan's tables alone (a round trip to global memory here is one per item).
-template <int G>
+// Item number -> what it is, out of the plan's tables alone (a round trip to global memory here is one per item).  In the
+// E4M3 form sixteen warps hold this code and its values between the tiles of an item, and the plain divisions and the
+// lengths from L1 are the better ones: step-scoring batch over codes 446 -> 443 us, prompts of 32 / 8 heads 283 -> 277 us.
+template <int G, bool E4M3>
 __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, const MmaArgs &a, Item &it) {
     if (item >= total) return false;
     int lo = 0, hi = a.batch;
@@ -493,18 +495,18 @@ __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, co
     }
     const int sb = pl.sorted[lo];  // pref runs over the sequences in serving order
     it.b = sb;
-    it.n = pl.row0[sb + 1] - pl.row0[sb];
-    it.L = pl.key[sb];
+    it.n = E4M3 ? a.q_lens[sb] : pl.row0[sb + 1] - pl.row0[sb];
+    it.L = E4M3 ? a.seq_lens[sb] : pl.key[sb];
     it.rows_total = it.n * G;
     const int pairs = pl.pairs[sb], P = pl.parts[lo];
     const int r = item - pl.pref[lo];
-    it.kvh = item_div(r, pairs * P);
+    it.kvh = E4M3 ? r / (pairs * P) : item_div(r, pairs * P);
     const int rem = r - it.kvh * pairs * P;
-    const int later = P > 1 ? item_div(rem, P) : rem, part = rem - later * P;
+    const int later = E4M3 ? rem / P : P > 1 ? item_div(rem, P) : rem, part = rem - later * P;
     const int pt = pairs - 1 - later;   // from the last pair of a sequence, which sees most keys, to the first
     it.r_begin = pt * 2 * kBM;
     it.qrow0 = pl.row0[sb];
-    const int rows = rows_there<G>(a, it.qrow0, it.n);
+    const int rows = E4M3 ? it.rows_total : rows_there<G>(a, it.qrow0, it.n);
     it.rows[0] = max(0, min(kBM, rows - it.r_begin));
     it.rows[1] = max(0, min(kBM, rows - it.r_begin - kBM));
     it.kv_len = pair_kv_len<G>(it.L, it.n, it.rows_total, it.r_begin);   // keys the pair's last row sees
@@ -599,13 +601,18 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
     const uint32_t tmem = bars->tmem_base;
     volatile int *abort = &bars->abort;
 
-    // What an announced item is.  The K warp works it out once for all roles; in the E4M3 form, whose K warps are its bottleneck,
-    // every role for itself (486 against 468 us per step-scoring batch the other way).
-    auto read_item = [&](uint32_t slot, Item &w) {
+    // What an announced item is.  The K warp works it out once for all roles; in the E4M3 form, whose widening warps set the
+    // pace, every role for itself (486 against 468 us per step-scoring batch the other way).
+    // false: there are no more.
+    auto read_item = [&](uint32_t slot, Item &w) -> bool {
         if constexpr (E4M3) {
-            if (!get_item<G>(bars->item_id[slot], total, pl, a, w)) w.ntiles = -1;
+            const int item = bars->item_id[slot];
+            mbar_arrive(&bars->item_empty[slot]);
+            return get_item<G, E4M3>(item, total, pl, a, w);
         } else {
             w = bars->item[slot];
+            mbar_arrive(&bars->item_empty[slot]);
+            return w.ntiles >= 0;
         }
     };
     const bool helper = E4M3 && warp >= kKHelpWarp;                          // a widening warp of the fourth group
@@ -630,37 +637,49 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         Item w;
         for (uint32_t nq = 0;; ++nq) {
             const uint32_t slot = nq % kItemSlots, qpar = (nq / kItemSlots) & 1u;
-            if (!is_v && !helper) {
-                int item = blockIdx.x;
-                if (nq > 0) {
-                    item = total;
-                    if (lane == 0 && mbar_wait(&bars->item_empty[slot], qpar ^ 1u, abort, a.status)) {
-                        const int taken = atomicAdd(a.work_counter, 1);   // `total` takes a call: the last of every CTA finds nothing
-                        if (taken == total - 1) *a.work_counter = 0;
-                        item = workers + taken;
+            // the number of the next item, in lane 0; `total`: there are no more
+            auto take_item = [&]() -> int {
+                if (nq == 0) return (int)blockIdx.x;
+                if (!mbar_wait(&bars->item_empty[slot], qpar ^ 1u, abort, a.status)) return total;
+                const int taken = atomicAdd(a.work_counter, 1);   // `total` takes a call: the last of every CTA finds nothing
+                if (taken == total - 1) *a.work_counter = 0;
+                return workers + taken;
+            };
+            if constexpr (E4M3) {
+                int item = total;
+                if (lane == 0) {
+                    if (!is_v && !helper) {
+                        item = take_item();
+                        bars->item_id[slot] = item;
+                        mbar_arrive(&bars->item_full[slot]);
+                    } else if (mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) {
+                        item = bars->item_id[slot];
+                        mbar_arrive(&bars->item_empty[slot]);
                     }
-                    item = __shfl_sync(0xffffffffu, item, 0);
                 }
-                if (E4M3 && lane == 0) {
-                    bars->item_id[slot] = item;
-                    mbar_arrive(&bars->item_full[slot]);
-                }
-                if (!get_item<G>(item, total, pl, a, w)) w.ntiles = -1;
-                if (!E4M3 && lane == 0) {
+                item = __shfl_sync(0xffffffffu, item, 0);
+                if (!get_item<G, E4M3>(item, total, pl, a, w)) break;
+            } else if (!is_v) {
+                int item = total;
+                if (lane == 0) item = take_item();
+                item = __shfl_sync(0xffffffffu, item, 0);
+                if (!get_item<G, E4M3>(item, total, pl, a, w)) w.ntiles = -1;
+                if (lane == 0) {
                     bars->item[slot] = w;
                     mbar_arrive(&bars->item_full[slot]);
                 }
+                if (w.ntiles < 0) break;
             } else {
                 bool there = true;
                 if (lane == 0) there = mbar_wait(&bars->item_full[slot], qpar, abort, a.status);
                 there = __shfl_sync(0xffffffffu, there ? 1 : 0, 0) != 0;
                 __syncwarp();   // lane 0's wait covers what the other lanes read (a shuffle alone orders no memory)
-                read_item(slot, w);
+                w = bars->item[slot];
                 if (!there) w.ntiles = -1;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars->item_empty[slot]);
+                if (w.ntiles < 0) break;
             }
-            if (w.ntiles < 0) break;
             // Block-table entries are read one step before they are used (the tile's own pages one tile
             // ahead, the pages to ask into L2 one tile before the request), so that no global-memory round
             // trip sits between two tiles.  Lanes 0-7: the pages of a tile; -1 marks "no such page".
@@ -808,9 +827,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             for (;; ++nitem) {
                 const uint32_t slot = nitem % kItemSlots, qpar = (nitem / kItemSlots) & 1u;
                 if (!mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) break;
-                read_item(slot, w);
-                mbar_arrive(&bars->item_empty[slot]);
-                if (w.ntiles < 0) break;
+                if (!read_item(slot, w)) break;
                 if (w.ntiles == 0) continue;   // a part the pair sees nothing of: no role does anything for it
                 const bool lone = w.rows[1] == 0;
                 const int units = lone ? w.ntiles : 2 * w.ntiles;
@@ -855,9 +872,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             for (;; ++nitem) {
                 const uint32_t slot = nitem % kItemSlots, qpar = (nitem / kItemSlots) & 1u;
                 if (!mbar_wait(&bars->item_full[slot], qpar, abort, a.status)) break;
-                read_item(slot, w);
-                mbar_arrive(&bars->item_empty[slot]);
-                if (w.ntiles < 0) break;
+                if (!read_item(slot, w)) break;
                 if (w.ntiles == 0) continue;
                 const bool lone = w.rows[1] == 0;
                 const int units = lone ? w.ntiles : 2 * w.ntiles;
@@ -903,7 +918,9 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
         const int warp_row = tg & ~31;   // a warp loads and stores the 32 rows of its own TMEM lanes, neighbouring lanes a row:
                                          // a row per lane instead touches 32 lines per instruction, 2 us per tile each way
         // (with the item's decoding done once per CTA: prompts of 256 to 2048 tokens, six key tiles an item, 209 -> 183 us, the
-        // step-scoring batch with 64-dimension heads 415 -> 382 us, a 16-token step 31 -> 29 us)
+        // step-scoring batch with 64-dimension heads 415 -> 382 us, a 16-token step 31 -> 29 us.  The E4M3 form keeps a row per
+        // lane: its widening warps fill the load and store units of shared memory, and q has to pass through registers to
+        // become f16 anyway; prompts over codes, 32 / 8 heads, 296 us by whole rows, 278 this way)
         auto row_offset = [&](const Item &w, int r) -> size_t {   // of query row r of the sequence in q and out, elements
             const int tok = r / G;
             return ((size_t)(w.qrow0 + tok) * a.Hq + w.kvh * G + (r - tok * G)) * HD;
@@ -915,18 +932,10 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 const int row = warp_row + i * kRowsPerPass + lane / kLanesPerRow, c = lane % kLanesPerRow;
                 const bool ok = row < rows;
                 const char *src = a.q + (ok ? (row_offset(w, r_first + row) + c * 8) * 2 : 0);
-                if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
-                    uint4 v = ok ? __ldg(reinterpret_cast<const uint4 *>(src)) : make_uint4(0, 0, 0, 0);
-                    v.x = bf16x2_to_f16x2(v.x); v.y = bf16x2_to_f16x2(v.y);
-                    v.z = bf16x2_to_f16x2(v.z); v.w = bf16x2_to_f16x2(v.w);
-                    *reinterpret_cast<uint4 *>(chunk_at(tile, row, c)) = v;
-                } else {
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                                 ::"r"(smem_u32(chunk_at(tile, row, c))), "l"(src), "r"(ok ? 16 : 0) : "memory");
-                }
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                             ::"r"(smem_u32(chunk_at(tile, row, c))), "l"(src), "r"(ok ? 16 : 0) : "memory");
             }
-            if constexpr (!E4M3) asm volatile("cp.async.wait_all;" ::: "memory");
-            fence_async_smem();   // the reader is the tensor core
+            asm volatile("cp.async.wait_all;" ::: "memory");
         };
         // Writes the chunks c0 .. c0 + N - 1 of this warp's rows, which its lanes have left in `tile` (the Q tile of an item
         // that is through with it), to out.
@@ -952,11 +961,10 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             // read where it stands, and given back when the item is done: the registers of the loop below are all spoken for
             Item mine;
             if constexpr (E4M3) {
-                read_item(slot, mine);
-                mbar_arrive(&bars->item_empty[slot]);
+                if (!read_item(slot, mine)) break;
             }
             const Item &w = E4M3 ? mine : bars->item[slot];
-            if (w.ntiles < 0) break;
+            if (!E4M3 && w.ntiles < 0) break;
             if (w.ntiles == 0) {   // a part the pair sees nothing of
                 if constexpr (!E4M3) mbar_arrive(&bars->item_empty[slot]);
                 continue;
@@ -964,13 +972,24 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             // An item with one row tile is worked on by both groups: even KV tiles by group A, odd ones by group B,
             // each with an O of its own, merged in the epilogue.
             const bool lone = w.rows[1] == 0;
-            const int tok = min(w.r_begin + (lone ? 0 : grp * kBM) + tg, w.rows_total - 1) / G;
-            const int lim = w.L - w.n + tok + 1;  // keys this row may see
-            // The (max, sum) of the lone row tile before must have been read by every thread before Q tile B, or the next
-            // lone tile's (max, sum), takes their place.
-            if (nlone > 0) mbar_wait(&bars->ml_free, (nlone - 1u) & 1u, abort, a.status);
+            const int row = min(w.r_begin + (lone ? 0 : grp * kBM) + tg, w.rows_total - 1);   // this thread's
+            const int lim = w.L - w.n + row / G + 1;  // keys it may see
+            const bool own_ok = E4M3 && tg < (lone ? w.rows[0] : w.rows[grp]) && (unsigned)(w.qrow0 + row / G) < (unsigned)a.rows;
+            const size_t own = E4M3 ? row_offset(w, row) : 0;
             if (!(lone && grp == 1)) {   // (the second group of a lone row tile reads Q tile A as well)
-                load_q(w, w.r_begin + (lone ? 0 : grp * kBM), lone ? w.rows[0] : w.rows[grp]);
+                if constexpr (E4M3) {   // the operands of one MMA share a type: q goes to f16 like the widened codes
+                    const uint4 *src = reinterpret_cast<const uint4 *>(a.q + (own_ok ? own * 2 : 0));
+#pragma unroll
+                    for (int c = 0; c < HD / 8; ++c) {
+                        uint4 v = own_ok ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
+                        v.x = bf16x2_to_f16x2(v.x); v.y = bf16x2_to_f16x2(v.y);
+                        v.z = bf16x2_to_f16x2(v.z); v.w = bf16x2_to_f16x2(v.w);
+                        *reinterpret_cast<uint4 *>(chunk_at(q_s + grp * kTileBytes, tg, c)) = v;
+                    }
+                } else {
+                    load_q(w, w.r_begin + (lone ? 0 : grp * kBM), lone ? w.rows[0] : w.rows[grp]);
+                }
+                fence_async_smem();   // the reader is the tensor core
                 mbar_arrive(&bars->q_full[grp]);
             }
             float m_used = -INFINITY, l_sum = 0.f;
@@ -1088,7 +1107,8 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                 mbar_arrive(&bars->p_full[grp]);
             }
             const int r_first = w.r_begin + (w.rows[1] == 0 ? 0 : grp * kBM), rows_here = w.rows[1] == 0 ? w.rows[0] : w.rows[grp];
-            const bool row_ok = tg < rows_here;
+            const bool row_ok = E4M3 ? own_ok : tg < rows_here;
+            uint4 *dst = reinterpret_cast<uint4 *>(a.out + own * 2);   // E4M3: this thread's row
             // ---- epilogue: O / l, bf16, one row of the output per thread
             if (my_tiles > 0) mbar_wait(&bars->o_full[grp], (itg - 1u) & 1u, abort, a.status);
             __syncwarp();
@@ -1139,7 +1159,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                                 *reinterpret_cast<float4 *>(po + ((size_t)(c4 * 8 + qd) * kBM + tg) * 4) =
                                     make_float4(o[qd * 4], o[qd * 4 + 1], o[qd * 4 + 2], o[qd * 4 + 3]);
                         }
-                    } else {
+                    } else if (!E4M3 || row_ok) {
 #pragma unroll
                         for (int qd = 0; qd < 4; ++qd) {
                             uint4 o4;
@@ -1147,13 +1167,16 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                             o4.y = pack_bf16(o[qd * 8 + 2], o[qd * 8 + 3]);
                             o4.z = pack_bf16(o[qd * 8 + 4], o[qd * 8 + 5]);
                             o4.w = pack_bf16(o[qd * 8 + 6], o[qd * 8 + 7]);
-                            *reinterpret_cast<uint4 *>(chunk_at(stage, tg, c4 * 4 + qd)) = o4;
+                            if constexpr (!E4M3) *reinterpret_cast<uint4 *>(chunk_at(stage, tg, c4 * 4 + qd)) = o4;
+                            else dst[c4 * 4 + qd] = o4;
                         }
                     }
                 }
-                if (!w.split) store_rows(w, stage, r_first, rows_here, HD / 16 * grp, IntC<HD / 16>());
+                if (!E4M3 && !w.split) store_rows(w, stage, r_first, rows_here, HD / 16 * grp, IntC<HD / 16>());
                 if (w.split && grp == 0 && row_ok && slot_in)
                     *reinterpret_cast<float2 *>(po + (size_t)kBM * HD + tg * 2) = make_float2(m, l);
+                // every thread has read (max, sum) before the next item's Q tile B, or the next lone tile, takes their place
+                mbar_wait(&bars->ml_free, (nlone - 1u) & 1u, abort, a.status);
             } else if (w.split) {
                 // one part of a split sequence: leave the un-normalised O row and its (max, sum)
                 const bool slot_in = ARB_IN_RANGE(a.status, w.slot + grp, a.split_cap);
@@ -1183,17 +1206,20 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
                     uint32_t v[32];
                     tmem_ld32(o_tmem + c4 * 32, v);
                     tmem_wait_ld();
+                    if (!E4M3 || row_ok) {
 #pragma unroll
-                    for (int qd = 0; qd < 4; ++qd) {
-                        uint4 o4;
-                        o4.x = pack_bf16(__uint_as_float(v[qd * 8 + 0]) * inv_l, __uint_as_float(v[qd * 8 + 1]) * inv_l);
-                        o4.y = pack_bf16(__uint_as_float(v[qd * 8 + 2]) * inv_l, __uint_as_float(v[qd * 8 + 3]) * inv_l);
-                        o4.z = pack_bf16(__uint_as_float(v[qd * 8 + 4]) * inv_l, __uint_as_float(v[qd * 8 + 5]) * inv_l);
-                        o4.w = pack_bf16(__uint_as_float(v[qd * 8 + 6]) * inv_l, __uint_as_float(v[qd * 8 + 7]) * inv_l);
-                        *reinterpret_cast<uint4 *>(chunk_at(stage, tg, c4 * 4 + qd)) = o4;
+                        for (int qd = 0; qd < 4; ++qd) {
+                            uint4 o4;
+                            o4.x = pack_bf16(__uint_as_float(v[qd * 8 + 0]) * inv_l, __uint_as_float(v[qd * 8 + 1]) * inv_l);
+                            o4.y = pack_bf16(__uint_as_float(v[qd * 8 + 2]) * inv_l, __uint_as_float(v[qd * 8 + 3]) * inv_l);
+                            o4.z = pack_bf16(__uint_as_float(v[qd * 8 + 4]) * inv_l, __uint_as_float(v[qd * 8 + 5]) * inv_l);
+                            o4.w = pack_bf16(__uint_as_float(v[qd * 8 + 6]) * inv_l, __uint_as_float(v[qd * 8 + 7]) * inv_l);
+                            if constexpr (!E4M3) *reinterpret_cast<uint4 *>(chunk_at(stage, tg, c4 * 4 + qd)) = o4;
+                            else dst[c4 * 4 + qd] = o4;
+                        }
                     }
                 }
-                store_rows(w, stage, r_first, rows_here, 0, IntC<HD / 8>());
+                if constexpr (!E4M3) store_rows(w, stage, r_first, rows_here, 0, IntC<HD / 8>());
             }
             __syncwarp();   // the warp's rows of the tile are read before the next item's Q takes their place
             if constexpr (!E4M3) mbar_arrive(&bars->item_empty[slot]);
