@@ -77,6 +77,16 @@ int size_of(const at::Tensor &t, int dim, const char *name) {
     return (int)t.size(dim);
 }
 
+// The sizes of a tensor mean what they should only at the right rank: a pool of all layers, or a batch of rows with a
+// dimension of its own, would be read with the wrong ones.
+const at::Tensor &of_rank(const at::Tensor &t, int rank, const char *name) {
+    if (t.dim() != rank) {
+        PyErr_Format(PyExc_ValueError, "%s must have %d dimensions, got %d", name, rank, (int)t.dim());
+        throw Raised();
+    }
+    return t;
+}
+
 long integer(PyObject *o) {
     const long v = PyLong_AsLong(o);
     if (v == -1 && PyErr_Occurred()) throw Raised();
@@ -119,16 +129,22 @@ arb_attn_params from_record(PyObject *record) {   // the caller's own AttnParams
 }
 
 arb_attn_params params_for(const at::Tensor &q, const at::Tensor &pool, const at::Tensor &table, int max_q_len, PyObject *scale,
-                           int flags, int head_dim, PyObject *record) {
-    if (record != Py_None) return from_record(record);
-    return {dtype_code(q), size_of(table, 0, "block_table"), size_of(q, 1, "q"), size_of(pool, 1, "pool"), head_dim,
-            size_of(pool, 2, "pool"), size_of(pool, 0, "pool"), size_of(table, 1, "block_table"), size_of(q, 0, "q"),
-            max_q_len, real(scale), (uint32_t)flags};
+                           int flags, PyObject *record, bool exact_q = true) {
+    if (record != Py_None) return from_record(record);   // the tensors' shapes are the caller's business then
+    if (exact_q) of_rank(q, 3, "q");
+    size_of(q, 2, "q");
+    of_rank(pool, 4, "the pool");
+    of_rank(table, 2, "block_table");
+    return {dtype_code(q), (int)table.size(0), (int)q.size(1), (int)pool.size(1), (int)q.size(2), (int)pool.size(2), (int)pool.size(0),
+            (int)table.size(1), (int)q.size(0), max_q_len, real(scale), (uint32_t)flags};
 }
-arb_attn_params params_for_append(const at::Tensor &rows, int dtype, const at::Tensor &pool, const at::Tensor &table, int head_dim) {
-    const int hkv = size_of(pool, 1, "pool");
-    return {dtype, size_of(table, 0, "block_table"), hkv, hkv, head_dim, size_of(pool, 2, "pool"), size_of(pool, 0, "pool"),
-            size_of(table, 1, "block_table"), 0, 0, 0.0f, 0u};
+// code_pack: dimensions per element of a pool row
+arb_attn_params params_for_append(int dtype, const at::Tensor &pool, const at::Tensor &table, int code_pack) {
+    of_rank(pool, 4, "the pool");
+    of_rank(table, 2, "block_table");
+    const int hkv = (int)pool.size(1);
+    return {dtype, (int)table.size(0), hkv, hkv, code_pack * (int)pool.size(3), (int)pool.size(2), (int)pool.size(0),
+            (int)table.size(1), 0, 0, 0.0f, 0u};
 }
 
 // Runs `body` (arguments checked, the call made without the GIL) and turns its status into a Python int.
@@ -172,7 +188,7 @@ constexpr auto kBf16 = at::kBFloat16;
 METHOD(attn) {
     return guarded(n, 12, [&] {
         const at::Tensor &q = tensor(a[1], "q"), &kp = tensor(a[2], "k_pages"), &bt = tensor(a[4], "block_table");
-        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[7]), a[9], 0, size_of(q, 2, "q"), a[11]);
+        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[7]), a[9], 0, a[11]);
         arb_ctx *h = context(a[0]);
         void *qp = dev(q, "q"), *k = dev(kp, "k_pages", q.scalar_type()), *v = dev(a[3], "v_pages", q.scalar_type());
         void *t = dev(bt, "block_table", kI32), *sl = dev(a[5], "seq_lens", kI32), *ql = dev(a[6], "q_lens", kI32);
@@ -187,11 +203,11 @@ METHOD(attn_host) {
     return guarded(n, 13, [&] {
         const at::Tensor &q = tensor(a[1], "q_host"), &kp = tensor(a[2], "k_pages"), &bt = tensor(a[4], "block_table_host");
         void *qp = host(q), *t = host(bt), *sl = host(a[5]), *ql = host(a[6]), *out = host(a[8]);
-        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[7]), a[9], (int)integer(a[10]), size_of(q, 2, "q_host"), Py_None);
+        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[7]), a[9], (int)integer(a[10]), Py_None);
         arb_ctx *h = context(a[0]);
         void *k = dev(kp, "k_pages"), *v = dev(tensor(a[3], "v_pages"), "v_pages");
         arb_stream_t s = stream_of(a[11]);
-        auto call = integer(a[12]) ? lib.arb_attn_host_begin : lib.arb_attn_host;
+        auto call = (int)integer(a[12]) ? lib.arb_attn_host_begin : lib.arb_attn_host;
         return without_gil([&] { return call(h, &p, qp, k, v, I32(t), I32(sl), I32(ql), out, s); });
     });
 }
@@ -208,7 +224,7 @@ METHOD(attn_host_wait) {
 METHOD(decode_step) {
     return guarded(n, 13, [&] {
         const at::Tensor &q = tensor(a[1], "q"), &kp = tensor(a[4], "k_pages"), &bt = tensor(a[6], "block_table");
-        const arb_attn_params p = params_for(q, kp, bt, 1, a[10], 0, size_of(q, 2, "q"), a[12]);
+        const arb_attn_params p = params_for(q, kp, bt, 1, a[10], 0, a[12]);
         arb_ctx *h = context(a[0]);
         const auto dt = q.scalar_type();
         void *qp = dev(q, "q"), *kn = dev(a[2], "k_new", dt), *vn = dev(a[3], "v_new", dt), *k = dev(kp, "k_pages", dt);
@@ -223,7 +239,7 @@ METHOD(decode_step) {
 METHOD(decode_step_e4m3) {
     return guarded(n, 17, [&] {
         const at::Tensor &q = tensor(a[1], "q"), &kp = tensor(a[4], "k_codes"), &bt = tensor(a[10], "block_table");
-        const arb_attn_params p = params_for(q, kp, bt, 1, a[14], 0, size_of(q, 2, "q"), a[16]);
+        const arb_attn_params p = params_for(q, kp, bt, 1, a[14], 0, a[16]);
         arb_ctx *h = context(a[0]);
         void *qp = dev(q, "q", kBf16), *kn = dev(a[2], "k_new", kBf16), *vn = dev(a[3], "v_new", kBf16);
         void *k = dev(kp, "k_codes", kU8), *v = dev(a[5], "v_codes", kU8), *t = dev(bt, "block_table", kI32);
@@ -240,7 +256,7 @@ METHOD(decode_step_e4m3) {
 METHOD(decode_step_i4) {
     return guarded(n, 15, [&] {
         const at::Tensor &q = tensor(a[1], "q"), &kp = tensor(a[4], "k_codes"), &bt = tensor(a[8], "block_table");
-        const arb_attn_params p = params_for(q, kp, bt, 1, a[12], 0, size_of(q, 2, "q"), a[14]);
+        const arb_attn_params p = params_for(q, kp, bt, 1, a[12], 0, a[14], false);
         arb_ctx *h = context(a[0]);
         void *qp = dev(q, "q", kBf16), *kn = dev(a[2], "k_new", kBf16), *vn = dev(a[3], "v_new", kBf16);
         void *k = dev(kp, "k_codes", kU8), *v = dev(a[5], "v_codes", kU8);
@@ -258,7 +274,7 @@ METHOD(kv_append) {
     return guarded(n, 10, [&] {
         const at::Tensor &kn = tensor(a[1], "k_new"), &bt = tensor(a[3], "block_table"), &kp = tensor(a[6], "k_pages");
         const auto dt = kp.scalar_type();
-        const arb_attn_params p = params_for_append(kn, dtype_code(kp), kp, bt, size_of(kp, 3, "k_pages"));
+        const arb_attn_params p = params_for_append(dtype_code(kp), kp, bt, 1);
         arb_ctx *h = context(a[0]);
         void *k = dev(kn, "k_new", dt), *v = dev(a[2], "v_new", dt), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[4], "seq_lens", kI32), *nl = dev(a[5], "new_lens", kI32), *ko = dev(kp, "k_pages"), *vo = dev(a[7], "v_pages", dt);
@@ -272,7 +288,7 @@ METHOD(kv_append) {
 METHOD(kv_append_e4m3) {
     return guarded(n, 12, [&] {
         const at::Tensor &kn = tensor(a[1], "k_new"), &bt = tensor(a[5], "block_table"), &kp = tensor(a[8], "k_codes");
-        const arb_attn_params p = params_for_append(kn, dtype_code(kn), kp, bt, size_of(kp, 3, "k_codes"));
+        const arb_attn_params p = params_for_append(dtype_code(kn), kp, bt, 1);
         arb_ctx *h = context(a[0]);
         void *k = dev(kn, "k_new"), *v = dev(a[2], "v_new", kn.scalar_type()), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[6], "seq_lens", kI32), *nl = dev(a[7], "new_lens", kI32), *ko = dev(kp, "k_codes", kU8), *vo = dev(a[9], "v_codes", kU8);
@@ -287,7 +303,7 @@ METHOD(kv_append_e4m3) {
 METHOD(kv_append_i4) {
     return guarded(n, 12, [&] {
         const at::Tensor &kn = tensor(a[1], "k_new"), &bt = tensor(a[3], "block_table"), &kp = tensor(a[6], "k_codes");
-        const arb_attn_params p = params_for_append(kn, dtype_code(kn), kp, bt, 2 * size_of(kp, 3, "k_codes"));
+        const arb_attn_params p = params_for_append(dtype_code(kn), kp, bt, 2);
         arb_ctx *h = context(a[0]);
         void *k = dev(kn, "k_new", kBf16), *v = dev(a[2], "v_new", kBf16), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[4], "seq_lens", kI32), *nl = dev(a[5], "new_lens", kI32), *ko = dev(kp, "k_codes", kU8), *vo = dev(a[7], "v_codes", kU8);
@@ -304,13 +320,13 @@ METHOD(kv_append_i4) {
 METHOD(attn_e4m3) {
     return guarded(n, 16, [&] {
         const at::Tensor &q = tensor(a[1], "q"), &kp = tensor(a[2], "k_codes"), &bt = tensor(a[6], "block_table");
-        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[9]), a[11], (int)integer(a[12]), size_of(q, 2, "q"), a[14]);
+        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[9]), a[11], (int)integer(a[12]), a[14]);
         arb_ctx *h = context(a[0]);
         void *qp = dev(q, "q", kBf16), *k = dev(kp, "k_codes", kU8), *v = dev(a[3], "v_codes", kU8), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[7], "seq_lens", kI32), *ql = dev(a[8], "q_lens", kI32), *out = dev(a[10], "out", kBf16);
         const float ks = real(a[4]), vs = real(a[5]);
         arb_stream_t s = stream_of(a[13]);
-        auto call = integer(a[15]) ? lib.arb_attn_decode_e4m3 : lib.arb_attn_e4m3;
+        auto call = (int)integer(a[15]) ? lib.arb_attn_decode_e4m3 : lib.arb_attn_e4m3;
         return without_gil([&] { return call(h, &p, qp, U8(k), U8(v), ks, vs, I32(t), I32(sl), I32(ql), out, s); });
     });
 }
@@ -318,7 +334,7 @@ METHOD(attn_e4m3) {
 // (h, hidden, w, b, tau, scores, decisions, stream)
 METHOD(route) {
     return guarded(n, 8, [&] {
-        const at::Tensor &x = tensor(a[1], "hidden");
+        const at::Tensor &x = of_rank(tensor(a[1], "hidden"), 2, "hidden");
         const int dt = dtype_code(x), steps = size_of(x, 0, "hidden"), dim = size_of(x, 1, "hidden");
         arb_ctx *h = context(a[0]);
         void *hp = dev(x, "hidden"), *w = dev(a[2], "w", x.scalar_type());
@@ -332,7 +348,7 @@ METHOD(route) {
 // (h, mode, hidden, w, biases (tuple of floats), tau, probs, scores, decisions, stream)
 METHOD(route_classes) {
     return guarded(n, 10, [&] {
-        const at::Tensor &x = tensor(a[2], "hidden");
+        const at::Tensor &x = of_rank(tensor(a[2], "hidden"), 2, "hidden");
         const int dt = dtype_code(x), steps = size_of(x, 0, "hidden"), dim = size_of(x, 1, "hidden"), mode = (int)integer(a[1]);
         if (!PyTuple_Check(a[4])) fail(PyExc_TypeError, "%s", "b must be a tuple of floats");
         const int classes = (int)PyTuple_GET_SIZE(a[4]);
