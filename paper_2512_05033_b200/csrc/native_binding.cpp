@@ -87,14 +87,34 @@ const at::Tensor &of_rank(const at::Tensor &t, int rank, const char *name) {
     return t;
 }
 
-long integer(PyObject *o) {
-    const long v = PyLong_AsLong(o);
-    if (v == -1 && PyErr_Occurred()) throw Raised();
-    return v;
+// a number, taken as a C field takes it
+int integer(PyObject *o) {
+    if (PyFloat_Check(o)) fail(PyExc_TypeError, "%s", "int expected instead of float");
+    const unsigned long v = PyLong_AsUnsignedLongMask(o);
+    if (v == (unsigned long)-1 && PyErr_Occurred()) throw Raised();
+    return (int)v;
 }
 float real(PyObject *o) {
     const double v = PyFloat_AsDouble(o);
     if (v == -1.0 && PyErr_Occurred()) throw Raised();
+    return (float)v;
+}
+// ... and as int() and float() take it
+int to_int(PyObject *o) {
+    if (PyLong_Check(o)) return integer(o);
+    PyObject *n = PyNumber_Long(o);
+    if (n == nullptr) throw Raised();
+    const unsigned long v = PyLong_AsUnsignedLongMask(n);
+    Py_DECREF(n);
+    if (v == (unsigned long)-1 && PyErr_Occurred()) throw Raised();
+    return (int)v;
+}
+float to_float(PyObject *o) {
+    if (PyFloat_Check(o)) return real(o);
+    PyObject *n = PyNumber_Float(o);
+    if (n == nullptr) throw Raised();
+    const double v = PyFloat_AS_DOUBLE(n);
+    Py_DECREF(n);
     return (float)v;
 }
 template <typename T>
@@ -188,7 +208,7 @@ constexpr auto kBf16 = at::kBFloat16;
 METHOD(attn) {
     return guarded(n, 12, [&] {
         const at::Tensor &q = tensor(a[1], "q"), &kp = tensor(a[2], "k_pages"), &bt = tensor(a[4], "block_table");
-        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[7]), a[9], 0, a[11]);
+        const arb_attn_params p = params_for(q, kp, bt, integer(a[7]), a[9], 0, a[11]);
         arb_ctx *h = context(a[0]);
         void *qp = dev(q, "q"), *k = dev(kp, "k_pages", q.scalar_type()), *v = dev(a[3], "v_pages", q.scalar_type());
         void *t = dev(bt, "block_table", kI32), *sl = dev(a[5], "seq_lens", kI32), *ql = dev(a[6], "q_lens", kI32);
@@ -203,11 +223,11 @@ METHOD(attn_host) {
     return guarded(n, 13, [&] {
         const at::Tensor &q = tensor(a[1], "q_host"), &kp = tensor(a[2], "k_pages"), &bt = tensor(a[4], "block_table_host");
         void *qp = host(q), *t = host(bt), *sl = host(a[5]), *ql = host(a[6]), *out = host(a[8]);
-        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[7]), a[9], (int)integer(a[10]), Py_None);
+        const arb_attn_params p = params_for(q, kp, bt, integer(a[7]), a[9], integer(a[10]), Py_None);
         arb_ctx *h = context(a[0]);
         void *k = dev(kp, "k_pages"), *v = dev(tensor(a[3], "v_pages"), "v_pages");
         arb_stream_t s = stream_of(a[11]);
-        auto call = (int)integer(a[12]) ? lib.arb_attn_host_begin : lib.arb_attn_host;
+        auto call = integer(a[12]) ? lib.arb_attn_host_begin : lib.arb_attn_host;
         return without_gil([&] { return call(h, &p, qp, k, v, I32(t), I32(sl), I32(ql), out, s); });
     });
 }
@@ -244,7 +264,7 @@ METHOD(decode_step_e4m3) {
         void *qp = dev(q, "q", kBf16), *kn = dev(a[2], "k_new", kBf16), *vn = dev(a[3], "v_new", kBf16);
         void *k = dev(kp, "k_codes", kU8), *v = dev(a[5], "v_codes", kU8), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[11], "seq_lens", kI32), *ql = dev(a[12], "q_lens", kI32), *out = dev(a[13], "out", kBf16);
-        const float ks = real(a[6]), vs = real(a[7]), ki = real(a[8]), vi = real(a[9]);
+        const float ks = to_float(a[6]), vs = to_float(a[7]), ki = to_float(a[8]), vi = to_float(a[9]);
         arb_stream_t s = stream_of(a[15]);
         return without_gil([&] {
             return lib.arb_decode_step_e4m3(h, &p, qp, kn, vn, U8(k), U8(v), ks, vs, ki, vi, I32(t), I32(sl), I32(ql), out, s);
@@ -278,7 +298,7 @@ METHOD(kv_append) {
         arb_ctx *h = context(a[0]);
         void *k = dev(kn, "k_new", dt), *v = dev(a[2], "v_new", dt), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[4], "seq_lens", kI32), *nl = dev(a[5], "new_lens", kI32), *ko = dev(kp, "k_pages"), *vo = dev(a[7], "v_pages", dt);
-        const int total = size_of(kn, 0, "k_new"), update = (int)integer(a[8]);
+        const int total = size_of(kn, 0, "k_new"), update = integer(a[8]);
         arb_stream_t s = stream_of(a[9]);
         return without_gil([&] { return lib.arb_kv_append(h, &p, total, k, v, I32(t), I32(sl), I32(nl), update, ko, vo, s); });
     });
@@ -292,8 +312,8 @@ METHOD(kv_append_e4m3) {
         arb_ctx *h = context(a[0]);
         void *k = dev(kn, "k_new"), *v = dev(a[2], "v_new", kn.scalar_type()), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[6], "seq_lens", kI32), *nl = dev(a[7], "new_lens", kI32), *ko = dev(kp, "k_codes", kU8), *vo = dev(a[9], "v_codes", kU8);
-        const float ki = real(a[3]), vi = real(a[4]);
-        const int total = size_of(kn, 0, "k_new"), update = (int)integer(a[10]);
+        const float ki = to_float(a[3]), vi = to_float(a[4]);
+        const int total = size_of(kn, 0, "k_new"), update = integer(a[10]);
         arb_stream_t s = stream_of(a[11]);
         return without_gil([&] { return lib.arb_kv_append_e4m3(h, &p, total, k, v, ki, vi, I32(t), I32(sl), I32(nl), update, U8(ko), U8(vo), s); });
     });
@@ -308,7 +328,7 @@ METHOD(kv_append_i4) {
         void *k = dev(kn, "k_new", kBf16), *v = dev(a[2], "v_new", kBf16), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[4], "seq_lens", kI32), *nl = dev(a[5], "new_lens", kI32), *ko = dev(kp, "k_codes", kU8), *vo = dev(a[7], "v_codes", kU8);
         void *ks = dev(a[8], "k_scales", at::kFloat), *vs = dev(a[9], "v_scales", at::kFloat);
-        const int total = size_of(kn, 0, "k_new"), update = (int)integer(a[10]);
+        const int total = size_of(kn, 0, "k_new"), update = integer(a[10]);
         arb_stream_t s = stream_of(a[11]);
         return without_gil([&] {
             return lib.arb_kv_append_i4(h, &p, total, k, v, I32(t), I32(sl), I32(nl), update, U8(ko), U8(vo), F32(ks), F32(vs), s);
@@ -320,13 +340,13 @@ METHOD(kv_append_i4) {
 METHOD(attn_e4m3) {
     return guarded(n, 16, [&] {
         const at::Tensor &q = tensor(a[1], "q"), &kp = tensor(a[2], "k_codes"), &bt = tensor(a[6], "block_table");
-        const arb_attn_params p = params_for(q, kp, bt, (int)integer(a[9]), a[11], (int)integer(a[12]), a[14]);
+        const arb_attn_params p = params_for(q, kp, bt, integer(a[9]), a[11], integer(a[12]), a[14]);
         arb_ctx *h = context(a[0]);
         void *qp = dev(q, "q", kBf16), *k = dev(kp, "k_codes", kU8), *v = dev(a[3], "v_codes", kU8), *t = dev(bt, "block_table", kI32);
         void *sl = dev(a[7], "seq_lens", kI32), *ql = dev(a[8], "q_lens", kI32), *out = dev(a[10], "out", kBf16);
-        const float ks = real(a[4]), vs = real(a[5]);
+        const float ks = to_float(a[4]), vs = to_float(a[5]);
         arb_stream_t s = stream_of(a[13]);
-        auto call = (int)integer(a[15]) ? lib.arb_attn_decode_e4m3 : lib.arb_attn_e4m3;
+        auto call = integer(a[15]) ? lib.arb_attn_decode_e4m3 : lib.arb_attn_e4m3;
         return without_gil([&] { return call(h, &p, qp, U8(k), U8(v), ks, vs, I32(t), I32(sl), I32(ql), out, s); });
     });
 }
@@ -339,7 +359,7 @@ METHOD(route) {
         arb_ctx *h = context(a[0]);
         void *hp = dev(x, "hidden"), *w = dev(a[2], "w", x.scalar_type());
         void *sc = dev(a[5], "scores", at::kFloat), *de = dev(a[6], "decisions", kU8);
-        const float b = real(a[3]), tau = real(a[4]);
+        const float b = to_float(a[3]), tau = to_float(a[4]);
         arb_stream_t s = stream_of(a[7]);
         return without_gil([&] { return lib.arb_route(h, dt, steps, dim, hp, w, b, tau, F32(sc), U8(de), s); });
     });
@@ -349,7 +369,7 @@ METHOD(route) {
 METHOD(route_classes) {
     return guarded(n, 10, [&] {
         const at::Tensor &x = of_rank(tensor(a[2], "hidden"), 2, "hidden");
-        const int dt = dtype_code(x), steps = size_of(x, 0, "hidden"), dim = size_of(x, 1, "hidden"), mode = (int)integer(a[1]);
+        const int dt = dtype_code(x), steps = size_of(x, 0, "hidden"), dim = size_of(x, 1, "hidden"), mode = integer(a[1]);
         if (!PyTuple_Check(a[4])) fail(PyExc_TypeError, "%s", "b must be a tuple of floats");
         const int classes = (int)PyTuple_GET_SIZE(a[4]);
         float bias[ARB_MAX_CLASSES] = {};
@@ -357,7 +377,7 @@ METHOD(route_classes) {
         arb_ctx *h = context(a[0]);
         void *hp = dev(x, "hidden"), *w = dev(a[3], "w", x.scalar_type()), *pr = dev(a[6], "probs", at::kFloat);
         void *sc = dev(a[7], "scores", at::kFloat), *de = dev(a[8], "decisions", kU8);
-        const float tau = real(a[5]);
+        const float tau = to_float(a[5]);
         arb_stream_t s = stream_of(a[9]);
         return without_gil([&] {
             return lib.arb_route_classes(h, dt, mode, steps, dim, classes, hp, w, bias, tau, F32(pr), F32(sc), U8(de), s);
@@ -381,7 +401,7 @@ METHOD(rollback) {
 METHOD(phase_lens) {
     return guarded(n, 8, [&] {
         const at::Tensor &st = tensor(a[1], "step_lens");
-        const int batch = size_of(st, 0, "step_lens"), want = (int)integer(a[3]), t = (int)integer(a[4]), tokens = (int)integer(a[5]);
+        const int batch = size_of(st, 0, "step_lens"), want = to_int(a[3]), t = to_int(a[4]), tokens = to_int(a[5]);
         arb_ctx *h = context(a[0]);
         void *l = dev(st, "step_lens", kI32), *de = dev_or_null(a[2], "decisions", kU8), *out = dev(a[6], "out", kI32);
         arb_stream_t s = stream_of(a[7]);
@@ -396,11 +416,11 @@ METHOD(phase_lens) {
 METHOD(policy) {
     return guarded(n, 9, [&] {
         const at::Tensor &sd = tensor(a[2], "s_d");
-        const int kind = (int)integer(a[1]), steps = size_of(sd, 0, "s_d"), budget = (int)integer(a[5]);
+        const int kind = integer(a[1]), steps = size_of(sd, 0, "s_d"), budget = to_int(a[5]);
         arb_ctx *h = context(a[0]);
         void *d = dev(sd, "s_d", at::kFloat), *t = dev_or_null(a[3], "s_t", at::kFloat), *de = dev(a[6], "decisions", kU8);
         void *st = dev_or_null(a[7], "stats", at::kDouble);
-        const float tau = real(a[4]);
+        const float tau = to_float(a[4]);
         arb_stream_t s = stream_of(a[8]);
         return without_gil([&] {
             return lib.arb_policy(h, kind, steps, F32(d), F32(t), tau, budget, U8(de), static_cast<arb_policy_stats *>(st), s);

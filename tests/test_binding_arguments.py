@@ -73,3 +73,16 @@ def test_a_record_of_parameters_leaves_the_shapes_to_the_caller():
         c.attn(_t(B, HQ * D), pool, pool, table, lens, lens, 1, params=p)
     with pytest.raises(ValueError, match=RIGHT):
         c.decode_step(_t(B, HQ * D), _t(B, HKV * D), _t(B, HKV * D), pool, pool, table, lens, lens, params=p)
+
+
+def test_numbers_are_taken_as_int_and_float_take_them():
+    c, binding = _context()
+    scores, lens = _t(4, dtype=F32), _t(B, dtype=I32)
+    with pytest.raises(ValueError, match=RIGHT):
+        c.policy(binding.POLICY_ORACLE_BUDGET, scores, scores, tau=torch.tensor(0.5), budget=2.0)
+    with pytest.raises(ValueError, match=RIGHT):
+        c.phase_lens(lens, want=1.0, t=0.0)
+    with pytest.raises(ValueError, match=RIGHT):
+        c.phase_lens_tokens(lens, 3, want=True)
+    with pytest.raises(TypeError):
+        c.attn(_t(B, HQ, D), _t(PAGES, HKV, P, D), _t(PAGES, HKV, P, D), _t(B, 3, dtype=I32), lens, lens, 1.0)
