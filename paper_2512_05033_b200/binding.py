@@ -379,7 +379,7 @@ class Context:
         """out int32 [B]: lengths of the next call of a phase of the step loop (see arb_phase_lens)."""
         if out is None:
             out = torch.empty_like(step_lens)
-        st = _native.phase_lens(self._p, step_lens, decisions, want, t, -1, out, stream)
+        st = _native.phase_lens(self._p, step_lens, decisions, want, t, out, stream)
         if st:
             _check(st, "arb_phase_lens")
         return out
@@ -388,7 +388,7 @@ class Context:
         """out int32 [n_tokens, B]: row t = phase_lens(..., t=t), all rows in one launch."""
         if out is None:
             out = torch.empty(n_tokens, step_lens.shape[0], dtype=torch.int32, device=step_lens.device)
-        st = _native.phase_lens(self._p, step_lens, decisions, want, -1, n_tokens, out, stream)
+        st = _native.phase_lens_tokens(self._p, step_lens, decisions, want, n_tokens, out, stream)
         if st:
             _check(st, "arb_phase_lens_tokens")
         return out

@@ -397,18 +397,27 @@ METHOD(rollback) {
     });
 }
 
-// (h, step_lens, decisions, want, t, n_tokens, out, stream): n_tokens < 0: one row for token t; else a row per token
+// (h, step_lens, decisions, want, t, out, stream)
 METHOD(phase_lens) {
-    return guarded(n, 8, [&] {
+    return guarded(n, 7, [&] {
         const at::Tensor &st = tensor(a[1], "step_lens");
-        const int batch = size_of(st, 0, "step_lens"), want = to_int(a[3]), t = to_int(a[4]), tokens = to_int(a[5]);
+        const int batch = size_of(st, 0, "step_lens"), want = to_int(a[3]), t = to_int(a[4]);
         arb_ctx *h = context(a[0]);
-        void *l = dev(st, "step_lens", kI32), *de = dev_or_null(a[2], "decisions", kU8), *out = dev(a[6], "out", kI32);
-        arb_stream_t s = stream_of(a[7]);
-        return without_gil([&] {
-            return tokens < 0 ? lib.arb_phase_lens(h, batch, I32(l), U8(de), want, t, I32(out), s)
-                              : lib.arb_phase_lens_tokens(h, batch, I32(l), U8(de), want, tokens, I32(out), s);
-        });
+        void *l = dev(st, "step_lens", kI32), *de = dev_or_null(a[2], "decisions", kU8), *out = dev(a[5], "out", kI32);
+        arb_stream_t s = stream_of(a[6]);
+        return without_gil([&] { return lib.arb_phase_lens(h, batch, I32(l), U8(de), want, t, I32(out), s); });
+    });
+}
+
+// (h, step_lens, decisions, want, n_tokens, out, stream)
+METHOD(phase_lens_tokens) {
+    return guarded(n, 7, [&] {
+        const at::Tensor &st = tensor(a[1], "step_lens");
+        const int batch = size_of(st, 0, "step_lens"), want = to_int(a[3]), tokens = to_int(a[4]);
+        arb_ctx *h = context(a[0]);
+        void *l = dev(st, "step_lens", kI32), *de = dev_or_null(a[2], "decisions", kU8), *out = dev(a[5], "out", kI32);
+        arb_stream_t s = stream_of(a[6]);
+        return without_gil([&] { return lib.arb_phase_lens_tokens(h, batch, I32(l), U8(de), want, tokens, I32(out), s); });
     });
 }
 
@@ -465,7 +474,7 @@ PyMethodDef methods[] = {
     {"bind", bind, METH_O, nullptr},
     ENTRY(attn), ENTRY(attn_host), ENTRY(attn_host_wait), ENTRY(decode_step), ENTRY(decode_step_e4m3), ENTRY(decode_step_i4),
     ENTRY(kv_append), ENTRY(kv_append_e4m3), ENTRY(kv_append_i4), ENTRY(attn_e4m3), ENTRY(route), ENTRY(route_classes),
-    ENTRY(rollback), ENTRY(phase_lens), ENTRY(policy), ENTRY(spearman),
+    ENTRY(rollback), ENTRY(phase_lens), ENTRY(phase_lens_tokens), ENTRY(policy), ENTRY(spearman),
     {nullptr, nullptr, 0, nullptr},
 };
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -86,3 +86,13 @@ def test_numbers_are_taken_as_int_and_float_take_them():
         c.phase_lens_tokens(lens, 3, want=True)
     with pytest.raises(TypeError):
         c.attn(_t(B, HQ, D), _t(PAGES, HKV, P, D), _t(PAGES, HKV, P, D), _t(B, 3, dtype=I32), lens, lens, 1.0)
+
+
+@pytest.mark.gpu
+def test_a_negative_number_of_tokens_is_refused():
+    from tests import helpers as H
+    from paper_2512_05033_b200 import binding
+    lens, out = torch.full((B,), 3, dtype=I32, device="cuda"), torch.full((B,), 77, dtype=I32, device="cuda")
+    with pytest.raises(binding.ArbError):
+        H.ctx().phase_lens_tokens(lens, -1, out=out)
+    assert H.ctx().poll_status() == 0 and bool((out == 77).all())
