@@ -291,7 +291,8 @@ arb_status arb_rollback(arb_ctx *ctx, int32_t batch, int32_t *seq_lens, const in
  *   decisions  uint8 [n_steps]: 1 = escalate to the target, 0 = keep the draft step.  Ties: RSD escalates
  *              at s_d == tau; the oracle rules keep the draft at Delta == tau / s_t == s_d; among equal
  *              advantages the budgeted rule takes the lower index first.
- *   stats      nullable; overwritten by the kernel (sums in fp64).
+ *   stats      nullable; overwritten by the kernel (sums in fp64).  Calls with stats use an arrival counter and records in
+ *              the ctx: one at a time per ctx, as every call.
  * Delta and every comparison are taken in fp32 (IEEE subtraction, no flush to zero).
  * Errors: ARB_ERR_INVALID_ARG (null pointer, unknown kind, s_t missing), ARB_ERR_UNSUPPORTED (budgeted
  * rule beyond 65536 steps).
@@ -498,10 +499,10 @@ arb_status arb_kv_append_i4(arb_ctx *ctx, const arb_attn_params *params, int32_t
  * replaced by its rank within its sample, equal values sharing the mean of the ranks they span, and
  * rho is the Pearson correlation of the two rank variables.
  *
- *   x, y   fp32 [n], finite;  n <= 65536 (ranks are found by counting, n^2 comparisons).
+ *   x, y   fp32 [n], finite;  n <= 65536 (what one cluster of eight CTAs sorts on chip).
  *   rho    DEVICE pointer to one double (8-byte aligned): the result, NaN when n < 2 or a sample is
- *          constant.  Sums are taken in fp64.
- * Uses three accumulators in the ctx: one call at a time per ctx.
+ *          constant.  Sums are exact, in 64-bit integers.
+ * Uses an arrival counter and two vectors of ranks in the ctx: one call at a time per ctx.
  */
 arb_status arb_spearman(arb_ctx *ctx, int32_t n, const float *x, const float *y, double *rho, arb_stream_t stream);
 
@@ -530,8 +531,8 @@ arb_status arb_phase_lens_tokens(arb_ctx *ctx, int32_t batch, const int32_t *ste
                                  arb_stream_t stream);
 
 /*
- * Synchronise `stream`, read the device status word into *bits (nullable) and clear it together
- * with the split-KV arrival counters.  Returns ARB_OK if the word was zero, else
+ * Synchronise `stream`, read the device status word into *bits (nullable) and, if it is not zero, clear it together
+ * with every arrival counter of the ctx.  Returns ARB_OK if the word was zero, else
  * ARB_ERR_DEVICE_STATUS.
  */
 arb_status arb_poll_status(arb_ctx *ctx, arb_stream_t stream, uint32_t *bits);

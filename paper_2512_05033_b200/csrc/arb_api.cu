@@ -163,7 +163,7 @@ arb_status arb_create(arb_ctx **out, int device, size_t workspace_bytes) {
     ok = ok && guarded_malloc(c, &c->rot, sizeof(int) * rot_ints);
     ok = ok && cudaMemset(c->rot, 0, sizeof(int) * rot_ints) == cudaSuccess;
     ok = ok && guarded_malloc(c, &c->rank_ws, rank_ws_bytes());
-    ok = ok && cudaMemset(c->rank_ws, 0, 256) == cudaSuccess;
+    ok = ok && cudaMemset(c->rank_ws, 0, kRankCounterBytes) == cudaSuccess;
     c->chunk_ws_bytes = 2 * c->workspace_bytes;   // partials of long step chunks that are split over their keys
     ok = ok && guarded_malloc(c, &c->chunk_ws, c->chunk_ws_bytes);
     ok = ok && guarded_malloc(c, &c->step_hint, decode_step_hint_bytes(sms));
@@ -749,6 +749,7 @@ arb_status arb_poll_status(arb_ctx *ctx, arb_stream_t stream, uint32_t *bits) {
     if (host != 0) {  // a kernel that gave up may have left arrival counters behind (the word between the two is the generation)
         if (cudaMemsetAsync(c->rot + (size_t)kRotSets * kRotCounters + kRotSets + 1, 0, sizeof(int) * 7, s) != cudaSuccess) return ARB_ERR_CUDA;
         if (cudaMemsetAsync(c->counters, 0, sizeof(int) * (c->counters_len + 4), s) != cudaSuccess) return ARB_ERR_CUDA;
+        if (cudaMemsetAsync(c->rank_ws, 0, kRankCounterBytes, s) != cudaSuccess) return ARB_ERR_CUDA;
         if (cudaMemsetAsync(c->rot, 0, sizeof(int) * ((size_t)kRotSets * kRotCounters + kRotSets), s) != cudaSuccess)
             return ARB_ERR_CUDA;
         if (cudaStreamSynchronize(s) != cudaSuccess) return ARB_ERR_CUDA;
@@ -787,6 +788,16 @@ int arb_debug_poke_guard(arb_ctx *ctx, int nbytes) {
     if (ctx == nullptr || nbytes < 1 || (size_t)nbytes > kGuardBytes) return 1;
     Ctx *c = reinterpret_cast<Ctx *>(ctx);
     return cudaMemset(c->workspace - nbytes, 0, (size_t)nbytes) == cudaSuccess ? 0 : 1;
+}
+
+// ... and for the test of what arb_poll_status clears: leaves the arrival counters of arb_policy and arb_spearman, and a
+// status bit, as calls that were mixed up would.
+int arb_debug_poke_rank_counters(arb_ctx *ctx) {
+    if (ctx == nullptr) return 1;
+    Ctx *c = reinterpret_cast<Ctx *>(ctx);
+    const uint32_t bit = ARB_DEV_CHECK_FAILED;
+    return cudaMemset(c->rank_ws, 1, 2 * sizeof(int)) == cudaSuccess &&
+                   cudaMemcpy(c->status, &bit, sizeof(bit), cudaMemcpyHostToDevice) == cudaSuccess ? 0 : 1;
 }
 #endif
 

@@ -57,8 +57,8 @@ struct Ctx {
     int *rot = nullptr;
     uint32_t decode_gen = 1000;          // generation of the next tensor-core decode call
     uint32_t rot_wait_through = 0;        // tensor-core decode calls up to this generation wait for their predecessor
-    char *rank_ws = nullptr;              // arb_policy, arb_spearman: two arrival counters (zero between calls), then at 256 the
-                                          // statistics of a policy's CTAs and the ranks of two samples
+    char *rank_ws = nullptr;              // arb_policy, arb_spearman: two arrival counters (zero between calls), then at
+                                          // kRankCounterBytes the statistics of a policy's CTAs and the ranks of two samples
     int *step_hint = nullptr;             // single-launch decode: the page tiles each CTA streamed last (arb_decode_step.cu)
     int step_min_chunk = 16;              // single-launch decode: fewest pages worth giving a CTA
     int step_boundary_pct = 100;          // single-launch decode: what a (sequence, kv head) boundary inside a CTA's range counts for
@@ -72,6 +72,7 @@ struct Ctx {
     unsigned long long *guard_bad = nullptr;
 };
 
+constexpr size_t kRankCounterBytes = 256;
 constexpr size_t kPolicyPartBytes = 8192;   // of rank_ws: the statistics of a policy's CTAs
 
 constexpr int kRotSets = 4;

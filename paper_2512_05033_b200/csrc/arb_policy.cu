@@ -208,7 +208,7 @@ arb_status launch_policy(Ctx *ctx, int kind, int n_steps, const float *s_d, cons
     const int need = (n_steps + kPolicyThreads - 1) / kPolicyThreads;
     const int grid = need < kPolicyMaxCtas ? need : kPolicyMaxCtas;
     policy_kernel<<<grid, kPolicyThreads, 0, stream>>>(kind, n_steps, s_d, s_t, tau, decisions, stats,
-                                                       reinterpret_cast<arb_policy_stats *>(ctx->rank_ws + 256),
+                                                       reinterpret_cast<arb_policy_stats *>(ctx->rank_ws + kRankCounterBytes),
                                                        reinterpret_cast<int *>(ctx->rank_ws) + 1);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? ARB_OK : ARB_ERR_CUDA;

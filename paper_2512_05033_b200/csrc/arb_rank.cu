@@ -422,7 +422,7 @@ policy_budget_kernel(int n, int lg, const float *__restrict__ s_d, const float *
 
 }  // namespace
 
-size_t rank_ws_bytes() { return 256 + kPolicyPartBytes + sizeof(uint32_t) * 2 * kCtas * kMaxPerCta; }
+size_t rank_ws_bytes() { return kRankCounterBytes + kPolicyPartBytes + sizeof(uint32_t) * 2 * kCtas * kMaxPerCta; }
 
 arb_status launch_spearman(Ctx *ctx, int n, const float *x, const float *y, double *rho, cudaStream_t stream) {
     static bool attr_set[64] = {};
@@ -432,7 +432,7 @@ arb_status launch_spearman(Ctx *ctx, int n, const float *x, const float *y, doub
         attr_set[ctx->device & 63] = true;
     }
     spearman_kernel<<<2 * kCtas, kThreads, sizeof(SortSmem), stream>>>(
-        n, log_per_cta(n), x, y, reinterpret_cast<uint32_t *>(ctx->rank_ws + 256 + kPolicyPartBytes), reinterpret_cast<int *>(ctx->rank_ws), rho);
+        n, log_per_cta(n), x, y, reinterpret_cast<uint32_t *>(ctx->rank_ws + kRankCounterBytes + kPolicyPartBytes), reinterpret_cast<int *>(ctx->rank_ws), rho);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? ARB_OK : ARB_ERR_CUDA;
 }

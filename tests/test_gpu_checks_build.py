@@ -51,3 +51,30 @@ def test_a_planted_overrun_is_seen_by_the_guard_check():
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, ARB_LIB_VARIANT="checks"),
                        capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "planted overrun seen" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+def test_poll_status_clears_the_counters_of_the_rank_kernels():
+    """Arrival counters that were left non-zero (here by an entry point of the bounds-check build) are zero again after a poll
+    that found a status bit: statistics and rho come out right."""
+    from paper_2512_05033_b200 import build
+    build.build(checks=True)
+    code = (
+        "import ctypes, torch\n"
+        "from paper_2512_05033_b200 import binding\n"
+        "from oracle import oracle\n"
+        "c = binding.Context(0)\n"
+        "poke = binding.lib.arb_debug_poke_rank_counters\n"
+        "poke.restype = ctypes.c_int; poke.argtypes = [ctypes.c_void_p]\n"
+        "assert poke(c._h) == 0 and c.poll_status() == binding.DEV_CHECK_FAILED\n"
+        "g = torch.Generator().manual_seed(3)\n"
+        "x, y = torch.rand(3000, generator=g), torch.rand(3000, generator=g)\n"
+        "for _ in range(3):\n"
+        "    stats, rho = c.new_policy_stats('cuda'), torch.full((1,), 9.0, dtype=torch.float64, device='cuda')\n"
+        "    c.policy(binding.POLICY_ORACLE_ARGMAX, x.cuda(), y.cuda(), stats=stats)\n"
+        "    c.spearman(x.cuda(), y.cuda(), rho=rho)\n"
+        "    assert c.policy_stats(stats)['escalated'] == int((y > x).sum())\n"
+        "    assert abs(rho.item() - oracle.spearman(x, y)) < 1e-12\n"
+        "print('counters cleared')\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, ARB_LIB_VARIANT="checks"),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "counters cleared" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
