@@ -75,10 +75,12 @@ namespace {
 // Decode rows over an E4M3 cache: a call of a back-to-back series takes the two-kernel form, a call on its own the single
 // launch: a target-shaped call 112 -> 104 us, a draft-shaped one 18.9 -> 10.5 us, two sequences of 300 to 500 tokens 11.2 ->
 // 6.6 us, and one launch instead of two in front of the chunks of a mixed one.
+bool e4m3_single_launch(const arb_attn_params &p) { return (p.flags & ARB_ATTN_OVERLAP_PREVIOUS) == 0 && decode_step_supported(p); }
+
 arb_status decode_e4m3(Ctx *c, const arb_attn_params &p, const void *q, const uint8_t *k_codes, const uint8_t *v_codes, float k_scale,
                        float v_scale, const int32_t *block_table, const int32_t *seq_lens, const int32_t *q_lens, void *out,
                        bool beside, cudaStream_t s) {
-    if ((p.flags & ARB_ATTN_OVERLAP_PREVIOUS) || !decode_step_supported(p))
+    if (!e4m3_single_launch(p))
         return launch_decode_e4m3(c, p, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, s);
     const float scales[4] = {k_scale, v_scale, 1.0f, 1.0f};
     return launch_decode_step(c, p, q, nullptr, nullptr, const_cast<uint8_t *>(k_codes), const_cast<uint8_t *>(v_codes), scales,
@@ -687,7 +689,8 @@ arb_status arb_attn_e4m3(arb_ctx *ctx, const arb_attn_params *params, const void
     if (decode_workspace_bytes(*params, c->num_sms) > c->workspace_bytes) return ARB_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const bool maybe_decode = params->max_q_len == 1 || params->total_q > params->max_q_len;
-    const bool beside = maybe_decode && params->max_q_len >= 2 && (params->flags & ARB_ATTN_OVERLAP_PREVIOUS) == 0;
+    // (side by side with the single launch only: the two-kernel form lets its successor start before what precedes it is done)
+    const bool beside = maybe_decode && params->max_q_len >= 2 && e4m3_single_launch(*params);
     if (maybe_decode) {
         st = decode_e4m3(c, *params, q, k_codes, v_codes, k_scale, v_scale, block_table, seq_lens, q_lens, out, beside, s);
         if (st != ARB_OK) return st;

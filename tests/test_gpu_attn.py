@@ -720,6 +720,23 @@ def test_decode_rows_beside_chunks_match_oracle(case):
         H.assert_close(got.double().cpu().numpy(), ref, BF, tight=3e-3)
 
 
+@pytest.mark.parametrize("case", BESIDE_CASES[:3])
+def test_e4m3_decode_rows_beside_chunks_match_oracle(case):
+    Hq, Hkv, D, sl, ql = case
+    inp = wl.small_attn_case(len(sl), Hq, Hkv, D, BF, sl, ql, seed=720 + Hq)
+    kc, vc = (torch.from_numpy(oracle.e4m3_encode(p, 1 / 0.0125)) for p in (inp.k_pages, inp.v_pages))
+    ref, st = oracle.attn_e4m3(inp.q, kc, vc, 0.0125, 0.0125, inp.block_table, inp.seq_lens, inp.q_lens)
+    d, c, dk, dv = inp.to("cuda"), H.ctx(), kc.cuda(), vc.cuda()
+    out, copies = torch.empty_like(d.q), []
+    for _ in range(4):
+        out.fill_(float("nan"))
+        c.attn_e4m3(d.q, dk, dv, 0.0125, 0.0125, d.block_table, d.seq_lens, d.q_lens, max(ql), out=out)
+        copies.append(out.clone())
+    assert c.poll_status() == 0 and st == 0
+    for got in copies:
+        H.assert_close(got.double().cpu().numpy(), ref, BF, tight=3e-3)
+
+
 LONE_CASES = [
     # (Hq, Hkv, seq_lens, q_lens): row tiles in threes (a lone one before its sequence's pair), and lone row tiles over a
     # single key tile one behind the other
