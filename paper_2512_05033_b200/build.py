@@ -10,6 +10,7 @@ ARB_LIB_VARIANT=checks is set; it is for test runs, not for timing.
 from __future__ import annotations
 
 import concurrent.futures
+import importlib.metadata
 import importlib.util
 import os
 import subprocess
@@ -67,9 +68,21 @@ def build(force: bool = False, verbose: bool = False, checks: bool = False) -> P
     return LIB
 
 
+def _native_abi() -> str:
+    """What an extension module is good for: this interpreter and this torch."""
+    return f"python {sys.version}\ntorch {importlib.metadata.version('torch')}\n"
+
+
+def native_stale() -> bool:
+    stamp = OBJ / "native_abi.txt"   # what the module there was built for
+    if not stamp.exists() or stamp.read_text() != _native_abi():
+        return True
+    return _stale(HERE / "_native.so", [CSRC / "native_binding.cpp", HERE.parent / "include" / "arb.h", Path(__file__)])
+
+
 def build_native(force: bool = False) -> Path:
     src, out = CSRC / "native_binding.cpp", HERE / "_native.so"
-    if force or _stale(out, [src, HERE.parent / "include" / "arb.h"]):
+    if force or native_stale():
         torch_dir = Path(importlib.util.find_spec("torch").origin).parent   # not imported: only its headers and libraries
         inc, lib = torch_dir / "include", torch_dir / "lib"
         tmp = out.with_suffix(f".tmp{os.getpid()}.so")
@@ -78,6 +91,8 @@ def build_native(force: bool = False) -> Path:
                                f"-I{Path(NVCC).parent.parent / 'include'}", str(src), "-o", str(tmp), f"-L{lib}",
                                "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
         os.replace(tmp, out)
+        OBJ.mkdir(exist_ok=True)
+        (OBJ / "native_abi.txt").write_text(_native_abi())
     return out
 
 

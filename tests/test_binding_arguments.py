@@ -88,6 +88,14 @@ def test_numbers_are_taken_as_int_and_float_take_them():
         c.attn(_t(B, HQ, D), _t(PAGES, HKV, P, D), _t(PAGES, HKV, P, D), _t(B, 3, dtype=I32), lens, lens, 1.0)
 
 
+def test_the_extension_module_is_built_again_for_another_interpreter_or_torch(monkeypatch):
+    from paper_2512_05033_b200 import build
+    build.build()
+    assert not build.native_stale()
+    monkeypatch.setattr(build, "_native_abi", lambda: "python 3.99\ntorch 9.9\n")
+    assert build.native_stale()
+
+
 @pytest.mark.gpu
 def test_a_negative_number_of_tokens_is_refused():
     from tests import helpers as H
