@@ -483,8 +483,8 @@ __device__ __forceinline__ int item_div(int a, int b) {
 }
 
 // Item number -> what it is, out of the plan's tables alone (a round trip to global memory here is one per item).  In the
-// E4M3 form sixteen warps hold this code and its values between the tiles of an item, and the plain divisions and the
-// lengths from L1 are the better ones: step-scoring batch over codes 446 -> 443 us, prompts of 32 / 8 heads 283 -> 277 us.
+// E4M3 form, whose sixteen warps all run this while the widening ones fill shared memory's queues, the lengths come from L1
+// instead: step-scoring batch over codes 447 -> 442 us, prompts of 32 / 8 heads 284 -> 278 us, short steps the same.
 template <int G, bool E4M3>
 __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, const MmaArgs &a, Item &it) {
     if (item >= total) return false;
@@ -500,9 +500,9 @@ __device__ __forceinline__ bool get_item(int item, int total, const Plan &pl, co
     it.rows_total = it.n * G;
     const int pairs = pl.pairs[sb], P = pl.parts[lo];
     const int r = item - pl.pref[lo];
-    it.kvh = E4M3 ? r / (pairs * P) : item_div(r, pairs * P);
+    it.kvh = item_div(r, pairs * P);
     const int rem = r - it.kvh * pairs * P;
-    const int later = E4M3 ? rem / P : P > 1 ? item_div(rem, P) : rem, part = rem - later * P;
+    const int later = P > 1 ? item_div(rem, P) : rem, part = rem - later * P;
     const int pt = pairs - 1 - later;   // from the last pair of a sequence, which sees most keys, to the first
     it.r_begin = pt * 2 * kBM;
     it.qrow0 = pl.row0[sb];
