@@ -472,10 +472,10 @@ arb_status arb_attn_host_begin(arb_ctx *ctx, const arb_attn_params *params, cons
     // A call flagged ARB_ATTN_OVERLAP_PREVIOUS whose out_host is page-locked (and so mapped into the device's
     // address space) moves its operands itself: the kernels read the slot's page-locked copy of the inputs over
     // the bus and write the rows of out straight into out_host; no copy is enqueued, only the event that marks
-    // the call complete.  Measured on the draft-shaped batch (34 MB of KV per call): 17 us per call against 24
-    // with the copies below and unflagged kernels.  It pays for flagged calls only: every CTA reads lengths,
-    // block-table entries and q rows over the bus in small requests, and an unflagged small call has twice the
-    // CTAs (41 us per call).
+    // the call complete.  Draft-shaped batch (34 MB of KV per call): 17 or 29 us per call, by host; with the copies
+    // below and the unflagged single launch, 15.7 to 16.8 us on either (24 us while unflagged calls were two kernels,
+    // which is when the rule was made).  It is for flagged calls only: every CTA reads lengths, block-table entries
+    // and q rows over the bus in small requests, and an unflagged small call has twice the CTAs (41 us per call).
     void *mapped_out = nullptr;
     if (!aligned16(out_host) || cudaHostGetDevicePointer(&mapped_out, out_host, 0) != cudaSuccess) {
         cudaGetLastError();   // out_host is ordinary memory

@@ -4,8 +4,8 @@
 //
 // k_new, v_new are [total_new, Hkv, D], packed by sequence; token j of sequence b lands at position
 // seq_lens[b] + j: page block_table[b][pos / 16], slot pos % 16 of the head-major pools
-// [num_pages, Hkv, 16, D].  Plain memory movement: a (token, kv head) row of D elements is 256 or 512
-// contiguous bytes on both sides, copied as 16-byte vectors, one row per half warp or warp, up to four rows of a
+// [num_pages, Hkv, 16, D].  Plain memory movement: a (token, kv head) row of D elements is 128, 256 or 512
+// contiguous bytes on both sides, copied as 16-byte vectors, one row per 8, 16 or 32 lanes, up to four rows of a
 // thread in flight.  Nothing
 // is known on the host but the total number of new tokens; every CTA derives the row offsets from
 // new_lens (scan in shared memory) and checks each sequence once, its pages side by side: new tokens that do not fit under

@@ -37,10 +37,10 @@
 // keys are k_scale * code, values v_scale * code): the chunk a quantised draft's cache absorbs when the target's
 // step replaces its own (Algorithm 1, escalation branch).  The codes widen to f16 exactly, so the products run as
 // f16 MMAs with fp32 accumulation; q is converted bf16 -> f16 as its tile is written, P is rounded to f16.  A page
-// of codes (16 rows x 128 bytes) arrives through one tiled TMA copy in a small staging ring of four pages per
-// operand; the producer warp of the operand widens it (cvt.rn.f16x2.e4m3x2) into the operand stage, in the
-// 128-byte-swizzled layout the bf16 tiles land in, and asks for the page four ahead.  The key scale folds into the
-// softmax scale, the value scale into the epilogue.
+// of codes (16 rows x 128 bytes) arrives through one tiled TMA copy in a staging ring of six pages per operand; three
+// warps per operand take them in pairs, widen them (cvt.rn.f16x2.e4m3x2) into the operand stage, in the 128-byte-swizzled
+// layout the bf16 tiles land in, and ask for the pair three ahead.  The key scale folds into the softmax scale, the value
+// scale into the epilogue.
 #include "arb_tma.cuh"
 
 namespace arb {
@@ -1109,7 +1109,7 @@ chunk_mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap k_map, con
             const int r_first = w.r_begin + (w.rows[1] == 0 ? 0 : grp * kBM), rows_here = w.rows[1] == 0 ? w.rows[0] : w.rows[grp];
             const bool row_ok = E4M3 ? own_ok : tg < rows_here;
             uint4 *dst = reinterpret_cast<uint4 *>(a.out + own * 2);   // E4M3: this thread's row
-            // ---- epilogue: O / l, bf16, one row of the output per thread
+            // ---- epilogue: O / l, bf16: a TMEM lane (a row) per thread; to out by whole rows per warp (E4M3: a row per thread)
             if (my_tiles > 0) mbar_wait(&bars->o_full[grp], (itg - 1u) & 1u, abort, a.status);
             __syncwarp();
             tc_fence_after();

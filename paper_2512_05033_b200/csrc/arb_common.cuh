@@ -241,9 +241,11 @@ __device__ __forceinline__ float fast_exp2(float x) {
 //  - let_successor_start: the next kernel on the stream, if launched as a programmatic dependent, may come up
 //    once every CTA of this grid has passed this point or exited.
 //  - wait_for_predecessor: returns when the preceding kernel has completed and its writes are visible.
-// Every kernel launched through launch_pdl passes wait_for_predecessor on all its paths before it touches global
-// memory (so that its own completion implies that of everything before it on the stream), and calls
-// let_successor_start at its top: a chain of small dependent kernels then pays no launch latency between them.
+// Every kernel launched through launch_pdl passes wait_for_predecessor on all its paths (so that its own completion implies
+// that of everything before it on the stream), and before it touches what an earlier kernel may be writing or reading: a
+// chain of small dependent kernels then pays no launch latency between them.  It calls let_successor_start at its top, with
+// one exception: decode rows beside chunks (arb_decode_step.cu, `beside`) call it behind their own wait, and the chunk kernel
+// behind them, which shares nothing with them, waits at its end only.
 __device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {

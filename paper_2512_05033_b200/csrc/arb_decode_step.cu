@@ -6,18 +6,19 @@
 // launches (append, decode, combine) become one.
 //
 // What is shared with the two-kernel decode (arb_decode_mma.cu): the flat (sequence, kv head, page) list cut
-// into equal ranges per CTA, a producer warp feeding a ring of 4 KB page tiles through tiled TMA copies, one
-// consumer warp per page with its own online softmax.  What differs:
+// into equal ranges per CTA, a ring of 4 KB page tiles fed through tiled TMA copies (here by two producer warps, one for K and
+// one for V), one consumer warp per page with its own online softmax.  What differs:
 //   - The product is transposed.  S^T = K q^T puts the 16 keys of a page on the 16 rows of an m16n8k16 tile and
 //     the group's heads (padded to 8) on its 8 columns; O^T += V^T P^T does the same for the second product.
 //     A page costs 8 + 8 MMAs instead of 16 + 16, the accumulators take 32 registers instead of 64, and the
 //     CTA runs eight consumer warps, two per scheduler, which hide one another's latencies.  P^T reaches the
 //     second product's B fragment through two movmatrix transposes; the row maximum is a reduction over the
 //     lanes that share a column pair (three shuffles).
-//   - The kernel waits for its predecessor at its top (griddepcontrol.wait) and lets its successor come up at
-//     once (griddepcontrol.launch_dependents): launched as a programmatic dependent it is resident, barriers
-//     initialised, when the kernel before it ends.  Nothing is read or written before the wait, so this is
-//     safe behind any kernel.
+//   - The kernel waits for its predecessor near its top (griddepcontrol.wait) and lets its successor come up at
+//     once (griddepcontrol.launch_dependents; beside chunks only behind its own wait): launched as a programmatic dependent
+//     it is resident, barriers initialised, when the kernel before it ends.  Before the wait it reads nothing but the hint
+//     record of the context, which only this kernel writes and whose rows are range-checked and only prefetched, so this
+//     is safe behind any kernel.
 //   - The combine is inside: a CTA that holds a part of a split (sequence, kv head) stores its partial, fences,
 //     and adds one to the item's arrival counter; the CTA that arrives last merges the parts (two round trips
 //     to L2) and writes the rows.  No CTA waits for another.
@@ -87,9 +88,13 @@ constexpr int kHintStride = kHintPages + 4;   // [tag, count, -, -, rows ...]
 // (65 of them 5 TB/s), beside chunks less.  Both kinds of work are known from the lengths; the decode rows get the share of
 // the SMs that kBesideWeight times their work is of the whole, counted in page tiles: a page of a kv head is 1, 128 keys of a
 // pair of chunk row tiles are kBesidePairTile (2.3 us against 0.106 us), of a lone row tile kBesideLoneTile.  A serving
-// iteration (32 decode rows, 32 steps, lognormal lengths) 806 -> 748 us, 900 -> 874 us under the power cap (weights 1.33 /
-// 1.9 / 2.6 / 3.5: 813 / 749 / 746 / 769 us); one 16-token step beside 15 decode rows of 4k to 32k 217 -> 199 us (on a fixed
-// 65 SMs 271), four of 32 tokens beside 60 rows of 500 to 3000 114 -> 100 us, one of 8 beside 7 draft-shaped rows 33 -> 24 us.
+// iteration (32 decode rows, 32 steps, lognormal lengths) 806 -> 748 us at full clock, 921 -> 871 us under the power cap (weights
+// 1.33 / 1.9 / 2.6 / 3.5: 813 / 749 / 746 / 769 us); one 16-token step beside 15 decode rows of 4k to 32k 217 -> 199 us (on a
+// fixed 65 SMs 271), four of 32 tokens beside 60 rows of 500 to 3000 114 -> 100 us, one of 8 beside 7 draft-shaped rows 33 -> 24 us.
+// The same numbers serve E4M3 calls and 64-dimension heads, whose pages are half the bytes.  With both tile weights times
+// 0.6 / 1 / 1.5 / 2 / 2.6: the serving iteration over E4M3 codes 828 / 834 / 843 / 940 / 1002 us (one after the other 828),
+// with 64-dimension heads 668 / 680 / 676 / 677 / 772 us; 8 rows beside 8 steps of 16 to 32 tokens, 28 / 4 heads, E4M3 265 / 267 /
+// 273 / 270 / 260 us (one after the other 297), 64 dimensions 240 / 239 / 240 / 238 / 234 us: flat around 1.
 constexpr float kBesideWeight = 2.2f;
 constexpr int kBesidePairTile = 22, kBesideLoneTile = 13;
 
