@@ -168,8 +168,8 @@ arb_status arb_create(arb_ctx **out, int device, size_t workspace_bytes) {
     ok = ok && cudaMemset(c->rank_ws, 0, kRankCounterBytes) == cudaSuccess;
     c->chunk_ws_bytes = 2 * c->workspace_bytes;   // partials of long step chunks that are split over their keys
     ok = ok && guarded_malloc(c, &c->chunk_ws, c->chunk_ws_bytes);
-    ok = ok && guarded_malloc(c, &c->step_hint, decode_step_hint_bytes(sms));
-    ok = ok && cudaMemset(c->step_hint, 0, decode_step_hint_bytes(sms)) == cudaSuccess;
+    ok = ok && guarded_malloc(c, &c->step_slots, decode_step_slot_bytes(sms));
+    ok = ok && cudaMemset(c->step_slots, 0xff, decode_step_slot_bytes(sms)) == cudaSuccess;
     if (ok && c->n_guards > 0) {
         ok = cudaMalloc(&c->guards_dev, sizeof(c->guards)) == cudaSuccess &&
              cudaMalloc(&c->guard_bad, sizeof(unsigned long long)) == cudaSuccess &&
@@ -186,7 +186,7 @@ arb_status arb_create(arb_ctx **out, int device, size_t workspace_bytes) {
         guarded_free(c->rot);
         guarded_free(c->rank_ws);
         guarded_free(c->chunk_ws);
-        guarded_free(c->step_hint);
+        guarded_free(c->step_slots);
         cudaFree(c->guards_dev);
         cudaFree(c->guard_bad);
         delete c;
@@ -207,7 +207,7 @@ arb_status arb_destroy(arb_ctx *ctx) {
     guarded_free(c->rot);
     guarded_free(c->rank_ws);
     guarded_free(c->chunk_ws);
-    guarded_free(c->step_hint);
+    guarded_free(c->step_slots);
     cudaFree(c->guards_dev);
     cudaFree(c->guard_bad);
     cudaFree(c->stage);
@@ -753,6 +753,7 @@ arb_status arb_poll_status(arb_ctx *ctx, arb_stream_t stream, uint32_t *bits) {
         if (cudaMemsetAsync(c->rot + (size_t)kRotSets * kRotCounters + kRotSets + 1, 0, sizeof(int) * 7, s) != cudaSuccess) return ARB_ERR_CUDA;
         if (cudaMemsetAsync(c->counters, 0, sizeof(int) * (c->counters_len + 4), s) != cudaSuccess) return ARB_ERR_CUDA;
         if (cudaMemsetAsync(c->rank_ws, 0, kRankCounterBytes, s) != cudaSuccess) return ARB_ERR_CUDA;
+        if (cudaMemsetAsync(c->step_slots, 0xff, decode_step_slot_bytes(c->num_sms), s) != cudaSuccess) return ARB_ERR_CUDA;
         if (cudaMemsetAsync(c->rot, 0, sizeof(int) * ((size_t)kRotSets * kRotCounters + kRotSets), s) != cudaSuccess)
             return ARB_ERR_CUDA;
         if (cudaStreamSynchronize(s) != cudaSuccess) return ARB_ERR_CUDA;

@@ -59,7 +59,7 @@ struct Ctx {
     uint32_t rot_wait_through = 0;        // tensor-core decode calls up to this generation wait for their predecessor
     char *rank_ws = nullptr;              // arb_policy, arb_spearman: two arrival counters (zero between calls), then at
                                           // kRankCounterBytes the statistics of a policy's CTAs and the ranks of two samples
-    int *step_hint = nullptr;             // single-launch decode: the page tiles each CTA streamed last (arb_decode_step.cu)
+    float *step_slots = nullptr;          // single-launch decode: the exchange slots of its CTAs, 0xff bytes between calls
     int step_min_chunk = 16;              // single-launch decode: fewest pages worth giving a CTA
     int step_boundary_pct = 100;          // single-launch decode: what a (sequence, kv head) boundary inside a CTA's range counts for
     float *chunk_ws = nullptr;            // partial results of split long sequences (step-chunk attention)
@@ -152,6 +152,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ void mbar_inval(uint64_t *bar) {   // before the same words become a new barrier
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ void mbar_fence_init() {
@@ -342,7 +346,7 @@ arb_status launch_kv_append_i4(Ctx *ctx, const arb_attn_params &p, int total_new
                                const int32_t *block_table, int32_t *seq_lens, const int32_t *new_lens, int update_lens,
                                void *k_codes, void *v_codes, float *k_scales, float *v_scales, cudaStream_t stream);
 bool decode_step_supported(const arb_attn_params &p);
-size_t decode_step_hint_bytes(int num_sms);
+size_t decode_step_slot_bytes(int num_sms);
 arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q, const void *k_new, const void *v_new,
                               void *k_pages, void *v_pages, const float *scales, const int32_t *block_table,
                               int32_t *seq_lens, const int32_t *q_lens, void *out, cudaStream_t stream,

@@ -16,12 +16,14 @@
 //     lanes that share a column pair (three shuffles).
 //   - The kernel waits for its predecessor near its top (griddepcontrol.wait) and lets its successor come up at
 //     once (griddepcontrol.launch_dependents; beside chunks only behind its own wait): launched as a programmatic dependent
-//     it is resident, barriers initialised, when the kernel before it ends.  Before the wait it reads nothing but the hint
-//     record of the context, which only this kernel writes and whose rows are range-checked and only prefetched, so this
-//     is safe behind any kernel.
-//   - The combine is inside: a CTA that holds a part of a split (sequence, kv head) stores its partial, fences,
-//     and adds one to the item's arrival counter; the CTA that arrives last merges the parts (two round trips
-//     to L2) and writes the rows.  No CTA waits for another.
+//     it is resident when the kernel before it ends, and by then it has read lengths and table and knows its work.  What it
+//     read is a guess, since the predecessor may be writing either: it is read again behind the wait, while the first
+//     tiles are on their way, and where anything differs the CTA starts over (see `guess`).
+//   - The combine is inside, and the partials are their own arrival signal: a CTA that holds a part of a split (sequence, kv
+//     head) stores it into its slot of an exchange buffer whose words hold a value no result has, and leaves; a CTA that
+//     merges reads the slots until every word has come, writes the rows and puts the value back.  It waits only for CTAs
+//     that drew an earlier ticket, which have started, so every wait ends whatever else is running.  The merging CTA is one
+//     with nothing else to do (the last tickets, see kMergerShare), or the one that holds the item's last part.
 //   - With k_new / v_new given, the warp that owns a sequence's last page puts the token's new row into the
 //     tile in shared memory (the tile arrives with whatever the slot held) and stores it to the pool; the
 //     lengths move forward once every CTA has read them (a counter in the prologue tells the last reader).
@@ -66,23 +68,32 @@ constexpr int kProdWarp = kCW;                // the producer warps, and behind 
 // tokens the same within 1 %, and where a tile is 2 KB or less more: 16 x 8 kv heads of 64 dimensions (150 MB) 38 -> 32 us,
 // draft-shaped tokens over 4-bit codes 17.6 -> 16.7 us.
 constexpr int kAuxWarp = kCW + 2;
+constexpr int kVerifyWarp = kCW - 1;          // the consumer warp that compares the guess (see decode_step_kernel) with what is final
 constexpr int kNT = 32 * (kCW + 3);
 
-constexpr int kMergeBatch = 12;               // parts of a split item merged per round of loads, straight into registers ...
-constexpr int kDirectParts = 2 * kMergeBatch; // ... up to this many; more go through the ring in one bulk copy
+// The exchange of a split item's parts.  A slot is what one CTA hands on: the group's outputs and (max, sum) per head, every
+// 32-bit word of it kEmpty until it is stored, and kEmpty again once it has been read.  A NaN of a result never has these bits
+// (see not_empty).  Against partials, a fence, an arrival counter and the last to arrive reading what the others left, a
+// draft-shaped token 12.4 -> 11.6 us, one of a single sequence of 256 tokens 7.3 -> 6.6 us.
+constexpr uint32_t kEmpty = 0xffffffffu;
+// A call of few items gives each a CTA that streams nothing and merges it: the others leave when they have stored their parts,
+// the next kernel's CTAs come up in their places, and where they would come late, behind a merge, there are the next
+// kernel's mergers, which have time.  Up to a kMergerShare-th of the CTAs (the SMs missed by the stream cost little, it is
+// bound by the memory): draft-shaped token (16 items) 11.0 -> 10.85 us, over E4M3 codes 10.0 -> 9.6 us, 8 x 8 heads (64
+// items, so not) the same.
+constexpr int kMergerShare = 4;
 // What a boundary costs is time (the warps meet, a second arrival, perhaps a second merge), a few microseconds
 // whatever the call's size: as pages it is the CTA's even share, but no more than this many.
 constexpr int kBoundaryCap = 32;
-// Hints for the next call: every CTA leaves the pool rows of the first kHintPages page tiles of its range in a record
-// of the context.  The next call of the same shape asks for those tiles into L2 before it waits for its predecessor
-// (the bookkeeping warp does, off every other warp's path): in a chain of dependent calls the bytes of call n + 1
-// cross from HBM while call n is in its latency-bound tail.  A prefetch is a hint: rows are range-checked, a stale or
-// foreign record costs some bandwidth and nothing else, and every real read comes after the wait.
-// 24 pages are about what HBM delivers while a kernel ends and the next one finds its plan.  More only stand in the way of the
-// lengths and the table: 64 / 32 / 24 / 16 / 8 pages, draft-shaped token 12.6 / 12.4 / 12.1 / 12.2 / 12.3 us, 32 x 8 kv
-// heads of 200 to 900 tokens 20.1 / 18.5 / 18.4 / 18.9 / 18.9 us, rounds of the step loop alike.
-constexpr int kHintPages = 24;
-constexpr int kHintStride = kHintPages + 4;   // [tag, count, -, -, rows ...]
+// The first kAheadPages page tiles of a CTA's range are asked into L2 before the wait for the predecessor (the bookkeeping warp
+// does, off every other warp's path): in a chain of dependent calls the bytes of call n + 1 cross from HBM while call n is in
+// its latency-bound tail.
+// Copies for L2 pass through the unit that brings the tiles, so many of them stand in front of the first: 0 / 4 / 8 / 16 / 24
+// pages, draft-shaped token 11.3 / 10.7 / 10.6 / 10.7 / 10.9 us, 48 x 2 kv heads of 512 to 2048 tokens 16.4 / 16.2 / 15.9 / 15.8 /
+// 15.3 us, 16 x 8 heads of 64 dimensions 30.5 / 30.1 / 30.0 / 29.7 / 29.8 us.  (By prefetch instructions the lines held up the
+// loads behind them: 11.8 us.)
+constexpr int kAheadPages = 16;
+constexpr int kLensCycles = 10000;   // a few microseconds: the lengths move one or two after the predecessor's end
 
 // The decode rows of a call with chunks stream while the chunks compute, on SMs of their own: alone an SM draws about 77 GB/s
 // (65 of them 5 TB/s), beside chunks less.  Both kinds of work are known from the lengths; the decode rows get the share of
@@ -106,18 +117,15 @@ struct StepArgs {
     int32_t *seq_lens;
     const int32_t *q_lens;
     char *out;
-    float *part_o;     // [slots][G][D]
-    float *part_ml;    // [slots][GP][2]
-    int *counters;     // [batch * Hkv] arrival counters, zero between calls
-    int *lens_counter; // CTAs that have read the lengths, zero between calls
-    int *hint;         // [grid][kHintStride] the page tiles each CTA streamed last time (see kHintPages)
-    int hint_tag;      // shape of this call; a record with another tag is ignored
+    float *part_o;     // [CTAs][2][G][D]  the exchange slots (see kEmpty): of an item's later parts, and of its first part
+    float *part_ml;    // [CTAs][2][kMaxGroup][2]
+    unsigned *ticket;  // the next CTA's number; back at zero when the last has drawn
+    int *lens_counter; // CTAs that have read the lengths, zero between calls and once the lengths have moved
+    int guess;         // lengths and table may be read before the predecessor has ended
     uint32_t *status;
     int batch, Hq, Hkv, num_pages, max_pages;
-    uint32_t grid_inv; // floor(2^32 / CTAs) + 1
     int beside;        // the kernel launched next runs beside this one (see launch_decode_step)
     int whole_rows;    // the tensor maps are 3-D: one copy per page tile instead of one per half
-    int slots;         // partial slots in the workspace region (bounds-check build)
     int rows;          // rows of q and out
     int min_chunk;     // fewest pages worth giving a CTA
     int boundary_pct;  // cost of a (sequence, kv head) boundary inside a CTA's range: percent of min(even share, kBoundaryCap) pages
@@ -131,15 +139,15 @@ template <int STAGES>
 struct Tail {
     uint64_t full[STAGES];
     uint64_t empty[STAGES];
-    uint64_t merge_bar;   // the bulk copies of a merge
+    uint64_t verdict;     // the guess has been compared with what is final
+    int differs;          // ... and this is what was found
     int abort;
-    int last[2];
+    int ticket;
 };
 
 template <int G, int HD>
 struct Cfg {
     static constexpr int kOStride = HD + 4;               // floats between two heads of a warp record (spreads the banks)
-    static constexpr int GP = (G + 3) / 4 * 4;
     static constexpr int WREC = 2 * 8 + G * kOStride;     // warp record: [m[8] | l[8] | o[G][kOStride]]
     static constexpr int OSM_BYTES = kCW * WREC * 4;
 };
@@ -149,13 +157,34 @@ size_t smem_bytes(int batch) {
     using C = Cfg<G, HD>;
     constexpr int kTileBytes = HD / 64 * kHalfTile;
     const size_t tiles = (size_t)STAGES * (KV == kKvE4m3 ? kCodeTileBytes : KV == kKvI4 ? kI4StageBytes : kTileBytes);
-    return 1024 + tiles + C::OSM_BYTES + sizeof(Tail<STAGES>) + sizeof(int) * (4 * (size_t)batch + 3);
+    return 1024 + tiles + C::OSM_BYTES + sizeof(Tail<STAGES>) + sizeof(int) * (6 * (size_t)batch + 3);
 }
 
-struct Split {   // a (sequence, kv head) of which this CTA holds a part
-    int bk, slot0, nparts;
-    size_t out_base;
-};
+__device__ __forceinline__ float4 load_slot4(const float4 *p) {   // not ordered among one another: each word is its own signal
+    float4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 load_slot2(const float2 *p) {
+    float2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_slot4(float4 *p, float4 v) {
+    asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void store_slot2(float2 *p, float2 v) {
+    asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ int load_now(const int32_t *p) {   // from L2, whoever wrote it and whenever
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ bool is_empty(float x) { return __float_as_uint(x) == kEmpty; }
+__device__ __forceinline__ bool any_empty(float4 v) { return is_empty(v.x) || is_empty(v.y) || is_empty(v.z) || is_empty(v.w); }
+// a word fit for a slot: a NaN with kEmpty's bits becomes another NaN
+__device__ __forceinline__ float not_empty(float x) { return is_empty(x) ? __uint_as_float(0x7fffffffu) : x; }
 
 __device__ __forceinline__ uint32_t tile_off(int r, int c) {   // 16-byte chunk c of row r of a swizzled bf16 tile
     return (uint32_t)((c >> 3) * kHalfTile + r * 128 + (((c & 7) ^ (r & 7)) << 4));
@@ -262,6 +291,8 @@ struct Plan {
     const int *act;    // [B + 1] sequences before b that take part
     const int *slen;   // [B] length of sequence b (with the new token)
     int B, Hkv, pen, chunk, total_padded;
+    int stream;        // CTAs that stream; with `mergers` those behind them have an item each to merge
+    bool mergers;
 
     __device__ __forceinline__ int pages_of(int b) const { return pref[b + 1] != pref[b] ? (slen[b] + kPage - 1) / kPage : 0; }
     __device__ __forceinline__ int padded_start(int b) const { return pref[b] + pen * Hkv * act[b]; }
@@ -320,14 +351,14 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     constexpr int kBatch = kOwnStages < 32 ? kOwnStages : 32;   // lanes of a producer warp issuing side by side
     using C = Cfg<G, HD>;
     using Tail = arb::Tail<STAGES>;
-    constexpr int GP = C::GP, WREC = C::WREC, kOStride = C::kOStride;
+    constexpr int WREC = C::WREC, kOStride = C::kOStride;
     constexpr int kD = HD, kTileBytes = HD / 64 * kHalfTile;   // a tile of a bf16 cache
     constexpr bool SPLIT_P = HD == 64;
     constexpr bool E4M3 = KV == kKvE4m3, I4 = KV == kKvI4, CODES = KV != kKvBf16;
     constexpr int kStageBytes = E4M3 ? kCodeTileBytes : I4 ? kI4StageBytes : kTileBytes;   // a ring stage
     constexpr int kTxBytes = I4 ? kI4CodeBytes + kI4ScaleBytes : kStageBytes;               // what the copies of a stage bring
     constexpr int kRowBytes = E4M3 ? kD : I4 ? kD / 2 : kD * 2;         // bytes of a cache row
-    constexpr int kRingBytes = STAGES * kStageBytes;                    // the merges use all of it
+    constexpr int kRingBytes = STAGES * kStageBytes;
     constexpr int kRowWords = E4M3 ? 8 : 4;                             // 32-bit words of codes a lane takes per key row for S^T
     static_assert(!CODES || HD == 128, "code caches have 128-dimension rows");
     static_assert(G >= 1 && G <= 8, "the group's heads are the 8 columns of the tile");
@@ -342,74 +373,68 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     int *row0 = pref + a.batch + 1;
     int *act = row0 + a.batch + 1;
     int *slen = act + a.batch + 1;
+    int *raw_n = slen + a.batch, *raw_len = raw_n + a.batch;   // q_lens and seq_lens as they were read
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int B = a.batch, Hkv = a.Hkv;
 
-    if (!a.beside) let_successor_start();
     if (tid == kCT) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&k_map)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&v_map)) : "memory");
     }
-    if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&tail->full[s], 1);
-            mbar_init(&tail->empty[s], 1);
+    // The CTA's number: in the order in which CTAs start, which is what the waits of the merge rest on (see kEmpty).  The
+    // successor may come up, and draw from the same counter, only once this has been drawn.
+    if (tid == kAuxWarp * 32) {
+        tail->ticket = (int)atomicInc(a.ticket, gridDim.x - 1);
+        if (!a.beside) let_successor_start();
+    }
+    if (warp == 0) {
+        for (int st = lane; st < STAGES; st += 32) {
+            mbar_init(&tail->full[st], 1);
+            mbar_init(&tail->empty[st], 1);
         }
-        mbar_init(&tail->merge_bar, 1);
-        tail->abort = 0;
+        if (lane == 0) {
+            mbar_init(&tail->verdict, 1);
+            tail->abort = 0;
+            pref[0] = 0;
+            row0[0] = 0;
+            act[0] = 0;
+        }
         mbar_fence_init();
-        pref[0] = 0;
-        row0[0] = 0;
-        act[0] = 0;
     }
-    __syncthreads();   // the barriers are initialised: off the path that begins below
-    int *hint = a.hint + (size_t)blockIdx.x * kHintStride;
-    if (warp == kAuxWarp) {
-        // the tiles this CTA streamed last time are asked into L2 while the predecessor is still at work
-        const int tag = __ldcg(hint), cnt = __ldcg(hint + 1);
-        if (tag == a.hint_tag) {
-            const int n = min(cnt, kHintPages);
-            for (int i = lane; i < n; i += 32) {
-                const int row = __ldcg(hint + 4 + i);
-                if ((unsigned)row < (unsigned)(a.num_pages * Hkv * kPage)) {
-                    const size_t off = (size_t)row * kRowBytes;
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.k_pool + off), "r"(kPage * kRowBytes) : "memory");
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.v_pool + off), "r"(kPage * kRowBytes) : "memory");
-                }
-            }
-        }
+    if (!a.guess) wait_for_predecessor();
+    for (int b = tid; b < B; b += kNT) {
+        raw_n[b] = load_now(a.q_lens + b);
+        raw_len[b] = load_now(a.seq_lens + b);
     }
-    // Everything below may read what the kernel before this one wrote (lengths, q, new rows, the cache).
-    wait_for_predecessor();
-    if (a.beside) let_successor_start();   // the successor does not wait for this kernel, but it may read what the predecessor wrote
+    __syncthreads();   // barriers, ticket and lengths are there
+    const int cta = tail->ticket;
 
     // ---- prologue: lengths -> page counts and q row offsets -------------------------------------------------
-    // Every warp works the plan out for itself: nothing but its own loads and shuffles lies between the predecessor's end
-    // and a warp's first look-up.  (One warp planning for all, with two barriers and a search of its tables, took 1.2 us; a
-    // draft-shaped token 12.9 -> 12.6 us, one of a single 256-token sequence 6.8 -> 6.5 us.)  All warps store the same values
-    // into the tables.  A batch of more than 32 is loaded by the whole block first.
+    // Every warp works the plan out for itself, and all store the same values into the tables.  (One warp planning for all, with
+    // two barriers and a search of its tables, took 1.2 us; a draft-shaped token 12.9 -> 12.6 us, one of a single 256-token
+    // sequence 6.8 -> 6.5 us.)  Of a batch of more than 32 the block makes the tables together.
     Plan pl;
     pl.pref = pref; pl.act = act; pl.slen = slen; pl.B = B; pl.Hkv = Hkv;
     // total work and items -> what a boundary counts for, the padded list's length, the even share of it
-    int ctas = (int)gridDim.x;   // that take part
-    auto per_cta = [&](int x) -> int {   // ceil(x / ctas), mostly through the launch's reciprocal, which is at most one too large
-        if (a.beside) return fast_div(x + ctas - 1, ctas);
-        const uint32_t y = (uint32_t)(x + ctas - 1), q = __umulhi(y, a.grid_inv);
-        return (int)(q * (uint32_t)ctas > y ? q - 1 : q);
-    };
+    int ctas;   // that take part
+    auto per_cta = [&](int x) -> int { return fast_div(x + ctas - 1, ctas); };
     auto chunk_work = [&](int n, int L) -> float {   // of one sequence, in page tiles
         if (n < 2 || L < n) return 0.f;
         const int tiles = (n * G + 127) / 128;
         return (float)Hkv * (float)((L + 127) / 128) * (float)((tiles >> 1) * kBesidePairTile + (tiles & 1) * kBesideLoneTile);
     };
     auto shares = [&](int total, int items, float chunks) {
+        ctas = (int)gridDim.x;
         if (a.beside) {
 #pragma unroll
             for (int off = 16; off >= 1; off >>= 1) chunks += __shfl_xor_sync(0xffffffffu, chunks, off);
             const float mine = kBesideWeight * (float)total;
             ctas = min(ctas, max(4, __float2int_ru((float)ctas * __fdividef(mine, mine + chunks + 1.f))));
         }
+        pl.mergers = !a.beside && items * kMergerShare <= ctas;
+        if (pl.mergers) ctas -= items;
+        pl.stream = ctas;
         const int even = max(a.min_chunk, per_cta(total));
         pl.pen = items > 1 ? (min(even, kBoundaryCap) * a.boundary_pct + 99) / 100 : 0;
         pl.total_padded = total + pl.pen * items;
@@ -417,7 +442,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     };
     int ends[2], seq0 = 0;   // this CTA's range, and the sequence it begins in
     auto lengths_of = [&](int b, int &pages, int &rows, int &ok, int &L) {
-        const int n = a.q_lens[b], L0 = a.seq_lens[b];
+        const int n = raw_n[b], L0 = raw_len[b];
         ok = step_ok<APPEND>(n, L0, a.max_pages) ? 1 : 0;
         L = L0 + (APPEND ? 1 : 0);
         pages = ok ? (L + kPage - 1) / kPage * Hkv : 0;
@@ -432,96 +457,227 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             if (lane >= off) { vp += tp; vr += tr; va += ta; }
         }
     };
-    if (B <= 32) {
-        int vp = 0, vr = 0, va = 0, L = 0;
-        if (lane < B) lengths_of(lane, vp, vr, va, L);
-        const int own = vp, ok = va, rows = vr;
-        scan3(vp, vr, va);
-        if (lane < B) { pref[lane + 1] = vp; row0[lane + 1] = vr; act[lane + 1] = va; slen[lane] = L; }
-        const int total = __shfl_sync(0xffffffffu, vp, 31);
-        shares(total, __shfl_sync(0xffffffffu, va, 31) * Hkv, a.beside ? chunk_work(rows, L) : 0.f);
-        // the lane whose sequence holds an end of the range works it out (see Plan)
-        const int pages = ok ? (L + kPage - 1) / kPage : 0, item = pages + pl.pen;
-        const int first = vp - own + pl.pen * Hkv * (va - ok);
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            const long long rel = (long long)(blockIdx.x + w) * pl.chunk - first;
-            const bool here = ok && rel >= 0 && rel < (long long)item * Hkv;
-            const int r = here ? (int)rel : 0, kvh = fast_div(r, max(item, 1));
-            const int pos = vp - own + kvh * pages + max(0, r - kvh * item - pl.pen);
-            const unsigned mask = __ballot_sync(0xffffffffu, here);
-            const int src = __ffs(mask) - 1;
-            const int at = __shfl_sync(0xffffffffu, pos, src & 31);
-            ends[w] = mask ? at : total;   // nobody's: behind the end of the list
-            if (w == 0) seq0 = max(src, 0);
+    auto make_plan = [&]() {
+        if (B <= 32) {
+            int vp = 0, vr = 0, va = 0, L = 0;
+            if (lane < B) lengths_of(lane, vp, vr, va, L);
+            const int own = vp, ok = va, rows = vr;
+            scan3(vp, vr, va);
+            if (lane < B) { pref[lane + 1] = vp; row0[lane + 1] = vr; act[lane + 1] = va; slen[lane] = L; }
+            const int total = __shfl_sync(0xffffffffu, vp, 31);
+            shares(total, __shfl_sync(0xffffffffu, va, 31) * Hkv, a.beside ? chunk_work(rows, L) : 0.f);
+            // the lane whose sequence holds an end of the range works it out (see Plan)
+            const int pages = ok ? (L + kPage - 1) / kPage : 0, item = pages + pl.pen;
+            const int first = vp - own + pl.pen * Hkv * (va - ok);
+    #pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                const long long rel = (long long)(cta + w) * pl.chunk - first;
+                const bool here = ok && rel >= 0 && rel < (long long)item * Hkv;
+                const int r = here ? (int)rel : 0, kvh = fast_div(r, max(item, 1));
+                const int pos = vp - own + kvh * pages + max(0, r - kvh * item - pl.pen);
+                const unsigned mask = __ballot_sync(0xffffffffu, here);
+                const int src = __ffs(mask) - 1;
+                const int at = __shfl_sync(0xffffffffu, pos, src & 31);
+                ends[w] = mask ? at : total;   // nobody's: behind the end of the list
+                if (w == 0) seq0 = max(src, 0);
+            }
+            __syncwarp();
+        } else {
+            for (int b = tid; b < B; b += kNT) {
+                int vp, vr, va, L;
+                lengths_of(b, vp, vr, va, L);
+                pref[b + 1] = vp; row0[b + 1] = vr; act[b + 1] = va; slen[b] = L;
+            }
+            __syncthreads();
+            if (warp == 0) {
+                int carry_p = 0, carry_r = 0, carry_a = 0;
+                for (int b0 = 0; b0 < B; b0 += 32) {
+                    const int b = b0 + lane;
+                    int vp = b < B ? pref[b + 1] : 0, vr = b < B ? row0[b + 1] : 0, va = b < B ? act[b + 1] : 0;
+                    scan3(vp, vr, va);
+                    if (b < B) { pref[b + 1] = vp + carry_p; row0[b + 1] = vr + carry_r; act[b + 1] = va + carry_a; }
+                    carry_p += __shfl_sync(0xffffffffu, vp, 31);
+                    carry_r += __shfl_sync(0xffffffffu, vr, 31);
+                    carry_a += __shfl_sync(0xffffffffu, va, 31);
+                }
+            }
+            __syncthreads();
+            // both ends of the range with one ballot per 32 sequences: the padded starts ascend, so the sequence that holds a
+            // position is the last one that starts at or before it
+            const int total = pref[B];
+            float chunks = 0.f;
+            if (a.beside)
+                for (int b = lane; b < B; b += 32) chunks += chunk_work(row0[b + 1] - row0[b], slen[b]);
+            shares(total, act[B] * Hkv, chunks);
+    #pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                const long long t = (long long)(cta + w) * pl.chunk;
+                int best = 0;
+                for (int b0 = 0; b0 < B; b0 += 32) {
+                    const int b = b0 + lane;
+                    const unsigned mask = __ballot_sync(0xffffffffu, b < B && pl.padded_start(b) <= t);
+                    if (mask) best = b0 + 31 - __clz(mask);
+                }
+                ends[w] = t >= pl.total_padded ? total : pl.real_in(best, t);
+                if (w == 0) seq0 = best;
+            }
         }
-        __syncwarp();
-    } else {
+    };
+
+    // ---- the producers' and consumers' first steps ----------------------------------------------------------
+    // The kv head of flat triple r, and where its page's number stands in the table.
+    auto find_page = [&](int r, const int32_t *&entry, int &kvh) {
+        const int lo = pl.seq_of(r, seq0);
+        int pg;
+        kvh = small_div(r - pref[lo], pl.pages_of(lo), pg);
+        const bool in = ARB_IN_RANGE(a.status, pg, a.max_pages) && ARB_IN_RANGE(a.status, kvh, Hkv);
+        entry = a.block_table + (in ? (size_t)lo * a.max_pages + pg : 0);
+    };
+    const int pw = warp - kProdWarp;       // of a producer warp: 0 brings K, 1 V
+    const bool is_v = pw == 1;
+    const CUtensorMap *map = is_v ? &v_map : &k_map;
+    auto issue = [&](uint32_t st, int row) {   // the copies of the page tile that begins at `row` of the 2-D view of the pool
+        mbar_arrive_expect_tx(&tail->full[st], kTxBytes);
+        if constexpr (I4) {   // 16 rows x 64 bytes of codes, then the rows' 16 scales
+            tma_box_load(ring + st * kStageBytes, map, 0, row, &tail->full[st]);
+            bulk_load(ring + st * kStageBytes + kI4CodeBytes, (is_v ? a.v_scales : a.k_scales) + row, kI4ScaleBytes, &tail->full[st]);
+        } else if constexpr (E4M3) {
+            tma_box_load(ring + st * kStageBytes, map, 0, row, &tail->full[st]);   // 16 rows x 128 codes
+        } else if constexpr (HD == 64) {
+            tma_box_load(ring + st * kTileBytes, map, 0, row, &tail->full[st]);    // 16 rows x 64 dims
+        } else if (a.whole_rows) {
+            tma_box_load3(ring + st * kTileBytes, map, 0, row, 0, &tail->full[st]);
+        } else {
+            tma_box_load(ring + st * kTileBytes, map, 0, row, &tail->full[st]);
+            tma_box_load(ring + st * kTileBytes + kHalfTile, map, 64, row, &tail->full[st]);
+        }
+    };
+    const int gq = lane >> 2, tq = lane & 3;   // fragment coordinates
+    const bool head_ok = gq < G;               // as a B-fragment column: this lane's head is a real one
+    // B fragments of q^T (kD dims x 8 heads): k-slice ks holds dims 16 ks + 2 tq, + 1 and + 8 of head gq.  The
+    // fragments of the next segment are asked for while this one streams.
+    uint32_t qb[kD / 16][2], qn[kD / 16][2];
+    auto load_q = [&](const Segment &g, uint32_t (&dst)[kD / 16][2]) {
+        const int row = row0[g.b];   // (guessed lengths may point anywhere)
+        const char *qh = a.q + ((size_t)((unsigned)row < (unsigned)a.rows ? row : 0) * a.Hq + g.kvh * G + (head_ok ? gq : 0)) * kD * 2;
+#pragma unroll
+        for (int ks = 0; ks < kD / 16; ++ks) {
+            if constexpr (CODES) {   // dimensions 32 tq + 4 ks .. + 3, in the order the codes come in
+                const uint2 w = head_ok ? __ldg(reinterpret_cast<const uint2 *>(qh + tq * 64 + ks * 8)) : make_uint2(0u, 0u);
+                dst[ks][0] = E4M3 ? bf16x2_to_f16x2(w.x) : w.x;   // (the operands of one MMA share a type)
+                dst[ks][1] = E4M3 ? bf16x2_to_f16x2(w.y) : w.y;
+                continue;
+            }
+            dst[ks][0] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + tq * 4)) : 0u;
+            dst[ks][1] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + 16 + tq * 4)) : 0u;
+        }
+    };
+    Segment s = {};
+    int cur = 0, seq_at = 0, page_next = 0, row_next = 0;   // (of a producer's lane: page number and row of its next triple)
+    bool have = false;
+
+    // `guess`: in the first round the plan comes from what lengths and table held before the predecessor was known to have
+    // ended.  Behind the wait the first ring of tiles and the first q are asked for, while one warp reads lengths and the
+    // look-ups' table entries again and tells everyone whether all of it still holds.  Until then nothing has been written
+    // and only tiles and q rows were read, in bounds whatever the guess.  Where something differs (lengths that the kernel right
+    // in front moves, as a rollback does) the copies are waited for, the barriers made new, and the second round plans from
+    // what is final.  Three dependent round trips (lengths, table, tile) and the plan become one behind the predecessor's end:
+    // tokens of one sequence of 256 / 2048 / 32768 tokens 7.3 / 8.1 / 15.7 -> 6.1 / 6.9 / 13.4 us, draft-shaped 12.4 -> 10.7 us
+    // with the mergers.
+#pragma unroll 1
+    for (bool guess = a.guess != 0;; guess = false) {
+        make_plan();
+        const int nflat = ends[1] - ends[0];
+        const int32_t *entry = a.block_table;
+        if (warp >= kVerifyWarp && lane < nflat) {
+            int kvh;
+            find_page(ends[0] + lane, entry, kvh);
+            page_next = load_now(entry);
+            row_next = ((unsigned)page_next < (unsigned)a.num_pages ? page_next * Hkv + kvh : 0) * kPage;
+        }
+        if (guess) {
+            if (warp == kAuxWarp && lane < min(nflat, kAheadPages)) {
+                const size_t off = (size_t)row_next * kRowBytes;
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.k_pool + off), "r"(kPage * kRowBytes) : "memory");
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.v_pool + off), "r"(kPage * kRowBytes) : "memory");
+            }
+            wait_for_predecessor();
+        }
+        if (guess && warp == kVerifyWarp) {
+            bool differs = lane < nflat && load_now(entry) != page_next;
+#pragma unroll 4
+            for (int b = lane; b < B; b += 32)
+                differs |= load_now(a.q_lens + b) != raw_n[b] || load_now(a.seq_lens + b) != raw_len[b];
+            differs = __any_sync(0xffffffffu, differs);
+            if (lane == 0) {
+                tail->differs = differs;
+                mbar_arrive(&tail->verdict);
+            }
+        }
+        const bool first_copy = (warp == kProdWarp || warp == kProdWarp + 1) && lane < min(nflat, kBatch);
+        if (first_copy && ARB_IN_RANGE(a.status, row_next, (long long)a.num_pages * Hkv * kPage)) issue(2u * lane + (uint32_t)pw, row_next);
+        if (warp < kCW) {
+            cur = ends[0];
+            seq_at = seq0;
+            have = next_segment(cur, ends[1], seq_at, pl, s);
+            if (have) load_q(s, qb);
+        }
+        if (!guess) break;
+        mbar_wait(&tail->verdict, 0, &tail->abort, a.status);
+        if (!*(volatile int *)&tail->differs) break;
+        if (first_copy) mbar_wait(&tail->full[2 * lane + pw], 0, &tail->abort, a.status);
+        __syncthreads();
+        if (tid == 0) {
+            for (int st = 0; st < STAGES; ++st) {
+                mbar_inval(&tail->full[st]);
+                mbar_inval(&tail->empty[st]);
+                mbar_init(&tail->full[st], 1);
+                mbar_init(&tail->empty[st], 1);
+            }
+            mbar_fence_init();
+        }
         for (int b = tid; b < B; b += kNT) {
-            int vp, vr, va, L;
-            lengths_of(b, vp, vr, va, L);
-            pref[b + 1] = vp; row0[b + 1] = vr; act[b + 1] = va; slen[b] = L;
+            raw_n[b] = load_now(a.q_lens + b);
+            raw_len[b] = load_now(a.seq_lens + b);
         }
         __syncthreads();
-        if (warp == 0) {
-            int carry_p = 0, carry_r = 0, carry_a = 0;
-            for (int b0 = 0; b0 < B; b0 += 32) {
-                const int b = b0 + lane;
-                int vp = b < B ? pref[b + 1] : 0, vr = b < B ? row0[b + 1] : 0, va = b < B ? act[b + 1] : 0;
-                scan3(vp, vr, va);
-                if (b < B) { pref[b + 1] = vp + carry_p; row0[b + 1] = vr + carry_r; act[b + 1] = va + carry_a; }
-                carry_p += __shfl_sync(0xffffffffu, vp, 31);
-                carry_r += __shfl_sync(0xffffffffu, vr, 31);
-                carry_a += __shfl_sync(0xffffffffu, va, 31);
-            }
-        }
-        __syncthreads();
-        // both ends of the range with one ballot per 32 sequences: the padded starts ascend, so the sequence that holds a
-        // position is the last one that starts at or before it
-        const int total = pref[B];
-        float chunks = 0.f;
-        if (a.beside)
-            for (int b = lane; b < B; b += 32) chunks += chunk_work(row0[b + 1] - row0[b], slen[b]);
-        shares(total, act[B] * Hkv, chunks);
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            const long long t = (long long)(blockIdx.x + w) * pl.chunk;
-            int best = 0;
-            for (int b0 = 0; b0 < B; b0 += 32) {
-                const int b = b0 + lane;
-                const unsigned mask = __ballot_sync(0xffffffffu, b < B && pl.padded_start(b) <= t);
-                if (mask) best = b0 + 31 - __clz(mask);
-            }
-            ends[w] = t >= pl.total_padded ? total : pl.real_in(best, t);
-            if (w == 0) seq0 = best;
-        }
     }
-    // Named barrier 3 counts the warps that have read the lengths: the bookkeeping warp waits for it, the others pass.
-    if (warp != kAuxWarp) asm volatile("bar.arrive 3, %0;" ::"r"(kNT) : "memory");
+    if (a.beside) let_successor_start();   // the successor does not wait for this kernel, but it may read what the predecessor wrote
 
     if (warp == kAuxWarp) {
         // ================================ bookkeeping warp ==========================================
-        // Lengths: once every warp has read them, the CTA counts itself in.  The CTA whose count completes the grid
+        // Lengths: nobody in this CTA reads them again, so it counts itself in.  The CTA whose count completes the grid
         // knows that nobody will read seq_lens again and moves them forward: for the sequences that take part
         // and whose new row has a page inside the pool to go to (the same test the writer of the row makes).
-        asm volatile("bar.sync 3, %0;" ::"r"(kNT) : "memory");
         if constexpr (APPEND) {
+            // (what the last one needs is on its way meanwhile)
+            const int L0 = lane < B ? slen[lane] - 1 : 0, n = lane < B ? row0[lane + 1] - row0[lane] : 0;
+            const bool moves = lane < B && step_ok<true>(n, L0, a.max_pages);
+            const int pid = moves ? load_now(a.block_table + (size_t)lane * a.max_pages + L0 / kPage) : -1;
             int last = 0;
             if (lane == 0) last = atomicAdd(a.lens_counter, 1) == (int)gridDim.x - 1;
             last = __shfl_sync(0xffffffffu, last, 0);
             if (last) {
-                for (int b = lane; b < B; b += 32) {
-                    const int L0 = slen[b] - 1;
-                    if (step_ok<true>(a.q_lens[b], L0, a.max_pages)) {
-                        const int pid = a.block_table[(size_t)b * a.max_pages + L0 / kPage];
-                        if ((unsigned)pid < (unsigned)a.num_pages) a.seq_lens[b] = L0 + 1;
+                if (moves && (unsigned)pid < (unsigned)a.num_pages) a.seq_lens[lane] = L0 + 1;
+                for (int b = lane + 32; b < B; b += 32) {
+                    const int L = slen[b] - 1;
+                    if (step_ok<true>(row0[b + 1] - row0[b], L, a.max_pages)) {
+                        const int page = load_now(a.block_table + (size_t)b * a.max_pages + L / kPage);
+                        if ((unsigned)page < (unsigned)a.num_pages) a.seq_lens[b] = L + 1;
                     }
                 }
+                __threadfence();
+                __syncwarp();
                 if (lane == 0) *a.lens_counter = 0;
+            }
+            // Where this CTA leaves, one of the next kernel comes up, and its guess is right once the lengths have moved.  A CTA with
+            // little or no work stays until then, or for as long as that should take: its place would only be waited in.
+            const long long t0 = clock64();
+            while (load_now(a.lens_counter) != 0 && clock64() - t0 < kLensCycles) {
             }
         }
         // Sequences that were asked to decode but cannot: status bit, rows of zeros.
-        if (blockIdx.x == 0) {
+        if (cta == 0) {
             for (int b = 0; b < B; ++b) {
                 const int n = row0[b + 1] - row0[b];
                 if (n != 1 || pref[b + 1] != pref[b]) continue;
@@ -534,10 +690,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     }
 
     const int r0 = ends[0], r1 = ends[1];
-    if (r0 >= r1) {
-        if (tid == 0) hint[1] = 0;   // nothing streamed: nothing to ask for next time
-        return;
-    }
+    const bool merges_only = r0 >= r1;
+    if (merges_only && (!pl.mergers || cta < pl.stream || warp >= kCW)) return;
     volatile int *abort = &tail->abort;
 
     if (warp >= kProdWarp) {
@@ -548,34 +702,24 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         // path after the first group, across sequence boundaries too.  Tiles enter the ring page by page, K then
         // V: one warp issues the K tiles, one the V tiles.  Lanes
         // 0 .. kBatch-1 of a warp each own one stage at a time.
-        const int pw = warp - kProdWarp;
-        const bool is_v = pw != 0;
-        const CUtensorMap *map = is_v ? &v_map : &k_map;
         const int nflat = r1 - r0;
-        auto tile_row = [&](int r) -> int {   // first row, in the 2-D view of the pool, of the tile of flat triple r
-            const int lo = pl.seq_of(r, seq0);
-            const int pages = pl.pages_of(lo);
-            int pg;
-            const int kvh = small_div(r - pref[lo], pages, pg);
-            int pid = ARB_IN_RANGE(a.status, pg, a.max_pages) && ARB_IN_RANGE(a.status, kvh, Hkv)
-                          ? a.block_table[(size_t)lo * a.max_pages + pg] : 0;
+        auto tile_row = [&](int r) -> int {
+            const int32_t *entry;
+            int kvh;
+            find_page(r, entry, kvh);
+            int pid = *entry;
             if ((unsigned)pid >= (unsigned)a.num_pages) {
                 atomicOr(a.status, (uint32_t)ARB_DEV_BAD_PAGE);
                 pid = 0;
             }
             return (pid * Hkv + kvh) * kPage;
         };
-        int row_next = lane < nflat ? tile_row(r0 + lane) : 0;
-        if (lane == 0 && pw == 0) {
-            hint[0] = a.hint_tag;
-            hint[1] = nflat;
-        }
+        if (lane < nflat && (unsigned)page_next >= (unsigned)a.num_pages) atomicOr(a.status, (uint32_t)ARB_DEV_BAD_PAGE);
         for (int g0 = 0; g0 < nflat; g0 += 32) {
             const int row_cur = row_next;
-            if (pw == 0 && g0 + lane < min(nflat, kHintPages)) hint[4 + g0 + lane] = row_cur;
             const int npages = min(32, nflat - g0);
 #pragma unroll 1
-            for (int i0 = 0; i0 < npages; i0 += kBatch) {
+            for (int i0 = g0 == 0 ? kBatch : 0; i0 < npages; i0 += kBatch) {   // (the first ring is on its way)
                 // the next group's look-up goes out behind this group's first copies, not in front of them
                 if (i0 == kBatch && g0 + 32 + lane < nflat) row_next = tile_row(r0 + g0 + 32 + lane);
                 const int i = i0 + lane;
@@ -589,21 +733,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 const long long t0 = clock64();
                 while (__any_sync(0xffffffffu, pending)) {
                     if (pending && mbar_test_wait(&tail->empty[st], par ^ 1u)) {
-                        mbar_arrive_expect_tx(&tail->full[st], kTxBytes);
-                        if constexpr (I4) {   // 16 rows x 64 bytes of codes, then the rows' 16 scales
-                            tma_box_load(ring + st * kStageBytes, map, 0, row, &tail->full[st]);
-                            bulk_load(ring + st * kStageBytes + kI4CodeBytes, (is_v ? a.v_scales : a.k_scales) + row,
-                                      kI4ScaleBytes, &tail->full[st]);
-                        } else if constexpr (E4M3) {
-                            tma_box_load(ring + st * kStageBytes, map, 0, row, &tail->full[st]);   // 16 rows x 128 codes
-                        } else if constexpr (HD == 64) {
-                            tma_box_load(ring + st * kTileBytes, map, 0, row, &tail->full[st]);    // 16 rows x 64 dims
-                        } else if (a.whole_rows) {
-                            tma_box_load3(ring + st * kTileBytes, map, 0, row, 0, &tail->full[st]);
-                        } else {
-                            tma_box_load(ring + st * kTileBytes, map, 0, row, &tail->full[st]);
-                            tma_box_load(ring + st * kTileBytes + kHalfTile, map, 64, row, &tail->full[st]);
-                        }
+                        issue(st, row);
                         pending = false;
                     }
                     if (pending && (*abort || clock64() - t0 > kWaitCycles)) {   // give up, like every other wait
@@ -632,18 +762,29 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     }
 
     // ==================================== consumer warps ==========================================
-    const int gq = lane >> 2, tq = lane & 3;   // fragment coordinates
-    const bool head_ok = gq < G;               // as a B-fragment column: this lane's head is a real one
     const int h0 = 2 * tq, h1 = 2 * tq + 1;    // as accumulator columns: the two heads this lane holds
     uint32_t seg_base = 0;                     // ring counter of the segment's first tile
-    int cur = r0;
-    Segment s;
-    // Only the first and the last segment of a CTA's range can be parts of a split item.
-    int n_split = 0;
-    Split sp[2];
-    constexpr int VECS = G * kD / 4;   // 4-dimension pieces of the group's outputs, one per consumer thread
-    constexpr int kPartBytes = G * kD * 4;
+    // A part of a split item is either in this CTA's last segment or its only one, and then it goes to a slot, or it is the last
+    // part of its item, in the CTA's first segment: that goes to a slot too, or, without mergers, this CTA merges.
+    constexpr int kLph = kD / 4;               // lanes of a head: one per 4-dimension piece
+    constexpr int VECS = G * kLph;             // 4-dimension pieces of the group's outputs, one per consumer thread
+    constexpr int kMergeBatch = 16;            // parts merged per round of loads, straight into registers (24: they spill, + 0.5 us)
+    constexpr int kMergeFan = 2 * kMergeBatch; // of so many parts the last hands on the sum: no CTA reads many slots
     static_assert(VECS <= kCT, "one piece per consumer thread");
+    static_assert(kMergeBatch <= kLph, "a lane of a head per part");
+    int gather_first = -1, gather_part = 0;    // the item to merge: the CTA of its first part, the number of this CTA's part
+    bool gather_last = false;                  // ... and whether that completes the item (else the sum of kMergeFan parts goes on)
+    size_t gather_out = 0;
+    float4 own = make_float4(0.f, 0.f, 0.f, 0.f);   // this CTA's part of it
+    float own_m = -INFINITY, own_l = 0.f;
+    auto publish = [&](float4 x, float M, float l, int part) {
+        if (!ARB_IN_RANGE(a.status, cta, gridDim.x)) return;
+        const int slot = 2 * cta + (part == 0);
+        store_slot4(reinterpret_cast<float4 *>(a.part_o) + (size_t)slot * VECS + tid,
+                    make_float4(not_empty(x.x), not_empty(x.y), not_empty(x.z), not_empty(x.w)));
+        if (tid % kLph == 0)
+            store_slot2(reinterpret_cast<float2 *>(a.part_ml) + (size_t)slot * kMaxGroup + tid / kLph, make_float2(not_empty(M), not_empty(l)));
+    };
     const int eh = tid / (kD / 4);     // head of this thread's piece
     auto write_row = [&](size_t out_base, float4 x, float inv) {
         if (!ARB_IN_RANGE(a.status, out_base + G * kD - 1, (size_t)a.rows * a.Hq * kD)) return;
@@ -651,30 +792,11 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             make_uint2(pack_bf16(x.x * inv, x.y * inv), pack_bf16(x.z * inv, x.w * inv));
     };
 
-    // B fragments of q^T (kD dims x 8 heads): k-slice ks holds dims 16 ks + 2 tq, + 1 and + 8 of head gq.  The
-    // fragments of the next segment are asked for while this one streams.
-    uint32_t qb[kD / 16][2], qn[kD / 16][2];
-    auto load_q = [&](const Segment &g, uint32_t (&dst)[kD / 16][2]) {
-        const char *qh = a.q + ((size_t)row0[g.b] * a.Hq + g.kvh * G + (head_ok ? gq : 0)) * kD * 2;
-#pragma unroll
-        for (int ks = 0; ks < kD / 16; ++ks) {
-            if constexpr (CODES) {   // dimensions 32 tq + 4 ks .. + 3, in the order the codes come in
-                const uint2 w = head_ok ? __ldg(reinterpret_cast<const uint2 *>(qh + tq * 64 + ks * 8)) : make_uint2(0u, 0u);
-                dst[ks][0] = E4M3 ? bf16x2_to_f16x2(w.x) : w.x;   // (the operands of one MMA share a type)
-                dst[ks][1] = E4M3 ? bf16x2_to_f16x2(w.y) : w.y;
-                continue;
-            }
-            dst[ks][0] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + tq * 4)) : 0u;
-            dst[ks][1] = head_ok ? __ldg(reinterpret_cast<const uint32_t *>(qh + ks * 32 + 16 + tq * 4)) : 0u;
-        }
-    };
     Segment s_next;
-    int seq_at = seq0;
-    bool have = next_segment(cur, r1, seq_at, pl, s);
-    if (have) load_q(s, qb);
     while (have) {
         const bool have_next = next_segment(cur, r1, seq_at, pl, s_next);
         if (have_next) load_q(s_next, qn);
+        parts_of(pl, s);   // (before the pages, the first of which is still on its way; behind them everyone waits 0.6 us for it)
         const int qrow = row0[s.b];
         // The token's new row: it belongs in slot (L - 1) mod 16 of the sequence's last page.  The warp that owns
         // that page fetches the row (lanes 0..15: K, lanes 16..31: V, 16 bytes each), stores it to the pool and
@@ -994,9 +1116,10 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         }
         named_barrier(1, kCT);
         // A whole item goes to `out`, a part of a split one to the workspace, from the registers the merge leaves it in.
-        parts_of(pl, s);
         const size_t out_base = ((size_t)qrow * a.Hq + s.kvh * G) * kD;
-        const size_t slot = (size_t)s.bk + blockIdx.x;
+        const int part = cta - s.c_first;   // (of s.nparts)
+        const bool last = part == s.nparts - 1 && !pl.mergers;   // of the item, and merged here
+        const bool gathers = s.nparts > 1 && (last || part % kMergeFan == kMergeFan - 1);
         if (tid < VECS) {
             float M = -INFINITY, mw[kCW];
 #pragma unroll
@@ -1013,14 +1136,19 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             if constexpr (E4M3) { x.x *= a.v_scale; x.y *= a.v_scale; x.z *= a.v_scale; x.w *= a.v_scale; }   // values are v_scale * code
             if (s.nparts == 1) {
                 write_row(out_base, x, 1.0f / l);
-            } else if (ARB_IN_RANGE(a.status, slot, a.slots)) {
-                reinterpret_cast<float4 *>(a.part_o + slot * G * kD)[tid] = x;
-                if (tid % (kD / 4) == 0) *reinterpret_cast<float2 *>(a.part_ml + (slot * GP + eh) * 2) = make_float2(M, l);
+            } else if (gathers) {
+                own = x;
+                own_m = M;
+                own_l = l;
+            } else {
+                publish(x, M, l, part);
             }
         }
-        if (s.nparts > 1) {
-            const Split here = {s.bk, s.bk + s.c_first, s.nparts, out_base};
-            if (n_split++ == 0) sp[0] = here; else sp[1] = here;
+        if (gathers) {
+            gather_first = s.c_first;
+            gather_part = part;
+            gather_last = last;
+            gather_out = out_base;
         }
         if (have_next) named_barrier(1, kCT);   // warp records are free for the next segment
         s = s_next;
@@ -1028,143 +1156,95 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) { qb[ks][0] = qn[ks][0]; qb[ks][1] = qn[ks][1]; }
     }
-    if (n_split == 0) return;
-    // Arrivals.  The barrier orders every thread's partials before thread 0's fence, whose release covers them; the last to
-    // arrive at an item acquires what the others released.  (A fence by every thread, and parking the results in shared memory
-    // first, cost 1.7 us more: a draft-shaped token 14.6 -> 12.9 us with the merge below, one of a single sequence of 256
-    // tokens 9.4 -> 7.1 us.)
-    named_barrier(1, kCT);
-    if (tid == 0) {
-        __threadfence();
-        int old[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-            if (j < n_split) old[j] = atomicAdd(&a.counters[sp[j].bk], 1);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int last = j < n_split && old[j] == sp[j].nparts - 1;
-            if (last) a.counters[sp[j].bk] = 0;   // everyone has arrived: ready for the next call
-            tail->last[j] = last;
+    if (merges_only) {   // the item this CTA is for: number cta - stream of those that take part
+        const int item = cta - pl.stream;
+        int b = 0;
+        while (b + 1 < B && act[b + 1] * Hkv <= item) ++b;
+        s.b = b;
+        s.kvh = item - act[b] * Hkv;
+        parts_of(pl, s);
+        if (s.nparts > 1) {
+            gather_first = s.c_first;
+            gather_part = s.nparts;
+            gather_last = true;
+            gather_out = ((size_t)row0[b] * a.Hq + s.kvh * G) * kD;
         }
-        __threadfence();
     }
-    named_barrier(1, kCT);
-    const bool last0 = tail->last[0] != 0, last1 = tail->last[1] != 0;
-    const int pend_n = (last0 ? 1 : 0) + (last1 ? 1 : 0);
-    if (pend_n == 0) return;
-    const Split pend[2] = {last0 ? sp[0] : sp[1], sp[1]};
+    if (gather_first < 0 || warp * 32 >= VECS) return;
 
-    // ---- merges of the split (sequence, kv head)s this CTA was the last to reach ------------------------
+    // ---- the merge of a split (sequence, kv head) ---------------------------------------------------------
     //     m = max_p m_p,  w_p = 2^(m_p - m),  out = sum_p w_p o_p / sum_p w_p l_p,
-    // one 4-dimension piece of the group's outputs per thread.  The parts of an item lie in consecutive workspace slots.  A few
-    // parts (the usual call: 148 CTAs over 16 items is 10 each) are loaded into registers, a round trip per kMergeBatch of them.
-    // Many parts (one sequence over the whole machine) come through the ring, which is idle by now (every tile has been
-    // consumed, the producer issues nothing more): one bulk copy brings the (max, sum) records, one the partial outputs, and
-    // the sum runs out of shared memory; more parts than the ring holds go in pieces.
-    if (max(pend[0].nparts, pend_n > 1 ? pend[1].nparts : 0) <= kDirectParts) {
-        if (tid >= VECS) return;
-#pragma unroll 1
-        for (int j = 0; j < pend_n; ++j) {
-            const Split it = j == 0 ? pend[0] : pend[1];
-            float M = -INFINITY, l = 0.f;
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int p0 = 0; p0 < it.nparts; p0 += kMergeBatch) {
-                float2 ml[kMergeBatch];
-                float4 v[kMergeBatch];
-#pragma unroll
-                for (int p = 0; p < kMergeBatch; ++p) {
-                    const bool in = p0 + p < it.nparts;
-                    const size_t slot = (size_t)it.slot0 + p0 + p;
-                    ml[p] = in ? __ldcg(reinterpret_cast<const float2 *>(a.part_ml) + slot * GP + eh) : make_float2(-INFINITY, 0.f);
-                    v[p] = in ? __ldcg(reinterpret_cast<const float4 *>(a.part_o) + slot * VECS + tid) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                float mb = M;
-#pragma unroll
-                for (int p = 0; p < kMergeBatch; ++p) mb = fmaxf(mb, ml[p].x);
-                const float f = fast_exp2(M - mb);
-                M = mb;
-                l *= f; x.x *= f; x.y *= f; x.z *= f; x.w *= f;
-#pragma unroll
-                for (int p = 0; p < kMergeBatch; ++p) {
-                    const float w = fast_exp2(ml[p].x - M);
-                    l = fmaf(w, ml[p].y, l);
-                    x.x = fmaf(w, v[p].x, x.x); x.y = fmaf(w, v[p].y, x.y); x.z = fmaf(w, v[p].z, x.z); x.w = fmaf(w, v[p].w, x.w);
-                }
-            }
-            write_row(it.out_base, x, 1.0f / l);
-        }
-        return;
-    }
-    // up to two merges, each in its own half of the ring, their first copies in flight together
-    const int cap = kRingBytes / pend_n;
+    // one 4-dimension piece of the group's outputs per thread.  Read are the parts of this CTA's own run of kMergeFan, as they
+    // are, and of every run before it the slot of its last part, which holds the run's sum; kMergeBatch of them at a time, in a
+    // fixed order whenever they come.  Lane p of a head's lanes has the (max, sum) of part p of a batch.
+    const int run0 = gather_part / kMergeFan * kMergeFan;        // first part of the own run
+    const int runs = gather_last ? gather_part / kMergeFan : 0;  // sums to read besides
+    const int n = runs + gather_part - run0;
     const bool mine = tid < VECS;
-    const int e = mine ? tid : 0, he = e / (kD / 4);
-    uint32_t merge_phase = 0;
-    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
-    float4 x[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-    int done[2] = {0, 0};
-    auto ml_area = [&](int j) -> uint32_t { return ((uint32_t)pend[j].nparts * GP * 8u + 127u) & ~127u; };
-    auto per_piece = [&](int j) -> int { return (cap - (int)ml_area(j)) / kPartBytes; };   // >= 6: at most 148 parts of 64-byte records
-    auto issue = [&](int j, int p0, uint32_t &bytes_out) {   // thread 0
-        const int np = min(per_piece(j), pend[j].nparts - p0);
-        const uint32_t bytes = (uint32_t)np * kPartBytes, ml_bytes = (uint32_t)pend[j].nparts * GP * 8u;
-        char *dst = ring + j * cap;
-        if (p0 == 0) bulk_load(dst, a.part_ml + (size_t)pend[j].slot0 * GP * 2, ml_bytes, &tail->merge_bar);
-        bulk_load(dst + ml_area(j), a.part_o + ((size_t)pend[j].slot0 + p0) * G * kD, bytes, &tail->merge_bar);
-        bytes_out += bytes + (p0 == 0 ? ml_bytes : 0u);
-    };
-    auto add_piece = [&](int j, int p0) {
-        const float2 *ml_s = reinterpret_cast<const float2 *>(ring + j * cap);
-        const float4 *po_s = reinterpret_cast<const float4 *>(ring + j * cap + ml_area(j));
-        const int np = min(per_piece(j), pend[j].nparts - p0);
-        if (p0 == 0)
-            for (int p = 0; p < pend[j].nparts; ++p) m[j] = fmaxf(m[j], ml_s[p * GP + he].x);
-#pragma unroll 4
-        for (int p = 0; p < np; ++p) {
-            const float2 ml = ml_s[(p0 + p) * GP + he];
-            const float w = fast_exp2(ml.x - m[j]);
-            const float4 v = po_s[p * VECS + e];
-            l[j] = fmaf(w, ml.y, l[j]);
-            x[j].x = fmaf(w, v.x, x[j].x);
-            x[j].y = fmaf(w, v.y, x[j].y);
-            x[j].z = fmaf(w, v.z, x[j].z);
-            x[j].w = fmaf(w, v.w, x[j].w);
-        }
-        done[j] = p0 + np;
-    };
-    while (true) {
-        bool more = false;
+    const int piece = mine ? tid : 0;
+    for (int p0 = 0; p0 < n; p0 += kMergeBatch) {
+        const int np = min(kMergeBatch, n - p0);
+        auto slot_of = [&](int i) -> int {   // of the i-th part to read; always an earlier CTA's
+            const int at = gather_first + (i < runs ? i * kMergeFan + kMergeFan - 1 : run0 + i - runs);
+            return 2 * (ARB_IN_RANGE(a.status, at, cta) ? at : 0) + (at == gather_first);
+        };
+        float4 v[kMergeBatch];
+        float2 ml = make_float2(-INFINITY, 0.f);
+        const bool has_ml = mine && lane % kLph < np;
+        float2 *ml_at = reinterpret_cast<float2 *>(a.part_ml) + (size_t)slot_of(has_ml ? p0 + lane % kLph : p0) * kMaxGroup + piece / kLph;
+        float4 *o_at = reinterpret_cast<float4 *>(a.part_o) + piece;
+        unsigned missing = mine ? (1u << np) - 1u : 0u;
+        bool ml_missing = has_ml;
+        long long t0 = 0;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) more = more || (j < pend_n && done[j] < pend[j].nparts);
-        if (!more) break;
-        if (tid == 0) {
-            asm volatile("fence.proxy.async;" ::: "memory");   // the partials were written by ordinary stores
-            uint32_t bytes = 0;
-            // the expected bytes are known before the copies are issued: same arithmetic as issue()
+        for (int p = 0; p < kMergeBatch; ++p) v[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        while (true) {
+            const unsigned before = missing;
+            if (ml_missing) ml = load_slot2(ml_at);
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
-                if (j < pend_n && done[j] < pend[j].nparts) {
-                    const int np = min(per_piece(j), pend[j].nparts - done[j]);
-                    bytes += (uint32_t)np * kPartBytes + (done[j] == 0 ? (uint32_t)pend[j].nparts * GP * 8u : 0u);
+            for (int p = 0; p < kMergeBatch; ++p)
+                if (missing >> p & 1u) v[p] = load_slot4(o_at + (size_t)slot_of(p0 + p) * VECS);
+            ml_missing = ml_missing && (is_empty(ml.x) || is_empty(ml.y));
+#pragma unroll
+            for (int p = 0; p < kMergeBatch; ++p)
+                if ((missing >> p & 1u) && !any_empty(v[p])) missing &= ~(1u << p);
+            if (!__any_sync(0xffffffffu, ml_missing || missing != 0u)) break;
+            if (merges_only && __all_sync(0xffffffffu, missing == before)) __nanosleep(200);
+            if (t0 == 0) t0 = clock64();
+            if (*abort || clock64() - t0 > kWaitCycles) {   // give up, like every other wait
+                if (!*abort) {
+                    *abort = 1;
+                    atomicOr(a.status, (uint32_t)ARB_DEV_WAIT_TIMEOUT);
                 }
-            mbar_arrive_expect_tx(&tail->merge_bar, bytes);
-            uint32_t issued = 0;
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-                if (j < pend_n && done[j] < pend[j].nparts) issue(j, done[j], issued);
+                break;
+            }
         }
         __syncwarp();
-        mbar_wait(&tail->merge_bar, merge_phase & 1u, abort, a.status);
-        ++merge_phase;
+        // read: empty again for the next call
+        const float e = __uint_as_float(kEmpty);
+        if (has_ml) store_slot2(ml_at, make_float2(e, e));
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-            if (j < pend_n && done[j] < pend[j].nparts) add_piece(j, done[j]);
-        named_barrier(1, kCT);   // everyone is done with the ring before the next pieces overwrite it
-    }
+        for (int p = 0; p < kMergeBatch; ++p)
+            if (mine && p < np) store_slot4(o_at + (size_t)slot_of(p0 + p) * VECS, make_float4(e, e, e, e));
+        float mb = fmaxf(own_m, ml.x);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        if (j < pend_n && mine) write_row(pend[j].out_base, x[j], 1.0f / l[j]);
+        for (int off = 1; off < kLph; off <<= 1) mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, off));
+        const float f = fast_exp2(own_m - mb), w = fast_exp2(ml.x - mb);
+        float l = w * ml.y;
+#pragma unroll
+        for (int off = 1; off < kLph; off <<= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+        own_m = mb;
+        own_l = fmaf(own_l, f, l);
+        own.x *= f; own.y *= f; own.z *= f; own.w *= f;
+#pragma unroll
+        for (int p = 0; p < kMergeBatch; ++p) {
+            const float wp = __shfl_sync(0xffffffffu, w, (lane / kLph) * kLph + p);   // 0 where the batch has no part p
+            own.x = fmaf(wp, v[p].x, own.x); own.y = fmaf(wp, v[p].y, own.y); own.z = fmaf(wp, v[p].z, own.z); own.w = fmaf(wp, v[p].w, own.w);
+        }
     }
+    if (!mine) return;
+    if (gather_last) write_row(gather_out, own, 1.0f / own_l);
+    else publish(own, own_m, own_l, gather_part);
 }
 
 // Ring depth: 32 stages, 128 KB of tiles in flight per SM with one CTA per SM.  A 16-stage ring with room for two
@@ -1219,7 +1299,8 @@ arb_status launch_g(Ctx *ctx, const StepArgs &a, int kv, int head_dim, const CUt
 
 }  // namespace
 
-size_t decode_step_hint_bytes(int num_sms) { return sizeof(int) * (size_t)num_sms * kHintStride; }
+// every word kEmpty between calls: memset to 0xff
+size_t decode_step_slot_bytes(int num_sms) { return sizeof(float) * 2 * (size_t)num_sms * kMaxGroup * (kD + 2); }
 
 bool decode_step_supported(const arb_attn_params &p) {
     const int g = p.num_q_heads / p.num_kv_heads;
@@ -1261,12 +1342,6 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
             return ARB_ERR_CUDA;
     }
     const int g = p.num_q_heads / p.num_kv_heads;
-    const int gp = (g + 3) / 4 * 4;
-    const size_t slots = (size_t)p.batch * p.num_kv_heads + (size_t)ctx->num_sms;
-    const size_t part_o_floats = (slots * g * p.head_dim + 63) & ~size_t(63);
-    const size_t bytes = (part_o_floats + slots * gp * 2) * sizeof(float);
-    if (bytes > ctx->workspace_bytes) return ARB_ERR_WORKSPACE;
-    note_unnumbered_decode(ctx, bytes);   // region 0 of the workspace: this kernel waits for its predecessor first
     StepArgs a;
     a.q = static_cast<const char *>(q);
     a.k_new = static_cast<const char *>(k_new);
@@ -1277,23 +1352,20 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
     a.seq_lens = seq_lens;
     a.q_lens = q_lens;
     a.out = static_cast<char *>(out);
-    a.part_o = reinterpret_cast<float *>(ctx->workspace);
-    a.part_ml = a.part_o + part_o_floats;
-    a.counters = ctx->rot;                                                       // [kRotCounters]
+    a.part_o = ctx->step_slots;
+    a.part_ml = a.part_o + 2 * (size_t)ctx->num_sms * kMaxGroup * kD;
+    a.ticket = reinterpret_cast<unsigned *>(ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 5);
     a.lens_counter = ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 4;
-    a.hint = ctx->step_hint;
-    a.hint_tag = ((int)(((uint32_t)p.batch * 2654435761u) ^ ((uint32_t)p.num_kv_heads * 40503u) ^
-                       ((uint32_t)p.num_pages * 2246822519u) ^ ((uint32_t)p.max_pages_per_seq * 3266489917u)) & ~3) | (beside ? 3 : 1);   // (another cut: another record)
+    // (a guessed length is at most what the table holds: its pages must be countable)
+    a.guess = (long long)p.batch * p.num_kv_heads * p.max_pages_per_seq < (1ll << 30) ? 1 : 0;
     a.status = ctx->status;
     a.batch = p.batch;
     a.beside = beside ? 1 : 0;
-    a.grid_inv = (uint32_t)((1ull << 32) / (unsigned)ctx->num_sms) + 1u;
     a.Hq = p.num_q_heads;
     a.Hkv = p.num_kv_heads;
     a.num_pages = p.num_pages;
     a.max_pages = p.max_pages_per_seq;
     a.whole_rows = whole_rows ? 1 : 0;
-    a.slots = (int)slots;
     a.rows = p.total_q;
     a.boundary_pct = ctx->step_boundary_pct;
     a.min_chunk = ctx->step_min_chunk;

@@ -522,3 +522,42 @@ def test_kv_append_i4_prefill_then_tokens():
     assert c.poll_status() == binding.DEV_BAD_SEQ_LEN
     for t_, b_ in zip(pools + [d.seq_lens], before):
         assert torch.equal(t_.view(torch.uint8) if t_.dtype == torch.float32 else t_, b_.view(torch.uint8) if b_.dtype == torch.float32 else b_)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,D", [(5, 12, 2, 128), (36, 6, 1, 128), (3, 8, 2, 64)])
+def test_token_right_behind_a_kernel_that_moves_the_lengths(B, Hq, Hkv, D):
+    """The token's kernel plans from the lengths it finds before the rollback in front of it has ended, and must notice that they
+    moved: by whole pages, within a page, to nothing, not at all."""
+    c = H.ctx()
+    sl = [(37 * b * b + 300 * b) % 2600 for b in range(B)]
+    inp = wl.small_attn_case(B, Hq, Hkv, D, BF, sl, [1] * B, seed=91 + B, extra_tokens=100)
+    k_new, v_new = _new_rows(inp, B, 9100 + Hq)
+    ok, ov, osl, _ = oracle.kv_append(k_new, v_new, inp.block_table, inp.seq_lens, inp.q_lens, inp.k_pages, inp.v_pages)
+    ref, _ = oracle.attn(inp.q, ok, ov, inp.block_table, osl, inp.q_lens)
+    d, kd, vd = inp.to("cuda"), k_new.cuda(), v_new.cuda()
+    steps = [[(b * 7 + 13 * r) % 97 if r else 0 for b in range(B)] for r in range(6)]
+    lens = [torch.tensor([s + n for s, n in zip(sl, step)], dtype=torch.int32, device="cuda") for step in steps]
+    step_t = [torch.tensor(step, dtype=torch.int32, device="cuda") for step in steps]
+    all_of_them = torch.ones(B, dtype=torch.uint8, device="cuda")
+    outs = [torch.full_like(d.q, float("nan")) for _ in steps]
+    torch.cuda.synchronize()
+    for ln, n, out in zip(lens, step_t, outs):
+        c.rollback(ln, n, all_of_them)
+        c.decode_step(d.q, kd, vd, d.k_pages, d.v_pages, d.block_table, ln, d.q_lens, out=out)
+    assert c.poll_status() == 0
+    for ln, out in zip(lens, outs):
+        assert np.array_equal(ln.cpu().numpy(), osl)
+        assert _same_bits(out, outs[0])
+    assert _same_bits(d.k_pages, ok) and _same_bits(d.v_pages, ov)
+    H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,D,L", [(37, 4, 1, 128, 900), (38, 4, 1, 128, 900),   # the most items with a merger each, one more
+                                          (1, 2, 1, 128, 33 * 16 * 16), (1, 7, 1, 64, 40000),   # runs of parts: 33 parts, 147
+                                          (2, 16, 2, 128, 20000), (4, 6, 1, 64, 8000)])
+def test_split_items_merge(B, Hq, Hkv, D, L):
+    sl = [L - 17 * b for b in range(B)]
+    inp = wl.small_attn_case(B, Hq, Hkv, D, BF, sl, [1] * B, seed=17 + B, extra_tokens=4)
+    k_new, v_new = _new_rows(inp, B, 1700 + Hq)
+    for _ in range(2):   # (the exchange slots are as they were)
+        _check(*_run(H.ctx(), inp, k_new, v_new), BF, 3e-3)
