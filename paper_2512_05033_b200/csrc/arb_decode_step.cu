@@ -78,10 +78,10 @@ constexpr int kNT = 32 * (kCW + 3);
 constexpr uint32_t kEmpty = 0xffffffffu;
 // A call of few items gives each a CTA that streams nothing and merges it: the others leave when they have stored their parts,
 // the next kernel's CTAs come up in their places, and where they would come late, behind a merge, there are the next
-// kernel's mergers, which have time.  Up to a kMergerShare-th of the CTAs (the SMs missed by the stream cost little, it is
-// bound by the memory): draft-shaped token (16 items) 11.0 -> 10.85 us, over E4M3 codes 10.0 -> 9.6 us, 8 x 8 heads (64
-// items, so not) the same.
-constexpr int kMergerShare = 4;
+// kernel's mergers, which have time: draft-shaped token (16 items) 11.0 -> 10.85 us, over E4M3 codes 10.0 -> 9.6 us.  Up to a
+// kMergerShare-th of the CTAs, and only where one of the others then streams at most kMergerPages more: that is a microsecond or
+// so, what a merger saves (with more, 32 items of 16 sequences of 2k to 8k over E4M3 codes 14 -> 15 us, 30 of 28k 69.5 -> 70.1 us).
+constexpr int kMergerShare = 4, kMergerPages = 5;
 // What a boundary costs is time (the warps meet, a second arrival, perhaps a second merge), a few microseconds
 // whatever the call's size: as pages it is the CTA's even share, but no more than this many.
 constexpr int kBoundaryCap = 32;
@@ -402,7 +402,10 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         }
         mbar_fence_init();
     }
-    if (!a.guess) wait_for_predecessor();
+    if (!a.guess) {
+        wait_for_predecessor();
+        if (a.beside) let_successor_start();   // it does not wait for this kernel, but it may read what the predecessor wrote
+    }
     for (int b = tid; b < B; b += kNT) {
         raw_n[b] = load_now(a.q_lens + b);
         raw_len[b] = load_now(a.seq_lens + b);
@@ -432,7 +435,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             const float mine = kBesideWeight * (float)total;
             ctas = min(ctas, max(4, __float2int_ru((float)ctas * __fdividef(mine, mine + chunks + 1.f))));
         }
-        pl.mergers = !a.beside && items * kMergerShare <= ctas;
+        pl.mergers = !a.beside && items * kMergerShare <= ctas && (long long)(ctas - items) * kMergerPages >= (long long)total / ctas * items;
         if (pl.mergers) ctas -= items;
         pl.stream = ctas;
         const int even = max(a.min_chunk, per_cta(total));
@@ -581,7 +584,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     // look-ups' table entries again and tells everyone whether all of it still holds.  Until then nothing has been written
     // and only tiles and q rows were read, in bounds whatever the guess.  Where something differs (lengths that the kernel right
     // in front moves, as a rollback does) the copies are waited for, the barriers made new, and the second round plans from
-    // what is final.  Three dependent round trips (lengths, table, tile) and the plan become one behind the predecessor's end:
+    // what is final.  Without a cache write the copies wait for the comparison: what precedes such a call is often the append that
+    // moved the lengths.  Three dependent round trips (lengths, table, tile) and the plan become one behind the predecessor's end:
     // tokens of one sequence of 256 / 2048 / 32768 tokens 7.3 / 8.1 / 15.7 -> 6.1 / 6.9 / 13.4 us, draft-shaped 12.4 -> 10.7 us
     // with the mergers.
 #pragma unroll 1
@@ -606,43 +610,51 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         if (guess && warp == kVerifyWarp) {
             bool differs = lane < nflat && load_now(entry) != page_next;
 #pragma unroll 4
-            for (int b = lane; b < B; b += 32)
-                differs |= load_now(a.q_lens + b) != raw_n[b] || load_now(a.seq_lens + b) != raw_len[b];
+            for (int b = lane; b < B; b += 32) {   // (what has moved goes where the next plan reads it)
+                const int n = load_now(a.q_lens + b), L0 = load_now(a.seq_lens + b);
+                if (n != raw_n[b] || L0 != raw_len[b]) {
+                    differs = true;
+                    raw_n[b] = n;
+                    raw_len[b] = L0;
+                }
+            }
             differs = __any_sync(0xffffffffu, differs);
             if (lane == 0) {
                 tail->differs = differs;
                 mbar_arrive(&tail->verdict);
             }
         }
+        auto right = [&]() -> bool {
+            mbar_wait(&tail->verdict, 0, &tail->abort, a.status);
+            return !*(volatile int *)&tail->differs;
+        };
         const bool first_copy = (warp == kProdWarp || warp == kProdWarp + 1) && lane < min(nflat, kBatch);
-        if (first_copy && ARB_IN_RANGE(a.status, row_next, (long long)a.num_pages * Hkv * kPage)) issue(2u * lane + (uint32_t)pw, row_next);
-        if (warp < kCW) {
-            cur = ends[0];
-            seq_at = seq0;
-            have = next_segment(cur, ends[1], seq_at, pl, s);
-            if (have) load_q(s, qb);
-        }
-        if (!guess) break;
-        mbar_wait(&tail->verdict, 0, &tail->abort, a.status);
-        if (!*(volatile int *)&tail->differs) break;
-        if (first_copy) mbar_wait(&tail->full[2 * lane + pw], 0, &tail->abort, a.status);
-        __syncthreads();
-        if (tid == 0) {
-            for (int st = 0; st < STAGES; ++st) {
-                mbar_inval(&tail->full[st]);
-                mbar_inval(&tail->empty[st]);
-                mbar_init(&tail->full[st], 1);
-                mbar_init(&tail->empty[st], 1);
+        const bool sure = !guess || (!APPEND && right());
+        if (APPEND || sure) {
+            if (first_copy && ARB_IN_RANGE(a.status, row_next, (long long)a.num_pages * Hkv * kPage)) issue(2u * lane + (uint32_t)pw, row_next);
+            if (warp < kCW) {
+                cur = ends[0];
+                seq_at = seq0;
+                have = next_segment(cur, ends[1], seq_at, pl, s);
+                if (have) load_q(s, qb);
             }
-            mbar_fence_init();
         }
-        for (int b = tid; b < B; b += kNT) {
-            raw_n[b] = load_now(a.q_lens + b);
-            raw_len[b] = load_now(a.seq_lens + b);
-        }
+        if (sure || (APPEND && right())) break;
+        if (APPEND && first_copy) mbar_wait(&tail->full[2 * lane + pw], 0, &tail->abort, a.status);
         __syncthreads();
+        if constexpr (APPEND) {
+            if (tid == 0) {
+                for (int st = 0; st < STAGES; ++st) {
+                    mbar_inval(&tail->full[st]);
+                    mbar_inval(&tail->empty[st]);
+                    mbar_init(&tail->full[st], 1);
+                    mbar_init(&tail->empty[st], 1);
+                }
+                mbar_fence_init();
+            }
+            __syncthreads();
+        }
     }
-    if (a.beside) let_successor_start();   // the successor does not wait for this kernel, but it may read what the predecessor wrote
 
     if (warp == kAuxWarp) {
         // ================================ bookkeeping warp ==========================================
@@ -1209,7 +1221,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             for (int p = 0; p < kMergeBatch; ++p)
                 if ((missing >> p & 1u) && !any_empty(v[p])) missing &= ~(1u << p);
             if (!__any_sync(0xffffffffu, ml_missing || missing != 0u)) break;
-            if (merges_only && __all_sync(0xffffffffu, missing == before)) __nanosleep(200);
+            if (__all_sync(0xffffffffu, missing == before)) __nanosleep(merges_only ? 200 : 100);
             if (t0 == 0) t0 = clock64();
             if (*abort || clock64() - t0 > kWaitCycles) {   // give up, like every other wait
                 if (!*abort) {
@@ -1356,8 +1368,9 @@ arb_status launch_decode_step(Ctx *ctx, const arb_attn_params &p, const void *q,
     a.part_ml = a.part_o + 2 * (size_t)ctx->num_sms * kMaxGroup * kD;
     a.ticket = reinterpret_cast<unsigned *>(ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 5);
     a.lens_counter = ctx->rot + (size_t)kRotSets * kRotCounters + kRotSets + 4;
-    // (a guessed length is at most what the table holds: its pages must be countable)
-    a.guess = (long long)p.batch * p.num_kv_heads * p.max_pages_per_seq < (1ll << 30) ? 1 : 0;
+    // (Beside chunks an append that moved the lengths is what precedes the call: its guess would always be wrong.  And a guessed
+    // length is at most what the table holds: its pages must be countable.)
+    a.guess = !beside && (long long)p.batch * p.num_kv_heads * p.max_pages_per_seq < (1ll << 30) ? 1 : 0;
     a.status = ctx->status;
     a.batch = p.batch;
     a.beside = beside ? 1 : 0;
