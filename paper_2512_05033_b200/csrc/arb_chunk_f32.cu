@@ -17,27 +17,26 @@ namespace arb {
 
 namespace {
 
-constexpr int kRows = 64;               // query rows of a tile
 constexpr int kKeys = 32;               // keys of a tile
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
-constexpr int kWarpRows = kRows / kWarps;
 constexpr int kMinUnits = 2;            // fewest key tiles worth giving a CTA
 constexpr int kCtasPerSm = 2;
 
-template <int D>
+// The kernel's template parameter R is the number of query rows of a tile: 64, 32 or 16, a warp owning R / 8 of them.
+template <int D, int R>
 struct Smem {
     static constexpr int kPitch = D + 4;    // neighbouring rows start 4 banks apart
-    float q[kRows][kPitch];
+    float q[R][kPitch];
     float k[2][kKeys][kPitch];
     float v[2][kKeys][kPitch];
-    float p[kWarps][kKeys][kWarpRows];
-    float row[kWarps][kWarpRows];           // a warp's rescale factors, then 1 / sum
+    float p[kWarps][kKeys][R / kWarps];
+    float row[kWarps][R / kWarps];           // a warp's rescale factors, then 1 / sum
     int last;
 };
 
-template <int D>
-__host__ __device__ constexpr size_t slot_floats() { return (size_t)kRows * D + 2 * kRows; }   // O [64][D], max [64], sum [64]
+template <int D, int R>
+__host__ __device__ constexpr size_t slot_floats() { return (size_t)R * D + 2 * R; }   // O [R][D], max [R], sum [R]
 
 struct F32Args {
     const float *q, *k_pages, *v_pages;
@@ -60,11 +59,16 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool real
 __device__ __forceinline__ int rows_there(const F32Args &a, int qrow0, int n) { return qrow0 < 0 ? 0 : max(0, min(n, a.rows - qrow0)); }
 
 // One row tile over the key tiles [t0, t1); nparts > 1: leaves partial `slot` and merges if it is the last to arrive.
-template <int D, int G>
-__device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, int t0, int t1, int qrow0, int nparts,
+template <int D, int G, int kRows>
+__device__ void row_tile(const F32Args &a, Smem<D, kRows> &s, int b, int kvh, int rt, int t0, int t1, int qrow0, int nparts,
                          long long slot, long long slot_first, int item) {
     constexpr int kVecs = D / 4;
-    constexpr int kLaneRows = D == 128 ? 8 : 4;     // rows of O a lane holds, 4 dimensions each
+    constexpr int kWarpRows = kRows / kWarps;
+    constexpr int kLaneRows = D == 128 ? kWarpRows : kWarpRows / 2;   // rows of O a lane holds, 4 dimensions each
+    constexpr int kRowLanes = kWarpRows < 4 ? 16 : 8;                 // S: lanes of a row,
+    constexpr int kSRows = kWarpRows < 4 ? 1 : kWarpRows / 4;         // a lane's rows, 32 / kRowLanes apart,
+    constexpr int kSKeys = kKeys / kRowLanes;                         // and its keys, kRowLanes apart
+    constexpr int kRowStep = 32 / kRowLanes;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = a.q_lens[b], L = a.seq_lens[b], rows = n * G, r_begin = rt * kRows;
     const int there = rows_there(a, qrow0, n) * G;   // rows that q and out have
@@ -76,16 +80,6 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
     };
     auto limit_of = [&](int i) { return L - n + min(r_begin + i, rows - 1) / G + 1; };   // keys row i sees
 
-    __syncthreads();   // the tile before this one is done with shared memory
-    for (int i = tid; i < kRows * kVecs; i += kThreads) {
-        const int r = i / kVecs, c = i - r * kVecs;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r_begin + r < there) {
-            x = __ldg(reinterpret_cast<const float4 *>(a.q + row_of(r)) + c);
-            x.x *= a.scale_log2; x.y *= a.scale_log2; x.z *= a.scale_log2; x.w *= a.scale_log2;
-        }
-        *reinterpret_cast<float4 *>(&s.q[r][c * 4]) = x;
-    }
     // Keys past the last visible one are zero-filled, not read: stale slots must not reach a product.
     auto load_tile = [&](int t, int st) {
 #pragma unroll
@@ -104,18 +98,33 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    const int rg = lane >> 3, kg = lane & 7;                      // S: rows rg, rg + 4; keys kg, kg + 8, ...
-    const int orow = D == 128 ? 0 : (lane >> 4) * 4;              // O: first row ...
+    const int rg = lane / kRowLanes, kg = lane % kRowLanes;
+    const int orow = D == 128 ? 0 : (lane >> 4) * kLaneRows;      // O: first row ...
     const int odim = (D == 128 ? lane : (lane & 15)) * 4;         // ... and first dimension of this lane
     const bool warp_ok = r_begin + warp * kWarpRows < rows;
-    const int lim[2] = {limit_of(warp * kWarpRows + rg), limit_of(warp * kWarpRows + rg + 4)};
+    int lim[kSRows];
+#pragma unroll
+    for (int i = 0; i < kSRows; ++i) lim[i] = limit_of(warp * kWarpRows + rg + kRowStep * i);
     const int lim_min = limit_of(warp * kWarpRows);
-    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+    float m[kSRows], l[kSRows];
+#pragma unroll
+    for (int i = 0; i < kSRows; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
     float o[kLaneRows][4];
 #pragma unroll
     for (int r = 0; r < kLaneRows; ++r) { o[r][0] = o[r][1] = o[r][2] = o[r][3] = 0.f; }
 
-    if (t0 < t1) load_tile(t0, 0);
+    __syncthreads();   // the tile before this one is done with shared memory
+    if (t0 < t1) load_tile(t0, 0);   // (the keys' way is the longer one: table, then rows)
+#pragma unroll
+    for (int i = tid; i < kRows * kVecs; i += kThreads) {
+        const int r = i / kVecs, c = i - r * kVecs;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r_begin + r < there) {
+            x = __ldg(reinterpret_cast<const float4 *>(a.q + row_of(r)) + c);
+            x.x *= a.scale_log2; x.y *= a.scale_log2; x.z *= a.scale_log2; x.w *= a.scale_log2;
+        }
+        *reinterpret_cast<float4 *>(&s.q[r][c * 4]) = x;
+    }
     for (int t = t0; t < t1; ++t) {
         const int st = (t - t0) & 1;
         if (t + 1 < t1) {
@@ -126,39 +135,41 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
         }
         __syncthreads();
         if (warp_ok) {
-            float sc[2][4] = {};
-            const float *q0 = s.q[warp * kWarpRows + rg], *q1 = s.q[warp * kWarpRows + rg + 4];
+            float sc[kSRows][kSKeys] = {};
 #pragma unroll 4
             for (int c = 0; c < D; c += 4) {
-                const float4 a0 = *reinterpret_cast<const float4 *>(q0 + c), a1 = *reinterpret_cast<const float4 *>(q1 + c);
+                float4 x[kSRows];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float4 kv = *reinterpret_cast<const float4 *>(&s.k[st][kg + 8 * j][c]);
-                    sc[0][j] = fmaf(a0.x, kv.x, fmaf(a0.y, kv.y, fmaf(a0.z, kv.z, fmaf(a0.w, kv.w, sc[0][j]))));
-                    sc[1][j] = fmaf(a1.x, kv.x, fmaf(a1.y, kv.y, fmaf(a1.z, kv.z, fmaf(a1.w, kv.w, sc[1][j]))));
+                for (int i = 0; i < kSRows; ++i) x[i] = *reinterpret_cast<const float4 *>(&s.q[warp * kWarpRows + rg + kRowStep * i][c]);
+#pragma unroll
+                for (int j = 0; j < kSKeys; ++j) {
+                    const float4 kv = *reinterpret_cast<const float4 *>(&s.k[st][kg + kRowLanes * j][c]);
+#pragma unroll
+                    for (int i = 0; i < kSRows; ++i)
+                        sc[i][j] = fmaf(x[i].x, kv.x, fmaf(x[i].y, kv.y, fmaf(x[i].z, kv.z, fmaf(x[i].w, kv.w, sc[i][j]))));
                 }
             }
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
+            for (int i = 0; i < kSRows; ++i) {
                 float mx = -INFINITY;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (t * kKeys + kg + 8 * j >= lim[i]) sc[i][j] = -INFINITY;
+                for (int j = 0; j < kSKeys; ++j) {
+                    if (t * kKeys + kg + kRowLanes * j >= lim[i]) sc[i][j] = -INFINITY;
                     mx = fmaxf(mx, sc[i][j]);
                 }
 #pragma unroll
-                for (int off = 1; off < 8; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                for (int off = 1; off < kRowLanes; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
                 const float mn = fmaxf(m[i], mx), base = mn == -INFINITY ? 0.f : mn;   // (a part may hold no key of a row)
                 const float f = fast_exp2(m[i] - base);
                 m[i] = mn;
                 l[i] *= f;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < kSKeys; ++j) {
                     const float p = fast_exp2(sc[i][j] - base);
                     l[i] += p;
-                    s.p[warp][kg + 8 * j][rg + 4 * i] = p;
+                    s.p[warp][kg + kRowLanes * j][rg + kRowStep * i] = p;
                 }
-                if (kg == 0) s.row[warp][rg + 4 * i] = f;
+                if (kg == 0) s.row[warp][rg + kRowStep * i] = f;
             }
             __syncwarp();
 #pragma unroll
@@ -172,8 +183,18 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
                     const float4 v = *reinterpret_cast<const float4 *>(&s.v[st][key][odim]);
                     float p[kLaneRows];
 #pragma unroll
-                    for (int r = 0; r < kLaneRows; r += 4)
-                        *reinterpret_cast<float4 *>(p + r) = *reinterpret_cast<const float4 *>(&s.p[warp][key][orow + r]);
+                    for (int r = 0; r < kLaneRows; r += 4) {
+                        const float *from = &s.p[warp][key][orow + r];
+                        if constexpr (kLaneRows >= 4) {
+                            const float4 x = *reinterpret_cast<const float4 *>(from);
+                            p[r] = x.x; p[r + 1] = x.y; p[r + 2] = x.z; p[r + 3] = x.w;
+                        } else if constexpr (kLaneRows == 2) {
+                            const float2 x = *reinterpret_cast<const float2 *>(from);
+                            p[0] = x.x; p[1] = x.y;
+                        } else {
+                            p[0] = *from;
+                        }
+                    }
 #pragma unroll
                     for (int r = 0; r < kLaneRows; ++r) {
                         o[r][0] = fmaf(p[r], v.x, o[r][0]); o[r][1] = fmaf(p[r], v.y, o[r][1]);
@@ -198,12 +219,15 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
     }
 
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kSRows; ++i) {
 #pragma unroll
-        for (int off = 1; off < 8; off <<= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+        for (int off = 1; off < kRowLanes; off <<= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
     }
     if (nparts == 1) {
-        if (kg == 0) { s.row[warp][rg] = 1.0f / l[0]; s.row[warp][rg + 4] = 1.0f / l[1]; }
+        if (kg == 0) {
+#pragma unroll
+            for (int i = 0; i < kSRows; ++i) s.row[warp][rg + kRowStep * i] = 1.0f / l[i];
+        }
         __syncwarp();
 #pragma unroll
         for (int r = 0; r < kLaneRows; ++r) {
@@ -216,16 +240,16 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
         }
         return;
     }
-    float *po = a.partials + (size_t)slot * slot_floats<D>();
+    float *po = a.partials + (size_t)slot * slot_floats<D, kRows>();
     if (ARB_IN_RANGE(a.status, slot, a.slots)) {
 #pragma unroll
         for (int r = 0; r < kLaneRows; ++r)
             *reinterpret_cast<float4 *>(po + (warp * kWarpRows + orow + r) * D + odim) = make_float4(o[r][0], o[r][1], o[r][2], o[r][3]);
         if (kg == 0) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                po[kRows * D + warp * kWarpRows + rg + 4 * i] = m[i];
-                po[kRows * D + kRows + warp * kWarpRows + rg + 4 * i] = l[i];
+            for (int i = 0; i < kSRows; ++i) {
+                po[kRows * D + warp * kWarpRows + rg + kRowStep * i] = m[i];
+                po[kRows * D + kRows + warp * kWarpRows + rg + kRowStep * i] = l[i];
             }
         }
     }
@@ -239,41 +263,61 @@ __device__ void row_tile(const F32Args &a, Smem<D> &s, int b, int kvh, int rt, i
     __syncthreads();
     if (!s.last) return;
     // m = max_p m_p, w_p = 2^(m_p - m), out = sum_p w_p o_p / sum_p w_p l_p; part 0 sees key 0: m is finite
-    const float *p0 = a.partials + (size_t)slot_first * slot_floats<D>();
-    const int i = tid / (kThreads / kRows), c0 = tid % (kThreads / kRows);   // four threads per row
+    const float *p0 = a.partials + (size_t)slot_first * slot_floats<D, kRows>();
+    constexpr int kRowThreads = kThreads / kRows, kPieces = kVecs / kRowThreads;   // threads of a row, and what each of them merges
+    constexpr int kAtOnce = kPieces > 2 ? 4 : kPieces > 1 ? 8 : 16;   // parts whose loads are in flight together
+    const int i = tid / kRowThreads, c0 = tid % kRowThreads;
     if (r_begin + i >= there || !ARB_IN_RANGE(a.status, qrow0 + (r_begin + i) / G, a.rows)) return;
-    float M = -INFINITY;
-#pragma unroll 8
-    for (int p = 0; p < nparts; ++p) M = fmaxf(M, __ldcg(p0 + p * slot_floats<D>() + kRows * D + i));
-    float4 acc[kVecs / 4];
+    float M = -INFINITY, sum = 0.f;
+    float4 acc[kPieces];
 #pragma unroll
-    for (int c = 0; c < kVecs / 4; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    float sum = 0.f;
-#pragma unroll 4
-    for (int p = 0; p < nparts; ++p) {
-        const float *pp = p0 + p * slot_floats<D>();
-        const float w = fast_exp2(__ldcg(pp + kRows * D + i) - M);
-        sum = fmaf(w, __ldcg(pp + kRows * D + kRows + i), sum);
+    for (int c = 0; c < kPieces; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int p = 0; p < nparts; p += kAtOnce) {
+        float pm[kAtOnce], pl[kAtOnce];
+        float4 x[kAtOnce][kPieces];
 #pragma unroll
-        for (int c = 0; c < kVecs / 4; ++c) {
-            const float4 x = __ldcg(reinterpret_cast<const float4 *>(pp + i * D) + c0 + 4 * c);
-            acc[c].x = fmaf(w, x.x, acc[c].x); acc[c].y = fmaf(w, x.y, acc[c].y);
-            acc[c].z = fmaf(w, x.z, acc[c].z); acc[c].w = fmaf(w, x.w, acc[c].w);
+        for (int j = 0; j < kAtOnce; ++j) {
+            const float *pp = p0 + (size_t)(p + j) * slot_floats<D, kRows>();
+            const bool in = p + j < nparts;
+            pm[j] = in ? __ldcg(pp + kRows * D + i) : -INFINITY;
+            pl[j] = in ? __ldcg(pp + kRows * D + kRows + i) : 0.f;
+#pragma unroll
+            for (int c = 0; c < kPieces; ++c)
+                x[j][c] = in ? __ldcg(reinterpret_cast<const float4 *>(pp + i * D) + c0 + kRowThreads * c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        float mx = M;
+#pragma unroll
+        for (int j = 0; j < kAtOnce; ++j) mx = fmaxf(mx, pm[j]);
+        const float base = mx == -INFINITY ? 0.f : mx, f = fast_exp2(M - base);   // (the first parts may hold no key of the row)
+        M = mx;
+        sum *= f;
+#pragma unroll
+        for (int c = 0; c < kPieces; ++c) { acc[c].x *= f; acc[c].y *= f; acc[c].z *= f; acc[c].w *= f; }
+#pragma unroll
+        for (int j = 0; j < kAtOnce; ++j) {
+            const float w = fast_exp2(pm[j] - base);
+            sum = fmaf(w, pl[j], sum);
+#pragma unroll
+            for (int c = 0; c < kPieces; ++c) {
+                acc[c].x = fmaf(w, x[j][c].x, acc[c].x); acc[c].y = fmaf(w, x[j][c].y, acc[c].y);
+                acc[c].z = fmaf(w, x[j][c].z, acc[c].z); acc[c].w = fmaf(w, x[j][c].w, acc[c].w);
+            }
         }
     }
     const float inv = 1.0f / sum;
 #pragma unroll
-    for (int c = 0; c < kVecs / 4; ++c)
-        reinterpret_cast<float4 *>(a.out + row_of(i))[c0 + 4 * c] = make_float4(acc[c].x * inv, acc[c].y * inv, acc[c].z * inv, acc[c].w * inv);
+    for (int c = 0; c < kPieces; ++c)
+        reinterpret_cast<float4 *>(a.out + row_of(i))[c0 + kRowThreads * c] = make_float4(acc[c].x * inv, acc[c].y * inv, acc[c].z * inv, acc[c].w * inv);
 }
 
-template <int D, int G>
+template <int D, int G, int kRows>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 chunk_f32_kernel(const F32Args a) {
     extern __shared__ __align__(16) char smem[];
-    Smem<D> &s = *reinterpret_cast<Smem<D> *>(smem);
+    using Shared = Smem<D, kRows>;
+    Shared &s = *reinterpret_cast<Shared *>(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, B = a.batch, Hkv = a.Hkv;
-    long long *units = reinterpret_cast<long long *>(smem + ((sizeof(Smem<D>) + 15) & ~size_t(15)));   // [B + 1] key tiles before b
+    long long *units = reinterpret_cast<long long *>(smem + ((sizeof(Shared) + 15) & ~size_t(15)));   // [B + 1] key tiles before b
     int *items = reinterpret_cast<int *>(units + B + 1);   // [B + 1] row tiles before b (times kv heads)
     int *row0 = items + B + 1;                             // [B + 1] rows of q before b
     pdl_enter();
@@ -336,27 +380,40 @@ chunk_f32_kernel(const F32Args a) {
         const int t1 = whole ? kts : (int)min((long long)kts, t0 + (end - cur));
         const long long first = units[lo] + (long long)in_seq * kts;   // the row tile's place in the list
         const int c_first = (int)(first / chunk), nparts = whole ? 1 : (int)((first + kts - 1) / chunk) - c_first + 1;
-        row_tile<D, G>(a, s, lo, in_seq / rts, in_seq % rts, t0, t1, row0[lo], nparts, (long long)item + blockIdx.x,
+        row_tile<D, G, kRows>(a, s, lo, in_seq / rts, in_seq % rts, t0, t1, row0[lo], nparts, (long long)item + blockIdx.x,
                        (long long)item + c_first, item);
         cur += whole ? grid : t1 - t0;
     }
 }
 
-template <int D, int G>
-arb_status launch_one(Ctx *ctx, F32Args a, cudaStream_t stream) {
+template <int D, int G, int R>
+arb_status launch_rows(Ctx *ctx, F32Args a, cudaStream_t stream) {
+    using Shared = Smem<D, R>;
     auto bytes = [](int batch) {
-        return ((sizeof(Smem<D>) + 15) & ~size_t(15)) + (sizeof(long long) + 2 * sizeof(int)) * ((size_t)batch + 1);
+        return ((sizeof(Shared) + 15) & ~size_t(15)) + (sizeof(long long) + 2 * sizeof(int)) * ((size_t)batch + 1);
     };
     static bool attr_set[64] = {};
     if (!attr_set[ctx->device & 63]) {
-        if (cudaFuncSetAttribute(chunk_f32_kernel<D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kMaxBatch)) != cudaSuccess)
+        if (cudaFuncSetAttribute(chunk_f32_kernel<D, G, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kMaxBatch)) != cudaSuccess)
             return ARB_ERR_CUDA;
         attr_set[ctx->device & 63] = true;
     }
-    a.slots = (int)(ctx->chunk_ws_bytes / (slot_floats<D>() * sizeof(float)));
-    const cudaError_t err = launch_pdl(chunk_f32_kernel<D, G>, dim3(kCtasPerSm * ctx->num_sms), dim3(kThreads), bytes(a.batch), stream, a);
+    a.slots = (int)(ctx->chunk_ws_bytes / (slot_floats<D, R>() * sizeof(float)));
+    const cudaError_t err = launch_pdl(chunk_f32_kernel<D, G, R>, dim3(kCtasPerSm * ctx->num_sms), dim3(kThreads), bytes(a.batch), stream, a);
     ctx->launches++;
     return err == cudaSuccess ? ARB_OK : ARB_ERR_CUDA;
+}
+
+// Rows of a tile: 64, or 32 or 16 where the call is so small that the CTAs cannot all have work with more.  Smaller tiles read
+// the keys more often and take less time each, and so does the merge of their parts.  The host knows the rows and the most keys
+// that the table can hold.  F32FIGURES
+template <int D, int G>
+arb_status launch_one(Ctx *ctx, const F32Args &a, cudaStream_t stream) {
+    const long long most = (long long)a.Hkv * ((long long)a.rows * G / 64 + a.batch) * ((a.max_pages * (long long)kPage + kKeys - 1) / kKeys);
+    const long long room = (long long)kMinUnits * kCtasPerSm * ctx->num_sms;
+    if (4 * most <= room) return launch_rows<D, G, 16>(ctx, a, stream);
+    if (2 * most <= room) return launch_rows<D, G, 32>(ctx, a, stream);
+    return launch_rows<D, G, 64>(ctx, a, stream);
 }
 
 template <int D>

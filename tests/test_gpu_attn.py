@@ -694,6 +694,17 @@ def test_fp32_chunk_matches_oracle(case, ws):
     H.assert_close(out, ref, F32)
 
 
+@pytest.mark.parametrize("ws", [0, 1_300_000])
+@pytest.mark.parametrize("case", [
+    (8, 2, 128, [530, 17], [4, 17]),          # row tiles of 16 (a row of the table holds 36 pages): one full, five with one of 4 rows
+    (7, 1, 64, [300, 64, 2], [5, 3, 2]),      # ... of 16, g = 7: 35, 21 and 14 rows
+    (3, 1, 128, [2500], [11]),                # ... of 32 and 16 keys of the last key tile: 33 rows
+    (16, 2, 64, [1200], [6]),                 # ... of 32: 48 rows, long merges
+])
+def test_fp32_chunks_of_small_calls_match_oracle(case, ws):
+    test_fp32_chunk_matches_oracle(case, ws)
+
+
 BESIDE_CASES = [
     # (Hq, Hkv, D, seq_lens, q_lens): decode rows and chunks of one call side by side, the SMs shared by their work
     (12, 2, 128, [40, 5000], [1, 2]),                                  # next to no decode work: the fewest CTAs
