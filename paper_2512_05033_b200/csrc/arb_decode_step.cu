@@ -70,6 +70,9 @@ constexpr int kProdWarp = kCW;                // the producer warps, and behind 
 constexpr int kAuxWarp = kCW + 2;
 constexpr int kVerifyWarp = kCW - 1;          // the consumer warp that compares the guess (see decode_step_kernel) with what is final
 constexpr int kNT = 32 * (kCW + 3);
+// Named barriers: the consumers', and behind the comparison of the guess one for each kind of warp, so that none waits for
+// another's copies or prefetches (the consumers behind the producers' first copies: 4-bit tokens 10.8 -> 12.0 us).
+enum { kBarConsumers = 1, kBarConsumersTold = 3, kBarProducersTold = 4, kBarAuxTold = 5 };
 
 // The exchange of a split item's parts.  A slot is what one CTA hands on: the group's outputs and (max, sum) per head, every
 // 32-bit word of it kEmpty until it is stored, and kEmpty again once it has been read.  A NaN of a result never has these bits
@@ -139,8 +142,7 @@ template <int STAGES>
 struct Tail {
     uint64_t full[STAGES];
     uint64_t empty[STAGES];
-    uint64_t verdict;     // the guess has been compared with what is final
-    int differs;          // ... and this is what was found
+    int differs;          // the comparing warp's finding: the guess does not hold
     int abort;
     int ticket;
 };
@@ -272,10 +274,11 @@ __device__ __forceinline__ int fast_div(int a, int b) {
     return q;
 }
 
-// a / b where the quotient is a kv head index (small): a few subtractions beat any division
+// a / b where the quotient is a kv head index (small): a few subtractions beat any division.  (Whoever asks holds a page of the
+// sequence, so b > 0; the loop ends for any b.)
 __device__ __forceinline__ int small_div(int a, int b, int &rem) {
     int q = 0;
-    while (a >= b) { a -= b; ++q; }
+    while (a >= b && b > 0) { a -= b; ++q; }
     rem = a;
     return q;
 }
@@ -394,7 +397,6 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             mbar_init(&tail->empty[st], 1);
         }
         if (lane == 0) {
-            mbar_init(&tail->verdict, 1);
             tail->abort = 0;
             pref[0] = 0;
             row0[0] = 0;
@@ -582,7 +584,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     // `guess`: in the first round the plan comes from what lengths and table held before the predecessor was known to have
     // ended.  Behind the wait the first ring of tiles and the first q are asked for, while one warp reads lengths and the
     // look-ups' table entries again and tells everyone whether all of it still holds.  Until then nothing has been written
-    // and only tiles and q rows were read, in bounds whatever the guess.  Where something differs (lengths that the kernel right
+    // and only tiles and q rows were read, in bounds whatever the guess: every warp plans from the same guessed lengths, which
+    // are replaced once the block has met.  Where something differs (lengths that the kernel right
     // in front moves, as a rollback does) the copies are waited for, the barriers made new, and the second round plans from
     // what is final.  Without a cache write the copies wait for the comparison: what precedes such a call is often the append that
     // moved the lengths.  Three dependent round trips (lengths, table, tile) and the plan become one behind the predecessor's end:
@@ -607,29 +610,36 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             }
             wait_for_predecessor();
         }
+        bool differs = false;
+        int n_now = 0, len_now = 0;   // a batch of at most 32: what is final, of sequence `lane`
         if (guess && warp == kVerifyWarp) {
-            bool differs = lane < nflat && load_now(entry) != page_next;
+            differs = lane < nflat && load_now(entry) != page_next;
 #pragma unroll 4
-            for (int b = lane; b < B; b += 32) {   // (what has moved goes where the next plan reads it)
-                const int n = load_now(a.q_lens + b), L0 = load_now(a.seq_lens + b);
-                if (n != raw_n[b] || L0 != raw_len[b]) {
+            for (int b = lane; b < B; b += 32) {
+                n_now = load_now(a.q_lens + b);
+                len_now = load_now(a.seq_lens + b);
+                if (n_now != raw_n[b] || len_now != raw_len[b]) {
                     differs = true;
-                    raw_n[b] = n;
-                    raw_len[b] = L0;
+                    // What has moved goes where the next plan reads it.  Of a batch of more than 32 the plan above has read it in front
+                    // of barriers of the block; of a smaller one the other warps may not have read it yet.
+                    if (B > 32) { raw_n[b] = n_now; raw_len[b] = len_now; }
                 }
             }
             differs = __any_sync(0xffffffffu, differs);
-            if (lane == 0) {
-                tail->differs = differs;
-                mbar_arrive(&tail->verdict);
-            }
+            if (lane == 0) tail->differs = differs;
+            barrier_arrive(kBarProducersTold, 96);
+            barrier_arrive(kBarAuxTold, 64);
         }
-        auto right = [&]() -> bool {
-            mbar_wait(&tail->verdict, 0, &tail->abort, a.status);
-            return !*(volatile int *)&tail->differs;
+        // Whether the guess was wrong: all but the comparing warp wait for it.  (Barriers of the block's own warps, like
+        // __syncthreads: everyone is told the same.)
+        auto wrong = [&]() -> bool {
+            if (warp < kCW) named_barrier(kBarConsumersTold, kCT);
+            else if (warp == kAuxWarp) named_barrier(kBarAuxTold, 64);
+            else named_barrier(kBarProducersTold, 96);
+            return *(volatile int *)&tail->differs != 0;
         };
         const bool first_copy = (warp == kProdWarp || warp == kProdWarp + 1) && lane < min(nflat, kBatch);
-        const bool sure = !guess || (!APPEND && right());
+        const bool sure = !guess || (!APPEND && !wrong());
         if (APPEND || sure) {
             if (first_copy && ARB_IN_RANGE(a.status, row_next, (long long)a.num_pages * Hkv * kPage)) issue(2u * lane + (uint32_t)pw, row_next);
             if (warp < kCW) {
@@ -639,9 +649,10 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 if (have) load_q(s, qb);
             }
         }
-        if (sure || (APPEND && right())) break;
+        if (sure || (APPEND && !wrong())) break;
         if (APPEND && first_copy) mbar_wait(&tail->full[2 * lane + pw], 0, &tail->abort, a.status);
-        __syncthreads();
+        __syncthreads();   // every warp is done with the plan, and with the lengths it came from
+        if (B <= 32 && warp == kVerifyWarp && lane < B) { raw_n[lane] = n_now; raw_len[lane] = len_now; }
         if constexpr (APPEND) {
             if (tid == 0) {
                 for (int st = 0; st < STAGES; ++st) {
@@ -652,8 +663,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 }
                 mbar_fence_init();
             }
-            __syncthreads();
         }
+        __syncthreads();
     }
 
     if (warp == kAuxWarp) {
@@ -1126,7 +1137,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             if (h0 < G) { rec[16 + h0 * kOStride + d] = o[mt][0]; rec[16 + h0 * kOStride + d + 8] = o[mt][2]; }
             if (h1 < G) { rec[16 + h1 * kOStride + d] = o[mt][1]; rec[16 + h1 * kOStride + d + 8] = o[mt][3]; }
         }
-        named_barrier(1, kCT);
+        named_barrier(kBarConsumers, kCT);
         // A whole item goes to `out`, a part of a split one to the workspace, from the registers the merge leaves it in.
         const size_t out_base = ((size_t)qrow * a.Hq + s.kvh * G) * kD;
         const int part = cta - s.c_first;   // (of s.nparts)
@@ -1162,7 +1173,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             gather_last = last;
             gather_out = out_base;
         }
-        if (have_next) named_barrier(1, kCT);   // warp records are free for the next segment
+        if (have_next) named_barrier(kBarConsumers, kCT);   // warp records are free for the next segment
         s = s_next;
         have = have_next;
 #pragma unroll

@@ -561,3 +561,86 @@ def test_split_items_merge(B, Hq, Hkv, D, L):
     k_new, v_new = _new_rows(inp, B, 1700 + Hq)
     for _ in range(2):   # (the exchange slots are as they were)
         _check(*_run(H.ctx(), inp, k_new, v_new), BF, 3e-3)
+
+
+def _guesses(final, room):
+    """Lengths that a kernel in front of the token replaces: none, all that fit, the final ones in another order, lengths that take
+    part in no call, a mixture."""
+    B = len(final)
+    return [[0] * B, [room] * B, final[::-1], [(-3, 1 << 30)[b % 2] for b in range(B)], [room if b % 3 else 0 for b in range(B)], final]
+
+
+def _token_over(kind, c, inp, k_new, v_new):
+    """A token over a cache of `kind`: (call on a lengths tensor and an output, device pools, oracle's lengths and rows)."""
+    d, kd, vd = inp.to("cuda"), k_new.cuda(), v_new.cuda()
+    if kind == "bf16":
+        ok, ov, osl, _ = oracle.kv_append(k_new, v_new, inp.block_table, inp.seq_lens, inp.q_lens, inp.k_pages, inp.v_pages)
+        ref, _ = oracle.attn(inp.q, ok, ov, inp.block_table, osl, inp.q_lens)
+        return (lambda ln, out: c.decode_step(d.q, kd, vd, d.k_pages, d.v_pages, d.block_table, ln, d.q_lens, out=out)), d, osl, ref
+    if kind == "e4m3":
+        kc, vc = (torch.from_numpy(oracle.e4m3_encode(p, 1 / s)) for p, s in ((inp.k_pages, KS), (inp.v_pages, VS)))
+        ok, ov, osl, _ = oracle.kv_append_e4m3(k_new, v_new, inp.block_table, inp.seq_lens, inp.q_lens, kc, vc, 1 / KS, 1 / VS)
+        ref, _ = oracle.attn_e4m3(inp.q, ok, ov, KS, VS, inp.block_table, osl, inp.q_lens)
+        pools = kc.cuda(), vc.cuda()
+        return (lambda ln, out: c.decode_step_e4m3(d.q, kd, vd, *pools, KS, VS, 1 / KS, 1 / VS, d.block_table, ln, d.q_lens,
+                                                   out=out)), d, osl, ref
+    kc, ks = map(torch.from_numpy, oracle.i4_encode(inp.k_pages))
+    vc, vs = map(torch.from_numpy, oracle.i4_encode(inp.v_pages))
+    ok, ov, oks, ovs, osl, _ = oracle.kv_append_i4(k_new, v_new, inp.block_table, inp.seq_lens, inp.q_lens, kc, vc, ks, vs)
+    ref, _ = oracle.attn_i4(inp.q, ok, ov, oks, ovs, inp.block_table, osl, inp.q_lens)
+    pools = kc.cuda(), vc.cuda(), ks.cuda(), vs.cuda()
+    return (lambda ln, out: c.decode_step_i4(d.q, kd, vd, *pools, d.block_table, ln, d.q_lens, out=out)), d, osl, ref
+
+
+@pytest.mark.parametrize("B", [1, 6, 32, 40])
+@pytest.mark.parametrize("kind", ["bf16", "e4m3", "i4"])
+def test_lengths_move_in_front_of_a_token(kind, B):
+    """A kernel that lets the token come up writes the lengths (arb_phase_lens): whatever stood there before, the token is the one
+    of the final lengths."""
+    c = H.ctx()
+    sl = [(37 * b * b + 700 * b + 45) % 1900 for b in range(B)]
+    inp = wl.small_attn_case(B, 6, 2, 128, BF, sl, [1] * B, seed=331 + B, extra_tokens=40)
+    k_new, v_new = _new_rows(inp, B, 3300 + B)
+    call, d, osl, ref = _token_over(kind, c, inp, k_new, v_new)
+    guesses = _guesses(sl, inp.block_table.shape[1] * 16 - 1)
+    final = torch.tensor(sl, dtype=torch.int32, device="cuda")
+    lens = [torch.tensor(g, dtype=torch.int32, device="cuda") for g in guesses]
+    outs = [torch.full_like(d.q, float("nan")) for _ in guesses]
+    torch.cuda.synchronize()
+    for ln, out in zip(lens, outs):
+        c.phase_lens(final, out=ln)
+        call(ln, out)
+    assert c.poll_status() == 0
+    for ln, out in zip(lens, outs):
+        assert np.array_equal(ln.cpu().numpy(), osl)
+        assert _same_bits(out, outs[0])
+    H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
+
+
+@pytest.mark.parametrize("B", [3, 40])
+@pytest.mark.parametrize("kind", ["bf16", "e4m3"])
+def test_lengths_move_in_front_of_decode_rows(kind, B):
+    """The same in front of a decode call that writes no cache."""
+    c = H.ctx()
+    sl = [(37 * b * b + 700 * b) % 1900 + 1 for b in range(B)]
+    inp = wl.small_attn_case(B, 6, 2, 128, BF, sl, [1] * B, seed=371 + B)
+    d = inp.to("cuda")
+    if kind == "bf16":
+        ref, _ = oracle.attn(inp.q, inp.k_pages, inp.v_pages, inp.block_table, inp.seq_lens, inp.q_lens)
+        call = lambda ln, out: c.attn(d.q, d.k_pages, d.v_pages, d.block_table, ln, d.q_lens, 1, out=out)
+    else:
+        kc, vc = (torch.from_numpy(oracle.e4m3_encode(p, 1 / s)) for p, s in ((inp.k_pages, KS), (inp.v_pages, VS)))
+        ref, _ = oracle.attn_e4m3(inp.q, kc, vc, KS, VS, inp.block_table, inp.seq_lens, inp.q_lens)
+        dk, dv = kc.cuda(), vc.cuda()
+        call = lambda ln, out: c.attn_decode_e4m3(d.q, dk, dv, KS, VS, d.block_table, ln, d.q_lens, out=out)
+    final = torch.tensor(sl, dtype=torch.int32, device="cuda")
+    lens = [torch.tensor(g, dtype=torch.int32, device="cuda") for g in _guesses(sl, inp.block_table.shape[1] * 16)]
+    outs = [torch.full_like(d.q, float("nan")) for _ in lens]
+    torch.cuda.synchronize()
+    for ln, out in zip(lens, outs):
+        c.phase_lens(final, out=ln)
+        call(ln, out)
+    assert c.poll_status() == 0
+    for out in outs:
+        assert _same_bits(out, outs[0])
+    H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
