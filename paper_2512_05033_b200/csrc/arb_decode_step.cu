@@ -72,7 +72,7 @@ constexpr int kVerifyWarp = kCW - 1;          // the consumer warp that compares
 constexpr int kNT = 32 * (kCW + 3);
 // Named barriers: the consumers', and behind the comparison of the guess one for each kind of warp, so that none waits for
 // another's copies or prefetches (the consumers behind the producers' first copies: 4-bit tokens 10.8 -> 12.0 us).
-enum { kBarConsumers = 1, kBarConsumersTold = 3, kBarProducersTold = 4, kBarAuxTold = 5 };
+enum { kBarConsumers = 1, kBarPages = 2, kBarConsumersTold = 3, kBarProducersTold = 4, kBarAuxTold = 5 };
 
 // The exchange of a split item's parts.  A slot is what one CTA hands on: the group's outputs and (max, sum) per head, every
 // 32-bit word of it kEmpty until it is stored, and kEmpty again once it has been read.  A NaN of a result never has these bits
@@ -142,6 +142,7 @@ template <int STAGES>
 struct Tail {
     uint64_t full[STAGES];
     uint64_t empty[STAGES];
+    int pages[32];        // guessed page numbers of the CTA's first look-ups
     int differs;          // the comparing warp's finding: the guess does not hold
     int abort;
     int ticket;
@@ -596,11 +597,20 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         make_plan();
         const int nflat = ends[1] - ends[0];
         const int32_t *entry = a.block_table;
-        if (warp >= kVerifyWarp && lane < nflat) {
-            int kvh;
-            find_page(ends[0] + lane, entry, kvh);
-            page_next = load_now(entry);
-            row_next = ((unsigned)page_next < (unsigned)a.num_pages ? page_next * Hkv + kvh : 0) * kPage;
+        if (warp >= kVerifyWarp) {
+            const bool there = lane < nflat;
+            int kvh = 0;
+            if (there) find_page(ends[0] + lane, entry, kvh);
+            if (there && (!guess || warp == kVerifyWarp)) page_next = load_now(entry);
+            // A guess is read once, by the warp that compares it, and handed on: what is compared is what is used.
+            if (guess && warp == kVerifyWarp) {
+                tail->pages[lane] = page_next;
+                barrier_arrive(kBarPages, 128);
+            } else if (guess) {
+                named_barrier(kBarPages, 128);
+                page_next = tail->pages[lane];
+            }
+            if (there) row_next = ((unsigned)page_next < (unsigned)a.num_pages ? page_next * Hkv + kvh : 0) * kPage;
         }
         if (guess) {
             if (warp == kAuxWarp && lane < min(nflat, kAheadPages)) {

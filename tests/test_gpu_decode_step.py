@@ -644,3 +644,37 @@ def test_lengths_move_in_front_of_decode_rows(kind, B):
     for out in outs:
         assert _same_bits(out, outs[0])
     H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
+
+
+@pytest.mark.parametrize("B", [1, 6, 40])
+@pytest.mark.parametrize("kind", ["bf16", "e4m3", "i4", "rows"])
+def test_block_table_is_rewritten_in_front_of_a_token(kind, B):
+    """The kernel in front writes every entry of the table (arb_phase_lens writes 32-bit words): pages of other sequences, and
+    numbers outside the pool, that stood there before are not attended, not reported and not written."""
+    c = H.ctx()
+    sl = [(37 * b * b + 700 * b + 45) % 1900 for b in range(B)]
+    inp = wl.small_attn_case(B, 6, 2, 128, BF, sl, [1] * B, seed=431 + B, extra_tokens=2)
+    final = inp.block_table.clamp(min=0).cuda()   # (entries behind a sequence's pages are never looked up)
+    if kind == "rows":
+        d = inp.to("cuda")
+        ref, _ = oracle.attn(inp.q, inp.k_pages, inp.v_pages, inp.block_table, inp.seq_lens, inp.q_lens)
+        call = lambda ln, out: c.attn(d.q, d.k_pages, d.v_pages, d.block_table, ln, d.q_lens, 1, out=out)
+        osl = np.array(sl, dtype=np.int32)
+    else:
+        k_new, v_new = _new_rows(inp, B, 4300 + B)
+        call, d, osl, ref = _token_over(kind, c, inp, k_new, v_new)
+    g = torch.Generator().manual_seed(B)
+    befores = [torch.randint(0, inp.k_pages.shape[0], final.shape, generator=g, dtype=torch.int32).cuda(),
+               torch.full_like(final, -7), torch.full_like(final, 1 << 30), final.flip(0).contiguous(), final]
+    lens = [torch.tensor(sl, dtype=torch.int32, device="cuda") for _ in befores]
+    outs = [torch.full_like(d.q, float("nan")) for _ in befores]
+    torch.cuda.synchronize()
+    for before, ln, out in zip(befores, lens, outs):
+        d.block_table.copy_(before)
+        c.phase_lens(final.view(-1), out=d.block_table.view(-1))
+        call(ln, out)
+    assert c.poll_status() == 0
+    for ln, out in zip(lens, outs):
+        assert np.array_equal(ln.cpu().numpy(), osl)
+        assert _same_bits(out, outs[0])
+    H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
