@@ -407,7 +407,9 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     }
     if (!a.guess) {
         wait_for_predecessor();
-        if (a.beside) let_successor_start();   // it does not wait for this kernel, but it may read what the predecessor wrote
+        // (beside: it does not wait for this kernel, but it may read what the predecessor wrote.  One thread's call counts for the
+        // CTA, so it is the one that has drawn the ticket: the kernel behind the next draws from the same counter.)
+        if (a.beside && tid == kAuxWarp * 32) let_successor_start();
     }
     for (int b = tid; b < B; b += kNT) {
         raw_n[b] = load_now(a.q_lens + b);

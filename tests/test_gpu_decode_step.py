@@ -678,3 +678,27 @@ def test_block_table_is_rewritten_in_front_of_a_token(kind, B):
         assert np.array_equal(ln.cpu().numpy(), osl)
         assert _same_bits(out, outs[0])
     H.assert_close(outs[0].double().cpu().numpy(), ref, BF, tight=3e-3)
+
+
+def test_tokens_between_calls_whose_rows_run_beside_chunks():
+    """Decode rows beside chunks, a token, and so on with nothing in between: the kernels number their CTAs by one counter."""
+    c = H.ctx()
+    mixed = wl.small_attn_case(4, 12, 2, 128, BF, [900, 40, 5000, 300], [1, 3, 1, 9], seed=521)
+    ref, _ = oracle.attn(mixed.q, mixed.k_pages, mixed.v_pages, mixed.block_table, mixed.seq_lens, mixed.q_lens)
+    inp = wl.small_attn_case(3, 12, 2, 128, BF, [700, 3100, 15], [1] * 3, seed=522, extra_tokens=2)
+    k_new, v_new = _new_rows(inp, 3, 5200)
+    call, d, osl, token_ref = _token_over("bf16", c, inp, k_new, v_new)
+    m = mixed.to("cuda")
+    lens = [torch.tensor(inp.seq_lens.tolist(), dtype=torch.int32, device="cuda") for _ in range(6)]
+    rows = [torch.full_like(m.q, float("nan")) for _ in lens]
+    tokens = [torch.full_like(d.q, float("nan")) for _ in lens]
+    torch.cuda.synchronize()
+    for ln, r, t in zip(lens, rows, tokens):
+        c.attn(m.q, m.k_pages, m.v_pages, m.block_table, m.seq_lens, m.q_lens, 9, out=r)
+        call(ln, t)
+    assert c.poll_status() == 0
+    for ln, r, t in zip(lens, rows, tokens):
+        assert np.array_equal(ln.cpu().numpy(), osl)
+        assert _same_bits(r, rows[0]) and _same_bits(t, tokens[0])
+    H.assert_close(rows[0].double().cpu().numpy(), ref, BF, tight=3e-3)
+    H.assert_close(tokens[0].double().cpu().numpy(), token_ref, BF, tight=3e-3)
