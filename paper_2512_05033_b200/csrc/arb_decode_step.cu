@@ -612,7 +612,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                 named_barrier(kBarPages, 128);
                 page_next = tail->pages[lane];
             }
-            if (there) row_next = ((unsigned)page_next < (unsigned)a.num_pages ? page_next * Hkv + kvh : 0) * kPage;
+            if (there) row_next = (((unsigned)page_next < (unsigned)a.num_pages ? page_next : 0) * Hkv + kvh) * kPage;
         }
         if (guess) {
             if (warp == kAuxWarp && lane < min(nflat, kAheadPages)) {

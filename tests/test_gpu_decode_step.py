@@ -702,3 +702,17 @@ def test_tokens_between_calls_whose_rows_run_beside_chunks():
         assert _same_bits(r, rows[0]) and _same_bits(t, tokens[0])
     H.assert_close(rows[0].double().cpu().numpy(), ref, BF, tight=3e-3)
     H.assert_close(tokens[0].double().cpu().numpy(), token_ref, BF, tight=3e-3)
+
+
+@pytest.mark.parametrize("sl", [[300, 2000], [60000, 2000]])   # the page is among a CTA's first look-ups, or behind them
+def test_page_outside_the_pool_reads_as_page_0(sl):
+    from paper_2512_05033_b200 import binding
+    c = H.ctx()
+    inp = wl.small_attn_case(2, 12, 2, 128, BF, sl, [1, 1], seed=611)
+    outs = []
+    for entry, bits in ((0, 0), (-1, binding.DEV_BAD_PAGE), (inp.k_pages.shape[0], binding.DEV_BAD_PAGE)):
+        d = inp.to("cuda")
+        d.block_table[0, ::3] = entry
+        outs.append(c.attn(d.q, d.k_pages, d.v_pages, d.block_table, d.seq_lens, d.q_lens, 1))
+        assert c.poll_status() == bits
+    assert _same_bits(outs[0], outs[1]) and _same_bits(outs[0], outs[2])
