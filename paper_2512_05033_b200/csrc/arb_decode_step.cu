@@ -49,6 +49,8 @@
 // the scales' copies, 118 without the products); the draft shape 16.5 -> 14.4 us, either cache.
 #include "arb_decode_tc.cuh"
 
+#include <type_traits>
+
 namespace arb {
 
 namespace {
@@ -804,11 +806,14 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     constexpr int kLph = kD / 4;               // lanes of a head: one per 4-dimension piece
     constexpr int VECS = G * kLph;             // 4-dimension pieces of the group's outputs, one per consumer thread
     constexpr int kMergeBatch = 16;            // parts merged per round of loads, straight into registers (24: they spill, + 0.5 us)
-    constexpr int kMergeFan = 2 * kMergeBatch; // of so many parts the last hands on the sum: no CTA reads many slots
+    // Of an item of more parts than two rounds bring, the last of every kMergeFan parts hands on the sum: a round for a run, one for
+    // the sums and the rest.  Runs of 32 took two and one: 4 items of 37 parts 11.8 -> 10.8 us, 2 of 74 11.8 -> 10.9 us.
+    constexpr int kLongBatch = 20, kMergeFan = kMergeBatch + 1, kDirectParts = 2 * kMergeBatch + 1;
     static_assert(VECS <= kCT, "one piece per consumer thread");
     static_assert(kMergeBatch <= kLph, "a lane of a head per part");
     int gather_first = -1, gather_part = 0;    // the item to merge: the CTA of its first part, the number of this CTA's part
-    bool gather_last = false;                  // ... and whether that completes the item (else the sum of kMergeFan parts goes on)
+    bool gather_last = false;                  // ... and whether that completes the item (else the sum of a run goes on)
+    bool in_runs = false;                      // ... of kMergeFan parts
     size_t gather_out = 0;
     float4 own = make_float4(0.f, 0.f, 0.f, 0.f);   // this CTA's part of it
     float own_m = -INFINITY, own_l = 0.f;
@@ -1154,7 +1159,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         const size_t out_base = ((size_t)qrow * a.Hq + s.kvh * G) * kD;
         const int part = cta - s.c_first;   // (of s.nparts)
         const bool last = part == s.nparts - 1 && !pl.mergers;   // of the item, and merged here
-        const bool gathers = s.nparts > 1 && (last || part % kMergeFan == kMergeFan - 1);
+        const bool gathers = s.nparts > 1 && (last || (s.nparts > kDirectParts && part % kMergeFan == kMergeFan - 1));
         if (tid < VECS) {
             float M = -INFINITY, mw[kCW];
 #pragma unroll
@@ -1182,6 +1187,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         if (gathers) {
             gather_first = s.c_first;
             gather_part = part;
+            in_runs = s.nparts > kDirectParts;
             gather_last = last;
             gather_out = out_base;
         }
@@ -1201,6 +1207,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         if (s.nparts > 1) {
             gather_first = s.c_first;
             gather_part = s.nparts;
+            in_runs = s.nparts > kDirectParts;
             gather_last = true;
             gather_out = ((size_t)row0[b] * a.Hq + s.kvh * G) * kD;
         }
@@ -1209,21 +1216,22 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
 
     // ---- the merge of a split (sequence, kv head) ---------------------------------------------------------
     //     m = max_p m_p,  w_p = 2^(m_p - m),  out = sum_p w_p o_p / sum_p w_p l_p,
-    // one 4-dimension piece of the group's outputs per thread.  Read are the parts of this CTA's own run of kMergeFan, as they
+    // one 4-dimension piece of the group's outputs per thread.  Read are the parts of this CTA's own run, as they
     // are, and of every run before it the slot of its last part, which holds the run's sum; kMergeBatch of them at a time, in a
     // fixed order whenever they come.  Lane p of a head's lanes has the (max, sum) of part p of a batch.
-    const int run0 = gather_part / kMergeFan * kMergeFan;        // first part of the own run
-    const int runs = gather_last ? gather_part / kMergeFan : 0;  // sums to read besides
+    const int run0 = in_runs ? gather_part / kMergeFan * kMergeFan : 0;        // first part of the own run
+    const int runs = in_runs && gather_last ? gather_part / kMergeFan : 0;     // sums to read besides
     const int n = runs + gather_part - run0;
     const bool mine = tid < VECS;
     const int piece = mine ? tid : 0;
-    for (int p0 = 0; p0 < n; p0 += kMergeBatch) {
-        const int np = min(kMergeBatch, n - p0);
+    auto merge = [&](int p0, auto batch) {
+        constexpr int kBatch = decltype(batch)::value;
+        const int np = min(kBatch, n - p0);
         auto slot_of = [&](int i) -> int {   // of the i-th part to read; always an earlier CTA's
             const int at = gather_first + (i < runs ? i * kMergeFan + kMergeFan - 1 : run0 + i - runs);
             return 2 * (ARB_IN_RANGE(a.status, at, cta) ? at : 0) + (at == gather_first);
         };
-        float4 v[kMergeBatch];
+        float4 v[kBatch];
         float2 ml = make_float2(-INFINITY, 0.f);
         const bool has_ml = mine && lane % kLph < np;
         float2 *ml_at = reinterpret_cast<float2 *>(a.part_ml) + (size_t)slot_of(has_ml ? p0 + lane % kLph : p0) * kMaxGroup + piece / kLph;
@@ -1232,16 +1240,16 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         bool ml_missing = has_ml;
         long long t0 = 0;
 #pragma unroll
-        for (int p = 0; p < kMergeBatch; ++p) v[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p = 0; p < kBatch; ++p) v[p] = make_float4(0.f, 0.f, 0.f, 0.f);
         while (true) {
             const unsigned before = missing;
             if (ml_missing) ml = load_slot2(ml_at);
 #pragma unroll
-            for (int p = 0; p < kMergeBatch; ++p)
+            for (int p = 0; p < kBatch; ++p)
                 if (missing >> p & 1u) v[p] = load_slot4(o_at + (size_t)slot_of(p0 + p) * VECS);
             ml_missing = ml_missing && (is_empty(ml.x) || is_empty(ml.y));
 #pragma unroll
-            for (int p = 0; p < kMergeBatch; ++p)
+            for (int p = 0; p < kBatch; ++p)
                 if ((missing >> p & 1u) && !any_empty(v[p])) missing &= ~(1u << p);
             if (!__any_sync(0xffffffffu, ml_missing || missing != 0u)) break;
             if (__all_sync(0xffffffffu, missing == before)) __nanosleep(merges_only ? 200 : 100);
@@ -1259,7 +1267,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         const float e = __uint_as_float(kEmpty);
         if (has_ml) store_slot2(ml_at, make_float2(e, e));
 #pragma unroll
-        for (int p = 0; p < kMergeBatch; ++p)
+        for (int p = 0; p < kBatch; ++p)
             if (mine && p < np) store_slot4(o_at + (size_t)slot_of(p0 + p) * VECS, make_float4(e, e, e, e));
         float mb = fmaxf(own_m, ml.x);
 #pragma unroll
@@ -1272,11 +1280,15 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         own_l = fmaf(own_l, f, l);
         own.x *= f; own.y *= f; own.z *= f; own.w *= f;
 #pragma unroll
-        for (int p = 0; p < kMergeBatch; ++p) {
+        for (int p = 0; p < kBatch; ++p) {
             const float wp = __shfl_sync(0xffffffffu, w, (lane / kLph) * kLph + p);   // 0 where the batch has no part p
             own.x = fmaf(wp, v[p].x, own.x); own.y = fmaf(wp, v[p].y, own.y); own.z = fmaf(wp, v[p].z, own.z); own.w = fmaf(wp, v[p].w, own.w);
         }
-    }
+    };
+    // 148 CTAs over 8 items are 18 and a half parts each: a round of twenty instead of two of sixteen
+    if (kLongBatch <= kLph && n > kMergeBatch && n <= kLongBatch) merge(0, std::integral_constant<int, kLongBatch <= kLph ? kLongBatch : kMergeBatch>());
+    else
+        for (int p0 = 0; p0 < n; p0 += kMergeBatch) merge(p0, std::integral_constant<int, kMergeBatch>());
     if (!mine) return;
     if (gather_last) write_row(gather_out, own, 1.0f / own_l);
     else publish(own, own_m, own_l, gather_part);

@@ -554,7 +554,9 @@ def test_token_right_behind_a_kernel_that_moves_the_lengths(B, Hq, Hkv, D):
 
 @pytest.mark.parametrize("B,Hq,Hkv,D,L", [(37, 4, 1, 128, 900), (38, 4, 1, 128, 900),   # the most items with a merger each, one more
                                           (1, 2, 1, 128, 33 * 16 * 16), (1, 7, 1, 64, 40000),   # runs of parts: 33 parts, 147
-                                          (2, 16, 2, 128, 20000), (4, 6, 1, 64, 8000)])
+                                          (2, 16, 2, 128, 20000), (4, 6, 1, 64, 8000),
+                                          (8, 6, 1, 128, 5000), (7, 6, 1, 128, 4800),      # rounds of twenty: 19 parts; two rounds: 22
+                                          (1, 8, 1, 128, 33 * 256), (1, 8, 1, 128, 34 * 256), (1, 3, 1, 64, 52 * 256)])   # 33 parts: no runs; 34 and 52: runs of 17
 def test_split_items_merge(B, Hq, Hkv, D, L):
     sl = [L - 17 * b for b in range(B)]
     inp = wl.small_attn_case(B, Hq, Hkv, D, BF, sl, [1] * B, seed=17 + B, extra_tokens=4)
