@@ -86,7 +86,10 @@ constexpr uint32_t kEmpty = 0xffffffffu;
 // kernel's mergers, which have time: draft-shaped token (16 items) 11.0 -> 10.85 us, over E4M3 codes 10.0 -> 9.6 us.  Up to a
 // kMergerShare-th of the CTAs, and only where one of the others then streams at most kMergerPages more: that is a microsecond or
 // so, what a merger saves (with more, 32 items of 16 sequences of 2k to 8k over E4M3 codes 14 -> 15 us, 30 of 28k 69.5 -> 70.1 us).
-constexpr int kMergerShare = 4, kMergerPages = 5;
+// Nor where there is less than a CTA's smallest range for each of the others (they would leave CTAs without work anyway, and an item's
+// last part is sooner merged where it is: 36 items of 50 pages 8.8 -> 7.8 us without, 8 over 4-bit codes 7.8 -> 7.5 us), nor for items of more
+// than kMergerParts parts (2 and 4 items: 0.1 us).
+constexpr int kMergerShare = 4, kMergerPages = 5, kMergerParts = 32;
 // What a boundary costs is time (the warps meet, a second arrival, perhaps a second merge), a few microseconds
 // whatever the call's size: as pages it is the CTA's even share, but no more than this many.
 constexpr int kBoundaryCap = 32;
@@ -442,7 +445,9 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             const float mine = kBesideWeight * (float)total;
             ctas = min(ctas, max(4, __float2int_ru((float)ctas * __fdividef(mine, mine + chunks + 1.f))));
         }
-        pl.mergers = !a.beside && items * kMergerShare <= ctas && (long long)(ctas - items) * kMergerPages >= (long long)total / ctas * items;
+        const int others = ctas - items;
+        pl.mergers = !a.beside && items * kMergerShare <= ctas && items * kMergerParts >= ctas && total >= a.min_chunk * others &&
+                     (long long)others * kMergerPages >= (long long)total / ctas * items;
         if (pl.mergers) ctas -= items;
         pl.stream = ctas;
         const int even = max(a.min_chunk, per_cta(total));
@@ -627,7 +632,8 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         bool differs = false;
         int n_now = 0, len_now = 0;   // a batch of at most 32: what is final, of sequence `lane`
         if (guess && warp == kVerifyWarp) {
-            differs = lane < nflat && load_now(entry) != page_next;
+            int entry_now = page_next;
+            if (lane < nflat) entry_now = load_now(entry);
 #pragma unroll 4
             for (int b = lane; b < B; b += 32) {
                 n_now = load_now(a.q_lens + b);
@@ -639,7 +645,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
                     if (B > 32) { raw_n[b] = n_now; raw_len[b] = len_now; }
                 }
             }
-            differs = __any_sync(0xffffffffu, differs);
+            differs = __any_sync(0xffffffffu, differs || entry_now != page_next);
             if (lane == 0) tail->differs = differs;
             barrier_arrive(kBarProducersTold, 96);
             barrier_arrive(kBarAuxTold, 64);
