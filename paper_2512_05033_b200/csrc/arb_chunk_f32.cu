@@ -1,14 +1,16 @@
 // Step-chunk attention over an fp32 cache (whose 1e-5 tolerance rules out tf32), on the CUDA cores.
 //
 // A chunk of n query tokens against one KV head is rows = n * group query rows (token-major) over the same keys.  A CTA of
-// eight warps takes a tile of 64 rows and walks keys in tiles of 32 (two pages, double-buffered with cp.async): every key
-// that reaches shared memory is used by all 64 rows.  A warp owns 8 rows, so the online softmax needs no barrier.  Per key
-// tile and lane: S as 2 rows x 4 keys (32 FMA per 6 conflict-free 16-byte loads per 4 dimensions), P through
-// the warp's own corner of shared memory, O += P V as 8 rows x 4 dimensions (4 x 4 at head_dim 64).
+// eight warps takes a tile of 64, 32 or 16 rows (see launch_one) and walks keys in tiles of 32 (two pages, double-buffered with
+// cp.async): every key that reaches shared memory is used by all rows of the tile.  A warp owns an eighth of the rows, so the online
+// softmax needs no barrier.  Per key tile and lane, of 64 rows: S as 2 rows x 4 keys (32 FMA per 6 conflict-free 16-byte loads per
+// 4 dimensions), of 32 as 1 x 4, of 16 as 1 x 2; P through the warp's own corner of shared memory; O += P V as 8, 4 or 2 rows x 4
+// dimensions (half the rows at head_dim 64).
 // What bounds it is shared-memory loads and FMA issue on large calls, latency on small ones, so the flat list of (sequence, kv head, row tile,
 // key tile) units is cut evenly over two CTAs per SM; a row tile that is cut leaves partials, and the CTA that arrives last
 // at the tile's counter merges them.  A CTA per (query row, kv head), which this replaces, re-read the keys for every
-// row and ran 528 keys as one chain: a 16-token step over 528 keys (8 / 2 heads of 64) 41.6 -> 17.3 us, two steps of 56 and
+// row and ran 528 keys as one chain: a 16-token step over 528 keys (8 / 2 heads of 64) 41.6 -> 17.3 us (in row tiles of 16 and with
+// the loads of a merge in flight together 13.1 us), two steps of 56 and
 // 104 tokens over 1.3k and 1.8k keys (8 / 2 heads of 128) 291 -> 61 us (a quarter of the FMA rate: the shared-memory
 // loads of the first product are the bound there).
 #include "arb_common.cuh"
@@ -406,7 +408,17 @@ arb_status launch_rows(Ctx *ctx, F32Args a, cudaStream_t stream) {
 
 // Rows of a tile: 64, or 32 or 16 where the call is so small that the CTAs cannot all have work with more.  Smaller tiles read
 // the keys more often and take less time each, and so does the merge of their parts.  The host knows the rows and the most keys
-// that the table can hold.  F32FIGURES
+// that the table can hold, not the lengths: a short sequence under a wide table keeps 64 rows.  us per call with tiles of
+// 16 / 32 / 64 rows, one sequence, 8 / 2 heads of 64 (of 128), the table as long as the sequence, by `most`:
+//   16 tokens over  528 keys,  68:  13.2 / 15.9 / 17.6  (18.0 / 23.6 / 25.5)
+//   16 tokens over 1100 keys, 140:  12.8 / 17.6 / 21.2  (17.5 / 25.2 / 36.7)
+//   64 tokens over  528 keys, 170:  13.4 / 15.7 / 18.7  (18.6 / 23.7 / 31.9)
+//   16 tokens over 2300 keys, 288:  14.4 / 18.1 / 23.7  (19.5 / 28.1 / 44.4)
+//   64 tokens over 1100 keys, 350:  18.7 / 18.3 / 21.7  (26.5 / 27.6 / 41.0)
+//   64 tokens over 4600 keys, 1440: 55.2 / 42.0 / 37.2  (81.1 / 70.0 / 77.5)
+// and two sequences of 64 tokens over 300 keys, 200: 18.1 / 16.5 / 20.5 (24.4 / 24.5 / 32.4).  At the first line (room / 4 = 148) 16 rows
+// win by a quarter, at the second (296) 32 do against 64.  Both lie low: they were drawn where a CTA's share falls below kMinUnits,
+// and tiles of the next smaller height still win somewhat above them, the less the more row tiles the call has.
 template <int D, int G>
 arb_status launch_one(Ctx *ctx, const F32Args &a, cudaStream_t stream) {
     const long long most = (long long)a.Hkv * ((long long)a.rows * G / 64 + a.batch) * ((a.max_pages * (long long)kPage + kKeys - 1) / kKeys);

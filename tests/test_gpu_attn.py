@@ -694,14 +694,28 @@ def test_fp32_chunk_matches_oracle(case, ws):
     H.assert_close(out, ref, F32)
 
 
+FP32_SMALL_CASES = [
+    # rows of a tile, (Hq, Hkv, D, seq_lens, q_lens)
+    (16, (8, 2, 128, [530, 17], [4, 17])),          # one full tile, five with one of 4 rows
+    (16, (7, 1, 64, [300, 64, 2], [5, 3, 2])),      # g = 7: 35, 21 and 14 rows
+    (16, (3, 1, 128, [2500], [11])),                # 33 rows, 4 keys of the last key tile
+    (16, (16, 2, 64, [1200], [6])),                 # 48 rows, long merges
+    (32, (3, 1, 128, [6000], [11])),                # 33 rows: a full tile and one row
+    (32, (16, 2, 64, [3000], [6])),                 # 48 rows: a full tile and half a one
+    (32, (7, 1, 64, [5000], [9])),                  # 63 rows
+    (32, (8, 1, 128, [2200, 40], [7, 2])),          # 56 and 16 rows
+]
+
+
 @pytest.mark.parametrize("ws", [0, 1_300_000])
-@pytest.mark.parametrize("case", [
-    (8, 2, 128, [530, 17], [4, 17]),          # row tiles of 16 (a row of the table holds 36 pages): one full, five with one of 4 rows
-    (7, 1, 64, [300, 64, 2], [5, 3, 2]),      # ... of 16, g = 7: 35, 21 and 14 rows
-    (3, 1, 128, [2500], [11]),                # ... of 32 and 16 keys of the last key tile: 33 rows
-    (16, 2, 64, [1200], [6]),                 # ... of 32: 48 rows, long merges
-])
-def test_fp32_chunks_of_small_calls_match_oracle(case, ws):
+@pytest.mark.parametrize("tile,case", FP32_SMALL_CASES)
+def test_fp32_chunks_of_small_calls_match_oracle(tile, case, ws):
+    Hq, Hkv, D, sl, ql = case
+    # the rule of arb_chunk_f32.cu, on the table that the inputs have (room for 20 tokens more than the longest sequence)
+    keys = (max(sl) + 20 + wl.PAGE - 1) // wl.PAGE * wl.PAGE
+    most = Hkv * (sum(ql) * (Hq // Hkv) // 64 + len(sl)) * ((keys + 31) // 32)
+    room = 2 * 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert tile == (16 if 4 * most <= room else 32 if 2 * most <= room else 64)
     test_fp32_chunk_matches_oracle(case, ws)
 
 
