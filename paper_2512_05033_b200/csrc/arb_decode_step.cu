@@ -143,12 +143,16 @@ struct StepArgs {
     float *k_scales, *v_scales;       // 4-bit cache: the scale pools [num_pages, Hkv, 16]
 };
 
+constexpr int kQPitch = kD * 2 + 16;   // of q in shared memory: neighbouring heads start 4 banks apart
+
 template <int STAGES>
 struct Tail {
     uint64_t full[STAGES];
     uint64_t empty[STAGES];
+    alignas(16) char q[kMaxGroup * kQPitch];   // the group's heads of q, of the first segment of a guess
     int pages[32];        // guessed page numbers of the CTA's first look-ups
     int differs;          // the comparing warp's finding: the guess does not hold
+    int ended;            // the predecessor is known to have ended
     int abort;
     int ticket;
 };
@@ -189,6 +193,18 @@ __device__ __forceinline__ int load_now(const int32_t *p) {   // from L2, whoeve
     asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void raise_flag(int *flag) {   // in shared memory; what happened before is seen by who sees it raised
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(flag)), "r"(1) : "memory");
+}
+__device__ __forceinline__ bool flag_raised(const int *flag) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(flag)) : "memory");
+    return v != 0;
+}
+__device__ __forceinline__ void cp_async16(void *dst_smem, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ bool is_empty(float x) { return __float_as_uint(x) == kEmpty; }
 __device__ __forceinline__ bool any_empty(float4 v) { return is_empty(v.x) || is_empty(v.y) || is_empty(v.z) || is_empty(v.w); }
 // a word fit for a slot: a NaN with kEmpty's bits becomes another NaN
@@ -404,6 +420,7 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
         }
         if (lane == 0) {
             tail->abort = 0;
+            tail->ended = 0;
             pref[0] = 0;
             row0[0] = 0;
             act[0] = 0;
@@ -572,6 +589,23 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     // B fragments of q^T (kD dims x 8 heads): k-slice ks holds dims 16 ks + 2 tq, + 1 and + 8 of head gq.  The
     // fragments of the next segment are asked for while this one streams.
     uint32_t qb[kD / 16][2], qn[kD / 16][2];
+    auto q_of = [&](const Segment &g, int head) -> const char * {   // of the group's heads
+        const int row = row0[g.b];   // (guessed lengths may point anywhere)
+        return a.q + ((size_t)((unsigned)row < (unsigned)a.rows ? row : 0) * a.Hq + g.kvh * G + head) * kD * 2;
+    };
+    auto q_fragments = [&](const char *qh, uint32_t (&dst)[kD / 16][2]) {   // this lane's head in memory of either kind
+#pragma unroll
+        for (int ks = 0; ks < kD / 16; ++ks) {
+            if constexpr (CODES) {   // dimensions 32 tq + 4 ks .. + 3, in the order the codes come in
+                const uint2 w = head_ok ? *reinterpret_cast<const uint2 *>(qh + tq * 64 + ks * 8) : make_uint2(0u, 0u);
+                dst[ks][0] = E4M3 ? bf16x2_to_f16x2(w.x) : w.x;   // (the operands of one MMA share a type)
+                dst[ks][1] = E4M3 ? bf16x2_to_f16x2(w.y) : w.y;
+                continue;
+            }
+            dst[ks][0] = head_ok ? *reinterpret_cast<const uint32_t *>(qh + ks * 32 + tq * 4) : 0u;
+            dst[ks][1] = head_ok ? *reinterpret_cast<const uint32_t *>(qh + ks * 32 + 16 + tq * 4) : 0u;
+        }
+    };
     auto load_q = [&](const Segment &g, uint32_t (&dst)[kD / 16][2]) {
         const int row = row0[g.b];   // (guessed lengths may point anywhere)
         const char *qh = a.q + ((size_t)((unsigned)row < (unsigned)a.rows ? row : 0) * a.Hq + g.kvh * G + (head_ok ? gq : 0)) * kD * 2;
@@ -597,32 +631,52 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
     // and only tiles and q rows were read, in bounds whatever the guess: every warp plans from the same guessed lengths, which
     // are replaced once the block has met.  Where something differs (lengths that the kernel right
     // in front moves, as a rollback does) the copies are waited for, the barriers made new, and the second round plans from
-    // what is final.  Without a cache write the copies wait for the comparison: what precedes such a call is often the append that
-    // moved the lengths.  Three dependent round trips (lengths, table, tile) and the plan become one behind the predecessor's end:
+    // what is final.  Three dependent round trips (lengths, table, tile) and the plan become one behind the predecessor's end:
     // tokens of one sequence of 256 / 2048 / 32768 tokens 7.3 / 8.1 / 15.7 -> 6.1 / 6.9 / 13.4 us, draft-shaped 12.4 -> 10.7 us
     // with the mergers.
+    // Without a cache write the copies wait for the comparison: what precedes such a call is often the append that
+    // moved the lengths.  Or it is a kernel that never lets its successor start early; then nothing was gained by guessing, and
+    // the comparison must not cost a round trip.  So where the predecessor has ended by the time of the look-ups, the lengths are
+    // compared beside them, and q is on its way into shared memory meanwhile: decode rows of 8 sequences of 2300 tokens, 2 kv heads,
+    // behind such a kernel 12.6 -> 11.9 us, behind one another 9.0 -> 8.5, behind an append 15.3 -> 15.6 us.  (With a cache write
+    // the first copies do not wait, and the same order made chains slower: 8.3 -> 8.5 us.)
 #pragma unroll 1
     for (bool guess = a.guess != 0;; guess = false) {
         make_plan();
         const int nflat = ends[1] - ends[0];
         const int32_t *entry = a.block_table;
+        // Without a cache write: has the predecessor ended by now?  (The consumers get to their wait a look-up earlier than the others.)
+        // Then what is read from here on is final, and nothing is left to ask into L2 ahead.
+        bool over = false;
+        int n_now = 0, len_now = 0;   // a batch of at most 32: what is final, of sequence `lane`
+        if constexpr (!APPEND) {
+            if (guess && warp < kVerifyWarp) {
+                wait_for_predecessor();
+                if (tid == 0) raise_flag(&tail->ended);
+            }
+        }
         if (warp >= kVerifyWarp) {
             const bool there = lane < nflat;
             int kvh = 0;
             if (there) find_page(ends[0] + lane, entry, kvh);
+            if constexpr (!APPEND)
+                if (guess && warp == kVerifyWarp) over = __all_sync(0xffffffffu, flag_raised(&tail->ended));
             if (there && (!guess || warp == kVerifyWarp)) page_next = load_now(entry);
             // A guess is read once, by the warp that compares it, and handed on: what is compared is what is used.
             if (guess && warp == kVerifyWarp) {
+                if constexpr (!APPEND)
+                    if (over && lane < B && B <= 32) { n_now = load_now(a.q_lens + lane); len_now = load_now(a.seq_lens + lane); }
                 tail->pages[lane] = page_next;
                 barrier_arrive(kBarPages, 128);
             } else if (guess) {
                 named_barrier(kBarPages, 128);
                 page_next = tail->pages[lane];
+                if constexpr (!APPEND) over = flag_raised(&tail->ended);
             }
             if (there) row_next = (((unsigned)page_next < (unsigned)a.num_pages ? page_next : 0) * Hkv + kvh) * kPage;
         }
         if (guess) {
-            if (warp == kAuxWarp && lane < min(nflat, kAheadPages)) {
+            if (warp == kAuxWarp && !over && lane < min(nflat, kAheadPages)) {
                 const size_t off = (size_t)row_next * kRowBytes;
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.k_pool + off), "r"(kPage * kRowBytes) : "memory");
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.v_pool + off), "r"(kPage * kRowBytes) : "memory");
@@ -630,22 +684,26 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             wait_for_predecessor();
         }
         bool differs = false;
-        int n_now = 0, len_now = 0;   // a batch of at most 32: what is final, of sequence `lane`
         if (guess && warp == kVerifyWarp) {
             int entry_now = page_next;
-            if (lane < nflat) entry_now = load_now(entry);
+            if (!over && lane < nflat) entry_now = load_now(entry);
+            if (!APPEND && over && B <= 32) {
+                differs = lane < B && (n_now != raw_n[lane] || len_now != raw_len[lane]);
+            } else {
 #pragma unroll 4
-            for (int b = lane; b < B; b += 32) {
-                n_now = load_now(a.q_lens + b);
-                len_now = load_now(a.seq_lens + b);
-                if (n_now != raw_n[b] || len_now != raw_len[b]) {
-                    differs = true;
-                    // What has moved goes where the next plan reads it.  Of a batch of more than 32 the plan above has read it in front
-                    // of barriers of the block; of a smaller one the other warps may not have read it yet.
-                    if (B > 32) { raw_n[b] = n_now; raw_len[b] = len_now; }
+                for (int b = lane; b < B; b += 32) {
+                    n_now = load_now(a.q_lens + b);
+                    len_now = load_now(a.seq_lens + b);
+                    if (n_now != raw_n[b] || len_now != raw_len[b]) {
+                        differs = true;
+                        // What has moved goes where the next plan reads it.  Of a batch of more than 32 the plan above has read it in
+                        // front of barriers of the block; of a smaller one the other warps may not have read it yet.
+                        if (B > 32) { raw_n[b] = n_now; raw_len[b] = len_now; }
+                    }
                 }
             }
-            differs = __any_sync(0xffffffffu, differs || entry_now != page_next);
+            differs = differs || entry_now != page_next;
+            differs = __any_sync(0xffffffffu, differs);
             if (lane == 0) tail->differs = differs;
             barrier_arrive(kBarProducersTold, 96);
             barrier_arrive(kBarAuxTold, 64);
@@ -659,13 +717,30 @@ decode_step_kernel(const StepArgs a, const __grid_constant__ CUtensorMap k_map, 
             return *(volatile int *)&tail->differs != 0;
         };
         const bool first_copy = (warp == kProdWarp || warp == kProdWarp + 1) && lane < min(nflat, kBatch);
-        const bool sure = !guess || (!APPEND && !wrong());
-        if (APPEND || sure) {
-            if (first_copy && ARB_IN_RANGE(a.status, row_next, (long long)a.num_pages * Hkv * kPage)) issue(2u * lane + (uint32_t)pw, row_next);
-            if (warp < kCW) {
+        if constexpr (!APPEND) {   // q comes into shared memory meanwhile: behind the first ring of tiles it takes a microsecond longer
+            if (guess && warp < kCW) {
                 cur = ends[0];
                 seq_at = seq0;
                 have = next_segment(cur, ends[1], seq_at, pl, s);
+                const char *from = q_of(s, 0);
+                for (int c = tid; have && c < G * kD / 8; c += kCT)
+                    cp_async16(tail->q + c / (kD / 8) * kQPitch + c % (kD / 8) * 16, from + c * 16);
+            }
+        }
+        const bool sure = !guess || (!APPEND && !wrong());
+        if (APPEND || sure) {
+            if (first_copy && ARB_IN_RANGE(a.status, row_next, (long long)a.num_pages * Hkv * kPage)) issue(2u * lane + (uint32_t)pw, row_next);
+            if (!APPEND && guess) {
+                if (warp < kCW) {
+                    cp_async_wait_all();
+                    named_barrier(kBarConsumers, kCT);
+                    q_fragments(tail->q + (head_ok ? gq : 0) * kQPitch, qb);
+                }
+            } else if (warp < kCW) {
+                cur = ends[0];
+                seq_at = seq0;
+                have = next_segment(cur, ends[1], seq_at, pl, s);
+                if constexpr (!APPEND) cp_async_wait_all();   // (a guess that was wrong has asked for q too)
                 if (have) load_q(s, qb);
             }
         }
