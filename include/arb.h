@@ -22,7 +22,7 @@
  *
  * Conventions shared by every call
  *   - Pointers are DEVICE pointers unless the argument says "host".  The caller owns every tensor;
- *     the library owns only the arb_ctx (split-KV partials, arrival counters, a status word and
+ *     the library owns only the arb_ctx (split-KV partials and exchange slots, arrival counters, a status word and
  *     staging buffers), allocated by arb_create / grown by the *_host calls, never by arb_attn,
  *     arb_route or arb_rollback.
  *   - Calls enqueue work on `stream` and return; they do not synchronise (arb_poll_status and the
@@ -532,7 +532,7 @@ arb_status arb_phase_lens_tokens(arb_ctx *ctx, int32_t batch, const int32_t *ste
 
 /*
  * Synchronise `stream`, read the device status word into *bits (nullable) and, if it is not zero, clear it together
- * with every arrival counter of the ctx.  Returns ARB_OK if the word was zero, else
+ * with every arrival counter and exchange slot of the ctx.  Returns ARB_OK if the word was zero, else
  * ARB_ERR_DEVICE_STATUS.
  */
 arb_status arb_poll_status(arb_ctx *ctx, arb_stream_t stream, uint32_t *bits);

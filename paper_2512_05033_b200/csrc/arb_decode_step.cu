@@ -23,7 +23,8 @@
 //     head) stores it into its slot of an exchange buffer whose words hold a value no result has, and leaves; a CTA that
 //     merges reads the slots until every word has come, writes the rows and puts the value back.  It waits only for CTAs
 //     that drew an earlier ticket, which have started, so every wait ends whatever else is running.  The merging CTA is one
-//     with nothing else to do (the last tickets, see kMergerShare), or the one that holds the item's last part.
+//     with nothing else to do (the last tickets, see kMergerShare), or the one that holds the item's last part; of an item of
+//     many parts the last CTA of a run of them hands on the run's sum.
 //   - With k_new / v_new given, the warp that owns a sequence's last page puts the token's new row into the
 //     tile in shared memory (the tile arrives with whatever the slot held) and stores it to the pool; the
 //     lengths move forward once every CTA has read them (a counter in the prologue tells the last reader).
@@ -46,7 +47,8 @@
 // memory and read back by ldmatrix, which this replaced, a page took a warp 1.4 us and the consumers set the pace of
 // every call: tokens of the target shape (16 sequences of 4k to 32k, 8 kv heads) E4M3 199 -> 108 us (6.0 TB/s, 0.93 of the
 // measured copy rate), 4-bit 192 -> 138 us (2.5 TB/s; the copies' issue and the page chain share the time: 132 us without
-// the scales' copies, 118 without the products); the draft shape 16.5 -> 14.4 us, either cache.
+// the scales' copies, 118 without the products); the draft shape 16.5 -> 14.4 us, either cache
+// (of the form of the call at the time; now 9.1 us over E4M3, 10.4 us over 4-bit codes).
 #include "arb_decode_tc.cuh"
 
 #include <type_traits>
@@ -307,7 +309,7 @@ __device__ __forceinline__ int small_div(int a, int b, int &rem) {
 
 // The cut of the flat (sequence, kv head, page) list into per-CTA ranges.  A CTA whose range crosses from one
 // (sequence, kv head) into the next pays for it (the warps meet, their records are merged, the next q is
-// loaded), and it then tends to be the last to arrive at both items and merges both.  So a boundary counts as
+// loaded), and both items wait for it.  So a boundary counts as
 // `pen` pages of work: the list is cut evenly in a padded coordinate in which every item is preceded by `pen`
 // virtual pages.  Item j (in list order) with real range [s, s + n) occupies [s + j pen, s + (j + 1) pen + n) there,
 // its real pages the last n of them.  Everything after the cut works in real coordinates.
